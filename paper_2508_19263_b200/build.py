@@ -1,6 +1,6 @@
 """Builds libzc.so (host logic + sm_100a kernels) in-tree with nvcc.
 
-Every source is compiled to an object file of its own (the decoder's to one per element format; in parallel, and
+Every source is compiled to an object file of its own (the encoder's and decoder's kernels to one per element format; in parallel, and
 only when it or a header is newer than its object), then the objects are linked into the shared library.
 """
 from __future__ import annotations
@@ -14,12 +14,13 @@ CSRC = os.path.join(HERE, "csrc")
 INCLUDE = os.path.join(os.path.dirname(HERE), "include")
 LIB = os.path.join(HERE, "libzc.so")
 OBJDIR = os.path.join(HERE, "build")
-SOURCES = ["zc_host.cpp", "zc_hist.cu", "zc_encode.cu", "zc_decode.cu"]
-# (source, extra flags, object name): the decoder's kernels are compiled one element format per object (ZC_DEC_PART),
-# so that the longest compile of the build runs four ways in parallel
+SOURCES = ["zc_host.cpp", "zc_hist.cu", "zc_encode.cu", "zc_encode_fmt.cu", "zc_decode.cu"]
+# (source, extra flags, object name): the encoder's and the decoder's kernels are compiled one element format per object
+# (ZC_ENC_FMT, ZC_DEC_PART), so that the longest compiles of the build run four ways in parallel
 UNITS = [("zc_host.cpp", [], "zc_host.cpp.o"), ("zc_hist.cu", [], "zc_hist.cu.o"), ("zc_encode.cu", [], "zc_encode.cu.o")] + \
+        [("zc_encode_fmt.cu", [f"-DZC_ENC_FMT={k}"], f"zc_encode.fmt{k}.o") for k in (1, 2, 3, 4)] + \
         [("zc_decode.cu", [f"-DZC_DEC_PART={k}"], f"zc_decode.part{k}.o") for k in (1, 2, 3, 4)]
-HEADERS = ["zc_internal.h", "zc_bits.cuh", "zc_device.cuh", "zc_encode_rows.cuh"]
+HEADERS = ["zc_internal.h", "zc_bits.cuh", "zc_device.cuh", "zc_encode.cuh"]
 ARCH = ["-gencode", "arch=compute_100a,code=sm_100a"]
 
 

@@ -42,26 +42,24 @@ struct zc_codebook_s {
     uint8_t len[2][256];
     uint32_t code[2][256];     // right-aligned canonical code values
     // derived once when the codebook is built, so that a compress call only copies them:
-    uint32_t enc[2][256];      // the encoder's table entry of every symbol: code << (32 - length) | length; 16: no code
-    uint8_t wide[2];           // the stream's codes are long on average: the encoder uses 12-bit pack slots
-    uint8_t brief[2];          // the stream's codes are short on average: half-size pack slots do for long subchunks
+    uint32_t enc[2][256];      // the encoder's table entry of every symbol: code << (32 - length) | length, or kNoCode
+    uint32_t fill[2];          // fill symbol (the one whose code is all zeros) | its code length << 8; 0xFF00: no code at all
 };
 
 namespace zc {
+// Entry of a symbol without a code.  A bit of its own: two of them add up to a bit that no sum of two lengths reaches.
+constexpr uint32_t kNoCode = 0x40;
+
 // Fills the derived fields of a codebook (call after len[] and code[] are final).
-// wide: with the symbol probabilities the code lengths imply (2^-length) the expected length is above 6.5 bits;
-// brief: it is at most 3.25 bits.
 inline void finish_codebook(zc_codebook_s* cb)
 {
     for (int s = 0; s < 2; ++s) {
-        uint64_t acc = 0;                        // sum of length * 2^(12 - length)
+        cb->fill[s] = 0xFF00u;
         for (int v = 0; v < 256; ++v) {
             const uint32_t l = cb->len[s][v];
-            cb->enc[s][v] = l ? (cb->code[s][v] << (32 - l)) | l : 16u;
-            if (l) acc += (uint64_t)l << (12 - l);
+            cb->enc[s][v] = l ? (cb->code[s][v] << (32 - l)) | l : kNoCode;
+            if (l && cb->code[s][v] == 0) cb->fill[s] = (uint32_t)v | (l << 8);
         }
-        cb->wide[s] = 2 * acc > (13ull << 12) ? 1 : 0;
-        cb->brief[s] = 4 * acc <= (13ull << 12) ? 1 : 0;
     }
 }
 
