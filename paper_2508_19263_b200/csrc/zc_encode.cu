@@ -11,49 +11,62 @@ using namespace zc;
 namespace {
 
 // Launch shape of the tensors of one launch (same format, chunk size and stream modes).
-struct EncShape { int kind; uint32_t lane_syms, tiles, team, teams, ring16; size_t smem; };
+struct EncShape { int kind; uint32_t unit_chunks, tiles, teams, ring16, buf_bytes; bool base_buf; size_t smem; };
 
-constexpr uint32_t kEncSmem = 220 * 1024;        // dynamic shared memory of a block; the rest is static
+constexpr uint32_t kEncSmem = 216 * 1024;        // dynamic shared memory of a block; the rest is static
 
 EncShape enc_shape(const zc_plan_t* p, uint32_t n_huff, bool any_base, uint64_t total_chunks)
 {
     EncShape s{};
-    // symbols per lane: the largest of 64, 48, 32, 16 that divides the subchunk (a multiple of 16 symbols)
-    const uint32_t units = p->syms_per_sub / 16;
-    const uint32_t g = units % 4 == 0 ? 4 : units % 3 == 0 ? 3 : units % 2 == 0 ? 2 : 1;
-    s.lane_syms = 16 * g;
-    s.tiles = units / g;
+    const uint32_t cs = p->syms_per_chunk, full = 32 * enc_lane_syms(kEncAny), small = 32 * enc_lane_syms(kEncAny48);
+    auto tiles = [&](uint32_t tile_syms) { return (cs + tile_syms - 1) / tile_syms; };
+    // a unit is as many whole chunks as fit a tile (1 and 2 KiB), or one chunk of one tile or several
+    s.unit_chunks = 2 * cs <= full && full % cs == 0 ? std::min(kMaxUnitChunks, full / cs) : 1;
+    if (cs == full) s.kind = kEncSolo;
+    else if (cs % full == 0) s.kind = kEncTeam;
+    else if (s.unit_chunks == 1 && tiles(small) * small < tiles(full) * full && tiles(small) <= enc_max_workers(kEncAny48, (int)n_huff)) s.kind = kEncAny48;
+    else s.kind = kEncAny;
+    s.tiles = tiles(32 * enc_lane_syms(s.kind));
+    if (s.tiles > enc_max_workers(s.kind, (int)n_huff)) s.kind = kEncBig;
+    const uint32_t tile_bytes = 64 * enc_lane_syms(s.kind);
     const uint32_t tables = 1024 * kTabSlots * std::max<uint32_t>(n_huff, 1);
-    const uint32_t buf = 64 * s.lane_syms * (any_base ? 2 : 1);
-    // a ring holds at least one chunk of 12-bit codes; typical chunks are a quarter to a half of that
-    const uint32_t min_ring = n_huff * (uint32_t)round_up((uint64_t)p->syms_per_chunk * kLmax / 8, 16);
-    const uint32_t max_w = enc_max_workers((int)n_huff);
-    // one warp per tile as long as the block has the warps and the memory; else the warps of a team take several tiles each
-    for (uint32_t turns = 1;; ++turns) {
-        s.team = (s.tiles + turns - 1) / turns;
-        if (s.team <= std::min(kEncMaxTeam, max_w) && tables + s.team * buf + min_ring <= kEncSmem) break;
-    }
-    s.teams = s.team < s.tiles ? 1 : std::min<uint32_t>(max_w / s.team, (kEncSmem - tables) / (s.team * buf + min_ring));
+    // a ring holds at least one unit of 12-bit codes; typical ones are a quarter to a half of that
+    const uint32_t min_ring = n_huff * s.unit_chunks * (uint32_t)round_up((uint64_t)cs * kLmax / 8, 16);
+    // The base tensor has an input buffer of its own, except for the largest chunks with both streams coded.  (The staged
+    // symbols take the input's place: a buffer of their own would let the next tile be requested earlier, but what it takes
+    // from the rings costs more: BF16 736 against 742 us, FP8 499 against 526 us.)
+    const uint32_t max_teams = enc_max_workers(s.kind, (int)n_huff) / s.tiles;
+    auto teams_with = [&](uint32_t worker_bytes) { return std::min<uint32_t>(max_teams, (kEncSmem - tables) / (s.tiles * worker_bytes + min_ring)); };
+    s.base_buf = any_base && teams_with(2 * tile_bytes) > 0;
+    s.buf_bytes = s.base_buf ? 2 * tile_bytes : tile_bytes;
+    s.teams = teams_with(s.buf_bytes);
+    const uint32_t buf = s.tiles * s.buf_bytes;
     // few chunks: rather more blocks than more teams in a block
-    s.teams = (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>(s.teams, (total_chunks + sm_count() - 1) / sm_count()));
-    s.ring16 = n_huff ? std::min<uint32_t>(((kEncSmem - tables) / s.teams - s.team * buf) / 16, std::max<uint32_t>(min_ring / 4, 1024)) : 0;
-    s.kind = s.lane_syms == 64 && s.team == s.tiles ? (s.tiles == 1 ? kEncSolo64 : kEncTeam64) : kEncAny;
-    s.smem = tables + (size_t)s.teams * (s.team * buf + 16 * s.ring16);
+    const uint64_t units = (total_chunks + s.unit_chunks - 1) / s.unit_chunks;
+    s.teams = (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>(s.teams, (units + sm_count() - 1) / sm_count()));
+    s.ring16 = n_huff ? std::min<uint32_t>(((kEncSmem - tables) / s.teams - buf) / 16, std::max<uint32_t>(min_ring / 4, 1024)) : 0;
+    s.smem = tables + (size_t)s.teams * (buf + 16 * s.ring16);
     return s;
 }
 
-void fill_common(EncParams& P, const zc_plan_t* p, const uint32_t mode[2], const EncShape& sh, bool any_base)
+void fill_common(EncParams& P, const zc_plan_t* p, const uint32_t mode[2], const EncShape& sh)
 {
     P.cs = p->syms_per_chunk; P.sub = p->syms_per_sub; P.chunk_bytes = p->chunk_bytes;
     P.format = p->format; P.group = p->group;
     P.sub_width = sub_end_width(p->chunk_bytes);
+    P.sub_magic = (uint32_t)(((1ull << 32) + p->syms_per_sub - 1) / p->syms_per_sub);
     P.mode[0] = mode[0]; P.mode[1] = mode[1];
-    P.lane_syms = sh.lane_syms; P.tiles = sh.tiles; P.team = sh.team; P.teams = sh.teams; P.ring16 = sh.ring16;
+    P.unit_syms = sh.unit_chunks * p->syms_per_chunk; P.unit_chunks = sh.unit_chunks;
+    P.tiles = sh.tiles; P.teams = sh.teams; P.ring16 = sh.ring16;
     P.spin_limit = test_knobs().spin_limit;
-    P.any_base = any_base ? 1u : 0u;
+    P.base_buf = sh.base_buf ? 1u : 0u;
+    P.buf_bytes = sh.buf_bytes;
 }
 
-void fill_item(EncItem& it, const zc_plan_t* p, const uint32_t mode[2], const void* d_in, const void* d_base, void* d_out,
+uint32_t units_of(const zc_plan_t* p, const EncShape& sh) { return (p->n_chunks + sh.unit_chunks - 1) / sh.unit_chunks; }
+uint32_t batches_of(const zc_plan_t* p, const EncShape& sh) { return (uint32_t)((units_of(p, sh) + (uint64_t)sh.teams - 1) / sh.teams); }
+
+void fill_item(EncItem& it, const zc_plan_t* p, const EncShape& sh, const uint32_t mode[2], const void* d_in, const void* d_base, void* d_out,
                uint32_t first_batch, uint32_t index, uint32_t table)
 {
     it.in = (const uint8_t*)d_in;
@@ -61,6 +74,8 @@ void fill_item(EncItem& it, const zc_plan_t* p, const uint32_t mode[2], const vo
     it.out = (uint8_t*)d_out;
     it.input_bytes = p->input_bytes; it.n_syms = p->n_syms; it.n_elems = p->n_elems;
     it.n_chunks = p->n_chunks;
+    it.n_units = units_of(p, sh);
+    it.pad = 0;
     it.first_batch = first_batch;
     it.index = index;
     it.table = table;
@@ -75,15 +90,13 @@ void fill_tables(EncTables& T, const zc_codebook_t* cb)
     T.pad[0] = T.pad[1] = 0;
 }
 
-uint32_t batches_of(const zc_plan_t* p, const EncShape& sh) { return (uint32_t)((p->n_chunks + (uint64_t)sh.teams - 1) / sh.teams); }
-
 cudaError_t launch_encode(EncParams& P, const EncShape& sh, const EncRanges& R, cudaStream_t st)
 {
     const uint32_t grid = std::min<uint32_t>(std::max<uint32_t>(P.total_batches, 1), (uint32_t)sm_count());
     // Holding a second batch lets the workers request its input while they code the first; with few batches per block it
     // would only keep them from idle blocks.
     P.ahead = P.total_batches >= 4 * grid ? 2 : 1;
-    const uint32_t threads = (sh.team * sh.teams + 1) * 32;
+    const uint32_t threads = (sh.tiles * sh.teams + kServiceWarps) * 32;
     switch (P.format) {
     case ZC_FMT_BF16: return enc_launch_bf16(sh.kind, grid, threads, sh.smem, st, P, R);
     case ZC_FMT_FP8_E4M3: case ZC_FMT_FP8_E5M2: return enc_launch_fp8(sh.kind, grid, threads, sh.smem, st, P, R);
@@ -173,7 +186,7 @@ uint32_t zc_test_encoder_workers(const zc_plan_t* p, uint32_t n_coded, uint32_t 
 {
     if (!p || n_coded > 2 || wide_slots > 2) return 0;
     const EncShape sh = enc_shape(p, n_coded, true, ~0ull >> 1);
-    return sh.smem <= kEncSmem ? sh.team * sh.teams : 0;
+    return sh.smem <= kEncSmem ? sh.tiles * sh.teams : 0;
 }
 
 zc_status zc_compress(const zc_plan_t* p, const zc_codebook_t* cb, const void* d_in, void* d_out, size_t out_capacity,
@@ -199,13 +212,13 @@ zc_status zc_compress_xor(const zc_plan_t* p, const zc_codebook_t* cb, const voi
     const EncShape sh = enc_shape(p, n_huff, d_base != nullptr, p->n_chunks);
 
     EncParams P{};
-    fill_common(P, p, mode, sh, d_base != nullptr);
+    fill_common(P, p, mode, sh);
     P.ctl = (Control*)d_workspace;
     P.counters = &P.ctl->tc;
     P.flags = (unsigned long long*)((uint8_t*)d_workspace + kControlBytes);
     P.n_tensors = 1;
     P.total_batches = batches_of(p, sh);
-    fill_item(P.one, p, mode, d_in, d_base, d_out, 0, 0, 0);
+    fill_item(P.one, p, sh, mode, d_in, d_base, d_out, 0, 0, 0);
     fill_tables(P.table, cb);
 
     if (cudaMemsetAsync(d_workspace, 0, kControlBytes + 8ull * P.total_batches, st) != cudaSuccess) return ZC_E_CUDA;
@@ -318,7 +331,7 @@ zc_status zc_compress_batch_xor(uint32_t n_tensors, const zc_plan_t* const* plan
     for (uint32_t t = 0; t < n_tensors; ++t) {
         const uint32_t combo = combo_of[t], i = at[combo]++;
         const uint32_t mode[2] = {combo & 1u, combo >> 1};
-        fill_item(items[i], plans[t], mode, d_in[t], d_base ? d_base[t] : nullptr, d_out[t], next[combo], t, table_of[t]);
+        fill_item(items[i], plans[t], shapes[combo], mode, d_in[t], d_base ? d_base[t] : nullptr, d_out[t], next[combo], t, table_of[t]);
         first[i] = next[combo];
         next[combo] += batches_of(plans[t], shapes[combo]);
     }
@@ -332,7 +345,7 @@ zc_status zc_compress_batch_xor(uint32_t n_tensors, const zc_plan_t* const* plan
         if (!per_combo[combo]) continue;
         const uint32_t mode[2] = {combo & 1u, combo >> 1};
         EncParams P{};
-        fill_common(P, p0, mode, shapes[combo], base[combo]);
+        fill_common(P, p0, mode, shapes[combo]);
         P.ctl = (Control*)ws;
         P.counters = (TensorCounters*)(ws + L.counters);
         P.flags = (unsigned long long*)(ws + L.flags) + flag_base;

@@ -1,19 +1,20 @@
 // Encoder kernel: field split, code lookup, bit packing and placement of the chunks in one pass over the input.
 //
-// Work unit of a warp: a tile, 32 lanes x n consecutive symbols of one chunk.  n is the largest of 64, 48, 32, 16 that
-// divides the subchunk length, so a subchunk is T = sub / n lanes long and a chunk is T tiles (T = 1 up to 4 KiB chunks).
-// Packing needs no serial walk over a subchunk: once every lane knows how many bits its symbols take, prefix sums give
-// every lane its bit position.  T warps form a team that codes one chunk together (T = 1: nothing to agree on); a block
-// is several teams plus one service warp, and its batch is as many consecutive chunks of a tensor as it has teams.
+// Work unit of a warp: a tile, 32 lanes x 64 (in one kernel shape 48) consecutive symbols, 4 KiB (3 KiB) of input.  Packing needs no serial walk over a
+// subchunk: once every lane knows how many bits its symbols take, prefix sums give every lane its bit position, and a
+// subchunk may end anywhere a lane has added up 16 symbols (subchunks are multiples of 16 symbols long).  A unit is one
+// chunk, or as many whole chunks as fit a tile (chunks of 1 and 2 KiB); T warps, one per tile of a unit, form a team that
+// codes one unit together (T = 1: nothing to agree on).  A block is several teams plus two service warps, and its batch is
+// as many consecutive units of a tensor as it has teams.
 //   A  the tile's input arrives in shared memory by a bulk asynchronous copy requested a tile ahead; it is split in
-//      registers, the raw stream is stored as it is, the coded stream goes back into the same buffer as one row of n bytes
-//      per lane (16-byte pieces swizzled so that neither side has bank conflicts)
+//      registers, the raw stream is stored as it is, the coded stream goes back into the same buffer as one row of 64
+//      (48) bytes per lane (16-byte pieces of 64-byte rows swizzled so that neither side has bank conflicts)
 //   B  every lane looks up its symbols and keeps the codes of two neighbouring symbols, joined, in one register each
 //      (24 bits of code, 5 bits of length), adding up the bits; the warp scans the bit counts
-//   C  the chunk's size is posted, subchunk ends are written, and every lane ORs its codes into the chunk's piece in the
+//   C  the unit's size is posted, subchunk ends are written, and every lane ORs its codes into the chunk's piece in the
 //      team's output ring in shared memory, at their final bit position
-// Pieces lie in the ring exactly as they will lie in the payload area.  Once a batch's place is known the service warp
-// sends each team's piece there with one bulk copy (cp.async.bulk shared -> global).  The place is the sum of the sizes
+// Pieces lie in the ring exactly as they will lie in the payload area.  Once a batch's place is known a service warp
+// sends each team's pieces there with one bulk copy (cp.async.bulk shared -> global).  The place is the sum of the sizes
 // of all earlier batches of the tensor, found by a look-back over one word per batch; workers never wait for it, only
 // for room in their ring (several chunks deep).
 #pragma once
@@ -35,10 +36,11 @@ struct EncItem {
     uint8_t* out;
     uint64_t input_bytes, n_syms, n_elems;
     Layout lay;
-    uint32_t n_chunks;
+    uint32_t n_chunks, n_units;
     uint32_t first_batch;                        // batches of all earlier tensors of the launch
     uint32_t index;                              // position in the caller's arrays (counters, error reports)
     uint32_t table;                              // its code tables among the uploaded ones (tensors may share a codebook)
+    uint32_t pad;
 };
 static_assert(sizeof(EncItem) % 8 == 0, "items are copied as 8-byte words");
 
@@ -52,13 +54,15 @@ struct EncParams {
     uint32_t cs, sub, chunk_bytes;               // symbols per chunk / per subchunk
     uint32_t format, group, sub_width;           // sub_width: bytes per sub_end entry (2 or 4)
     uint32_t mode[2];
-    uint32_t lane_syms, tiles;                   // n, T
-    uint32_t team, teams;                        // warps per chunk (T, or fewer: then each takes several tiles), chunks per batch
+    uint32_t sub_magic;                          // ceil(2^32 / sub): k / sub == umulhi(k, sub_magic) for k < 2^17
+    uint32_t unit_syms, unit_chunks;             // symbols and chunks of a unit
+    uint32_t tiles, teams;                       // T (tiles of a unit = warps of a team), units of a batch
     uint32_t ring16;                             // a team's output ring, in 16-byte units
     uint32_t n_tensors, total_batches;
     uint32_t ahead;                              // batches a block may hold beyond those it has packed
     uint32_t spin_limit;                         // polls after which a bounded wait gives up
-    uint32_t any_base;                           // some tensor has a base: every worker has a second input buffer
+    uint32_t base_buf;                           // every worker has a second input buffer for the base tensor
+    uint32_t buf_bytes;                          // a worker's input buffers
     EncItem one;
     EncTables table;
 };
@@ -167,13 +171,17 @@ constexpr uint32_t kNoSlot = 0xFFFFFFFFu;        // "no more batches"
 constexpr uint32_t kConstTile = 0x80000000u;     // tile of nothing but the fill symbol
 constexpr int kLookWide = 4;                     // look-back rounds cover 32 * kLookWide predecessors
 
-// Kernel shapes: lanes of 64 symbols and one warp per chunk (4 KiB chunks); lanes of 64 symbols and a warp per tile (chunks
-// of 8, 12, 16, .. KiB); everything else.
-constexpr int kEncSolo64 = 0, kEncTeam64 = 1, kEncAny = 2;
-// Worker warps per block: the joined codes take 32 registers per lane and coded stream; with the service warp that makes
-// 6 warps of 80 registers per scheduler with one coded stream, 4 of 128 with two.
-__host__ __device__ constexpr uint32_t enc_max_workers(int n_huff) { return n_huff == 2 ? 15u : 23u; }
-constexpr uint32_t kEncMaxTeam = 16;
+// Kernel shapes: a chunk is one tile (4 KiB); a chunk is T whole tiles (8, 12, 16, .. KiB); everything else, with lanes of
+// 64 symbols (1 and 2 KiB: several chunks to a tile; odd sizes: the last tile is not full) or of 48 where that fills the
+// tiles better (3, 6, 9 KiB; BF16 weights at 6 KiB: 95 against 119 us); and chunks of 16 tiles with both streams coded,
+// whose team is larger than the other shapes' blocks.
+constexpr int kEncSolo = 0, kEncTeam = 1, kEncAny = 2, kEncAny48 = 3, kEncBig = 4;
+__host__ __device__ constexpr uint32_t enc_lane_syms(int shape) { return shape == kEncAny48 ? 48u : 64u; }
+constexpr uint32_t kMaxUnitChunks = 4;           // chunks of a unit (kEncAny)
+// Worker warps per block: the joined codes take 32 registers per lane and coded stream; with the two service warps that
+// makes 5 warps of 96 registers per scheduler with one coded stream, 4 of 128 with two.
+constexpr uint32_t kServiceWarps = 2;
+__host__ __device__ constexpr uint32_t enc_max_workers(int shape, int n_huff) { return shape == kEncBig ? 16u : n_huff == 2 || shape == kEncAny ? 14u : 18u; }
 
 __device__ __forceinline__ uint32_t add_low_byte(uint32_t x, uint32_t acc) { return __dp4a(x, 1u, acc); }
 // Joins the table entries of two neighbouring symbols: codes behind one another in bits 31..8, length in bits 7..0.
@@ -182,62 +190,60 @@ __device__ __forceinline__ uint32_t join_codes(uint32_t a, uint32_t b)
     return add_low_byte(b, a | (__funnelshift_r(b, 0, a) & 0xFFFFFF00u));   // the funnel shift takes the low five bits of a: its length
 }
 
-// Phase B for one coded stream: looks up the lane's symbols (its row of 16 * parts staged bytes at row_s, 16-byte pieces
+// Phase B for one coded stream: looks up the lane's symbols (its row of 2 N staged bytes at row_s, 16-byte pieces
 // XORed with `swz`), leaves the joined codes in e[] and returns the lane's bit count.  `ok` turns false when a symbol has
 // no code: the caller then uses lookup_checked.
-__device__ __forceinline__ uint32_t lookup_quick(uint32_t (&e)[32], const uint32_t row_s, const uint32_t swz, const uint32_t parts,
+template <uint32_t N>
+__device__ __forceinline__ uint32_t lookup_quick(uint32_t (&e)[N], const uint32_t row_s, const uint32_t swz,
                                                  const uint32_t tab_s, bool& ok, bool& long_quad)
 {
     uint32_t bits = 0, seen = 0, over = 0;
 #pragma unroll
-    for (uint32_t p = 0; p < 4; ++p) {
-        if (p < parts) {
-            const uint4 v = lds128(row_s + ((p ^ swz) << 4));
-            const uint32_t q[4] = {v.x, v.y, v.z, v.w};
+    for (uint32_t p = 0; p < N / 8; ++p) {
+        const uint4 v = lds128(row_s + ((p ^ swz) << 4));
+        const uint32_t q[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
-            for (uint32_t i = 0; i < 4; ++i) {
-                // tab_s + 4 * byte k of the word, in one dot product
-                const uint32_t a0 = lds32(__dp4a(q[i], 0x00000004u, tab_s)), a1 = lds32(__dp4a(q[i], 0x00000400u, tab_s));
-                const uint32_t a2 = lds32(__dp4a(q[i], 0x00040000u, tab_s)), a3 = lds32(__dp4a(q[i], 0x04000000u, tab_s));
-                const uint32_t e0 = join_codes(a0, a1), e1 = join_codes(a2, a3);
-                seen |= e0 | e1;
-                e[8 * p + 2 * i] = e0;
-                e[8 * p + 2 * i + 1] = e1;
-                const uint32_t len = e0 + e1 + 95;               // bit 7 of it: more than 32 bits
-                over |= len;
-                bits = add_low_byte(len, bits);
-            }
+        for (uint32_t i = 0; i < 4; ++i) {
+            // tab_s + 4 * byte k of the word, in one dot product
+            const uint32_t a0 = lds32(__dp4a(q[i], 0x00000004u, tab_s)), a1 = lds32(__dp4a(q[i], 0x00000400u, tab_s));
+            const uint32_t a2 = lds32(__dp4a(q[i], 0x00040000u, tab_s)), a3 = lds32(__dp4a(q[i], 0x04000000u, tab_s));
+            const uint32_t e0 = join_codes(a0, a1), e1 = join_codes(a2, a3);
+            seen |= e0 | e1;
+            e[8 * p + 2 * i] = e0;
+            e[8 * p + 2 * i + 1] = e1;
+            const uint32_t len = e0 + e1 + 95;               // bit 7 of it: more than 32 bits
+            over |= len;
+            bits = add_low_byte(len, bits);
         }
     }
     ok = (seen & (3u * kNoCode)) == 0;                           // one or two of them in a pair
     long_quad = (over & 0x80u) != 0;
-    return bits - 4 * 95 * parts;
+    return bits - 95 * (N / 2);
 }
 
 // The same symbol by symbol for tiles that need care: a ragged end (only the first n_my symbols count) and symbols
 // without a code (they take no bits; `bad` is set).
-__device__ __forceinline__ uint32_t lookup_checked(uint32_t (&e)[32], const uint32_t row_s, const uint32_t swz, const uint32_t parts,
+template <uint32_t N>
+__device__ __forceinline__ uint32_t lookup_checked(uint32_t (&e)[N], const uint32_t row_s, const uint32_t swz,
                                                    const uint32_t tab_s, const uint32_t n_my, bool& bad)
 {
     uint32_t bits = 0;
 #pragma unroll
-    for (uint32_t p = 0; p < 4; ++p) {
-        if (p < parts) {
-            const uint4 v = lds128(row_s + ((p ^ swz) << 4));
-            const uint32_t q[4] = {v.x, v.y, v.z, v.w};
+    for (uint32_t p = 0; p < N / 8; ++p) {
+        const uint4 v = lds128(row_s + ((p ^ swz) << 4));
+        const uint32_t q[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
-            for (uint32_t i = 0; i < 4; ++i) {
-                uint32_t a[4];
+        for (uint32_t i = 0; i < 4; ++i) {
+            uint32_t a[4];
 #pragma unroll
-                for (uint32_t k = 0; k < 4; ++k) {
-                    a[k] = 0;
-                    if (16 * p + 4 * i + k < n_my) a[k] = lds32(tab_s + 4u * __byte_perm(q[i], 0, 0x4440 + k));
-                    if (a[k] & kNoCode) { bad = true; a[k] = 0; }
-                }
-                e[8 * p + 2 * i] = join_codes(a[0], a[1]);
-                e[8 * p + 2 * i + 1] = join_codes(a[2], a[3]);
-                bits = add_low_byte(e[8 * p + 2 * i] + e[8 * p + 2 * i + 1], bits);
+            for (uint32_t k = 0; k < 4; ++k) {
+                a[k] = 0;
+                if (16 * p + 4 * i + k < n_my) a[k] = lds32(tab_s + 4u * __byte_perm(q[i], 0, 0x4440 + k));
+                if (a[k] & kNoCode) { bad = true; a[k] = 0; }
             }
+            e[8 * p + 2 * i] = join_codes(a[0], a[1]);
+            e[8 * p + 2 * i + 1] = join_codes(a[2], a[3]);
+            bits = add_low_byte(e[8 * p + 2 * i] + e[8 * p + 2 * i + 1], bits);
         }
     }
     return bits;
@@ -245,31 +251,29 @@ __device__ __forceinline__ uint32_t lookup_checked(uint32_t (&e)[32], const uint
 
 // Phase C for one coded stream: ORs the joined codes into shared memory from bit `at` of the piece at piece_s on.
 // QUADS: four codes at a time (no group of four in the warp is longer than 32 bits), else two at a time.
-template <bool QUADS>
-__device__ __forceinline__ void emit_codes(const uint32_t (&e)[32], const uint32_t parts, const uint32_t piece_s, const uint32_t at)
+template <bool QUADS, uint32_t N>
+__device__ __forceinline__ void emit_codes(const uint32_t (&e)[N], const uint32_t piece_s, const uint32_t at)
 {
     uint32_t addr = piece_s + 4 * (at >> 5), t = at & 31u, w = 0;
 #pragma unroll
-    for (uint32_t p = 0; p < 4; ++p) {
-        if (p < parts) {
+    for (uint32_t p = 0; p < N / 8; ++p) {
 #pragma unroll
-            for (uint32_t i = 0; i < 4; ++i) {
-                const uint32_t e0 = e[8 * p + 2 * i], e1 = e[8 * p + 2 * i + 1], c0 = e0 & 0xFFFFFF00u, c1 = e1 & 0xFFFFFF00u;
-                if (QUADS) {
-                    put_bits(c0 | __funnelshift_r(c1, 0, e0), add_low_byte(e0 + e1, t), t, w, addr);
-                } else {
-                    put_bits(c0, add_low_byte(e0, t), t, w, addr);
-                    put_bits(c1, add_low_byte(e1, t), t, w, addr);
-                }
+        for (uint32_t i = 0; i < 4; ++i) {
+            const uint32_t e0 = e[8 * p + 2 * i], e1 = e[8 * p + 2 * i + 1], c0 = e0 & 0xFFFFFF00u, c1 = e1 & 0xFFFFFF00u;
+            if (QUADS) {
+                put_bits(c0 | __funnelshift_r(c1, 0, e0), add_low_byte(e0 + e1, t), t, w, addr);
+            } else {
+                put_bits(c0, add_low_byte(e0, t), t, w, addr);
+                put_bits(c1, add_low_byte(e1, t), t, w, addr);
             }
         }
     }
     if (t & 31u) red_or(addr, w);
 }
 
-// Whether the n_my staged symbols of every lane all equal `symbol`; the whole warp calls it.  Rarely needed (tiles that
-// might be constant), so it is kept out of line.
-static __device__ __noinline__ bool all_symbols_are(uint32_t row_s, uint32_t swz, uint32_t n_my, uint32_t symbol)
+// The lanes whose n_my staged symbols all equal `symbol`; the whole warp calls it.  Rarely needed (tiles that might be
+// constant), so it is kept out of line.
+static __device__ __noinline__ uint32_t lanes_of_only(uint32_t row_s, uint32_t swz, uint32_t n_my, uint32_t symbol)
 {
     bool same = true;
     for (uint32_t k = 0; k < n_my; k += 4) {
@@ -277,7 +281,7 @@ static __device__ __noinline__ bool all_symbols_are(uint32_t row_s, uint32_t swz
         const uint32_t x = lds32(row_s + (((k >> 4) ^ swz) << 4) + (k & 15u)) ^ (symbol * 0x01010101u);
         same = same && (x & (0xFFFFFFFFu >> (32 - 8 * left))) == 0;
     }
-    return __all_sync(0xFFFFFFFFu, same);
+    return __ballot_sync(0xFFFFFFFFu, same);
 }
 
 __device__ __forceinline__ uint32_t warp_scan(uint32_t v, uint32_t lane)
@@ -291,39 +295,39 @@ __device__ __forceinline__ uint32_t warp_scan(uint32_t v, uint32_t lane)
 }
 
 template <int FMT, bool H0, bool H1, int SHAPE>
-__global__ void __launch_bounds__((enc_max_workers((H0 ? 1 : 0) + (H1 ? 1 : 0)) + 1) * 32, 1)
+__global__ void __launch_bounds__((enc_max_workers(SHAPE, (H0 ? 1 : 0) + (H1 ? 1 : 0)) + kServiceWarps) * 32, 1)
 encode_kernel(const __grid_constant__ EncParams P)
 {
     constexpr int kHuff = (H0 ? 1 : 0) + (H1 ? 1 : 0);
     constexpr int kTabs = kHuff ? kHuff : 1;
-    constexpr uint32_t kMaxW = enc_max_workers(kHuff);
-    constexpr uint32_t kMaxTiles = SHAPE == kEncAny ? 64 : kMaxW;        // tiles of a batch
-    constexpr bool kSolo = SHAPE == kEncSolo64;
+    constexpr uint32_t kMaxW = enc_max_workers(SHAPE, kHuff);
+    constexpr bool kSolo = SHAPE == kEncSolo, kAny = SHAPE >= kEncAny;
+    constexpr uint32_t kN = enc_lane_syms(SHAPE);               // symbols of a lane
+    constexpr uint32_t kTileSyms = 32 * kN;
     extern __shared__ __align__(16) uint8_t smem[];
     const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const uint32_t n_workers = (blockDim.x >> 5) - 1;
-    const uint32_t T = kSolo ? 1u : P.tiles, team = kSolo ? 1u : P.team, teams = kSolo ? n_workers : P.teams;
-    const uint32_t n = SHAPE != kEncAny ? 64u : P.lane_syms;            // symbols per lane
+    const uint32_t n_workers = (blockDim.x >> 5) - kServiceWarps;
+    const uint32_t T = kSolo ? 1u : P.tiles, teams = kSolo ? n_workers : P.teams;
+    const uint32_t unit_syms = kSolo ? kTileSyms : P.unit_syms, unit_chunks = SHAPE == kEncAny ? P.unit_chunks : 1u;
 
-    // shared: rings[teams] | input buffers[workers][1 or 2][64 n] | tables[kTabSlots][kTabs][256]
+    // shared: rings[teams] | input buffers[workers] | tables[kTabSlots][kTabs][256]
     const uint32_t rings_s = smem_u32(smem);
     const uint32_t bufs_s = rings_s + teams * 16 * P.ring16;
-    const uint32_t buf_bytes = P.any_base ? 128 * n : 64 * n;
-    const uint32_t tabs_s = bufs_s + n_workers * buf_bytes;
+    const uint32_t tabs_s = bufs_s + n_workers * P.buf_bytes;
 
     __shared__ EncItem s_item[kTabSlots];
     __shared__ uint32_t s_fill[kTabSlots][2];
-    __shared__ uint32_t s_slot[kEncRing], s_c0[kEncRing], s_ticket[kEncRing], s_cnt[kEncRing], s_done[kEncRing], s_tot[kEncRing];
-    __shared__ uint32_t s_bits[kEncRing][kTabs][kMaxW], s_src[kEncRing][kMaxW];
-    __shared__ uint32_t s_tile[2][kTabs][kMaxTiles];
-    __shared__ uint32_t s_freed_seq, s_fail;
-    __shared__ uint64_t mb_in[kMaxW], mb_team[kMaxW], mb_info[kEncRing];
+    __shared__ uint32_t s_slot[kEncRing], s_c0[kEncRing], s_ticket[kEncRing], s_tensor[kEncRing], s_tot[kEncRing];
+    __shared__ uint32_t s_bits[kEncRing][kTabs][kMaxW * (SHAPE == kEncAny ? kMaxUnitChunks : 1)], s_src[kEncRing][kMaxW];
+    __shared__ uint32_t s_tile[2][kTabs][kMaxW];
+    __shared__ uint32_t s_freed_seq, s_end, s_fail;
+    __shared__ uint64_t mb_in[kMaxW], mb_team[kMaxW], mb_info[kEncRing], mb_size[kEncRing], mb_posted[kEncRing], mb_done[kEncRing];
 
-    if (threadIdx.x < kEncRing) s_cnt[threadIdx.x] = s_done[threadIdx.x] = 0;
     if (threadIdx.x == 0) {
         s_freed_seq = s_fail = 0;
-        for (uint32_t i = 0; i < kEncRing; ++i) mbar_init(&mb_info[i], 1);
-        for (uint32_t i = 0; i < n_workers; ++i) { mbar_init(&mb_in[i], 1); mbar_init(&mb_team[i], team); }
+        s_end = 0xFFFFFFFFu;
+        for (uint32_t i = 0; i < kEncRing; ++i) { mbar_init(&mb_info[i], 1); mbar_init(&mb_size[i], teams); mbar_init(&mb_posted[i], 1); mbar_init(&mb_done[i], n_workers); }
+        for (uint32_t i = 0; i < n_workers; ++i) { mbar_init(&mb_in[i], 1); mbar_init(&mb_team[i], T); }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
@@ -331,37 +335,156 @@ encode_kernel(const __grid_constant__ EncParams P)
 
     auto vol32 = [](const uint32_t* p) { return *reinterpret_cast<const volatile uint32_t*>(p); };
     auto counters = [&](const uint32_t index) -> TensorCounters* { return P.counters + index; };
+    const EncItem* const items = P.items ? P.items : &P.one;
 
     if (warp == n_workers) {
-        // =========================== the service warp ===========================
-        // It never blocks on one thing: in a loop it publishes batches, posts the sizes of packed ones, advances the
-        // look-back of the oldest batch without a place by one round, and sends out the batch whose place is known.
-        const EncItem* const items = P.items ? P.items : &P.one;
-        if (blockIdx.x == 0)                                     // tensors without chunks are all header
-            for (uint32_t t = lane; t < P.n_tensors; t += 32)
-                if (items[t].n_chunks == 0) write_header(P, items[t], counters(items[t].index));
-
-        uint32_t published = 0, posted = 0, placed = 0, freed = 0;     // batches of this block
+        // =========================== the dealer warp ===========================
+        // Takes tickets, turns them into batches and publishes those; posts the sizes of batches that have been packed.
+        uint32_t published = 0, posted = 0;                      // batches of this block
         uint32_t ticket = 0;                                     // lane 0: ticket taken for the next batch
         bool have_ticket = false;
         uint32_t tcur = 0, next_first = 0;                       // tensor of the last ticket (tickets only grow), first batch of the next one
         uint32_t slot = 0, slot_tensor = kNoSlot;                // the newest table slot and whose it is
         uint32_t slot_last[kTabSlots] = {};                      // 1 + last batch that uses the slot
-        bool ended = false, lb_on = false, lb_done = false;
-        unsigned long long lb_sum = 0;
-        long long lb_pos = 0;
+        bool ended = false;
+        uint32_t idle = 0;
+        for (;;) {
+            bool did = false;
+            // ---- sizes of batches that have been packed ----
+            while (posted < published && __all_sync(0xFFFFFFFFu, mbar_test(&mb_size[posted % kEncRing], (posted / kEncRing) & 1u))) {
+                const uint32_t r = posted % kEncRing;
+                uint32_t p16 = 0;
+#pragma unroll
+                for (int h = 0; h < kHuff; ++h)
+                    for (uint32_t k = 0; k < unit_chunks; ++k) p16 += lane < teams ? (s_bits[r][h][lane * unit_chunks + k] + 127) >> 7 : 0u;
+                const uint32_t total = __reduce_add_sync(0xFFFFFFFFu, p16);
+                if (lane == 0) {
+                    if (kHuff) st_flag(P.flags + s_ticket[r], (s_c0[r] == 0 ? kFlagPrefix : kFlagAggregate) | total);
+                    s_tot[r] = total;
+                    mbar_arrive(&mb_posted[r]);
+                }
+                __syncwarp();
+                ++posted;
+                did = true;
+            }
+            if (ended && posted == published) break;
+            // ---- a new batch ----
+            const uint32_t freed = __shfl_sync(0xFFFFFFFFu, vol32(&s_freed_seq), 0);
+            if (!ended && published < posted + P.ahead && published < freed + kEncRing) {
+                if (!have_ticket && lane == 0) ticket = atomicAdd(&P.ctl->ticket, 1u);
+                have_ticket = true;
+                const uint32_t g = __shfl_sync(0xFFFFFFFFu, ticket, 0);
+                const uint32_t r = published % kEncRing;
+                if (g >= P.total_batches) {
+                    ended = true;
+                    if (lane == 0) {
+                        s_slot[r] = kNoSlot;
+                        *reinterpret_cast<volatile uint32_t*>(&s_end) = published;
+                        mbar_arrive(&mb_info[r]);
+                    }
+                    __syncwarp();
+                    continue;
+                }
+                // the last tensor that starts at or before the batch (tensors without chunks share their start with the next)
+                if (P.items && g >= next_first) {
+                    for (;;) {
+                        const uint32_t cand = tcur + 1 + lane;
+                        const uint32_t k = __popc(__ballot_sync(0xFFFFFFFFu, cand < P.n_tensors && P.first_batch[cand] <= g));
+                        tcur += k;
+                        if (k < 32) break;
+                    }
+                    next_first = tcur + 1 < P.n_tensors ? P.first_batch[tcur + 1] : 0xFFFFFFFFu;
+                }
+                bool publish = true;
+                if (tcur != slot_tensor) {
+                    // another tensor: it takes the next slot once every batch that uses it has left the block
+                    const uint32_t ns = (slot + 1) % kTabSlots;
+                    const uint32_t last = ns == 0 ? slot_last[0] : ns == 1 ? slot_last[1] : ns == 2 ? slot_last[2] : slot_last[3];
+                    publish = freed >= last;
+                    if (publish) {
+                        slot = ns;
+                        slot_tensor = tcur;
+                        const unsigned long long* src = reinterpret_cast<const unsigned long long*>(items + tcur);
+                        unsigned long long* dst = reinterpret_cast<unsigned long long*>(&s_item[ns]);
+                        for (uint32_t i = lane; i < sizeof(EncItem) / 8; i += 32) dst[i] = src[i];
+                        const EncTables& E = P.tables ? P.tables[items[tcur].table] : P.table;
+                        uint32_t h = 0;
+#pragma unroll
+                        for (int s = 0; s < 2; ++s) {
+                            if (!(s == 0 ? H0 : H1)) continue;
+#pragma unroll
+                            for (uint32_t i = 0; i < 8; ++i) sts32(tabs_s + 1024 * (kTabs * ns + h) + 4 * (lane + 32 * i), E.enc[s][lane + 32 * i]);
+                            if (lane == 0) s_fill[ns][h] = E.fill[s];
+                            ++h;
+                        }
+                        __syncwarp();
+                    }
+                }
+                if (publish) {
+                    const EncItem& I = s_item[slot];
+                    const uint32_t c0 = (g - I.first_batch) * teams;
+                    ++published;
+                    have_ticket = false;
+#pragma unroll
+                    for (uint32_t k = 0; k < kTabSlots; ++k) if (k == slot) slot_last[k] = published;
+                    if (lane == 0) {
+                        s_slot[r] = slot; s_c0[r] = c0; s_ticket[r] = g; s_tensor[r] = tcur;
+                        mbar_arrive(&mb_info[r]);
+                    }
+                    __syncwarp();
+                    if (P.ahead > 1) {                           // the next one's ticket travels until it is looked at
+                        if (lane == 0) ticket = atomicAdd(&P.ctl->ticket, 1u);
+                        have_ticket = true;
+                    }
+                    if (c0 == 0) {
+                        // the fixed parts of the tensor's container: code lengths, padding of the chunk offset table, tail
+                        // padding of raw bodies
+                        uint32_t h = 0;
+#pragma unroll
+                        for (int s = 0; s < 2; ++s) {
+                            if (s == 0 ? H0 : H1) {
+                                for (uint32_t v = lane; v < 256; v += 32)
+                                    I.out[I.lay.section_off[s] + v] = (uint8_t)(lds32(tabs_s + 1024 * (kTabs * slot + h) + 4 * v) & 15u);
+                                const uint32_t padded = (I.n_chunks + 3) & ~3u;
+                                for (uint32_t i = I.n_chunks + lane; i < padded; i += 32)
+                                    reinterpret_cast<uint32_t*>(I.out + I.lay.chunk_off_tab[s])[i] = 0;
+                                ++h;
+                            } else {
+                                const uint64_t lo = (I.n_syms + 7) & ~7ull, hi = (I.n_syms + 15) & ~15ull;
+                                for (uint64_t i = lo + lane; i < hi; i += 32) I.out[I.lay.section_off[s] + i] = 0;
+                            }
+                        }
+                    }
+                    did = true;
+                }
+            }
+            if (__shfl_sync(0xFFFFFFFFu, vol32(&s_fail), 0)) break;
+            if (did) { idle = 0; continue; }
+            if (++idle > P.spin_limit) { s_fail = 1; break; }
+            __nanosleep(200);                                    // nothing to do right now: leave the issue slots to the workers
+        }
+    } else if (warp == n_workers + 1) {
+        // =========================== the placer warp ===========================
+        // Finds the place of the block's oldest batch without one by a look-back over other blocks' words, sends its pieces
+        // there, gives the ring space back, and keeps the tensors' counters.
+        if (blockIdx.x == 0)                                     // tensors without chunks are all header
+            for (uint32_t t = lane; t < P.n_tensors; t += 32)
+                if (items[t].n_chunks == 0) write_header(P, items[t], counters(items[t].index));
+        uint32_t placed = 0, freed = 0;                          // batches of this block
+        bool lb_on = false, lb_done = false;
+        uint32_t lb_sum = 0, lb_pos = 0;
         uint32_t idle = 0;
         // chunks this block has placed, per tensor; added to the tensor's counters when the tensor changes
-        uint32_t acc_slot = kNoSlot, acc_index = 0, acc_n = 0;
+        uint32_t acc_t = kNoSlot, acc_n = 0;
         unsigned long long acc_bits[2] = {0, 0};                 // per lane: payload bits of those chunks
-        auto flush_acc = [&]() {                                 // before its slot is given to another tensor
+        auto flush_acc = [&]() {
             if (acc_n == 0) return;
 #pragma unroll
             for (int h = 0; h < kHuff; ++h)
 #pragma unroll
                 for (int o = 16; o > 0; o >>= 1) acc_bits[h] += __shfl_xor_sync(0xFFFFFFFFu, acc_bits[h], o);
             if (lane == 0) {
-                const EncItem& I = s_item[acc_slot];
+                const EncItem& I = items[acc_t];
                 TensorCounters* tc = counters(I.index);
                 if (H0) atomicAdd(&tc->payload_bits[0], acc_bits[0]);
                 if (H1) atomicAdd(&tc->payload_bits[1], acc_bits[H0 ? 1 : 0]);
@@ -378,187 +501,80 @@ encode_kernel(const __grid_constant__ EncParams P)
         };
         for (;;) {
             bool did = false;
-            // ---- post the sizes of batches that have been packed ----
-            while (posted < published - (ended ? 1u : 0u) && __shfl_sync(0xFFFFFFFFu, vol32(&s_cnt[posted % kEncRing]), 0) == teams) {
-                __threadfence_block();
-                const uint32_t r = posted % kEncRing;
-                uint32_t p16 = 0;
-#pragma unroll
-                for (int h = 0; h < kHuff; ++h) p16 += lane < teams ? (s_bits[r][h][lane] + 127) >> 7 : 0u;
-                const uint32_t total = __reduce_add_sync(0xFFFFFFFFu, p16);
-                if (lane == 0) {
-                    s_cnt[r] = 0;
-                    s_tot[r] = total;
-                    if (kHuff) st_flag(P.flags + s_ticket[r], (s_c0[r] == 0 ? kFlagPrefix : kFlagAggregate) | total);
-                }
-                __syncwarp();
-                ++posted;
+            const uint32_t r = placed % kEncRing;
+            if (!lb_on && __all_sync(0xFFFFFFFFu, mbar_test(&mb_posted[r], (placed / kEncRing) & 1u))) {
+                lb_sum = 0;                                      // sizes are 16-byte units: chunk_off16 has 32 bits
+                lb_pos = 1;                                      // lane i looks lb_pos + i batches back
+                lb_done = !kHuff || s_c0[r] == 0;
+                lb_on = true;
                 did = true;
             }
-            // ---- a new batch ----
-            if (!ended && published < posted + P.ahead && published < freed + kEncRing) {
-                if (!have_ticket && lane == 0) ticket = atomicAdd(&P.ctl->ticket, 1u);
-                have_ticket = true;
-                const uint32_t next_g = __shfl_sync(0xFFFFFFFFu, ticket, 0);
-                const uint32_t r = published % kEncRing;
-                bool publish = true;
-                uint32_t use = kNoSlot, c0 = 0;
-                if (next_g < P.total_batches) {
-                    // the last tensor that starts at or before the batch (tensors without chunks share their start with the next)
-                    if (P.items && next_g >= next_first) {
-                        for (;;) {
-                            const uint32_t cand = tcur + 1 + lane;
-                            const uint32_t k = __popc(__ballot_sync(0xFFFFFFFFu, cand < P.n_tensors && P.first_batch[cand] <= next_g));
-                            tcur += k;
-                            if (k < 32) break;
-                        }
-                        next_first = tcur + 1 < P.n_tensors ? P.first_batch[tcur + 1] : 0xFFFFFFFFu;
-                    }
-                    if (tcur != slot_tensor) {
-                        // another tensor: it takes the next slot once every batch that uses it is placed
-                        const uint32_t ns = (slot + 1) % kTabSlots;
-                        const uint32_t last = ns == 0 ? slot_last[0] : ns == 1 ? slot_last[1] : ns == 2 ? slot_last[2] : slot_last[3];
-                        if (placed < last) {
-                            publish = false;
-                        } else {
-                            if (acc_slot == ns) flush_acc();
-                            slot = ns;
-                            slot_tensor = tcur;
-                            const unsigned long long* src = reinterpret_cast<const unsigned long long*>(items + tcur);
-                            unsigned long long* dst = reinterpret_cast<unsigned long long*>(&s_item[ns]);
-                            for (uint32_t i = lane; i < sizeof(EncItem) / 8; i += 32) dst[i] = src[i];
-                            const EncTables& E = P.tables ? P.tables[items[tcur].table] : P.table;
-                            uint32_t h = 0;
-#pragma unroll
-                            for (int s = 0; s < 2; ++s) {
-                                if (!(s == 0 ? H0 : H1)) continue;
-#pragma unroll
-                                for (uint32_t i = 0; i < 8; ++i) sts32(tabs_s + 1024 * (kTabs * ns + h) + 4 * (lane + 32 * i), E.enc[s][lane + 32 * i]);
-                                if (lane == 0) s_fill[ns][h] = E.fill[s];
-                                ++h;
-                            }
-                            __syncwarp();
-                        }
-                    }
-                    if (publish) {
-                        use = slot;
-                        const EncItem& I = s_item[slot];
-                        c0 = (next_g - I.first_batch) * teams;
-                        if (c0 == 0) {
-                            // the fixed parts of the tensor's container: code lengths, padding of the chunk offset table,
-                            // tail padding of raw bodies
-                            uint32_t h = 0;
-#pragma unroll
-                            for (int s = 0; s < 2; ++s) {
-                                if (s == 0 ? H0 : H1) {
-                                    for (uint32_t v = lane; v < 256; v += 32)
-                                        I.out[I.lay.section_off[s] + v] = (uint8_t)(lds32(tabs_s + 1024 * (kTabs * slot + h) + 4 * v) & 15u);
-                                    const uint32_t padded = (I.n_chunks + 3) & ~3u;
-                                    for (uint32_t i = I.n_chunks + lane; i < padded; i += 32)
-                                        reinterpret_cast<uint32_t*>(I.out + I.lay.chunk_off_tab[s])[i] = 0;
-                                    ++h;
-                                } else {
-                                    const uint64_t lo = (I.n_syms + 7) & ~7ull, hi = (I.n_syms + 15) & ~15ull;
-                                    for (uint64_t i = lo + lane; i < hi; i += 32) I.out[I.lay.section_off[s] + i] = 0;
-                                }
-                            }
-                        }
-                    }
-                } else {
-                    ended = true;
-                }
-                if (publish) {
-                    ++published;
-                    have_ticket = false;
-                    if (use != kNoSlot) {
-#pragma unroll
-                        for (uint32_t k = 0; k < kTabSlots; ++k) if (k == use) slot_last[k] = published;
-                    }
-                    if (lane == 0) {
-                        s_slot[r] = use; s_c0[r] = c0; s_ticket[r] = next_g;
-                    }
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(&mb_info[r]);
-                    if (P.ahead > 1 && !ended) {                 // the next one's ticket travels until it is looked at
-                        if (lane == 0) ticket = atomicAdd(&P.ctl->ticket, 1u);
-                        have_ticket = true;
-                    }
-                    did = true;
-                }
-            }
-            // ---- placement of the oldest batch without a place ----
-            if (placed < posted) {
-                const uint32_t r = placed % kEncRing;
-                const uint32_t use = s_slot[r], c0 = s_c0[r];
-                const EncItem& I = s_item[use];
-                unsigned long long* const flags = P.flags + s_ticket[r];   // the batch's own word; the look-back stays inside the tensor
-                const uint32_t total = s_tot[r];
-                if (!lb_on) {
-                    lb_sum = 0;
-                    lb_pos = 1;                                  // lane i looks lb_pos + i batches back
-                    lb_done = !kHuff || c0 == 0;
-                    lb_on = true;
-                }
+            if (lb_on) {
+                const EncItem& I = s_item[s_slot[r]];
+                const uint32_t c0 = s_c0[r], total = s_tot[r];
                 if (!lb_done) {
                     // One round: 32 * kLookWide predecessors at a time, newest first, up to the first one that already knows
-                    // its prefix.  All loads of a round are in flight together.
-                    const long long b = s_ticket[r] - I.first_batch;
+                    // its prefix.  All loads of a round are in flight together.  The look-back stays inside the tensor.
+                    unsigned long long* const flags = P.flags + s_ticket[r];
+                    const uint32_t b = s_ticket[r] - I.first_batch;
                     unsigned long long f[kLookWide];
 #pragma unroll
                     for (int k = 0; k < kLookWide; ++k) {
-                        const long long back = lb_pos + 32 * k + lane;
+                        const uint32_t back = lb_pos + 32 * k + lane;
                         f[k] = back <= b ? ld_flag(flags - back) : kFlagPrefix;      // before batch 0: prefix 0
                     }
 #pragma unroll
                     for (int k = 0; k < kLookWide; ++k) {
-                        if (lb_done) continue;
                         const uint32_t ready = __ballot_sync(0xFFFFFFFFu, (f[k] >> 62) != 0);
                         const uint32_t prefix = __ballot_sync(0xFFFFFFFFu, (f[k] >> 62) == 2);
                         const uint32_t first = prefix ? (uint32_t)__ffs(prefix) - 1 : 32u;
                         const uint32_t need = first == 32 ? 0xFFFFFFFFu : (0xFFFFFFFFu >> (31 - first));
                         if ((ready & need) != need) break;       // somebody has not posted yet: again from here later
-                        unsigned long long x = lane <= first ? f[k] & kFlagValue : 0;
-#pragma unroll
-                        for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xFFFFFFFFu, x, o);
-                        lb_sum += x;
-                        lb_done = first != 32;
+                        lb_sum += __reduce_add_sync(0xFFFFFFFFu, lane <= first ? (uint32_t)f[k] : 0u);
                         lb_pos += 32;
                         did = true;
+                        if (first != 32) { lb_done = true; break; }
                     }
-                    if (lb_done && lane == 0) st_flag(flags, kFlagPrefix | (lb_sum + total));
+                    if (lb_done && lane == 0) st_flag(flags, kFlagPrefix | ((unsigned long long)lb_sum + total));
                 }
-                if (lb_done && __shfl_sync(0xFFFFFFFFu, vol32(&s_done[r]), 0) == n_workers) {
-                    __threadfence_block();
-                    const uint32_t n_mine = min(teams, I.n_chunks - c0);
-                    if (use != acc_slot || I.index != acc_index) { flush_acc(); acc_slot = use; acc_index = I.index; }
-                    acc_n += n_mine;
+                if (lb_done && __all_sync(0xFFFFFFFFu, mbar_test(&mb_done[r], (placed / kEncRing) & 1u))) {
+                    const uint32_t n_mine = min(teams, I.n_units - c0);
+                    if (s_tensor[r] != acc_t) { flush_acc(); acc_t = s_tensor[r]; }
+                    acc_n += min(n_mine * unit_chunks, I.n_chunks - c0 * unit_chunks);
                     if (kHuff) {
-                        uint32_t bits[2] = {0, 0}, p16[2] = {0, 0};
+                        uint32_t mine = 0;
+                        for (uint32_t k = 0; k < unit_chunks; ++k)
 #pragma unroll
-                        for (int h = 0; h < kHuff; ++h) {
-                            if (lane < n_mine) bits[h] = s_bits[r][h][lane];
-                            p16[h] = (bits[h] + 127) >> 7;
-                            acc_bits[h] += bits[h];
-                        }
-                        const uint32_t mine = p16[0] + p16[1];
-                        const unsigned long long off = lb_sum + warp_scan(mine, lane) - mine;
-                        if (lane < n_mine) {
-                            reinterpret_cast<uint32_t*>(I.out + I.lay.chunk_off_tab[H0 ? 0 : 1])[c0 + lane] = (uint32_t)off;
-                            if (kHuff == 2) reinterpret_cast<uint32_t*>(I.out + I.lay.chunk_off_tab[1])[c0 + lane] = (uint32_t)off + p16[0];
-                            if (mine) bulk_s2g(I.out + I.lay.payload_off + 16 * off, rings_s + 16 * (lane * P.ring16 + s_src[r][lane]), 16 * mine);
-                        }
+                            for (int h = 0; h < kHuff; ++h)
+                                if (lane < n_mine) {
+                                    const uint32_t bits = s_bits[r][h][lane * unit_chunks + k];
+                                    mine += (bits + 127) >> 7;
+                                    acc_bits[h] += bits;
+                                }
+                        const uint32_t off = lb_sum + warp_scan(mine, lane) - mine;
+                        if (lane < n_mine && mine)
+                            bulk_s2g(I.out + I.lay.payload_off + 16ull * off, rings_s + 16 * (lane * P.ring16 + s_src[r][lane]), 16 * mine);
                         asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+                        if (lane < n_mine) {
+                            uint32_t at = off;
+                            for (uint32_t k = 0; k < unit_chunks; ++k) {
+                                const uint32_t c = (c0 + lane) * unit_chunks + k;
+#pragma unroll
+                                for (int h = 0; h < kHuff; ++h) {
+                                    if (c < I.n_chunks) reinterpret_cast<uint32_t*>(I.out + I.lay.chunk_off_tab[H0 ? h : 1])[c] = at;
+                                    at += (s_bits[r][h][lane * unit_chunks + k] + 127) >> 7;
+                                }
+                            }
+                        }
                         // the block that owns the last chunk knows the size of the whole payload area
-                        if (lane == 0 && c0 + n_mine == I.n_chunks) counters(I.index)->total16 = lb_sum + total;
+                        if (lane == 0 && c0 + n_mine == I.n_units) counters(I.index)->total16 = lb_sum + total;
                     }
                     __syncwarp();
-                    if (lane == 0) s_done[r] = 0;
                     ++placed;
                     lb_on = false;
                     did = true;
                 }
             }
-            if (ended && freed == published - 1) break;
             if (__shfl_sync(0xFFFFFFFFu, vol32(&s_fail), 0)) break;
             // ---- ring space of batches that have been sent: the newest one's copies are given time until nothing else is to do ----
             if (freed < placed) {
@@ -569,10 +585,12 @@ encode_kernel(const __grid_constant__ EncParams P)
                 did = did || now != freed;
                 freed = now;
                 if (lane == 0) *reinterpret_cast<volatile uint32_t*>(&s_freed_seq) = freed;
+            } else if (freed == __shfl_sync(0xFFFFFFFFu, vol32(&s_end), 0)) {
+                break;
             }
             if (did) { idle = 0; continue; }
             if (++idle > P.spin_limit) { s_fail = 1; break; }
-            __nanosleep(100);                                    // nothing to do right now: leave the issue slots to the workers
+            __nanosleep(50);
         }
         asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
         __syncwarp();
@@ -582,14 +600,14 @@ encode_kernel(const __grid_constant__ EncParams P)
         // Bounded wait of the whole warp for a phase of an mbarrier; false on the failure flag or when the wait gives up.
         // (A try_wait sleeps in hardware until the phase completes or a time limit is reached.)
         auto wait_phase = [&](uint64_t* bar, const uint32_t parity) -> bool {
-            bool ok = mbar_try_wait(bar, parity);
+            bool ok = mbar_try_wait_ns(bar, parity, 2000u);
             for (uint32_t k = 0; !ok && k < P.spin_limit; ++k) {
                 if (vol32(&s_fail)) break;
-                ok = mbar_try_wait(bar, parity);
+                ok = mbar_try_wait_ns(bar, parity, 2000u);
             }
             return __all_sync(0xFFFFFFFFu, ok);                  // decisions of the whole warp: no lane may leave alone
         };
-        const uint32_t my_team = kSolo ? warp : warp / team, tw = kSolo ? 0u : warp - my_team * team;    // my team, my place in it
+        const uint32_t my_team = kSolo ? warp : warp / T, tw = kSolo ? 0u : warp - my_team * T;    // my team, my tile of its unit
         uint32_t ph_team = 0;
         auto team_sync = [&]() -> bool {
             __syncwarp();
@@ -598,34 +616,32 @@ encode_kernel(const __grid_constant__ EncParams P)
             ++ph_team;
             return ok;
         };
-        const uint32_t parts = n / 16;                           // 16-byte pieces of a lane's row
-        const uint32_t tile_syms = 32 * n;
-        const uint32_t buf_s = bufs_s + warp * buf_bytes;
+        const uint32_t t_lo = tw * kTileSyms;                                          // my tile in the unit,
+        const uint32_t t_full = kAny ? min(kTileSyms, unit_syms - t_lo) : kTileSyms;   // and its symbols (a multiple of 256)
+        const uint32_t buf_s = bufs_s + warp * P.buf_bytes;
         const uint32_t ring_s = rings_s + my_team * 16 * P.ring16;
-        // rows of 64 bytes: 16-byte piece p of row r sits at p ^ (r >> 1 & 3); of 32 bytes: p ^ (r >> 2 & 1); the others as they are
-        const uint32_t swz_shift = n == 64 ? 1u : 2u, swz_mask = n == 64 ? 3u : n == 32 ? 1u : 0u;
-        const uint32_t swz = (lane >> swz_shift) & swz_mask;
-        const uint32_t row_groups = n / 8, row_magic = (0xFFFFFFFFu / row_groups) + 1;   // g / row_groups == umulhi(g, magic), g < 2^16
-        auto at_of = [&](const uint32_t g) {                     // where group g's 8 symbols are staged
-            const uint32_t row = __umulhi(g, row_magic), k = g - row * row_groups;
-            return row * n + (((k >> 1) ^ ((row >> swz_shift) & swz_mask)) << 4) + 8 * (k & 1u);
-        };
-        // lanes of 64 symbols: lane l's groups l + 32 i go to row 4 i + l / 8; from one i to the next the swizzle flips bit 1
-        // of the piece index
-        const uint32_t at0 = (lane >> 3) * 64 + ((((lane & 7) >> 1) ^ (lane >> 4)) << 4) + 8 * (lane & 1u);
+        // Staged symbols.  Rows of 64 bytes: 16-byte piece p of row r sits at p ^ (r >> 1 & 3); group g (8 symbols) is half of a
+        // piece of row g / 8.  Lane l's groups l + 32 i go to row 4 i + l / 8: from one i to the next the swizzle flips bit 1
+        // of the piece index.  Rows of 48 bytes have no bank conflicts as they are.
+        const uint32_t swz = kN == 64 ? (lane >> 1) & 3u : 0u;
+        const uint32_t at0 = kN == 64 ? (lane >> 3) * 64 + ((((lane & 7) >> 1) ^ (lane >> 4)) << 4) + 8 * (lane & 1u) : 8 * lane;
+        auto stage_at = [&](const uint32_t i) { return (kN == 64 ? at0 ^ ((i & 1u) << 5) : at0) + 256 * i; };
+        // several chunks in a unit: the lanes of my chunk
+        const uint32_t chunk_lanes = (SHAPE == kEncAny && unit_chunks > 1) ? P.cs / kN : 32u, my_k = kAny ? lane / chunk_lanes : 0u, k_lane = my_k * chunk_lanes;
 
         bool loaded = false;                                     // the next tile's input has been requested
         uint32_t ph_in = 0;
-        auto whole_tile = [&](const EncItem& I, const uint64_t s_lo) { return s_lo + tile_syms <= I.n_syms && 2 * (s_lo + tile_syms) <= I.input_bytes; };
-        // Requests tile j of chunk c of tensor I, if it is a complete one (the buffer is free: every lane has passed a __syncwarp).
-        auto request = [&](const EncItem& I, const uint32_t c, const uint32_t j) {
-            const uint64_t s_lo = (uint64_t)c * P.cs + j * tile_syms;
-            if (c >= I.n_chunks || !whole_tile(I, s_lo)) return;
+        auto whole_tile = [&](const EncItem& I, const uint64_t s_lo) { return s_lo + t_full <= I.n_syms && 2 * (s_lo + t_full) <= I.input_bytes; };
+        // Requests my tile of unit u of tensor I, if it is a complete one (the buffer is free: every lane has passed a __syncwarp).
+        auto request = [&](const EncItem& I, const uint32_t u) {
+            const uint64_t s_lo = (uint64_t)u * unit_syms + t_lo;
+            if (u >= I.n_units || !whole_tile(I, s_lo)) return;
             if (lane == 0) {
+                const bool two = I.base && P.base_buf;
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-                mbar_expect_tx(&mb_in[warp], I.base ? 128 * n : 64 * n);
-                bulk_g2s_addr(buf_s, I.in + 2 * s_lo, 64 * n, &mb_in[warp]);
-                if (I.base) bulk_g2s_addr(buf_s + 64 * n, I.base + 2 * s_lo, 64 * n, &mb_in[warp]);
+                mbar_expect_tx(&mb_in[warp], two ? 4 * t_full : 2 * t_full);
+                bulk_g2s_addr(buf_s, I.in + 2 * s_lo, 2 * t_full, &mb_in[warp]);
+                if (two) bulk_g2s_addr(buf_s + 2 * kTileSyms, I.base + 2 * s_lo, 2 * t_full, &mb_in[warp]);
             }
             loaded = true;
         };
@@ -640,21 +656,25 @@ encode_kernel(const __grid_constant__ EncParams P)
             const uint32_t use = vol32(&s_slot[r]);
             if (use == kNoSlot) break;
             const EncItem& I = s_item[use];
-            const uint32_t c = vol32(&s_c0[r]) + my_team;
-            const bool active = c < I.n_chunks;
-            const uint64_t c_lo = (uint64_t)c * P.cs;
-            const uint32_t c_syms = active ? (uint32_t)min((uint64_t)P.cs, I.n_syms - c_lo) : 0u;
+            const uint32_t u = vol32(&s_c0[r]) + my_team;
+            const bool active = u < I.n_units;
             const uint32_t tab_s = tabs_s + 1024 * kTabs * use;
 
-            uint32_t e[kTabs][32];                               // joined codes of my symbols
-            uint32_t inc[kTabs], mine[kTabs];                    // my symbols' bits, and their inclusive scan over the tile
-            uint32_t tile_bits[kTabs];
-            bool quads[kTabs];                                   // no four neighbouring codes of the tile are longer than 32 bits
-            // Phases A and B of tile j of my chunk; `raw`: store the raw stream too; next(): requests the tile after it.
-            auto do_tile = [&](const uint32_t j, const bool raw, auto next) -> bool {
-                const uint32_t t_lo = j * tile_syms;
-                const uint32_t t_syms = c_syms > t_lo ? min(tile_syms, c_syms - t_lo) : 0u;
-                const uint64_t s_lo = c_lo + t_lo;               // first symbol of the tile in its stream
+            uint32_t e[kTabs][kN / 2];                             // joined codes of my symbols
+            uint32_t mine[kTabs] = {}, end[kTabs] = {};          // bits of my symbols, and where they end in their chunk
+            uint32_t chunk_bits[kTabs] = {};                     // bits of my chunk (0: constant)
+            bool quads[kTabs] = {};                              // no four neighbouring codes of the tile are longer than 32 bits
+            const uint64_t s_lo = (uint64_t)u * unit_syms + t_lo;       // first symbol of the tile in its stream
+            auto request_next = [&]() {                          // my tile of the next batch, if that is known already
+                const uint32_t r1 = (it + 1) % kEncRing;
+                if (!__all_sync(0xFFFFFFFFu, mbar_test(&mb_info[r1], ((it + 1) / kEncRing) & 1u))) return;
+                const uint32_t use1 = vol32(&s_slot[r1]);
+                if (use1 != kNoSlot) request(s_item[use1], vol32(&s_c0[r1]) + my_team);
+            };
+            if (active) {
+                // ---- phase A ----
+                const uint32_t t_syms = s_lo < I.n_syms ? (uint32_t)min((uint64_t)t_full, I.n_syms - s_lo) : 0u;
+                const bool whole = whole_tile(I, s_lo);
                 uint8_t* const raw0 = I.out + I.lay.section_off[0] + s_lo;
                 uint8_t* const raw1 = I.out + I.lay.section_off[1] + s_lo;
                 // With both streams coded (delta checkpoints: stretches of unchanged weights are constant chunks in both
@@ -666,144 +686,150 @@ encode_kernel(const __grid_constant__ EncParams P)
                     fill4[0] = (s_fill[use][0] & 0xFFu) * 0x01010101u;
                     fill4[1] = (s_fill[use][1] & 0xFFu) * 0x01010101u;
                 }
-                auto stage = [&](const uint4 x, const uint32_t g, const uint32_t at) {
+                auto stage = [&](const uint4 x, const uint32_t g, const uint32_t at, const bool on) {
                     const uint32_t w[4] = {x.x, x.y, x.z, x.w};
                     uint32_t sy[2][2];
                     split16<FMT>(w, sy[0], sy[1]);
                     if (H0) sts64(buf_s + at, sy[0][0], sy[0][1]);
-                    else if (raw) st_cs_v2(raw0 + 8 * g, make_uint2(sy[0][0], sy[0][1]));
-                    if (H1) sts64(buf_s + (H0 ? tile_syms : 0u) + at, sy[1][0], sy[1][1]);
-                    else if (raw) st_cs_v2(raw1 + 8 * g, make_uint2(sy[1][0], sy[1][1]));
-                    if (kSpotConstant) {
+                    else if (!kAny || on) st_cs_v2(raw0 + 8 * g, make_uint2(sy[0][0], sy[0][1]));
+                    if (H1) sts64(buf_s + (H0 ? kTileSyms : 0u) + at, sy[1][0], sy[1][1]);
+                    else if (!kAny || on) st_cs_v2(raw1 + 8 * g, make_uint2(sy[1][0], sy[1][1]));
+                    if (kSpotConstant && (!kAny || on)) {
                         differs[0] |= (sy[0][0] ^ fill4[0]) | (sy[0][1] ^ fill4[0]);
                         differs[1] |= (sy[1][0] ^ fill4[1]) | (sy[1][1] ^ fill4[1]);
                     }
                 };
                 auto x4 = [](const uint4 a, const uint4 b) { return make_uint4(a.x ^ b.x, a.y ^ b.y, a.z ^ b.z, a.w ^ b.w); };
-                const bool whole = t_syms == tile_syms;
-                if (whole && whole_tile(I, s_lo)) {
-                    if (!loaded) request(I, c, j);
-                    if (!wait_phase(&mb_in[warp], ph_in & 1u)) return false;
+                if (whole) {
+                    if (!loaded) request(I, u);
+                    if (!wait_phase(&mb_in[warp], ph_in & 1u)) { failed = true; break; }
                     ++ph_in;
                     loaded = false;
-                    uint4 x[8];
+                    // (a tile that is not full is read and staged to its end all the same: what lies behind is not looked at)
+                    uint4 x[kN / 8];
 #pragma unroll
-                    for (uint32_t i = 0; i < 8; ++i)
-                        if (SHAPE != kEncAny || i < row_groups) x[i] = lds128(buf_s + 16 * (lane + 32 * i));
+                    for (uint32_t i = 0; i < kN / 8; ++i) x[i] = lds128(buf_s + 16 * (lane + 32 * i));
                     if (I.base) {
 #pragma unroll
-                        for (uint32_t i = 0; i < 8; ++i)
-                            if (SHAPE != kEncAny || i < row_groups) x[i] = x4(x[i], lds128(buf_s + 64 * n + 16 * (lane + 32 * i)));
+                        for (uint32_t i = 0; i < kN / 8; ++i) {
+                            const uint32_t on = kAny ? min(i, t_full / 256 - 1) : i;
+                            x[i] = x4(x[i], P.base_buf ? lds128(buf_s + 2 * kTileSyms + 16 * (lane + 32 * i)) : ld_nc_v4(I.base + 2 * s_lo + 16 * (lane + 32 * on)));
+                        }
                     }
                     __syncwarp();                                // everybody has read: the buffer takes the staged symbols
 #pragma unroll
-                    for (uint32_t i = 0; i < 8; ++i)
-                        if (SHAPE != kEncAny || i < row_groups)
-                            stage(x[i], lane + 32 * i, SHAPE != kEncAny ? (at0 ^ ((i & 1u) << 5)) + 256 * i : at_of(lane + 32 * i));
+                    for (uint32_t i = 0; i < kN / 8; ++i) stage(x[i], lane + 32 * i, stage_at(i), 256 * i < t_full);
                 } else {
-                    for (uint32_t g = lane; g < (t_syms + 7) / 8; g += 32) {
+                    for (uint32_t i = 0; 256 * i + 8 * lane < t_syms; ++i) {
+                        const uint32_t g = lane + 32 * i;
                         uint4 x = load16_guarded(I.in, 2 * (s_lo + 8ull * g), I.input_bytes);
                         if (I.base) x = x4(x, load16_guarded(I.base, 2 * (s_lo + 8ull * g), I.input_bytes));
-                        stage(x, g, at_of(g));
+                        stage(x, g, stage_at(i), true);
                     }
                 }
                 __syncwarp();
 
-                const uint32_t n_my = t_syms > lane * n ? min(n, t_syms - lane * n) : 0u;
+                // ---- phase B ----
+                const uint32_t n_my = t_syms > kN * lane ? min(kN, t_syms - kN * lane) : 0u;
+                const uint32_t k_syms = (SHAPE == kEncAny && unit_chunks > 1) ? (t_syms > my_k * P.cs ? min(P.cs, t_syms - my_k * P.cs) : 0u) : t_syms;   // of my chunk in the tile
+                uint32_t tile_bits[kTabs];
 #pragma unroll
                 for (int h = 0; h < kHuff; ++h) {
-                    const uint32_t row = buf_s + h * tile_syms + lane * n;
+                    const uint32_t row = buf_s + h * kTileSyms + lane * kN;
                     const uint32_t fill = s_fill[use][h], fill_len = fill >> 8;
                     bool constant = false;
                     if (kSpotConstant && whole && fill_len <= kLmax && __all_sync(0xFFFFFFFFu, differs[h] == 0)) {
                         // nothing but the fill symbol (which has the all-zero code)
 #pragma unroll
-                        for (uint32_t i = 0; i < 32; ++i) e[h][i] = 2 * fill_len;
-                        mine[h] = n * fill_len;
+                        for (uint32_t i = 0; i < kN / 2; ++i) e[h][i] = 2 * fill_len;
+                        mine[h] = n_my * fill_len;
                         constant = true;
                         quads[h] = fill_len <= 8;
                     } else {
                         bool ok = false, long_quad = true;
-                        if (whole) mine[h] = lookup_quick(e[h], row, swz, parts, tab_s + 1024 * h, ok, long_quad);
+                        if (whole) {
+                            if (!kAny || n_my) {
+                                mine[h] = lookup_quick(e[h], row, swz, tab_s + 1024 * h, ok, long_quad);
+                            } else {
+                                ok = true; long_quad = false;
+                            }
+                        }
                         quads[h] = __all_sync(0xFFFFFFFFu, ok && !long_quad);
                         if (!quads[h] && !__all_sync(0xFFFFFFFFu, ok)) {
                             bool no_code = false;
-                            mine[h] = lookup_checked(e[h], row, swz, parts, tab_s + 1024 * h, n_my, no_code);
+                            mine[h] = lookup_checked(e[h], row, swz, tab_s + 1024 * h, n_my, no_code);
                             if (no_code) bad = I.index + 1;
                         }
                     }
-                    inc[h] = warp_scan(mine[h], lane);
-                    uint32_t bits = __shfl_sync(0xFFFFFFFFu, inc[h], 31);
-                    if (!constant && t_syms && bits == t_syms * fill_len) constant = all_symbols_are(row, swz, n_my, fill & 0xFFu);
-                    // tiles without symbols (behind the end of a ragged chunk) do not keep a chunk from being constant
-                    if (constant || t_syms == 0) bits |= kConstTile;
-                    tile_bits[h] = bits;
-                }
-                __syncwarp();                                    // the buffer is free
-                next();
-                return true;
-            };
-            auto next_batch = [&]() {                            // the first tile of my next chunk, if that is known already
-                const uint32_t r1 = (it + 1) % kEncRing;
-                if (!__all_sync(0xFFFFFFFFu, mbar_test(&mb_info[r1], ((it + 1) / kEncRing) & 1u))) return;
-                const uint32_t use1 = vol32(&s_slot[r1]);
-                if (use1 != kNoSlot) request(s_item[use1], vol32(&s_c0[r1]) + my_team, tw);
-            };
-
-            // per coded stream: bits of the chunk, and of the tiles of it before mine (lane = tile when a warp has several)
-            uint32_t chunk_bits[kTabs] = {}, before[kTabs] = {}, before2[kTabs] = {};
-            const bool several = SHAPE == kEncAny && team < T;
-            if (active) {
-                if (several) {
-                    for (uint32_t j = tw; j < T && !failed; j += team) {
-                        failed = !do_tile(j, true, [&] { if (kHuff || j + team < T) request(I, c, j + team < T ? j + team : tw); else next_batch(); });
-                        if (lane == 0)
-                            for (int h = 0; h < kHuff; ++h) s_tile[it & 1u][h][j] = tile_bits[h];
+                    const uint32_t inc = warp_scan(mine[h], lane);
+                    uint32_t bits = __shfl_sync(0xFFFFFFFFu, inc, 31), lead = 0;         // of my chunk in the tile; of the chunks before it
+                    if (SHAPE == kEncAny && unit_chunks > 1) {
+                        lead = __shfl_sync(0xFFFFFFFFu, inc, k_lane ? k_lane - 1 : 0);
+                        if (k_lane == 0) lead = 0;
+                        bits = __shfl_sync(0xFFFFFFFFu, inc, k_lane + chunk_lanes - 1) - lead;
                     }
-                } else {
-                    failed = !do_tile(tw, true, next_batch);
-                    if (!kSolo && lane == 0)
-                        for (int h = 0; h < kHuff; ++h) s_tile[it & 1u][h][warp] = tile_bits[h];
+                    const bool maybe = !constant && k_syms && bits == k_syms * fill_len;
+                    if (__any_sync(0xFFFFFFFFu, maybe)) {
+                        const uint32_t want = (0xFFFFFFFFu >> (32 - chunk_lanes)) << k_lane;
+                        if ((lanes_of_only(row, swz, n_my, fill & 0xFFu) & want) == want) constant = constant || maybe;
+                    }
+                    end[h] = inc - lead;
+                    // tiles without symbols (behind the end of a ragged chunk) do not keep a chunk from being constant
+                    tile_bits[h] = bits | ((constant || k_syms == 0) ? kConstTile : 0u);
                 }
-                if (failed) break;
-                if (kSolo) {
+                __syncwarp();                                    // the staged symbols are used up
+                request_next();
+                if (T == 1) {
 #pragma unroll
                     for (int h = 0; h < kHuff; ++h) chunk_bits[h] = (tile_bits[h] & kConstTile) ? 0u : tile_bits[h];
                 } else if (kHuff) {
                     // every warp of the team learns the bit counts of the chunk's tiles
+                    if (lane == 0)
+#pragma unroll
+                        for (int h = 0; h < kHuff; ++h) s_tile[it & 1u][h][warp] = tile_bits[h];
                     if (!team_sync()) { failed = true; break; }
 #pragma unroll
                     for (int h = 0; h < kHuff; ++h) {
-                        const uint32_t* tiles = &s_tile[it & 1u][h][several ? 0u : my_team * team];
-                        const uint32_t v0 = lane < T ? tiles[lane] : kConstTile, v1 = lane + 32 < T ? tiles[lane + 32] : kConstTile;
-                        const uint32_t a = warp_scan(v0 & ~kConstTile, lane), a31 = __shfl_sync(0xFFFFFFFFu, a, 31);
-                        uint32_t b = 0;
-                        if (SHAPE == kEncAny && T > 32) b = warp_scan(v1 & ~kConstTile, lane);
-                        const bool none = __all_sync(0xFFFFFFFFu, (v0 & v1 & kConstTile) != 0);
-                        chunk_bits[h] = none ? 0u : a31 + __shfl_sync(0xFFFFFFFFu, b, 31);
-                        before[h] = a - (v0 & ~kConstTile);
-                        before2[h] = a31 + b - (v1 & ~kConstTile);
-                        if (!several) before[h] = __shfl_sync(0xFFFFFFFFu, before[h], tw);
+                        const uint32_t v = lane < T ? s_tile[it & 1u][h][my_team * T + lane] : kConstTile;
+                        const uint32_t a = warp_scan(v & ~kConstTile, lane);
+                        const bool none = __all_sync(0xFFFFFFFFu, (v & kConstTile) != 0);
+                        const uint32_t bits = __shfl_sync(0xFFFFFFFFu, a, 31);
+                        chunk_bits[h] = none ? 0u : bits;
+                        end[h] += __shfl_sync(0xFFFFFFFFu, a - (v & ~kConstTile), tw);
                     }
                 }
             }
 
-            // ---- the piece: its size is posted, it gets a stretch of the ring (every warp of the team follows the allocation) ----
-            uint32_t p16[kTabs], total = 0;
+            // ---- the pieces: their sizes are posted, they get a stretch of the ring (every warp of the team follows the allocation) ----
+            uint32_t p16[kTabs], total = 0, my_at = 0;           // my chunk's pieces; the unit's; where mine start among them
 #pragma unroll
             for (int h = 0; h < kHuff; ++h) { p16[h] = (chunk_bits[h] + 127) >> 7; total += p16[h]; }
+            if (SHAPE == kEncAny && unit_chunks > 1) {
+                const uint32_t own = total;
+                total = 0;
+                for (uint32_t k = 0; k < unit_chunks; ++k) {
+                    const uint32_t x = __shfl_sync(0xFFFFFFFFu, own, k * chunk_lanes);
+                    if ((int)k < (int)my_k) my_at += x;
+                    total += x;
+                }
+            }
             if (ring_pos + total > P.ring16) { virt += P.ring16 - ring_pos; ring_pos = 0; }
             const uint32_t piece_at = ring_pos;
             ring_pos += total;
             virt += total;
             if (lane == (it & 31u)) vend = virt;
-            if (tw == 0 && lane == 0) {
+            if (tw == 0) {
+                if (lane == k_lane) {
 #pragma unroll
-                for (int h = 0; h < kHuff; ++h) s_bits[r][h][my_team] = chunk_bits[h];
-                s_src[r][my_team] = piece_at;
-                __threadfence_block();
-                atomicAdd(&s_cnt[r], 1u);
+                    for (int h = 0; h < kHuff; ++h) s_bits[r][h][my_team * unit_chunks + my_k] = chunk_bits[h];
+                }
+                if (kAny) __syncwarp();
+                if (lane == 0) {
+                    s_src[r][my_team] = piece_at;
+                    mbar_arrive(&mb_size[r]);
+                }
             }
+            // ---- phase C ----
             if (kHuff && active) {
                 if (total) {
                     bool room = false;
@@ -815,49 +841,45 @@ encode_kernel(const __grid_constant__ EncParams P)
                         __nanosleep(50);
                     }
                     if (!room) { failed = true; break; }
-                    // my share of the piece starts from zero
-                    for (uint32_t u = tw * 32 + lane; u < total; u += 32 * team) sts128_zero(ring_s + 16 * (piece_at + u));
-                    if (kSolo) __syncwarp();
+                    // my share of the pieces starts from zero
+                    for (uint32_t q = tw * 32 + lane; q < total; q += 32 * T) sts128_zero(ring_s + 16 * (piece_at + q));
+                    if (T == 1) __syncwarp();
                     else if (!team_sync()) { failed = true; break; }
                 }
-                auto finish_tile = [&](const uint32_t j, const uint32_t (&pre)[kTabs]) {
-                    // subchunk ends: lane g of the chunk (counting through its tiles) ends subchunk (g + 1) / T - 1 if T divides g + 1
-                    const uint32_t gl = j * 32 + lane + 1, sub_i = kSolo ? gl : gl / T;
+                const uint32_t c = u * unit_chunks + my_k;
 #pragma unroll
-                    for (int h = 0; h < kHuff; ++h) {
-                        const int s = H0 ? h : 1;
-                        const uint32_t end = chunk_bits[h] ? pre[h] + inc[h] : 0u;
-                        if (sub_i * T == gl) {
-                            if (SHAPE == kEncSolo64 || P.sub_width == 2) reinterpret_cast<uint16_t*>(I.out + I.lay.sub_end_tab[s] + 64ull * c)[sub_i - 1] = (uint16_t)end;
-                            else reinterpret_cast<uint32_t*>(I.out + I.lay.sub_end_tab[s] + 128ull * c)[sub_i - 1] = end;
-                        }
-                        if (chunk_bits[h]) {
-                            const uint32_t piece_s = ring_s + 16 * (piece_at + (h ? p16[0] : 0u));
-                            if (quads[h]) emit_codes<true>(e[h], parts, piece_s, end - mine[h]);
-                            else emit_codes<false>(e[h], parts, piece_s, end - mine[h]);
-                        }
-                    }
-                };
-                if (several) {
-                    for (uint32_t j = tw; j < T && !failed; j += team) {
-                        uint32_t pre[kTabs];
+                for (int h = 0; h < kHuff; ++h) {
+                    const int s = H0 ? h : 1;
+                    uint8_t* const tab = I.out + I.lay.sub_end_tab[s] + (uint64_t)(32 * P.sub_width) * c;
+                    auto put_end = [&](const uint32_t i, const uint32_t at) {
+                        if (kSolo || P.sub_width == 2) reinterpret_cast<uint16_t*>(tab)[i] = (uint16_t)at;
+                        else reinterpret_cast<uint32_t*>(tab)[i] = at;
+                    };
+                    if (kAny) {
+                        // subchunks end where a lane has added up a multiple of 16 symbols
+                        uint32_t at = end[h] - mine[h];
 #pragma unroll
-                        for (int h = 0; h < kHuff; ++h) pre[h] = __shfl_sync(0xFFFFFFFFu, j < 32 ? before[h] : before2[h], j & 31u);
-                        // looked up again: the codes of one tile at a time are kept
-                        failed = !do_tile(j, false, [&] { if (j + team < T) request(I, c, j + team); else next_batch(); });
-                        if (!failed) finish_tile(j, pre);
+                        for (uint32_t p = 0; p < kN / 16; ++p) {
+#pragma unroll
+                            for (uint32_t i = 0; i < 8; ++i) at = add_low_byte(e[h][8 * p + i], at);
+                            const uint32_t k = t_lo + kN * (lane - k_lane) + 16 * (p + 1), i = __umulhi(k, P.sub_magic);
+                            if (c < I.n_chunks && k <= P.cs && i * P.sub == k) put_end(i - 1, chunk_bits[h] ? at : 0u);
+                        }
+                    } else {
+                        // T lanes are a subchunk: lane g of the chunk (counting through its tiles) ends subchunk (g + 1) / T - 1 if T divides g + 1
+                        const uint32_t g1 = tw * 32 + lane + 1, i = kSolo ? g1 : g1 / T;
+                        if (i * T == g1) put_end(i - 1, chunk_bits[h] ? end[h] : 0u);
                     }
-                    if (failed) break;
-                } else {
-                    finish_tile(tw, before);
+                    if (chunk_bits[h] && (!kAny || mine[h])) {
+                        const uint32_t piece_s = ring_s + 16 * (piece_at + my_at + (h ? p16[0] : 0u));
+                        if (quads[h]) emit_codes<true>(e[h], piece_s, end[h] - mine[h]);
+                        else emit_codes<false>(e[h], piece_s, end[h] - mine[h]);
+                    }
                 }
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             }
             __syncwarp();
-            if (lane == 0) {
-                __threadfence_block();
-                atomicAdd(&s_done[r], 1u);
-            }
+            if (lane == 0) mbar_arrive(&mb_done[r]);
         }
         if (failed) s_fail = 1;
         if (loaded) mbar_wait(&mb_in[warp], ph_in & 1u, P.spin_limit);   // a copy that was requested must land before the block leaves

@@ -25,9 +25,11 @@ cudaError_t enc_launch_t(int shape, uint32_t grid, uint32_t threads, size_t smem
     else if (h0) launch(encode_kernel<F, true, false, SHAPE>);              \
     else if (h1) launch(encode_kernel<F, false, true, SHAPE>);              \
     else launch(encode_kernel<F, false, false, SHAPE>);
-    if (shape == kEncSolo64) { ZC_ENC_CASE(kEncSolo64) }
-    else if (shape == kEncTeam64) { ZC_ENC_CASE(kEncTeam64) }
-    else { ZC_ENC_CASE(kEncAny) }
+    if (shape == kEncSolo) { ZC_ENC_CASE(kEncSolo) }
+    else if (shape == kEncTeam) { ZC_ENC_CASE(kEncTeam) }
+    else if (shape == kEncAny) { ZC_ENC_CASE(kEncAny) }
+    else if (shape == kEncAny48) { ZC_ENC_CASE(kEncAny48) }
+    else { ZC_ENC_CASE(kEncBig) }
 #undef ZC_ENC_CASE
     return e;
 }
