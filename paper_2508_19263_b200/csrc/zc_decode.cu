@@ -26,6 +26,7 @@ struct DecParams {
     uint32_t spin_limit;     // polls after which a wait for a staged piece gives up
     uint32_t skip_copy;      // test hook: the copies of the pieces are not started
     uint32_t sliced;         // large chunks: pieces are staged slice by slice and lane by lane (see run_chunks)
+    uint32_t active;         // warps of a block that decode chunks (they share the pools); the others only help to build the tables
     unsigned long long call_id;
 };
 
@@ -56,6 +57,12 @@ constexpr uint32_t kDecMaxWarps = 28;              // 896 threads: 72 registers 
 constexpr uint32_t kDecMaxWarpsBoth = 20;          // 640 threads: 96 registers per thread
 template <int FMT, bool XOR>
 constexpr uint32_t dec_block_warps() { return (XOR || FMT == ZC_FMT_SCALE_U8) ? kDecMaxWarpsBoth : kDecMaxWarps; }
+// Launches of few chunks (at most kDecFewActive per SM) run kernels of their own: every SM takes a share of the chunks
+// however few they are, all 16 warps of a block build the tables, and only as many warps as the block has chunks decode,
+// each with room to stage whole pieces of both streams and with registers for two bit readers.  What such a launch takes
+// is one lane's serial walk over its subchunk: 16 chunks of 64 KiB with both streams coded (FP8) took 230 us as 16 warps of
+// one block that staged slices.
+constexpr uint32_t kDecFewWarps = 16, kDecFewActive = 8;
 constexpr uint32_t kDecFixedSmem = 2 * kLutBytes + kScratchBytes;
 constexpr uint32_t kSliceSyms = 128;               // symbols a lane decodes from one slice of its subchunk
 constexpr uint32_t kSliceBytes = 256;              // copied per slice: 15 bytes of alignment + 128 * 12 bits + the window's look-ahead fit
@@ -131,40 +138,42 @@ static __device__ bool build_lut(uint32_t my_len, uint32_t* lut, uint16_t* singl
         }
     }
     __syncthreads();
-    if (tid >= 1 && tid <= kLmax) {                              // thread l adds up length l over the 8 warps
+    if (warp == 0) {
+        // Lane l looks after length l: adds up its codes over the 8 warps; the rest are prefix sums over the lengths.
+        // weight = the share of the 2^12 windows that start with a code of length l (a code of length k < l takes 2^(l - k)
+        // values of length l, so the first value of length l is the weight of all shorter ones >> (12 - l)).
+        const uint32_t l = lane, use = l >= 1 && l <= kLmax;
         uint32_t cnt = 0;
-        for (uint32_t w = 0; w < 8; ++w) { const uint32_t t = b.wcount[w * 16 + tid]; b.wcount[w * 16 + tid] = cnt; cnt += t; }
-        b.count[tid] = cnt;
-    }
-    __syncthreads();
-    if (tid == 0) {
-        uint32_t code = 0, off = 0, active = 0;
-        uint32_t p[kLmax + 2];                                    // weight of length l in units of 2^-12
-        for (uint32_t l = 1; l <= kLmax; ++l) {
-            const uint32_t cnt = b.count[l];
-            code = (code + b.count[l - 1]) << 1;
-            b.first[l] = code;
-            b.offset[l] = off;
-            b.limit[l] = (code + cnt) << (kLmax - l);
-            off += cnt;
-            active += cnt;
-            p[l] = cnt << (kLmax - l);
-            // codes at or next to the length limit belong to symbols that are rarer than 2^-length says: the limit
-            // clipped them, or they are the never-seen symbols of a static dictionary
-            if (l + 1 >= kLmax) p[l] >>= 3;
+        if (use)
+            for (uint32_t w = 0; w < 8; ++w) { const uint32_t t = b.wcount[w * 16 + l]; b.wcount[w * 16 + l] = cnt; cnt += t; }
+        const uint32_t weight = use ? cnt << (kLmax - l) : 0u;
+        // weight of length l in units of 2^-12; codes at or next to the length limit belong to symbols that are rarer than
+        // 2^-length says: the limit clipped them, or they are the never-seen symbols of a static dictionary
+        const uint32_t p = l + 1 >= kLmax ? weight >> 3 : weight;
+        uint32_t sum_w = weight, sum_c = cnt, sum_p = p;
+#pragma unroll
+        for (int o = 1; o < 16; o <<= 1) {
+            const uint32_t xw = __shfl_up_sync(0xFFFFFFFFu, sum_w, o), xc = __shfl_up_sync(0xFFFFFFFFu, sum_c, o), xp = __shfl_up_sync(0xFFFFFFFFu, sum_p, o);
+            if (lane >= (uint32_t)o) { sum_w += xw; sum_c += xc; sum_p += xp; }
         }
-        const bool complete = b.limit[kLmax] == kLutEntries;      // Kraft sum is exactly one
-        const bool one = active == 1 && b.count[1] == 1;
-        if (!(complete || one || active == 0)) b.ok[0] = 0;
-        // probability (units of 2^-24) that two consecutive codes need more than 12 bits
-        uint64_t long_pairs = 0;
-        uint32_t tail = 0;                                        // sum of p[l2] for l2 >= 13 - l1
-        for (uint32_t l1 = 1; l1 <= kLmax; ++l1) {
-            tail += p[kLmax + 1 - l1];
-            long_pairs += (uint64_t)p[l1] * tail;
+        const uint32_t total = __shfl_sync(0xFFFFFFFFu, sum_w, kLmax), active = __shfl_sync(0xFFFFFFFFu, sum_c, kLmax);
+        const uint32_t all_p = __shfl_sync(0xFFFFFFFFu, sum_p, kLmax), shorter_p = __shfl_sync(0xFFFFFFFFu, sum_p, use ? kLmax - l : 0u);
+        const bool one = active == 1 && __shfl_sync(0xFFFFFFFFu, cnt, 1) == 1;
+        // probability (units of 2^-24) that two consecutive codes need more than 12 bits: the first is of length l, the
+        // second of length 13 - l or more
+        unsigned long long pairs = use ? (unsigned long long)p * (all_p - shorter_p) : 0ull;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) pairs += __shfl_xor_sync(0xFFFFFFFFu, pairs, o);
+        if (use) {
+            b.count[l] = cnt;
+            b.first[l] = (sum_w - weight) >> (kLmax - l);
+            b.offset[l] = sum_c - cnt;
+            b.limit[l] = (l == 1 && one) ? kLutEntries : sum_w;   // the unused half of the windows reads as the one symbol
         }
-        b.ok[1] = long_pairs <= (1ull << 24) / 32 ? 2u : 1u;
-        if (one) b.limit[1] = kLutEntries;                        // the unused half of the windows reads as the one symbol
+        if (lane == 0) {
+            if (!(total == kLutEntries || one || active == 0)) b.ok[0] = 0;      // Kraft sum is exactly one
+            b.ok[1] = pairs <= (1ull << 24) / 32 ? 2u : 1u;
+        }
     }
     __syncthreads();
     const uint32_t mode = b.ok[1];
@@ -436,7 +445,8 @@ struct DecShared {                   // what the block's prologue leaves for the
 template <bool V> struct BoolTag { static constexpr bool value = V; };
 
 // PPL = 16-symbol parts each lane merges per round = R / 16, R in {16, 32, 64}.
-template <int FMT, int PPL, bool H0, bool H1, bool XOR>
+// SIDE: the streams of chunks with both streams coded are decoded side by side.
+template <int FMT, int PPL, bool H0, bool H1, bool XOR, bool SIDE>
 __device__ __forceinline__ uint32_t run_chunks(const DecParams& P, const DecShared& S, uint8_t* pool, uint64_t* bar,
                                                uint32_t first_end0, uint32_t first_off0,
                                                uint32_t c, const uint32_t c_end, const uint32_t step,
@@ -639,8 +649,8 @@ __device__ __forceinline__ uint32_t run_chunks(const DecParams& P, const DecShar
                     const uint32_t done = r * R;
                     // a ragged end decodes up to 15 symbols too many (from the bits that follow); they are not used
                     const uint32_t n_quads = FULL ? (uint32_t)PPL : (n_my > done ? (min(R, n_my - done) + 15) / 16 : 0u);
-                    // (only in the kernels built for launches that expect two coded streams: they have the registers for it)
-                    constexpr bool kSideBySide = H0 && H1 && (XOR || FMT == ZC_FMT_SCALE_U8);
+                    // (only in the kernels that have the registers for it)
+                    constexpr bool kSideBySide = H0 && H1 && SIDE;
                     if (kSideBySide && n_quads && staged0 && staged1 && piece0 != 0 && piece1 != 0) {
                         // both streams come from staged pieces: their words are decoded side by side
                         const uint32_t wra_s = rows0_s + wr_off, wrb_s = rows1_s + wr_off;
@@ -753,7 +763,7 @@ struct DecSmem {                     // the block's dynamic shared memory, carve
     uint64_t* bar;                   // this warp's two mbarriers
 };
 
-__device__ __forceinline__ DecSmem carve_smem(uint8_t* smem, uint32_t pool_bytes)
+__device__ __forceinline__ DecSmem carve_smem(uint8_t* smem, uint32_t pool_bytes, uint32_t active)
 {
     const uint32_t warp = threadIdx.x >> 5, n_warps = blockDim.x >> 5;
     DecSmem m;
@@ -762,7 +772,7 @@ __device__ __forceinline__ DecSmem carve_smem(uint8_t* smem, uint32_t pool_bytes
     m.scratch = reinterpret_cast<uint32_t*>(smem + 2 * kLutBytes);
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem + kDecFixedSmem);
     m.pools = reinterpret_cast<uint8_t*>(bars + 2 * n_warps);
-    m.pool = m.pools + (size_t)warp * pool_bytes;
+    m.pool = m.pools + (size_t)min(warp, active - 1) * pool_bytes;
     m.bar = bars + 2 * warp;
     if ((threadIdx.x & 31) == 0) { mbar_init(&m.bar[0], 1); mbar_init(&m.bar[1], 1); }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -773,13 +783,13 @@ __device__ __forceinline__ DecSmem carve_smem(uint8_t* smem, uint32_t pool_bytes
 // Decodes the chunks c0, c0 + step, ... (< c_end) of one tensor with this warp; the whole block calls it
 // together (the header check and the table build are block-wide).  Returns a zc_status, the same in every
 // thread for the block-wide checks.
-template <int FMT, int PPL, bool XOR>
+template <int FMT, int PPL, bool XOR, bool SIDE>
 __device__ __forceinline__ uint32_t decode_one(const DecParams& P, const DecSmem& M, const uint32_t chunk_base, const uint32_t c_end,
                                                const uint32_t block_index, const uint32_t n_blocks, uint32_t& parity0, uint32_t& parity1)
 {
-    const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5, n_warps = blockDim.x >> 5;
-    // chunk chunk_base + k goes to block (k / n_warps) % n_blocks, warp k % n_warps
-    uint32_t c0 = chunk_base + block_index * n_warps + warp, step = n_blocks * n_warps;
+    const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    // chunk chunk_base + k goes to block k % n_blocks, warp (k / n_blocks) % P.active
+    uint32_t c0 = warp < P.active ? chunk_base + block_index + warp * n_blocks : c_end, step = n_blocks * P.active;
     const uint32_t sub_w = P.chunk_bytes <= 8192 ? 2u : 4u;     // bytes per sub_end entry
     const uint64_t tab_chunk = 256, tab_sub = 256 + (((uint64_t)4 * P.n_chunks + 15) & ~15ull);
     // Nearly every container has stream 0 coded, its table section right behind the header.  Its code lengths
@@ -863,10 +873,10 @@ __device__ __forceinline__ uint32_t decode_one(const DecParams& P, const DecSmem
     if (P.sliced && huff0 && huff1) {
         const uint32_t need = 2 * (512 * PPL + 32 * kSliceSlot);
         if (need > P.pool_bytes) {
-            const uint32_t active = max(1u, n_warps * P.pool_bytes / need);
+            const uint32_t active = max(1u, P.active * P.pool_bytes / need);
             pool = M.pools + (size_t)min(warp, active - 1) * need;
             pool_bytes = need;
-            c0 = warp < active ? chunk_base + block_index * active + warp : c_end;
+            c0 = warp < active ? chunk_base + block_index + warp * n_blocks : c_end;
             step = n_blocks * active;
             spec_end = spec_off = 0;
             if (c0 < c_end) {
@@ -887,22 +897,22 @@ __device__ __forceinline__ uint32_t decode_one(const DecParams& P, const DecSmem
         first_end0 = load_sub_end(P.comp + S.sec0 + tab_sub, sub_w, c0, lane);
         first_off0 = reinterpret_cast<const uint32_t*>(P.comp + S.sec0 + tab_chunk)[c0];
     }
-    if (huff0 && !huff1) return run_chunks<FMT, PPL, true, false, XOR>(P, S, pool, M.bar, first_end0, first_off0, c0, c_end, step, parity0, parity1);
-    if (!huff0 && !huff1) return run_chunks<FMT, PPL, false, false, XOR>(P, S, pool, M.bar, 0, 0, c0, c_end, step, parity0, parity1);
-    if (huff0) return run_chunks<FMT, PPL, true, true, XOR>(P, S, pool, M.bar, first_end0, first_off0, c0, c_end, step, parity0, parity1);
-    return run_chunks<FMT, PPL, false, true, XOR>(P, S, pool, M.bar, 0, 0, c0, c_end, step, parity0, parity1);
+    if (huff0 && !huff1) return run_chunks<FMT, PPL, true, false, XOR, SIDE>(P, S, pool, M.bar, first_end0, first_off0, c0, c_end, step, parity0, parity1);
+    if (!huff0 && !huff1) return run_chunks<FMT, PPL, false, false, XOR, SIDE>(P, S, pool, M.bar, 0, 0, c0, c_end, step, parity0, parity1);
+    if (huff0) return run_chunks<FMT, PPL, true, true, XOR, SIDE>(P, S, pool, M.bar, first_end0, first_off0, c0, c_end, step, parity0, parity1);
+    return run_chunks<FMT, PPL, false, true, XOR, SIDE>(P, S, pool, M.bar, 0, 0, c0, c_end, step, parity0, parity1);
 }
 
-// One tensor per launch: the warps of all blocks take the chunks in turn.
-template <int FMT, int PPL>
-__global__ void __launch_bounds__(dec_block_warps<FMT, false>() * 32, 1)
+// One tensor per launch: the warps of all blocks take the chunks in turn.  FEW: see kDecFewWarps.
+template <int FMT, int PPL, bool FEW>
+__global__ void __launch_bounds__((FEW ? kDecFewWarps : dec_block_warps<FMT, false>()) * 32, 1)
 decode_kernel(const __grid_constant__ DecParams P)
 {
     extern __shared__ __align__(16) uint8_t smem[];
-    const DecSmem M = carve_smem(smem, P.pool_bytes);
+    const DecSmem M = carve_smem(smem, P.pool_bytes, P.active);
     if (P.ctl && blockIdx.x == 0 && threadIdx.x == 0) P.ctl->call_id = P.call_id;
     uint32_t parity0 = 0, parity1 = 0;
-    const uint32_t err = decode_one<FMT, PPL, false>(P, M, P.c_begin, P.c_end, blockIdx.x, gridDim.x, parity0, parity1);
+    const uint32_t err = decode_one<FMT, PPL, false, FEW || FMT == ZC_FMT_SCALE_U8>(P, M, P.c_begin, P.c_end, blockIdx.x, gridDim.x, parity0, parity1);
     if (err) raise_status(P.ctl, P.call_id, err);
 }
 
@@ -914,7 +924,7 @@ __global__ void __launch_bounds__(dec_block_warps<FMT, XOR>() * 32, 1)
 decode_batch_kernel(const __grid_constant__ DecBatchParams B)
 {
     extern __shared__ __align__(16) uint8_t smem[];
-    const DecSmem M = carve_smem(smem, B.pool_bytes);
+    const DecSmem M = carve_smem(smem, B.pool_bytes, blockDim.x >> 5);
     if (blockIdx.x == 0 && threadIdx.x == 0 && B.tensor_base == 0) B.ctl->call_id = B.call_id;
     uint32_t parity0 = 0, parity1 = 0;
 
@@ -925,11 +935,11 @@ decode_batch_kernel(const __grid_constant__ DecBatchParams B)
         P.n_syms = B.item[t].n_syms; P.n_elems = B.item[t].n_elems; P.n_chunks = B.item[t].n_chunks;
         P.cs = B.cs; P.sub = B.sub; P.chunk_bytes = B.chunk_bytes; P.format = B.format; P.group = B.group;
         P.pool_bytes = B.pool_bytes; P.call_id = B.call_id; P.c_begin = 0; P.c_end = P.n_chunks;
-        P.spin_limit = B.spin_limit; P.skip_copy = B.skip_copy; P.sliced = B.sliced;
+        P.spin_limit = B.spin_limit; P.skip_copy = B.skip_copy; P.sliced = B.sliced; P.active = blockDim.x >> 5;
         const uint64_t tables = 256 + (((uint64_t)4 * P.n_chunks + 15) & ~15ull) + 32ull * (P.chunk_bytes <= 8192 ? 2u : 4u) * P.n_chunks;
         P.spec = P.comp_bytes >= kHeaderBytes + tables ? 1u : 0u;
         __syncthreads();                                         // everybody is done with the previous tensor's tables
-        const uint32_t err = decode_one<FMT, PPL, XOR>(P, M, seg_lo, seg_hi, 0, 1, parity0, parity1);
+        const uint32_t err = decode_one<FMT, PPL, XOR, XOR || FMT == ZC_FMT_SCALE_U8>(P, M, seg_lo, seg_hi, 0, 1, parity0, parity1);
         if (err && raise_status(B.ctl, B.call_id, err)) B.ctl->failed = B.tensor_base + t + 1;
     };
 
@@ -988,7 +998,7 @@ decode_batch_kernel(const __grid_constant__ DecBatchParams B)
 struct DecRanges { const void* in; size_t in_bytes; const void* out; size_t out_bytes; const void* ws; size_t ws_bytes; };
 
 template <int F>
-cudaError_t dec_launch_single_t(uint32_t ppl, uint32_t grid, uint32_t threads, size_t smem, cudaStream_t st, const DecParams& P,
+cudaError_t dec_launch_single_t(uint32_t ppl, bool few, uint32_t grid, uint32_t threads, size_t smem, cudaStream_t st, const DecParams& P,
                                 const DecRanges& R)
 {
     cudaError_t e = cudaSuccess;
@@ -1003,9 +1013,15 @@ cudaError_t dec_launch_single_t(uint32_t ppl, uint32_t grid, uint32_t threads, s
         kern<<<grid, threads, smem, st>>>(P);
         e = cudaGetLastError();
     };
-    if (ppl == 4) launch(decode_kernel<F, 4>);
-    else if (ppl == 2) launch(decode_kernel<F, 2>);
-    else launch(decode_kernel<F, 1>);
+    if (few) {
+        if (ppl == 4) launch(decode_kernel<F, 4, true>);
+        else if (ppl == 2) launch(decode_kernel<F, 2, true>);
+        else launch(decode_kernel<F, 1, true>);
+    } else {
+        if (ppl == 4) launch(decode_kernel<F, 4, false>);
+        else if (ppl == 2) launch(decode_kernel<F, 2, false>);
+        else launch(decode_kernel<F, 1, false>);
+    }
     return e;
 }
 
@@ -1038,7 +1054,7 @@ cudaError_t dec_launch_batch_t(uint32_t ppl, bool any_base, uint32_t grid, uint3
 }
 
 #define ZC_DEC_DECLARE(NAME)                                                                                              \
-    cudaError_t dec_launch_single_##NAME(uint32_t ppl, uint32_t grid, uint32_t threads, size_t smem, cudaStream_t st,     \
+    cudaError_t dec_launch_single_##NAME(uint32_t ppl, bool few, uint32_t grid, uint32_t threads, size_t smem, cudaStream_t st,     \
                                          const DecParams& P, const DecRanges& R);                                        \
     cudaError_t dec_launch_batch_##NAME(uint32_t ppl, bool any_base, uint32_t grid, uint32_t threads, size_t smem,        \
                                         cudaStream_t st, const DecBatchParams& B, const DecRanges& R);                   \
@@ -1055,9 +1071,9 @@ ZC_DEC_DECLARE(fp4)
 #define ZC_DEC_COUNTS(out) (void)(out)
 #endif
 #define ZC_DEC_DEFINE(NAME, F)                                                                                            \
-    cudaError_t dec_launch_single_##NAME(uint32_t ppl, uint32_t grid, uint32_t threads, size_t smem, cudaStream_t st,     \
+    cudaError_t dec_launch_single_##NAME(uint32_t ppl, bool few, uint32_t grid, uint32_t threads, size_t smem, cudaStream_t st,     \
                                          const DecParams& P, const DecRanges& R)                                         \
-    { return dec_launch_single_t<F>(ppl, grid, threads, smem, st, P, R); }                                                \
+    { return dec_launch_single_t<F>(ppl, few, grid, threads, smem, st, P, R); }                                                \
     cudaError_t dec_launch_batch_##NAME(uint32_t ppl, bool any_base, uint32_t grid, uint32_t threads, size_t smem,        \
                                         cudaStream_t st, const DecBatchParams& B, const DecRanges& R)                    \
     { return dec_launch_batch_t<F>(ppl, any_base, grid, threads, smem, st, B, R); }                                       \
@@ -1124,6 +1140,26 @@ zc_status dec_shape(const zc_plan_t* p, bool both_coded, DecShape* out)
     return ZC_OK;
 }
 
+// Launch shape for n_chunks chunks of one tensor when they are few: `warps` build the tables, `active` of them decode.
+DecShape few_shape(const zc_plan_t* p, uint32_t n_chunks, uint32_t* active)
+{
+    DecShape s{};
+    s.ppl = (p->syms_per_sub % 64 == 0) ? 4 : (p->syms_per_sub % 32 == 0) ? 2 : 1;
+    s.warps = kDecFewWarps;
+    const size_t slack = (size_t)round_up(p->syms_per_sub + p->syms_per_sub / 2 + 16, 16);
+    const size_t room = kMaxSmem - 1024 - kDecFixedSmem - 512 - 16 * s.warps - slack;
+    *active = std::max<uint32_t>(1, (n_chunks + sm_count() - 1) / sm_count());
+    // rows of both streams and room for whole pieces of 12-bit codes (less when the warps' shares are smaller: slices then)
+    const uint32_t most = 2 * (512 * s.ppl + (uint32_t)round_up((uint64_t)p->syms_per_chunk * kLmax / 8, 16) + 32);
+    const uint32_t share = (uint32_t)(room / *active) & ~15u;
+    s.pool_bytes = std::max<uint32_t>(std::min(most, share), 8192);          // the table build uses 8 KiB of the pools
+    // slices only where whole pieces might not fit (then the pools fill the block's memory, as decode_one's sharing of them
+    // among fewer warps expects)
+    s.sliced = share < most && p->syms_per_sub % kSliceSyms == 0 ? 1u : 0u;
+    s.smem = kDecFixedSmem + 16 * s.warps + (size_t)*active * s.pool_bytes + slack;
+    return s;
+}
+
 // no clearing of the workspace: errors are tagged with the id of the call that raised them
 unsigned long long new_call_id()
 {
@@ -1179,8 +1215,15 @@ zc_status zc_decompress_chunks(const zc_plan_t* p, const void* d_comp, size_t co
     if (comp_bytes < kHeaderBytes) return ZC_E_CORRUPT;
     cudaStream_t st = (cudaStream_t)cuda_stream;
     DecShape shape;
-    const zc_status ss = dec_shape(p, false, &shape);
-    if (ss != ZC_OK) return ss;
+    uint32_t active = 0;
+    const bool few = n_chunks <= kDecFewActive * (uint32_t)sm_count();
+    if (few) {
+        shape = few_shape(p, n_chunks, &active);
+    } else {
+        const zc_status ss = dec_shape(p, false, &shape);
+        if (ss != ZC_OK) return ss;
+        active = shape.warps;
+    }
     DecParams P{};
     P.comp = (const uint8_t*)d_comp;
     P.base = nullptr;
@@ -1194,21 +1237,21 @@ zc_status zc_decompress_chunks(const zc_plan_t* p, const void* d_comp, size_t co
     P.call_id = new_call_id();
     P.spec = comp_bytes >= kHeaderBytes + table_section_bytes(p->n_chunks, p->chunk_bytes) ? 1u : 0u;
     P.pool_bytes = shape.pool_bytes;
-    P.spin_limit = test_knobs().spin_limit; P.skip_copy = test_knobs().skip_copy; P.sliced = shape.sliced;
+    P.spin_limit = test_knobs().spin_limit; P.skip_copy = test_knobs().skip_copy; P.sliced = shape.sliced; P.active = active;
     const uint32_t warps = shape.warps, ppl = shape.ppl;
     const size_t smem = shape.smem;
     // at least one block even for an empty range: the header is still checked
-    const uint32_t want = std::max<uint32_t>((n_chunks + warps - 1) / warps, 1);
+    const uint32_t want = std::max<uint32_t>(few ? n_chunks : (n_chunks + warps - 1) / warps, 1);
     const uint32_t grid = std::min<uint32_t>(want, (uint32_t)sm_count());
     const DecRanges R{d_comp, comp_bytes, d_out,
                       (size_t)std::min<uint64_t>((uint64_t)n_chunks * p->chunk_bytes, p->input_bytes - (uint64_t)first_chunk * p->chunk_bytes),
                       d_workspace, sizeof(Control)};
     cudaError_t e;
     switch (p->format) {
-    case ZC_FMT_BF16: e = dec_launch_single_bf16(ppl, grid, warps * 32, smem, st, P, R); break;
-    case ZC_FMT_FP8_E4M3: case ZC_FMT_FP8_E5M2: e = dec_launch_single_fp8(ppl, grid, warps * 32, smem, st, P, R); break;
-    case ZC_FMT_SCALE_U8: e = dec_launch_single_scale(ppl, grid, warps * 32, smem, st, P, R); break;
-    default: e = dec_launch_single_fp4(ppl, grid, warps * 32, smem, st, P, R); break;
+    case ZC_FMT_BF16: e = dec_launch_single_bf16(ppl, few, grid, warps * 32, smem, st, P, R); break;
+    case ZC_FMT_FP8_E4M3: case ZC_FMT_FP8_E5M2: e = dec_launch_single_fp8(ppl, few, grid, warps * 32, smem, st, P, R); break;
+    case ZC_FMT_SCALE_U8: e = dec_launch_single_scale(ppl, few, grid, warps * 32, smem, st, P, R); break;
+    default: e = dec_launch_single_fp4(ppl, few, grid, warps * 32, smem, st, P, R); break;
     }
     return e == cudaSuccess ? ZC_OK : ZC_E_CUDA;
 }
