@@ -31,7 +31,7 @@ struct DecParams {
 };
 
 // One tensor of a batch, and the parameters of a batched launch.  The tensors share format and chunk size;
-// the chunks of all of them form one index space that is cut into equal contiguous ranges, one per block.
+// the chunks of all of them form one index space that is cut into contiguous ranges (see kDecMaxRounds).
 struct DecItem {
     const uint8_t* comp;
     const uint8_t* base;
@@ -39,12 +39,19 @@ struct DecItem {
     uint64_t comp_bytes, input_bytes, n_syms, n_elems;
     uint32_t n_chunks, first_chunk;          // first_chunk = chunks of all earlier tensors of the launch
 };
+// The chunk index space of a batched launch is dealt out in rounds, every round in as many equal contiguous ranges as there
+// are blocks; the blocks take ranges from a ticket counter.  The first round is most of it and the others shrink, so that
+// blocks end together although tensors, and SMs, differ in how fast they get through a range.  A range costs a block about
+// 12 us (waiting for its last warp, header, tables, first pieces), so there are few: with eight equal ones per block the
+// BF16 stack of 1.74 GB took 707 us.
+constexpr uint32_t kDecMaxRounds = 5;
 constexpr uint32_t kDecBatchMax = 448;       // tensors per launch: the parameter block stays below 32 KiB
 struct DecBatchParams {
     Control* ctl;
     unsigned long long call_id;
     uint32_t cs, sub, chunk_bytes, format, group, pool_bytes;
-    uint32_t n_tensors, total_chunks, tensor_base, n_ranges;
+    uint32_t n_tensors, total_chunks, tensor_base, n_rounds;
+    uint32_t round_end[kDecMaxRounds];       // chunks of the first rounds
     uint32_t spin_limit, skip_copy, sliced;
     DecItem item[kDecBatchMax];
 };
@@ -943,9 +950,8 @@ decode_batch_kernel(const __grid_constant__ DecBatchParams B)
         if (err && raise_status(B.ctl, B.call_id, err)) B.ctl->failed = B.tensor_base + t + 1;
     };
 
-    // The concatenated chunk index space is cut into n_ranges equal ranges which the blocks take one after the
-    // other from a ticket counter (tensors, and SMs, differ in how fast they get through a range).  Block 0
-    // first walks over the tensors without chunks: their headers are still checked.
+    // The ranges of all rounds come one after the other from a ticket counter.  Block 0 first walks over the tensors without
+    // chunks: their headers are still checked.
     __shared__ uint32_t s_range;
     uint32_t empties = blockIdx.x == 0 ? 0u : B.n_tensors;      // cursor of that walk
     uint32_t t = 0, g = 0, g_hi = 0;
@@ -961,9 +967,11 @@ decode_batch_kernel(const __grid_constant__ DecBatchParams B)
                 if (threadIdx.x == 0) s_range = atomicAdd(&B.ctl->ticket, 1u);
                 __syncthreads();
                 const uint32_t r = s_range;
-                if (r >= B.n_ranges) break;
-                g = (uint32_t)((uint64_t)r * B.total_chunks / B.n_ranges);
-                g_hi = (uint32_t)((uint64_t)(r + 1) * B.total_chunks / B.n_ranges);
+                const uint32_t round = r / gridDim.x, j = r % gridDim.x;
+                if (round >= B.n_rounds) break;
+                const uint32_t lo_c = round ? B.round_end[round - 1] : 0u, n_c = B.round_end[round] - lo_c;
+                g = lo_c + (uint32_t)((uint64_t)j * n_c / gridDim.x);
+                g_hi = lo_c + (uint32_t)((uint64_t)(j + 1) * n_c / gridDim.x);
                 // the last tensor that starts at or before g (tensors without chunks share their start with the next one)
                 uint32_t lo = 0, hi = B.n_tensors;
                 while (hi - lo > 1) {
@@ -1307,21 +1315,26 @@ zc_status zc_decompress_batch_xor(uint32_t n_tensors, const zc_plan_t* const* pl
             ++n;
         }
         B.n_tensors = n; B.total_chunks = (uint32_t)total;
-        uint32_t with_chunks = 0;
-        for (uint32_t i = 0; i < n; ++i) with_chunks += B.item[i].n_chunks != 0;
-        // enough blocks for one chunk per warp, and (many small tensors, say the K/V pages of a step) for one
-        // tensor per block, so that their tables are built side by side
-        const uint32_t want = std::max<uint32_t>({(uint32_t)((total + shape.warps - 1) / shape.warps), with_chunks, 1u});
-        const uint32_t grid = std::min<uint32_t>(want, (uint32_t)sm_count());
-        // up to 8 ranges per block, none shorter than 16 chunks per warp (a range costs a table build); with fewer
-        // tensors than blocks, one range per tensor at least
-        B.n_ranges = grid * (uint32_t)std::min<uint64_t>(8, std::max<uint64_t>(1, total / ((uint64_t)grid * shape.warps * 16)));
-        if (with_chunks <= grid) B.n_ranges = std::max<uint32_t>(B.n_ranges, with_chunks);
-        B.n_ranges = (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>(B.n_ranges, total));
-        // the ranges are handed out through the ticket word of the control block
-        if (cudaMemsetAsync(&B.ctl->ticket, 0, sizeof(uint32_t), st) != cudaSuccess) return ZC_E_CUDA;
+        // one block per SM unless there are fewer chunks (a lane's walk over its subchunk is what a small launch takes, so
+        // its chunks are spread as far as they go)
+        const uint32_t grid = std::max<uint32_t>(1, std::min<uint32_t>((uint32_t)std::min<uint64_t>(total, 0xFFFFFFFFu), (uint32_t)sm_count()));
         bool any_base = false;
         for (uint32_t i = 0; i < n; ++i) any_base = any_base || B.item[i].base != nullptr;
+        // Rounds: three quarters (deltas: half, since unchanged stretches take a fraction of the time) of what is left go to the
+        // next one, in whole chunks per warp, until a range is down to two chunks per warp; the last one takes the rest.  With
+        // fewer than 32 chunks per warp in all, another range costs more than it evens out (FP8 at 16 KiB chunks, 9 chunks per
+        // warp: 219 us in one round, 270 us in three).
+        const uint64_t turn = (uint64_t)grid * shape.warps;      // one chunk per warp
+        uint64_t done = 0;
+        B.n_rounds = 0;
+        while (done < total) {
+            const uint64_t left = total - done, part = (any_base ? left / 2 : left - left / 4) / turn * turn;
+            const bool last = B.n_rounds + 1 == kDecMaxRounds || total < 32 * turn || left - part < turn || part < 2 * turn;
+            done = last ? total : done + part;
+            B.round_end[B.n_rounds++] = (uint32_t)done;
+        }
+        // the ranges are handed out through the ticket word of the control block
+        if (cudaMemsetAsync(&B.ctl->ticket, 0, sizeof(uint32_t), st) != cudaSuccess) return ZC_E_CUDA;
         DecRanges R{nullptr, 0, nullptr, 0, d_workspace, sizeof(Control)};
 #if ZC_DEBUG_CHECKS
         DbgHull rd, wr;
