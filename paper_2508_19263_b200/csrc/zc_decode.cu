@@ -621,11 +621,14 @@ __device__ __forceinline__ uint32_t run_chunks(const DecParams& P, const DecShar
             uint32_t pos0 = 0, pos1 = 0, w00 = 0, w01 = 0, w10 = 0, w11 = 0, next0 = 0, next1 = 0;
             uint32_t lim0 = 0, lim1 = 0;
             for (uint32_t r = 0; r <= last_r; ++r) {
-                // ---- raw sign+mantissa bytes of this round go to registers before the decoding starts ----
+                // ---- what this round is merged with (raw stream, base tensor) travels to the L2 while it is decoded ----
 #pragma unroll
-                for (int i = 0; i < PPL; ++i)
+                for (int i = 0; i < PPL; ++i) {
                     if (!H1 && (FULL || k_lane + i * k_step + r * R < c_syms))
                         asm volatile("prefetch.global.L2 [%0];" :: "l"(raw1 + i * k_step + r * R));
+                    if (XOR && P.base && (FULL || 2 * (k_lane + i * k_step + r * R) < out_bytes))
+                        asm volatile("prefetch.global.L2 [%0];" :: "l"(P.base + (dst_lane - P.out) + 2 * (i * k_step + r * R)));
+                }
                 if (kHuff && (sliced0 || sliced1) && r % kRoundsPerSlice == 0) {
                     // the slice requested after the previous one was used up (or, for the chunk's first one, while
                     // the chunk before was merged) is needed now
@@ -733,7 +736,8 @@ __device__ __forceinline__ uint32_t run_chunks(const DecParams& P, const DecShar
                     uint8_t* dst = dst_lane + 2 * (i * k_step + r * R);
                     if (XOR && P.base) {                              // delta form: XOR the base tensor back in
                         const uint64_t off = (uint64_t)(dst - P.out);
-                        const uint4 b0 = load16_guarded(P.base, off, P.input_bytes), b1 = load16_guarded(P.base, off + 16, P.input_bytes);
+                        const uint4 b0 = FULL ? ld_nc_v4(P.base + off) : load16_guarded(P.base, off, P.input_bytes);
+                        const uint4 b1 = FULL ? ld_nc_v4(P.base + off + 16) : load16_guarded(P.base, off + 16, P.input_bytes);
                         o[0] ^= b0.x; o[1] ^= b0.y; o[2] ^= b0.z; o[3] ^= b0.w;
                         o[4] ^= b1.x; o[5] ^= b1.y; o[6] ^= b1.z; o[7] ^= b1.w;
                     }
