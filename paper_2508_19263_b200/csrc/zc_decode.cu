@@ -493,6 +493,7 @@ __device__ __forceinline__ uint32_t run_chunks(const DecParams& P, const DecShar
     const uint32_t rl = lane / PPL, rq = lane % PPL;
     const uint32_t rd_off = 16 * (rl * PPL + (rq ^ ((rl >> (3 - kLog)) & (PPL - 1))));   // part i: + 512 * i
     uint32_t err = 0;
+    const bool out32 = ((uintptr_t)P.out & 16) == 0;           // chunks start at multiples of 1024 bytes behind it
 
     // this lane's parts of a round: part i covers symbols k_lane + i * k_step (+ round offset) of the chunk
     const uint32_t k_lane = rl * P.sub + rq * 16, k_step = (32 / PPL) * P.sub;
@@ -742,7 +743,12 @@ __device__ __forceinline__ uint32_t run_chunks(const DecParams& P, const DecShar
                         o[4] ^= b1.x; o[5] ^= b1.y; o[6] ^= b1.z; o[7] ^= b1.w;
                     }
                     if (FULL || 2 * k + 32 <= out_bytes) {
-                        st_cs_v8(dst, o);
+                        if (out32) {
+                            st_cs_v8(dst, o);
+                        } else {                                 // an output that is aligned to 16 bytes only
+                            st_cs_v4(dst, make_uint4(o[0], o[1], o[2], o[3]));
+                            st_cs_v4(dst + 16, make_uint4(o[4], o[5], o[6], o[7]));
+                        }
                     } else {
 #pragma unroll
                         for (int t = 0; t < 32; ++t)

@@ -165,3 +165,25 @@ def test_largest_chunk_size_with_both_streams_coded(fmt):
     zc.decompress(p, d_out, nbytes, d_back, ws)
     assert zc.device_status(p, ws) == zc.OK
     assert np.array_equal(d_back.cpu().numpy(), data[: p.input_bytes])
+
+
+@pytest.mark.parametrize("batched", [False, True])
+def test_output_aligned_to_16_bytes_only(batched):
+    fmt, chunk_bytes, n = zc.FMT_BF16, 4096, 5 * 2048 + 77
+    data = _bf16_weights(n, 31)
+    cont = _oracle_container(fmt, data, n, chunk_bytes)
+    p = zc.plan(fmt, n, chunk_bytes)
+    buf = torch.full((p.input_bytes + 64,), 0xEE, dtype=torch.uint8, device=DEV)
+    assert buf.data_ptr() % 32 == 0
+    d_out = buf[16: 16 + p.input_bytes]
+    d_comp = torch.from_numpy(cont).to(DEV)
+    ws = torch.zeros(256, dtype=torch.uint8, device=DEV)
+    if batched:
+        zc.decompress_batch(zc.DecompressBatch([p], [d_comp], [cont.size], [d_out]), ws)
+        assert zc.batch_status(ws) == (zc.OK, None)
+    else:
+        zc.decompress(p, d_comp, cont.size, d_out, ws)
+        assert zc.device_status(p, ws) == zc.OK
+    back = buf.cpu().numpy()
+    assert np.array_equal(back[16: 16 + p.input_bytes], data[: p.input_bytes])
+    assert (back[:16] == 0xEE).all() and (back[16 + p.input_bytes:] == 0xEE).all()
