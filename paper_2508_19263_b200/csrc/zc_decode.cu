@@ -26,6 +26,7 @@ struct DecParams {
     uint32_t spin_limit;     // polls after which a wait for a staged piece gives up
     uint32_t skip_copy;      // test hook: the copies of the pieces are not started
     uint32_t sliced;         // large chunks: pieces are staged slice by slice and lane by lane (see run_chunks)
+    uint32_t groups;         // decode_split_kernel: blocks a chunk's subchunks are dealt to (1, 2, 4 or 8)
     uint32_t active;         // warps of a block that decode chunks (they share the pools); the others only help to build the tables
     unsigned long long call_id;
 };
@@ -70,6 +71,7 @@ constexpr uint32_t dec_block_warps() { return (XOR || FMT == ZC_FMT_SCALE_U8) ? 
 // is one lane's serial walk over its subchunk: 16 chunks of 64 KiB with both streams coded (FP8) took 230 us as 16 warps of
 // one block that staged slices.
 constexpr uint32_t kDecFewWarps = 16, kDecFewActive = 8;
+constexpr int kDecMany = 0, kDecFew = 1, kDecSplit = 2;   // kernels of a single-tensor launch
 constexpr uint32_t kDecFixedSmem = 2 * kLutBytes + kScratchBytes;
 constexpr uint32_t kSliceSyms = 128;               // symbols a lane decodes from one slice of its subchunk
 constexpr uint32_t kSliceBytes = 256;              // copied per slice: 15 bytes of alignment + 128 * 12 bits + the window's look-ahead fit
@@ -797,29 +799,21 @@ __device__ __forceinline__ DecSmem carve_smem(uint8_t* smem, uint32_t pool_bytes
     return m;
 }
 
-// Decodes the chunks c0, c0 + step, ... (< c_end) of one tensor with this warp; the whole block calls it
-// together (the header check and the table build are block-wide).  Returns a zc_status, the same in every
-// thread for the block-wide checks.
-template <int FMT, int PPL, bool XOR, bool SIDE>
-__device__ __forceinline__ uint32_t decode_one(const DecParams& P, const DecSmem& M, const uint32_t chunk_base, const uint32_t c_end,
-                                               const uint32_t block_index, const uint32_t n_blocks, uint32_t& parity0, uint32_t& parity1)
+struct DecOpened {                   // what open_container leaves
+    DecShared S;
+    bool huff0, huff1;
+};
+
+// Checks the header against the plan and builds the decode tables of the coded streams; the whole block calls it.  Returns a
+// zc_status, the same in every thread.
+__device__ __forceinline__ uint32_t open_container(const DecParams& P, const DecSmem& M, DecOpened& H)
 {
     const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    // chunk chunk_base + k goes to block k % n_blocks, warp (k / n_blocks) % P.active
-    uint32_t c0 = warp < P.active ? chunk_base + block_index + warp * n_blocks : c_end, step = n_blocks * P.active;
     const uint32_t sub_w = P.chunk_bytes <= 8192 ? 2u : 4u;     // bytes per sub_end entry
-    const uint64_t tab_chunk = 256, tab_sub = 256 + (((uint64_t)4 * P.n_chunks + 15) & ~15ull);
-    // Nearly every container has stream 0 coded, its table section right behind the header.  Its code lengths
-    // and this warp's first table entries are requested now, together with the header, and thrown away if the
-    // header says otherwise.
-    uint32_t spec_len = 0, spec_end = 0, spec_off = 0;
-    if (P.spec) {
-        if (threadIdx.x < 256) spec_len = P.comp[kHeaderBytes + threadIdx.x];
-        if (c0 < c_end) {
-            spec_end = load_sub_end(P.comp + kHeaderBytes + tab_sub, sub_w, c0, lane);
-            spec_off = reinterpret_cast<const uint32_t*>(P.comp + kHeaderBytes + tab_chunk)[c0];
-        }
-    }
+    // Nearly every container has stream 0 coded, its table section right behind the header.  Its code lengths are requested
+    // together with the header, and thrown away if the header says otherwise.
+    uint32_t spec_len = 0;
+    if (P.spec && threadIdx.x < 256) spec_len = P.comp[kHeaderBytes + threadIdx.x];
     // ---- header check against the plan ----
     __shared__ uint32_t s_mode[2], s_per_lookup[2];
     __shared__ uint32_t s_ok;
@@ -863,17 +857,17 @@ __device__ __forceinline__ uint32_t decode_one(const DecParams& P, const DecSmem
     __syncthreads();
     if (!s_ok) return ZC_E_CORRUPT;
 
-    const bool huff0 = s_mode[0] == ZC_MODE_HUFF, huff1 = s_mode[1] == ZC_MODE_HUFF;
+    H.huff0 = s_mode[0] == ZC_MODE_HUFF; H.huff1 = s_mode[1] == ZC_MODE_HUFF;
     {
         // the warps' pools are free until the chunk loop: 8 KiB of them hold the one-symbol scratch table
         uint16_t* single = reinterpret_cast<uint16_t*>(M.pools);
         bool tables_ok = true;
-        if (huff0) {
+        if (H.huff0) {
             uint32_t len = spec_len;                             // stream 0's section always starts behind the header
             if (!P.spec && threadIdx.x < 256) len = P.comp[s_sec[0] + threadIdx.x];
             tables_ok = build_lut(len, M.lut0, single, M.scratch, &s_per_lookup[0]) && tables_ok;
         }
-        if (huff1) {
+        if (H.huff1) {
             uint32_t len = 0;
             if (threadIdx.x < 256) len = P.comp[s_sec[1] + threadIdx.x];
             tables_ok = build_lut(len, M.lut1, single, M.scratch, &s_per_lookup[1]) && tables_ok;
@@ -881,7 +875,38 @@ __device__ __forceinline__ uint32_t decode_one(const DecParams& P, const DecSmem
         __syncthreads();
         if (!tables_ok) return ZC_E_CORRUPT;
     }
+    H.S.pool_bytes = P.pool_bytes;
+    H.S.lut0_s = smem_u32(M.lut0); H.S.lut1_s = smem_u32(M.lut1);
+    H.S.pairs0 = H.huff0 && s_per_lookup[0] == 2;
+    H.S.pairs1 = H.huff1 && s_per_lookup[1] == 2;
+    H.S.sec0 = s_sec[0]; H.S.sec1 = s_sec[1];
+    H.S.payload_off = s_payload_off; H.S.payload_bytes = s_payload_bytes;
+    return ZC_OK;
+}
 
+// Decodes the chunks c0, c0 + step, ... (< c_end) of one tensor with this warp; the whole block calls it
+// together (the header check and the table build are block-wide).  Returns a zc_status, the same in every
+// thread for the block-wide checks.
+template <int FMT, int PPL, bool XOR, bool SIDE>
+__device__ __forceinline__ uint32_t decode_one(const DecParams& P, const DecSmem& M, const uint32_t chunk_base, const uint32_t c_end,
+                                               const uint32_t block_index, const uint32_t n_blocks, uint32_t& parity0, uint32_t& parity1)
+{
+    const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    // chunk chunk_base + k goes to block k % n_blocks, warp (k / n_blocks) % P.active
+    uint32_t c0 = warp < P.active ? chunk_base + block_index + warp * n_blocks : c_end, step = n_blocks * P.active;
+    const uint32_t sub_w = P.chunk_bytes <= 8192 ? 2u : 4u;     // bytes per sub_end entry
+    const uint64_t tab_chunk = 256, tab_sub = 256 + (((uint64_t)4 * P.n_chunks + 15) & ~15ull);
+    // this warp's first table entries, on the guess that stream 0 is coded (see open_container)
+    uint32_t spec_end = 0, spec_off = 0;
+    if (P.spec && c0 < c_end) {
+        spec_end = load_sub_end(P.comp + kHeaderBytes + tab_sub, sub_w, c0, lane);
+        spec_off = reinterpret_cast<const uint32_t*>(P.comp + kHeaderBytes + tab_chunk)[c0];
+    }
+    DecOpened H;
+    const uint32_t opened = open_container(P, M, H);
+    if (opened != ZC_OK) return opened;
+    const bool huff0 = H.huff0, huff1 = H.huff1;
+    DecShared& S = H.S;
     // Large chunks with both streams coded: a warp's pool was sized for one coded stream's lane slots (the plan
     // does not say how many streams a container codes); fewer warps then share the block's pools, each with room
     // for both, and the chunks are dealt to those warps only.
@@ -902,13 +927,7 @@ __device__ __forceinline__ uint32_t decode_one(const DecParams& P, const DecSmem
             }
         }
     }
-    DecShared S;
     S.pool_bytes = pool_bytes;
-    S.lut0_s = smem_u32(M.lut0); S.lut1_s = smem_u32(M.lut1);
-    S.pairs0 = huff0 && s_per_lookup[0] == 2;
-    S.pairs1 = huff1 && s_per_lookup[1] == 2;
-    S.sec0 = s_sec[0]; S.sec1 = s_sec[1];
-    S.payload_off = s_payload_off; S.payload_bytes = s_payload_bytes;
     uint32_t first_end0 = spec_end, first_off0 = spec_off;
     if (huff0 && !P.spec && c0 < c_end) {
         first_end0 = load_sub_end(P.comp + S.sec0 + tab_sub, sub_w, c0, lane);
@@ -931,6 +950,239 @@ decode_kernel(const __grid_constant__ DecParams P)
     uint32_t parity0 = 0, parity1 = 0;
     const uint32_t err = decode_one<FMT, PPL, false, FEW || FMT == ZC_FMT_SCALE_U8>(P, M, P.c_begin, P.c_end, blockIdx.x, gridDim.x, parity0, parity1);
     if (err) raise_status(P.ctl, P.call_id, err);
+}
+
+// Launches of a few large chunks (see zc_decompress_chunks).  A lane's walk over its subchunk is serial, 1024 symbols at
+// 64 KiB, and with a few chunks most of the GPU would watch.  Here a block takes a group of a chunk's subchunks, and every
+// subchunk is cut into `parts` stretches of equal bits, a thread each: every thread decodes from its cut on, as if a code
+// started there, up to the first code boundary at or behind the next cut, and counts.  Prefix codes find back into step within
+// some codes, so where a thread ends is nearly always right even if it began inside a code; where its predecessor ended is
+// where it must begin, and the threads whose beginning was wrong decode once more until nothing changes (the first is right
+// from the start, so that ends after `parts` rounds whatever the payload is).  A code whose codes all have one length never
+// finds back into step; its cuts are multiples of that length.  Then everybody's symbols have their place, and a last pass
+// writes them.
+// 1 MiB FP8 tensor, 64 KiB chunks, both streams coded: 63 us with a lane per subchunk (decode_kernel), 50 us here (its nearly
+// uniform sign+mantissa code finds back into step late); one stream coded 57 against 25 us.
+struct SplitBits {                   // 33 to 64 bits of the payload from the current position on, and the word behind them
+    uint32_t hi, lo, n, next, addr;
+};
+__device__ __forceinline__ void split_start(SplitBits& B, uint32_t base_s, uint32_t at)
+{
+    B.addr = base_s + 4 * (at >> 5);
+    const uint32_t w0 = lds32(B.addr), w1 = lds32(B.addr + 4);
+    B.next = lds32(B.addr + 8);
+    B.hi = __funnelshift_l(w1, w0, at);
+    B.lo = w1 << (at & 31u);
+    B.n = 64 - (at & 31u);
+    B.addr += 12;
+}
+// back to 33 bits and more; two codes (of at most 12 bits, or whatever four bits of a damaged table say) fit between two calls
+__device__ __forceinline__ void split_refill(SplitBits& B)
+{
+    if (B.n <= 32) {
+        B.hi |= B.n == 32 ? 0u : B.next >> (B.n & 31u);
+        B.lo = B.n == 32 ? B.next : B.next << (32 - B.n);
+        B.n += 32;
+        B.next = lds32(B.addr);
+        B.addr += 4;
+    }
+}
+// the table entry of the code at the current position; the position moves behind it
+__device__ __forceinline__ uint32_t split_code(SplitBits& B, uint32_t lut_s, uint32_t len_shift, uint32_t& pos)
+{
+    const uint32_t e = lut_peek(B.hi, lut_s), l = (e >> len_shift) & 15u;
+    B.hi = __funnelshift_l(B.lo, B.hi, l);
+    B.lo <<= l;
+    B.n -= l;
+    pos += l;
+    return e;
+}
+
+constexpr uint32_t kSplitThreads = 512;
+// Shortest subchunk it is used for (chunks from 32 KiB on).  With one coded stream, 16 chunks of BF16 weights, here against
+// decode_kernel: 16 KiB 24.6 / 18.4 us, 32 KiB 25.4 / 30.6 us, 64 KiB 26.6 / 51 us.
+constexpr uint32_t kSplitMinSub = 512;
+
+template <int FMT>
+__global__ void __launch_bounds__(kSplitThreads, 1)
+decode_split_kernel(const __grid_constant__ DecParams P)
+{
+    extern __shared__ __align__(16) uint8_t smem[];
+    __shared__ uint32_t s_end[2][32], s_off[2], s_lens[2];
+    const DecSmem M = carve_smem(smem, P.pool_bytes, 1);
+    const uint32_t tid = threadIdx.x, lane = tid & 31;
+    uint64_t* const bars = M.bar - 2 * (tid >> 5);               // the first warp's: one per stream
+    if (tid < 2) s_lens[tid] = 0;
+    if (P.ctl && blockIdx.x == 0 && tid == 0) P.ctl->call_id = P.call_id;
+    DecOpened H;
+    const uint32_t opened = open_container(P, M, H);
+    if (opened != ZC_OK) { raise_status(P.ctl, P.call_id, opened); return; }
+    const DecShared& S = H.S;
+    const bool coded[2] = {H.huff0, H.huff1};
+    const uint32_t sub_w = P.chunk_bytes <= 8192 ? 2u : 4u;
+    const uint64_t tab_chunk = 256, tab_sub = 256 + (((uint64_t)4 * P.n_chunks + 15) & ~15ull);
+    // my work: subchunks g_lo .. g_lo + g_subs - 1 of chunk c
+    const uint32_t g_subs = 32 / P.groups, c = P.c_begin + blockIdx.x / P.groups, g_lo = (blockIdx.x % P.groups) * g_subs;
+    const uint64_t c_lo = (uint64_t)c * P.cs;
+    const uint32_t c_syms = c < P.c_end ? (uint32_t)min((uint64_t)P.cs, P.n_syms - c_lo) : 0u;
+    const uint32_t out_bytes = c < P.c_end ? (uint32_t)min((uint64_t)P.chunk_bytes, P.input_bytes - 2 * c_lo) : 0u;
+    if (c_syms <= g_lo * P.sub) return;                          // nothing of the (ragged) chunk is in my group; block-uniform
+    // pool: the group's symbols of both streams, then its pieces (12 bits per symbol and 48 bytes each)
+    const uint32_t g_syms = g_subs * P.sub, syms_s = smem_u32(M.pools), piece_room = ((g_syms + g_syms / 2 + 15) & ~15u) + 48;
+    const uint32_t pieces_s = syms_s + 2 * g_syms;
+
+    // ---- table entries (warp 0: stream 0, warp 1: stream 1), checked before anything is staged; code lengths in use ----
+    bool bad = false;
+    if (tid < 64 && coded[tid >> 5]) {
+        const uint32_t s = tid >> 5;
+        const uint8_t* sec = P.comp + (s == 0 ? S.sec0 : S.sec1);
+        const uint32_t end = load_sub_end(sec + tab_sub, sub_w, c, lane), off16 = reinterpret_cast<const uint32_t*>(sec + tab_chunk)[c];
+        uint32_t start = __shfl_up_sync(0xFFFFFFFFu, end, 1);
+        if (lane == 0) start = 0;
+        const uint32_t piece16 = (__shfl_sync(0xFFFFFFFFu, end, 31) + 127) / 128;
+        bad = !(start <= end && end - start <= P.sub * kLmax && (uint64_t)off16 + piece16 <= (S.payload_bytes >> 4));
+        s_end[s][lane] = end;
+        if (lane == 0) s_off[s] = off16;
+    }
+    if (tid < 512 && coded[tid >> 8]) {
+        const uint32_t m = __reduce_or_sync(0xFFFFFFFFu, 1u << (P.comp[(tid >> 8 ? S.sec1 : S.sec0) + (tid & 255)] & 31u));
+        if (lane == 0) atomicOr(&s_lens[tid >> 8], m & ~1u);
+    }
+    if (__syncthreads_or(bad)) { if (tid == 0) raise_status(P.ctl, P.call_id, ZC_E_CORRUPT); return; }
+
+    // ---- the group's part of the pieces ----
+    const uint32_t bits[2] = {H.huff0 ? s_end[0][31] : 0u, H.huff1 ? s_end[1][31] : 0u};     // of the chunk
+    uint32_t from_byte[2] = {0, 0};
+#pragma unroll
+    for (int s = 0; s < 2; ++s) {
+        if (!bits[s]) continue;
+        const uint32_t lo = g_lo ? s_end[s][g_lo - 1] : 0u, hi = s_end[s][g_lo + g_subs - 1];
+        from_byte[s] = (lo >> 7) * 16;
+        if (tid == 0 && !P.skip_copy) {
+            // 16 bytes more (bits of the next subchunk or piece, or the guard) for the window's look-ahead
+            const uint32_t bytes = ((hi + 127) / 128) * 16 + 16 - from_byte[s];
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            mbar_expect_tx(&bars[s], bytes);
+            bulk_g2s_addr(pieces_s + s * piece_room, P.comp + S.payload_off + 16ull * s_off[s] + from_byte[s], bytes, &bars[s]);
+        }
+    }
+#pragma unroll
+    for (int s = 0; s < 2; ++s)                                  // (a copy that was started must land before the block may leave: once more where the wait gave up)
+        if (bits[s] && !mbar_wait(&bars[s], 0, P.spin_limit)) bad = P.skip_copy || !mbar_wait(&bars[s], 0, P.spin_limit) || bad;
+    if (__syncthreads_or(bad)) { if (tid == 0) raise_status(P.ctl, P.call_id, ZC_E_DEVICE_TIMEOUT); return; }
+
+    // ---- decode: my stream, subchunk and stretch ----
+    const uint32_t per_stream = H.huff0 && H.huff1 ? kSplitThreads / 2 : kSplitThreads;
+    uint32_t parts = per_stream / g_subs;                        // a power of two, at most 32 and of 64 symbols or more
+    while (parts > 32 || (parts > 1 && parts * 64 > P.sub)) parts /= 2;
+    const uint32_t st = H.huff0 ? tid / per_stream : 1u, q = tid % per_stream;
+    if ((H.huff0 || H.huff1) && bits[st]) {
+        const bool on = q < g_subs * parts;
+        const uint32_t sub = g_lo + (on ? q / parts : 0u), part = q % parts;
+        const uint32_t lut_s = st ? S.lut1_s : S.lut0_s, pairs = st ? S.pairs1 : S.pairs0;
+        const uint32_t len_shift = pairs ? 24u : 0u, sym_shift = pairs ? 8u : 24u;   // of an entry's first code
+        const uint32_t piece_s = pieces_s + st * piece_room, base = 8 * from_byte[st];
+        const uint32_t lo = (sub ? s_end[st][sub - 1] : 0u) - base, end_bit = s_end[st][sub] - base, len = end_bit - lo;
+        const uint32_t lens = s_lens[st], unit = (lens & (lens - 1)) == 0 && lens ? (uint32_t)__ffs(lens) - 1 : 1u;
+        auto cut_at = [&](const uint32_t k) { return k == parts ? end_bit : lo + len * k / parts / unit * unit; };
+        const uint32_t cut = cut_at(part), stop = on ? cut_at(part + 1) : cut;
+        // counts the codes from `at` to the first boundary at or behind `stop`
+        uint32_t count = 0, end = cut, from = cut;
+        auto walk = [&]() {
+            count = 0;
+            end = from;
+            if (end < stop) {
+                SplitBits B;
+                split_start(B, piece_s, from);
+                for (;;) {
+                    split_code(B, lut_s, len_shift, end);
+                    ++count;
+                    if (end >= stop) break;
+                    split_code(B, lut_s, len_shift, end);
+                    ++count;
+                    if (end >= stop) break;
+                    split_refill(B);
+                }
+            }
+        };
+        walk();
+        for (uint32_t round = 1; round < parts; ++round) {
+            uint32_t should = __shfl_up_sync(0xFFFFFFFFu, end, 1);
+            if (part == 0) should = lo;
+            const bool wrong = on && should != from;
+            if (!__any_sync(0xFFFFFFFFu, wrong)) break;
+            if (wrong) { from = should; walk(); }
+        }
+        // symbols of the subchunk before mine
+        uint32_t upto = count;
+        for (uint32_t o = 1; o < parts; o <<= 1) {
+            const uint32_t x = __shfl_up_sync(0xFFFFFFFFu, upto, o);
+            if (part >= o) upto += x;
+        }
+        // A subchunk must hold exactly its symbols and end with its last bit; anything else means that the payload does not
+        // belong to the tables.
+        const uint32_t first = sub * P.sub, want = c_syms > first ? min(P.sub, c_syms - first) : 0u;
+        const uint32_t got = __shfl_sync(0xFFFFFFFFu, upto, lane | (parts - 1)), last = __shfl_sync(0xFFFFFFFFu, end, lane | (parts - 1));
+        if (on && (got != want || last != end_bit)) {
+            bad = true;
+        } else if (count) {
+            // the last pass: single symbols up to a word boundary, then whole words, then single symbols again
+            SplitBits B;
+            split_start(B, piece_s, from);
+            uint32_t at = syms_s + st * g_syms + (sub - g_lo) * P.sub + upto - count, left = count, pos = 0;
+            while (left) {
+                if ((at & 3u) == 0 && left >= 4) {
+                    uint32_t w = (split_code(B, lut_s, len_shift, pos) >> sym_shift) & 0xFFu;
+                    w |= ((split_code(B, lut_s, len_shift, pos) >> sym_shift) & 0xFFu) << 8;
+                    split_refill(B);
+                    w |= ((split_code(B, lut_s, len_shift, pos) >> sym_shift) & 0xFFu) << 16;
+                    w |= ((split_code(B, lut_s, len_shift, pos) >> sym_shift) & 0xFFu) << 24;
+                    sts32(at, w);
+                    at += 4;
+                    left -= 4;
+                } else {
+                    sts8(at, (split_code(B, lut_s, len_shift, pos) >> sym_shift) & 0xFFu);
+                    ++at;
+                    --left;
+                }
+                split_refill(B);
+            }
+        }
+    }
+    if (__syncthreads_or(bad)) { if (tid == 0) raise_status(P.ctl, P.call_id, ZC_E_CORRUPT); return; }
+
+    // ---- merge: 16 symbols of each stream, 32 output bytes per thread and step ----
+    const uint8_t* raw[2] = {P.comp + S.sec0 + c_lo, P.comp + S.sec1 + c_lo};
+    uint32_t fill4[2];                                           // a chunk without bits: nothing but the fill symbol
+#pragma unroll
+    for (int s = 0; s < 2; ++s) {
+        const uint32_t e = lds32(s ? S.lut1_s : S.lut0_s);
+        fill4[s] = ((s ? S.pairs1 : S.pairs0) ? (e >> 8) & 0xFFu : e >> 24) * 0x01010101u;
+    }
+    const uint32_t k_lo = g_lo * P.sub, k_hi = min(c_syms, k_lo + g_syms);
+    for (uint32_t k = k_lo + 16 * tid; k < k_hi; k += 16 * kSplitThreads) {
+        uint32_t f[2][4];
+#pragma unroll
+        for (int s = 0; s < 2; ++s) {
+            uint4 v;
+            if (!coded[s]) v = ld_nc_v4(raw[s] + k);
+            else if (bits[s]) v = lds128(syms_s + s * g_syms + k - k_lo);
+            else v = make_uint4(fill4[s], fill4[s], fill4[s], fill4[s]);
+            f[s][0] = v.x; f[s][1] = v.y; f[s][2] = v.z; f[s][3] = v.w;
+        }
+        uint32_t o[8];
+        merge16<FMT>(f[0], f[1], o);
+        merge16<FMT>(f[0] + 2, f[1] + 2, o + 4);
+        uint8_t* dst = P.out + 2 * (c_lo + k);
+        if (2 * k + 32 <= out_bytes) {
+            st_cs_v4(dst, make_uint4(o[0], o[1], o[2], o[3]));
+            st_cs_v4(dst + 16, make_uint4(o[4], o[5], o[6], o[7]));
+        } else {
+#pragma unroll
+            for (int t = 0; t < 32; ++t)
+                if (2 * k + t < out_bytes) dst[t] = (uint8_t)(o[t >> 2] >> (8 * (t & 3)));
+        }
+    }
 }
 
 // Many tensors per launch: block b takes the chunks [b * total / grid, (b + 1) * total / grid) of the
@@ -1016,7 +1268,7 @@ decode_batch_kernel(const __grid_constant__ DecBatchParams B)
 struct DecRanges { const void* in; size_t in_bytes; const void* out; size_t out_bytes; const void* ws; size_t ws_bytes; };
 
 template <int F>
-cudaError_t dec_launch_single_t(uint32_t ppl, bool few, uint32_t grid, uint32_t threads, size_t smem, cudaStream_t st, const DecParams& P,
+cudaError_t dec_launch_single_t(uint32_t ppl, int kind, uint32_t grid, uint32_t threads, size_t smem, cudaStream_t st, const DecParams& P,
                                 const DecRanges& R)
 {
     cudaError_t e = cudaSuccess;
@@ -1031,7 +1283,9 @@ cudaError_t dec_launch_single_t(uint32_t ppl, bool few, uint32_t grid, uint32_t 
         kern<<<grid, threads, smem, st>>>(P);
         e = cudaGetLastError();
     };
-    if (few) {
+    if (kind == kDecSplit) {
+        launch(decode_split_kernel<F>);
+    } else if (kind == kDecFew) {
         if (ppl == 4) launch(decode_kernel<F, 4, true>);
         else if (ppl == 2) launch(decode_kernel<F, 2, true>);
         else launch(decode_kernel<F, 1, true>);
@@ -1072,7 +1326,7 @@ cudaError_t dec_launch_batch_t(uint32_t ppl, bool any_base, uint32_t grid, uint3
 }
 
 #define ZC_DEC_DECLARE(NAME)                                                                                              \
-    cudaError_t dec_launch_single_##NAME(uint32_t ppl, bool few, uint32_t grid, uint32_t threads, size_t smem, cudaStream_t st,     \
+    cudaError_t dec_launch_single_##NAME(uint32_t ppl, int kind, uint32_t grid, uint32_t threads, size_t smem, cudaStream_t st,     \
                                          const DecParams& P, const DecRanges& R);                                        \
     cudaError_t dec_launch_batch_##NAME(uint32_t ppl, bool any_base, uint32_t grid, uint32_t threads, size_t smem,        \
                                         cudaStream_t st, const DecBatchParams& B, const DecRanges& R);                   \
@@ -1089,9 +1343,9 @@ ZC_DEC_DECLARE(fp4)
 #define ZC_DEC_COUNTS(out) (void)(out)
 #endif
 #define ZC_DEC_DEFINE(NAME, F)                                                                                            \
-    cudaError_t dec_launch_single_##NAME(uint32_t ppl, bool few, uint32_t grid, uint32_t threads, size_t smem, cudaStream_t st,     \
+    cudaError_t dec_launch_single_##NAME(uint32_t ppl, int kind, uint32_t grid, uint32_t threads, size_t smem, cudaStream_t st,     \
                                          const DecParams& P, const DecRanges& R)                                         \
-    { return dec_launch_single_t<F>(ppl, few, grid, threads, smem, st, P, R); }                                                \
+    { return dec_launch_single_t<F>(ppl, kind, grid, threads, smem, st, P, R); }                                                \
     cudaError_t dec_launch_batch_##NAME(uint32_t ppl, bool any_base, uint32_t grid, uint32_t threads, size_t smem,        \
                                         cudaStream_t st, const DecBatchParams& B, const DecRanges& R)                    \
     { return dec_launch_batch_t<F>(ppl, any_base, grid, threads, smem, st, B, R); }                                       \
@@ -1178,6 +1432,20 @@ DecShape few_shape(const zc_plan_t* p, uint32_t n_chunks, uint32_t* active)
     return s;
 }
 
+// Launch shape of decode_split_kernel: as many blocks per chunk as there are SMs for, up to 8 (4 subchunks each).
+DecShape split_shape(const zc_plan_t* p, uint32_t n_chunks, uint32_t* groups)
+{
+    DecShape s{};
+    s.ppl = 1;
+    s.warps = kSplitThreads / 32;
+    *groups = 1;
+    while (*groups < 8 && 2ull * *groups * n_chunks <= (uint64_t)sm_count()) *groups *= 2;
+    const uint32_t syms = p->syms_per_chunk / *groups;
+    s.pool_bytes = std::max<uint32_t>(2 * syms + 2 * ((uint32_t)round_up((uint64_t)syms * kLmax / 8, 16) + 48), 8192);
+    s.smem = kDecFixedSmem + 16 * s.warps + s.pool_bytes + 64;   // the bit readers look a few words past a piece's copy
+    return s;
+}
+
 // no clearing of the workspace: errors are tagged with the id of the call that raised them
 unsigned long long new_call_id()
 {
@@ -1234,8 +1502,15 @@ zc_status zc_decompress_chunks(const zc_plan_t* p, const void* d_comp, size_t co
     cudaStream_t st = (cudaStream_t)cuda_stream;
     DecShape shape;
     uint32_t active = 0;
-    const bool few = n_chunks <= kDecFewActive * (uint32_t)sm_count();
-    if (few) {
+    uint32_t groups = 1;
+    // decode_split_kernel's rounds cost more than a lane's walk where subchunks are short, and more than other warps' walks
+    // where a block would have several chunks.
+    const int kind = p->syms_per_sub >= kSplitMinSub && n_chunks <= (uint32_t)sm_count() ? kDecSplit
+                     : n_chunks <= kDecFewActive * (uint32_t)sm_count() ? kDecFew : kDecMany;
+    if (kind == kDecSplit) {
+        shape = split_shape(p, n_chunks, &groups);
+        active = 1;
+    } else if (kind == kDecFew) {
         shape = few_shape(p, n_chunks, &active);
     } else {
         const zc_status ss = dec_shape(p, false, &shape);
@@ -1255,21 +1530,21 @@ zc_status zc_decompress_chunks(const zc_plan_t* p, const void* d_comp, size_t co
     P.call_id = new_call_id();
     P.spec = comp_bytes >= kHeaderBytes + table_section_bytes(p->n_chunks, p->chunk_bytes) ? 1u : 0u;
     P.pool_bytes = shape.pool_bytes;
-    P.spin_limit = test_knobs().spin_limit; P.skip_copy = test_knobs().skip_copy; P.sliced = shape.sliced; P.active = active;
+    P.spin_limit = test_knobs().spin_limit; P.skip_copy = test_knobs().skip_copy; P.sliced = shape.sliced; P.active = active; P.groups = groups;
     const uint32_t warps = shape.warps, ppl = shape.ppl;
     const size_t smem = shape.smem;
     // at least one block even for an empty range: the header is still checked
-    const uint32_t want = std::max<uint32_t>(few ? n_chunks : (n_chunks + warps - 1) / warps, 1);
-    const uint32_t grid = std::min<uint32_t>(want, (uint32_t)sm_count());
+    const uint32_t want = std::max<uint32_t>(kind != kDecMany ? n_chunks : (n_chunks + warps - 1) / warps, 1);
+    const uint32_t grid = kind == kDecSplit ? std::max<uint32_t>(n_chunks, 1) * groups : std::min<uint32_t>(want, (uint32_t)sm_count());
     const DecRanges R{d_comp, comp_bytes, d_out,
                       (size_t)std::min<uint64_t>((uint64_t)n_chunks * p->chunk_bytes, p->input_bytes - (uint64_t)first_chunk * p->chunk_bytes),
                       d_workspace, sizeof(Control)};
     cudaError_t e;
     switch (p->format) {
-    case ZC_FMT_BF16: e = dec_launch_single_bf16(ppl, few, grid, warps * 32, smem, st, P, R); break;
-    case ZC_FMT_FP8_E4M3: case ZC_FMT_FP8_E5M2: e = dec_launch_single_fp8(ppl, few, grid, warps * 32, smem, st, P, R); break;
-    case ZC_FMT_SCALE_U8: e = dec_launch_single_scale(ppl, few, grid, warps * 32, smem, st, P, R); break;
-    default: e = dec_launch_single_fp4(ppl, few, grid, warps * 32, smem, st, P, R); break;
+    case ZC_FMT_BF16: e = dec_launch_single_bf16(ppl, kind, grid, warps * 32, smem, st, P, R); break;
+    case ZC_FMT_FP8_E4M3: case ZC_FMT_FP8_E5M2: e = dec_launch_single_fp8(ppl, kind, grid, warps * 32, smem, st, P, R); break;
+    case ZC_FMT_SCALE_U8: e = dec_launch_single_scale(ppl, kind, grid, warps * 32, smem, st, P, R); break;
+    default: e = dec_launch_single_fp4(ppl, kind, grid, warps * 32, smem, st, P, R); break;
     }
     return e == cudaSuccess ? ZC_OK : ZC_E_CUDA;
 }
