@@ -201,6 +201,8 @@ def plan(fmt: int, n_elems: int, chunk_bytes: int) -> Plan:
 class Codebook:
     """zc_build_codebook result: per stream a mode, 256 code lengths and 256 canonical code values."""
 
+    __slots__ = ("_h", "_owned")
+
     def __init__(self, handle, owned: bool = True):
         self._h = handle
         self._owned = owned                      # a dictionary's codebook belongs to the dictionary
@@ -217,10 +219,9 @@ class Codebook:
     def modes(self):
         return [self.get(0)[0], self.get(1)[0]]
 
-    def __del__(self):
-        h = getattr(self, "_h", None)
-        if h and _lib is not None and getattr(self, "_owned", True):
-            _lib.zc_codebook_destroy(h)
+    def __del__(self, _destroy=_lib.zc_codebook_destroy):
+        if self._owned and self._h:
+            _destroy(self._h)
             self._h = None
 
 
@@ -297,16 +298,19 @@ class Dictionary:
         _keep, ptr = _hist_ptr(h_hist)
         self._h = C.c_void_p()
         _check(_lib.zc_dict_create(p._h, ptr, tolerance, C.byref(self._h)), "zc_dict_create")
+        self._flag = C.c_int(0)                  # a dictionary is used from one thread at a time
+        self._flag_ref = C.byref(self._flag)
 
     @property
     def codebook(self) -> Codebook:
         """The current codebook (not owned: valid until rebuild())."""
         return Codebook(C.c_void_p(_lib.zc_dict_codebook(self._h)), owned=False)
 
-    def observe(self, input_bytes: int, container_bytes: int) -> bool:
-        flag = C.c_int(0)
-        _check(_lib.zc_dict_observe(self._h, input_bytes, container_bytes, C.byref(flag)), "zc_dict_observe")
-        return bool(flag.value)
+    def observe(self, input_bytes: int, container_bytes: int, _observe=_lib.zc_dict_observe) -> bool:
+        status = _observe(self._h, input_bytes, container_bytes, self._flag_ref)
+        if status != OK:
+            raise ZcError(status, "zc_dict_observe")
+        return self._flag.value != 0
 
     def rebuild(self, p: Plan, h_hist) -> None:
         _keep, ptr = _hist_ptr(h_hist)
@@ -339,7 +343,7 @@ def build_codebooks(plans, h_hists, policy: int = POLICY_AUTO, n_threads: int = 
     plan_arr = (C.c_void_p * max(n, 1))(*[p._h.value for p in plans])
     _check(_lib.zc_build_codebooks(n, plan_arr, C.cast(h.ctypes.data, C.POINTER(C.c_uint64)), policy, n_threads, handles),
            "zc_build_codebooks")
-    return [Codebook(C.c_void_p(handles[i])) for i in range(n)]
+    return [Codebook(C.c_void_p(h)) for h in handles[:n]]
 
 
 def compress(p: Plan, cb: Codebook, d_in: torch.Tensor, d_out: torch.Tensor, d_workspace: torch.Tensor,
@@ -434,7 +438,7 @@ def compress_batch(batch: CompressBatch, d_workspace: torch.Tensor, sync: bool =
     _check(_lib.zc_compress_batch_xor(batch.n, batch.plans, batch.cbs, batch.ins, batch.bases, batch.outs, batch.caps,
                                       d_workspace.data_ptr(), d_workspace.numel(), sizes if sync else None, _stream_ptr(stream)),
            "zc_compress_batch")
-    return [int(v) for v in sizes[: batch.n]] if sync else None
+    return sizes[: batch.n] if sync else None
 
 
 class DecompressBatch:

@@ -22,12 +22,18 @@
 
 namespace zc {
 
-// Per symbol: the code left-aligned in bits 31..20 and its length in bits 3..0; a symbol without a code is kNoCode.
+// The code tables of a codebook as they travel to the device: per symbol the code left-aligned in bits 15..4 and its
+// length in bits 3..0, 0 for a symbol without a code.
 struct EncTables {
-    uint32_t enc[2][256];
+    uint16_t enc[2][256];
     uint32_t fill[2];                            // fill symbol (the one with the all-zero code) | its code length << 8
     uint32_t pad[2];
 };
+
+// The entries of the tables in shared memory: the code left-aligned in bits 31..20, the length in bits 3..0.  A symbol
+// without a code has a bit of its own; two of them add up to a bit that no sum of two lengths reaches.
+constexpr uint32_t kNoCode = 0x40;
+__device__ __forceinline__ uint32_t enc_entry(uint32_t v) { return v ? ((v & 0xFFF0u) << 16) | (v & 15u) : kNoCode; }
 
 // One tensor of a launch.
 struct EncItem {
@@ -59,7 +65,7 @@ struct EncParams {
     uint32_t tiles, teams;                       // T (tiles of a unit = warps of a team), units of a batch
     uint32_t ring16;                             // a team's output ring, in 16-byte units
     uint32_t n_tensors, total_batches;
-    uint32_t ahead;                              // batches a block may hold beyond those it has packed
+    uint32_t ahead;                              // 1: a block holds one batch at a time, 2: the next one too, 3: and the ticket after it
     uint32_t spin_limit;                         // polls after which a bounded wait gives up
     uint32_t base_buf;                           // every worker has a second input buffer for the base tensor
     uint32_t buf_bytes;                          // a worker's input buffers
@@ -370,7 +376,7 @@ encode_kernel(const __grid_constant__ EncParams P)
             if (ended && posted == published) break;
             // ---- a new batch ----
             const uint32_t freed = __shfl_sync(0xFFFFFFFFu, vol32(&s_freed_seq), 0);
-            if (!ended && published < posted + P.ahead && published < freed + kEncRing) {
+            if (!ended && published < posted + min(P.ahead, 2u) && published < freed + kEncRing) {
                 if (!have_ticket && lane == 0) ticket = atomicAdd(&P.ctl->ticket, 1u);
                 have_ticket = true;
                 const uint32_t g = __shfl_sync(0xFFFFFFFFu, ticket, 0);
@@ -413,7 +419,10 @@ encode_kernel(const __grid_constant__ EncParams P)
                         for (int s = 0; s < 2; ++s) {
                             if (!(s == 0 ? H0 : H1)) continue;
 #pragma unroll
-                            for (uint32_t i = 0; i < 8; ++i) sts32(tabs_s + 1024 * (kTabs * ns + h) + 4 * (lane + 32 * i), E.enc[s][lane + 32 * i]);
+                            for (uint32_t i = 0; i < 4; ++i) {
+                                const uint32_t two = reinterpret_cast<const uint32_t*>(E.enc[s])[lane + 32 * i];
+                                sts64(tabs_s + 1024 * (kTabs * ns + h) + 8 * (lane + 32 * i), enc_entry(two & 0xFFFFu), enc_entry(two >> 16));
+                            }
                             if (lane == 0) s_fill[ns][h] = E.fill[s];
                             ++h;
                         }
@@ -432,7 +441,7 @@ encode_kernel(const __grid_constant__ EncParams P)
                         mbar_arrive(&mb_info[r]);
                     }
                     __syncwarp();
-                    if (P.ahead > 1) {                           // the next one's ticket travels until it is looked at
+                    if (P.ahead > 2) {                           // the next one's ticket travels until it is looked at
                         if (lane == 0) ticket = atomicAdd(&P.ctl->ticket, 1u);
                         have_ticket = true;
                     }

@@ -42,14 +42,11 @@ struct zc_codebook_s {
     uint8_t len[2][256];
     uint32_t code[2][256];     // right-aligned canonical code values
     // derived once when the codebook is built, so that a compress call only copies them:
-    uint32_t enc[2][256];      // the encoder's table entry of every symbol: code << (32 - length) | length, or kNoCode
+    uint16_t enc[2][256];      // what the encoder needs of every symbol: code << (16 - length) | length; 0: no code
     uint32_t fill[2];          // fill symbol (the one whose code is all zeros) | its code length << 8; 0xFF00: no code at all
 };
 
 namespace zc {
-// Entry of a symbol without a code.  A bit of its own: two of them add up to a bit that no sum of two lengths reaches.
-constexpr uint32_t kNoCode = 0x40;
-
 // Fills the derived fields of a codebook (call after len[] and code[] are final).
 inline void finish_codebook(zc_codebook_s* cb)
 {
@@ -57,7 +54,7 @@ inline void finish_codebook(zc_codebook_s* cb)
         cb->fill[s] = 0xFF00u;
         for (int v = 0; v < 256; ++v) {
             const uint32_t l = cb->len[s][v];
-            cb->enc[s][v] = l ? (cb->code[s][v] << (32 - l)) | l : kNoCode;
+            cb->enc[s][v] = (uint16_t)(l ? (cb->code[s][v] << (16 - l)) | l : 0u);
             if (l && cb->code[s][v] == 0) cb->fill[s] = (uint32_t)v | (l << 8);
         }
     }
