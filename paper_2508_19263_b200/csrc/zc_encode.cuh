@@ -197,11 +197,12 @@ __device__ __forceinline__ uint32_t join_codes(uint32_t a, uint32_t b)
 }
 
 // Phase B for one coded stream: looks up the lane's symbols (its row of 2 N staged bytes at row_s, 16-byte pieces
-// XORed with `swz`), leaves the joined codes in e[] and returns the lane's bit count.  `ok` turns false when a symbol has
-// no code: the caller then uses lookup_checked.
+// XORed with `swz`), leaves the joined codes in e[] and returns the lane's bit count.  longer: not 0 when some four
+// neighbouring codes are longer than 32 bits together.  `ok` turns false when a symbol has no code: the caller then uses
+// lookup_checked.
 template <uint32_t N>
 __device__ __forceinline__ uint32_t lookup_quick(uint32_t (&e)[N], const uint32_t row_s, const uint32_t swz,
-                                                 const uint32_t tab_s, bool& ok, bool& long_quad)
+                                                 const uint32_t tab_s, bool& ok, uint32_t& longer)
 {
     uint32_t bits = 0, seen = 0, over = 0;
 #pragma unroll
@@ -223,7 +224,7 @@ __device__ __forceinline__ uint32_t lookup_quick(uint32_t (&e)[N], const uint32_
         }
     }
     ok = (seen & (3u * kNoCode)) == 0;                           // one or two of them in a pair
-    long_quad = (over & 0x80u) != 0;
+    longer = over & 0x80u;
     return bits - 95 * (N / 2);
 }
 
@@ -256,22 +257,20 @@ __device__ __forceinline__ uint32_t lookup_checked(uint32_t (&e)[N], const uint3
 }
 
 // Phase C for one coded stream: ORs the joined codes into shared memory from bit `at` of the piece at piece_s on.
-// QUADS: four codes at a time (no group of four in the warp is longer than 32 bits), else two at a time.
+// QUADS: four codes at a time (no four neighbouring ones in the warp are longer than 32 bits), else two at a time (choosing
+// anew for every four costs more than it saves: FP8 505 against 474 us).
 template <bool QUADS, uint32_t N>
 __device__ __forceinline__ void emit_codes(const uint32_t (&e)[N], const uint32_t piece_s, const uint32_t at)
 {
     uint32_t addr = piece_s + 4 * (at >> 5), t = at & 31u, w = 0;
 #pragma unroll
-    for (uint32_t p = 0; p < N / 8; ++p) {
-#pragma unroll
-        for (uint32_t i = 0; i < 4; ++i) {
-            const uint32_t e0 = e[8 * p + 2 * i], e1 = e[8 * p + 2 * i + 1], c0 = e0 & 0xFFFFFF00u, c1 = e1 & 0xFFFFFF00u;
-            if (QUADS) {
-                put_bits(c0 | __funnelshift_r(c1, 0, e0), add_low_byte(e0 + e1, t), t, w, addr);
-            } else {
-                put_bits(c0, add_low_byte(e0, t), t, w, addr);
-                put_bits(c1, add_low_byte(e1, t), t, w, addr);
-            }
+    for (uint32_t i = 0; i < N / 2; ++i) {
+        const uint32_t e0 = e[2 * i], e1 = e[2 * i + 1], c0 = e0 & 0xFFFFFF00u, c1 = e1 & 0xFFFFFF00u;
+        if (QUADS) {
+            put_bits(c0 | __funnelshift_r(c1, 0, e0), add_low_byte(e0 + e1, t), t, w, addr);
+        } else {
+            put_bits(c0, add_low_byte(e0, t), t, w, addr);
+            put_bits(c1, add_low_byte(e1, t), t, w, addr);
         }
     }
     if (t & 31u) red_or(addr, w);
@@ -672,7 +671,7 @@ encode_kernel(const __grid_constant__ EncParams P)
             uint32_t e[kTabs][kN / 2];                             // joined codes of my symbols
             uint32_t mine[kTabs] = {}, end[kTabs] = {};          // bits of my symbols, and where they end in their chunk
             uint32_t chunk_bits[kTabs] = {};                     // bits of my chunk (0: constant)
-            bool quads[kTabs] = {};                              // no four neighbouring codes of the tile are longer than 32 bits
+            uint32_t longer[kTabs] = {};                         // not 0: some four neighbouring codes of the tile are longer than 32 bits
             const uint64_t s_lo = (uint64_t)u * unit_syms + t_lo;       // first symbol of the tile in its stream
             auto request_next = [&]() {                          // my tile of the next batch, if that is known already
                 const uint32_t r1 = (it + 1) % kEncRing;
@@ -753,18 +752,20 @@ encode_kernel(const __grid_constant__ EncParams P)
                         for (uint32_t i = 0; i < kN / 2; ++i) e[h][i] = 2 * fill_len;
                         mine[h] = n_my * fill_len;
                         constant = true;
-                        quads[h] = fill_len <= 8;
+                        longer[h] = fill_len > 8;
                     } else {
-                        bool ok = false, long_quad = true;
+                        bool ok = false;
+                        uint32_t mine_longer = 0;
                         if (whole) {
                             if (!kAny || n_my) {
-                                mine[h] = lookup_quick(e[h], row, swz, tab_s + 1024 * h, ok, long_quad);
+                                mine[h] = lookup_quick(e[h], row, swz, tab_s + 1024 * h, ok, mine_longer);
                             } else {
-                                ok = true; long_quad = false;
+                                ok = true;
                             }
                         }
-                        quads[h] = __all_sync(0xFFFFFFFFu, ok && !long_quad);
-                        if (!quads[h] && !__all_sync(0xFFFFFFFFu, ok)) {
+                        longer[h] = __reduce_or_sync(0xFFFFFFFFu, mine_longer);
+                        if (!__all_sync(0xFFFFFFFFu, ok)) {
+                            longer[h] = 1;
                             bool no_code = false;
                             mine[h] = lookup_checked(e[h], row, swz, tab_s + 1024 * h, n_my, no_code);
                             if (no_code) bad = I.index + 1;
@@ -881,7 +882,7 @@ encode_kernel(const __grid_constant__ EncParams P)
                     }
                     if (chunk_bits[h] && (!kAny || mine[h])) {
                         const uint32_t piece_s = ring_s + 16 * (piece_at + my_at + (h ? p16[0] : 0u));
-                        if (quads[h]) emit_codes<true>(e[h], piece_s, end[h] - mine[h]);
+                        if (longer[h] == 0) emit_codes<true>(e[h], piece_s, end[h] - mine[h]);
                         else emit_codes<false>(e[h], piece_s, end[h] - mine[h]);
                     }
                 }
