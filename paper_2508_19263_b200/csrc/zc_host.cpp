@@ -95,6 +95,13 @@ bool huffman_lengths(const uint64_t* w, size_t n, uint32_t L, uint8_t* depth)
     return true;
 }
 
+// What package-merge keeps of its levels.  The caller's, so that the threads of a batched call work in memory that has been
+// touched before (a new thread's own would cost it a page fault per 4 KiB).
+struct MergeScratch {
+    uint64_t w[2][512];
+    uint16_t leaves_in[kLmax][513];                              // [r][k]: leaves among the first k items of level r
+};
+
 // Optimal code lengths under a maximum length, by package-merge in its prefix-count form:
 // only the weights and the number of leaves in every prefix of each level's merged list are kept.  Because
 // the leaves are sorted, the leaves chosen at a level are always a prefix of the sorted list,
@@ -103,7 +110,7 @@ bool huffman_lengths(const uint64_t* w, size_t n, uint32_t L, uint8_t* depth)
 // (count, symbol); at equal weight a leaf is taken before a package.
 // A tensor's two codes take 10 us (BF16 weights) or 17 us (FP8), single-threaded on a 2.7 GHz Xeon; with a comparison sort
 // and branching merges of every level it was 25 and 60 us.
-bool limited_lengths(const uint64_t hist[256], uint32_t L, uint8_t len[256])
+bool limited_lengths(const uint64_t hist[256], uint32_t L, uint8_t len[256], MergeScratch& scratch)
 {
     std::memset(len, 0, 256);
     for (int v = 0; v < 256; ++v)
@@ -131,8 +138,8 @@ bool limited_lengths(const uint64_t hist[256], uint32_t L, uint8_t len[256])
     // more than 2n - 1 items.  Only the weights are needed to build the next level; of a level itself, only how many
     // leaves its prefixes hold.  A merge is cut in the middle and both halves run from both ends (four independent chains of
     // compare, select and advance, without branches).
-    static thread_local uint64_t w[2][512];
-    static thread_local uint16_t leaves_in[kLmax][513];          // [r][k]: leaves among the first k items of level r
+    auto& w = scratch.w;
+    auto& leaves_in = scratch.leaves_in;
     size_t size[kLmax];
     for (size_t i = 0; i < n; ++i) { w[0][i] = lw[i]; leaves_in[0][i] = (uint16_t)i; }
     leaves_in[0][n] = (uint16_t)n;
@@ -309,12 +316,9 @@ static bool known_policy(zc_policy policy)
     return policy == ZC_POLICY_AUTO || policy == ZC_POLICY_HUFF_ALL || policy == ZC_POLICY_RAW_ALL || policy == ZC_POLICY_STATIC;
 }
 
-zc_status zc_build_codebook(const zc_plan_t* plan, const uint64_t* h_hist, zc_policy policy, zc_codebook_t** out)
+// Fills a codebook from a histogram (see zc_build_codebook).
+static zc_status fill_codebook(const uint64_t* h_hist, zc_policy policy, MergeScratch& scratch, zc_codebook_s* cb)
 {
-    if (!plan || !h_hist || !out) return ZC_E_INVALID_ARG;
-    if (!known_policy(policy)) return ZC_E_UNSUPPORTED;
-    zc_codebook_s* cb = new (std::nothrow) zc_codebook_s;
-    if (!cb) return ZC_E_NOMEM;
     for (int s = 0; s < 2; ++s) {
         const uint64_t* h = h_hist + 256 * s;
         uint64_t n = 0;
@@ -322,10 +326,10 @@ zc_status zc_build_codebook(const zc_plan_t* plan, const uint64_t* h_hist, zc_po
         // a static dictionary codes tensors it has not seen: every symbol counts as 1/256 of an occurrence more
         uint64_t smoothed[256];
         if (policy == ZC_POLICY_STATIC) {
-            if (n >> 54) { delete cb; return ZC_E_INVALID_ARG; }
+            if (n >> 54) return ZC_E_INVALID_ARG;
             for (int v = 0; v < 256; ++v) smoothed[v] = 256 * h[v] + 1;
         }
-        if (!limited_lengths(policy == ZC_POLICY_STATIC ? smoothed : h, kLmax, cb->len[s])) { delete cb; return ZC_E_INVALID_ARG; }
+        if (!limited_lengths(policy == ZC_POLICY_STATIC ? smoothed : h, kLmax, cb->len[s], scratch)) return ZC_E_INVALID_ARG;
         canonical(cb->len[s], cb->code[s]);
         uint32_t mode = ZC_MODE_RAW;
         if (n != 0 && policy == ZC_POLICY_HUFF_ALL) mode = ZC_MODE_HUFF;
@@ -334,6 +338,18 @@ zc_status zc_build_codebook(const zc_plan_t* plan, const uint64_t* h_hist, zc_po
         cb->mode[s] = mode;
     }
     finish_codebook(cb);
+    return ZC_OK;
+}
+
+zc_status zc_build_codebook(const zc_plan_t* plan, const uint64_t* h_hist, zc_policy policy, zc_codebook_t** out)
+{
+    if (!plan || !h_hist || !out) return ZC_E_INVALID_ARG;
+    if (!known_policy(policy)) return ZC_E_UNSUPPORTED;
+    zc_codebook_s* cb = new (std::nothrow) zc_codebook_s;
+    if (!cb) return ZC_E_NOMEM;
+    MergeScratch scratch;
+    const zc_status st = fill_codebook(h_hist, policy, scratch, cb);
+    if (st != ZC_OK) { delete cb; return st; }
     *out = cb;
     return ZC_OK;
 }
@@ -344,29 +360,41 @@ zc_status zc_build_codebooks(uint32_t n_tensors, const zc_plan_t* const* plans, 
     if (n_tensors == 0) return ZC_OK;
     if (!plans || !h_hists || !out) return ZC_E_INVALID_ARG;
     if (!known_policy(policy)) return ZC_E_UNSUPPORTED;
+    for (uint32_t t = 0; t < n_tensors; ++t) if (!plans[t]) return ZC_E_INVALID_ARG;
     if (n_threads == 0) {
         const uint32_t hw = std::max(1u, std::thread::hardware_concurrency());
-        n_threads = std::min<uint32_t>({hw, 16u, (n_tensors + 7) / 8});     // a codebook takes tens of microseconds
+        n_threads = std::min<uint32_t>({hw, 16u, (n_tensors + 7) / 8});     // a codebook takes about ten microseconds, a thread twice that
     }
     n_threads = std::max<uint32_t>(1, std::min<uint32_t>(n_threads, n_tensors));
+    // The memory of all threads is the caller's: a new thread that allocates sets up an arena of its own first.
+    static thread_local std::vector<MergeScratch> scratch;
     std::vector<zc_codebook_t*> made(n_tensors, nullptr);
-    std::atomic<int> first_error{ZC_OK};
+    std::vector<std::thread> pool;
+    bool room = true;
+    try {
+        if (scratch.size() < n_threads) scratch.resize(n_threads);
+        pool.reserve(n_threads);
+    } catch (...) {
+        room = false;
+    }
+    for (uint32_t t = 0; t < n_tensors && room; ++t) room = (made[t] = new (std::nothrow) zc_codebook_s) != nullptr;
+    std::atomic<int> first_error{room ? ZC_OK : ZC_E_NOMEM};
     // every thread takes the next tensor until none is left: the first ones are at work while the others are still being
-    // started (which takes about as long as a codebook)
-    std::atomic<uint32_t> next{0};
-    auto work = [&]() {
+    // started
+    std::atomic<uint32_t> next{room ? 0u : n_tensors};
+    MergeScratch* const shared_scratch = scratch.data();         // (thread_local: the others must not name it)
+    auto work = [&](uint32_t i) {
         for (uint32_t t; (t = next.fetch_add(1, std::memory_order_relaxed)) < n_tensors;) {
-            const zc_status st = zc_build_codebook(plans[t], h_hists + 512ull * t, policy, &made[t]);
+            const zc_status st = fill_codebook(h_hists + 512ull * t, policy, shared_scratch[i], made[t]);
             if (st != ZC_OK) { int expected = ZC_OK; first_error.compare_exchange_strong(expected, (int)st); }
         }
     };
-    std::vector<std::thread> pool;
     try {
-        for (uint32_t i = 1; i < n_threads && next.load(std::memory_order_relaxed) < n_tensors; ++i) pool.emplace_back(work);
+        for (uint32_t i = 1; i < n_threads && next.load(std::memory_order_relaxed) < n_tensors; ++i) pool.emplace_back(work, i);
     } catch (...) {
         // fewer threads than asked for: the ones that run do it all
     }
-    work();
+    if (room) work(0);
     for (auto& th : pool) th.join();
     if (first_error.load() != ZC_OK) {
         for (auto* cb : made) delete cb;
