@@ -199,14 +199,21 @@ __device__ __forceinline__ uint32_t join_codes(uint32_t a, uint32_t b)
 // Phase B for one coded stream: looks up the lane's symbols (its row of 2 N staged bytes at row_s, 16-byte pieces
 // XORed with `swz`), leaves the joined codes in e[] and returns the lane's bit count.  longer: not 0 when some four
 // neighbouring codes are longer than 32 bits together.  `ok` turns false when a symbol has no code: the caller then uses
-// lookup_checked.
+// lookup_checked.  Tiles are multiples of 256 symbols, so only a lane of 48 can be filled in part, by 16 or 32 of them: what
+// lies behind is left by another tile.
 template <uint32_t N>
 __device__ __forceinline__ uint32_t lookup_quick(uint32_t (&e)[N], const uint32_t row_s, const uint32_t swz,
-                                                 const uint32_t tab_s, bool& ok, uint32_t& longer)
+                                                 const uint32_t tab_s, const uint32_t n_my, bool& ok, uint32_t& longer)
 {
     uint32_t bits = 0, seen = 0, over = 0;
 #pragma unroll
     for (uint32_t p = 0; p < N / 8; ++p) {
+        if (N == 24 && 16 * p >= n_my) {
+#pragma unroll
+            for (uint32_t i = 0; i < 8; ++i) e[8 * p + i] = 0;
+            bits += 4 * 95;
+            continue;
+        }
         const uint4 v = lds128(row_s + ((p ^ swz) << 4));
         const uint32_t q[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
@@ -749,7 +756,7 @@ encode_kernel(const __grid_constant__ EncParams P)
                     if (kSpotConstant && whole && fill_len <= kLmax && __all_sync(0xFFFFFFFFu, differs[h] == 0)) {
                         // nothing but the fill symbol (which has the all-zero code)
 #pragma unroll
-                        for (uint32_t i = 0; i < kN / 2; ++i) e[h][i] = 2 * fill_len;
+                        for (uint32_t i = 0; i < kN / 2; ++i) e[h][i] = kN != 48 || 16 * (i / 8) < n_my ? 2 * fill_len : 0u;
                         mine[h] = n_my * fill_len;
                         constant = true;
                         longer[h] = fill_len > 8;
@@ -758,7 +765,7 @@ encode_kernel(const __grid_constant__ EncParams P)
                         uint32_t mine_longer = 0;
                         if (whole) {
                             if (!kAny || n_my) {
-                                mine[h] = lookup_quick(e[h], row, swz, tab_s + 1024 * h, ok, mine_longer);
+                                mine[h] = lookup_quick(e[h], row, swz, tab_s + 1024 * h, n_my, ok, mine_longer);
                             } else {
                                 ok = true;
                             }

@@ -477,3 +477,24 @@ def test_whole_containers_at_bench_size_equal_the_oracle_s(fmt, chunk_bytes):
     assert zc.batch_status(ws) == (zc.OK, None)
     for p, b, x in zip(plans, d_backs, d_ins):
         assert torch.equal(b[: p.input_bytes], x[: p.input_bytes])
+
+
+@pytest.mark.parametrize("fmt,chunk_bytes,chunks", [(zc.FMT_BF16, 4096, k) for k in (1, 31, 149, 2500, 5500)] +
+                         [(zc.FMT_FP8_E4M3, 16384, k) for k in (1, 149, 700)] + [(zc.FMT_BF16, 1024, k) for k in (60000, 150000)])
+def test_batches_from_one_chunk_to_several_rounds(fmt, chunk_bytes, chunks):
+    """The batched decoder deals its chunks out in one to five rounds and the batched encoder holds one to three batches,
+    by the number of chunks: totals on both sides of those lines, in a large, a ragged and an empty tensor."""
+    cs = chunk_bytes // 2 * zo.group(fmt)
+    a = chunks * 2 // 3
+    sizes = [a * cs, 0, max((chunks - a) * cs - 3, 1)]
+    datas, plans, ocbs, d_outs, batch, ws = _batch_compress(fmt, sizes, chunk_bytes, 40 + chunks, [zc.POLICY_AUTO, zc.POLICY_HUFF_ALL])
+    got_sizes = zc.compress_batch(batch, ws)
+    assert zc.batch_status(ws) == (zc.OK, None)
+    for n, data, ocb, out, nbytes in zip(sizes, datas, ocbs, d_outs, got_sizes):
+        assert np.array_equal(out[:nbytes].cpu().numpy(), zo.compress(fmt, data, n, chunk_bytes, ocb))
+    backs = [torch.full((p.input_bytes + 16,), 0xEE, dtype=torch.uint8, device=DEV) for p in plans]
+    zc.decompress_batch(zc.DecompressBatch(plans, d_outs, got_sizes, backs), ws)
+    assert zc.batch_status(ws) == (zc.OK, None)
+    for p, data, back in zip(plans, datas, backs):
+        back = back.cpu().numpy()
+        assert np.array_equal(back[: p.input_bytes], data[: p.input_bytes]) and (back[p.input_bytes:] == 0xEE).all()

@@ -340,3 +340,36 @@ def test_large_tensor_sampled_chunks():
     zc.decompress(p, d_out, nbytes, d_back, d_ws)
     assert zc.device_status(p, d_ws) == zc.OK
     assert torch.equal(d_back, d_in)
+
+
+@pytest.mark.parametrize("fmt", [zc.FMT_BF16, zc.FMT_FP8_E4M3])
+@pytest.mark.parametrize("policy", [zc.POLICY_AUTO, zc.POLICY_HUFF_ALL])
+@pytest.mark.parametrize("chunk_kib,extra", [(1, 0), (2, 1), (4, 0), (5, -1), (6, 17), (7, 1), (9, 0), (12, -16), (13, 1), (28, -1), (32, 16),
+                                             (33, 0), (61, 1), (64, 0)])
+def test_encoder_at_every_kind_of_chunk_size(fmt, policy, chunk_kib, extra):
+    """Chunks that fill a worker's lanes exactly, several workers, part of one, and more symbols than the workers of a block
+    hold at once; 11 chunks and a tail that ends just before or behind a chunk's, a subchunk's or a word's edge."""
+    n = (11 * 512 * chunk_kib + extra) * zo.group(fmt)
+    _gpu_round_trip(fmt, _weights(fmt, n, chunk_kib + fmt), n, 1024 * chunk_kib, policy)
+
+
+@pytest.mark.parametrize("fmt,policy", [(zc.FMT_BF16, zc.POLICY_AUTO), (zc.FMT_BF16, zc.POLICY_HUFF_ALL), (zc.FMT_FP8_E4M3, zc.POLICY_AUTO)])
+@pytest.mark.parametrize("chunk_kib", [4, 31, 32, 64])
+def test_decoder_at_the_chunk_counts_where_its_kernel_changes(fmt, policy, chunk_kib):
+    """Ranges of one chunk up to a few per SM and beyond, below and from the subchunk length on that is cut into stretches."""
+    sm = torch.cuda.get_device_properties(0).multi_processor_count
+    counts = sorted({1, 2, 18, 19, 37, 74, 75, sm, sm + 1, 8 * sm, 8 * sm + 1} if chunk_kib == 4 else {1, 2, 18, 19, 37, 74, 75, sm, sm + 1})
+    cs = 512 * chunk_kib
+    n = ((counts[-1] + 1) * cs - cs // 3 - 5) * zo.group(fmt)        # a ragged chunk follows the longest range
+    data = _weights(fmt, n, chunk_kib)
+    cont = zo.compress(fmt, data, n, 1024 * chunk_kib, zo.build_codebook(zo.histogram(fmt, data, n), policy))
+    p = zc.plan(fmt, n, 1024 * chunk_kib)
+    d_comp, d_ws = torch.from_numpy(cont).to(DEV), torch.zeros(p.workspace_bytes, dtype=torch.uint8, device=DEV)
+    want = torch.from_numpy(data).to(DEV)
+    for count in counts:
+        for first in (0, p.n_chunks - count):
+            lo, hi = first * p.chunk_bytes, min((first + count) * p.chunk_bytes, p.input_bytes)
+            back = torch.full((hi - lo + 64,), 0xEE, dtype=torch.uint8, device=DEV)
+            zc.decompress_chunks(p, d_comp, cont.size, first, count, back, d_ws)
+            assert zc.device_status(p, d_ws) == zc.OK
+            assert torch.equal(back[: hi - lo], want[lo:hi]) and bool((back[hi - lo:] == 0xEE).all())
