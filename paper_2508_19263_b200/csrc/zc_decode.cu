@@ -92,6 +92,27 @@ __device__ __forceinline__ uint32_t lds32_if(bool p, uint32_t addr)
     return v;
 }
 
+__device__ __forceinline__ void sts128(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d)
+{
+    ZC_DBG_SHARED(addr, 16, return);
+    asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};" :: "r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
+}
+__device__ __forceinline__ uint4 lds128(uint32_t addr)
+{
+    ZC_DBG_SHARED(addr, 16, return make_uint4(0, 0, 0, 0));
+    uint4 v;
+    asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr));
+    return v;
+}
+
+__device__ __forceinline__ uint32_t lds16(uint32_t addr)
+{
+    ZC_DBG_SHARED(addr, 2, return 0);
+    uint16_t v;
+    asm volatile("ld.shared.u16 %0, [%1];" : "=h"(v) : "r"(addr));
+    return v;
+}
+
 // ------------------------------------------------------------------------------------------------
 // decode tables, built by every block from the container's code-length table
 // ------------------------------------------------------------------------------------------------
@@ -191,28 +212,42 @@ static __device__ bool build_lut(uint32_t my_len, uint32_t* lut, uint16_t* singl
 #pragma unroll
     for (uint32_t l = 1; l <= kLmax; ++l) lim[l] = b.limit[l];
     __syncthreads();
-    // first code of every window: its length is the number of limits at or below the window value, plus one
-    for (uint32_t idx = tid; idx < kLutEntries; idx += blockDim.x) {
+    // First code of every window: its length is the number of limits at or below the window value, plus one.  A thread takes
+    // eight neighbouring windows at a time: they start with the same code when that is of 9 bits or less.
+    const uint32_t single_s = smem_u32(single), lut_s = smem_u32(lut);
+    auto first_code = [&](const uint32_t idx) -> uint32_t {
         uint32_t l = 1;
 #pragma unroll
         for (uint32_t k = 1; k < kLmax; ++k) l += idx >= lim[k] ? 1u : 0u;
         uint32_t rel = (idx >> (kLmax - l)) - b.first[l];
         if (rel >= b.count[l]) rel = 0;                           // only reachable with damaged or one-symbol tables
-        single[idx] = (uint16_t)((l << 8) | b.sorted[b.offset[l] + rel]);
+        return (l << 8) | b.sorted[b.offset[l] + rel];
+    };
+    for (uint32_t idx = 8 * tid; idx < kLutEntries; idx += 8 * blockDim.x) {
+        uint32_t e = first_code(idx) * 0x10001u, w[4] = {e, e, e, e};
+        if ((e & 0xFF00u) > 0x900u) {
+#pragma unroll
+            for (uint32_t i = 0; i < 4; ++i) w[i] = first_code(idx + 2 * i) | first_code(idx + 2 * i + 1) << 16;
+        }
+        sts128(single_s + 2 * idx, w[0], w[1], w[2], w[3]);
     }
     __syncthreads();
-    for (uint32_t idx = tid; idx < kLutEntries; idx += blockDim.x) {
-        const uint32_t e1 = single[idx];
-        const uint32_t l1 = e1 >> 8, s1 = e1 & 0xFF;
-        uint32_t e = l1 | (s1 << 24);                             // one-symbol mode: length | symbol << 24
-        if (mode == 2) {
-            e = l1 | (s1 << 8) | (l1 << 24);
-            const uint32_t e2 = single[(idx << l1) & (kLutEntries - 1)];
-            const uint32_t l2 = e2 >> 8, s2 = e2 & 0xFF;
-            if (l1 + l2 <= kLmax) e = (l1 + l2) | (s1 << 8) | (s2 << 16) | (l1 << 24);
-            else e |= 0x80000000u;
+    for (uint32_t idx = 8 * tid; idx < kLutEntries; idx += 8 * blockDim.x) {
+        const uint4 v = lds128(single_s + 2 * idx);
+        const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+        uint32_t e[8];
+#pragma unroll
+        for (uint32_t i = 0; i < 8; ++i) {
+            const uint32_t e1 = (w[i / 2] >> (16 * (i & 1u))) & 0xFFFFu, l1 = e1 >> 8, s1 = e1 & 0xFF;
+            e[i] = l1 | (s1 << 24);                               // one-symbol mode: length | symbol << 24
+            if (mode == 2) {
+                const uint32_t e2 = lds16(single_s + 2 * (((idx + i) << l1) & (kLutEntries - 1)));
+                const uint32_t l2 = e2 >> 8, s2 = e2 & 0xFF;
+                e[i] = l1 + l2 <= kLmax ? (l1 + l2) | (s1 << 8) | (s2 << 16) | (l1 << 24) : l1 | (s1 << 8) | (l1 << 24) | 0x80000000u;
+            }
         }
-        lut[idx] = e;
+        sts128(lut_s + 4 * idx, e[0], e[1], e[2], e[3]);
+        sts128(lut_s + 4 * idx + 16, e[4], e[5], e[6], e[7]);
     }
     __syncthreads();
     if (tid == 0) *per_lookup = mode;
@@ -276,19 +311,6 @@ __device__ __forceinline__ uint32_t lut_peek(uint32_t win, uint32_t lut_s)
 }
 // pos + low byte of x, in one multiply-add-like instruction off the integer ALU pipe
 __device__ __forceinline__ uint32_t add_low_byte(uint32_t pos, uint32_t x) { return __dp4a(x, 1u, pos); }
-
-__device__ __forceinline__ void sts128(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d)
-{
-    ZC_DBG_SHARED(addr, 16, return);
-    asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};" :: "r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
-}
-__device__ __forceinline__ uint4 lds128(uint32_t addr)
-{
-    ZC_DBG_SHARED(addr, 16, return make_uint4(0, 0, 0, 0));
-    uint4 v;
-    asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr));
-    return v;
-}
 
 // Decode one word of 4 symbols from a piece staged in shared memory.  K = symbols per lookup (1 or 2).
 // A window of 32 bits serves two lookups of at most 12 bits each.

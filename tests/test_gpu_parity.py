@@ -373,3 +373,19 @@ def test_decoder_at_the_chunk_counts_where_its_kernel_changes(fmt, policy, chunk
             zc.decompress_chunks(p, d_comp, cont.size, first, count, back, d_ws)
             assert zc.device_status(p, d_ws) == zc.OK
             assert torch.equal(back[: hi - lo], want[lo:hi]) and bool((back[hi - lo:] == 0xEE).all())
+
+
+@pytest.mark.parametrize("counts", [[255 - k for k in range(256)], [2 ** max(0, 40 - k) for k in range(256)], [1] * 256,
+                                    [2 ** max(0, 11 - k) for k in range(256)], [10 ** 6] + [1] * 255, [7] + [0] * 255, [7, 7] + [0] * 254])
+def test_decode_tables_of_every_shape_of_code(counts):
+    """Codes of all lengths from 1 to 12, of one length only, and of one or two symbols: windows that start with a code of up
+    to 9 bits, of 10 to 12 bits, and of no symbol."""
+    rng = np.random.default_rng(5)
+    c = np.array(counts, dtype=np.float64)
+    n = 40 * 2048
+    lo = rng.choice(256, n, p=c / c.sum()).astype(np.uint32)         # the exponent byte of BF16 carries the counts
+    rest = rng.integers(0, 256, n, dtype=np.uint32)
+    v = ((rest & 0x80) << 8) | (lo << 7) | (rest & 0x7F)
+    data = v.astype(np.uint16).view(np.uint8)
+    for chunk_bytes in (4096, 65536):
+        _gpu_round_trip(zc.FMT_BF16, data, n, chunk_bytes, zc.POLICY_HUFF_ALL)
