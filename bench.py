@@ -41,8 +41,8 @@ ORACLE_SAMPLE_BYTES = int(os.environ.get("ZC_ORACLE_SAMPLE_BYTES", 768 << 20))  
 # stack of 872.4 MB, 4 KiB chunks, batched kernels); traffic grows in proportion to the input, so the figure for a
 # launch over the whole stack is this ratio times its input bytes.  The write part is undercounted in a capture
 # because some of the output is still in L2 when the kernel ends.
-NCU_DRAM_BYTES_PER_INPUT_BYTE = {"decode_kernel": (607251968.0 + 827155200.0) / 872415232.0,
-                                 "encode_kernel": (872882944.0 + 535107840.0) / 872415232.0}
+NCU_DRAM_BYTES_PER_INPUT_BYTE = {"decode_kernel": (603383040.0 + 825236480.0) / 872415232.0,
+                                 "encode_kernel": (872557824.0 + 553053952.0) / 872415232.0}
 
 
 def measured_peaks():
@@ -643,7 +643,7 @@ def measure(args, ctx):
         for t in tensors:
             key = tuple(t["cb"].modes) if t["n"] else (0, 0)
             combos[key] = combos.get(key, 0) + 1
-        n_enc_launch = sum((c + 255) // 256 for c in combos.values())
+        n_enc_launch = len(combos)
         n_dec_launch = (n_t + 447) // 448
         n_hist_launch = (n_t + 767) // 768
         # the step encodes group by group: one launch per group and combination of stream modes in it
@@ -653,7 +653,7 @@ def measure(args, ctx):
             for i in g["idx"]:
                 key = tuple(tensors[i]["cb"].modes) if tensors[i]["n"] else (0, 0)
                 gc[key] = gc.get(key, 0) + 1
-            n_enc_launch_step += sum((c + 255) // 256 for c in gc.values())
+            n_enc_launch_step += len(gc)
     else:
         n_enc_launch = n_dec_launch = n_hist_launch = n_enc_launch_step = n_t
     # delta form: the earlier checkpoint is read once more by every kernel

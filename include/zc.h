@@ -298,7 +298,7 @@ zc_status zc_decompress_chunks(const zc_plan_t* plan, const void* d_comp, size_t
  *      tensors, each compressed on its own with its own codes; Sec. 3.3: K and V of all layers) -
  * The containers are byte for byte those of n_tensors calls of zc_compress; the chunks of all
  * tensors are handed out through one ticket counter, so that small tensors do not pay a launch
- * each (one launch per combination of stream modes that occurs and per 256 tensors of it).
+ * each (one launch per combination of stream modes that occurs).
  * n_tensors        number of tensors (0 returns ZC_OK and launches nothing)
  * plans            host array of n_tensors plans; all must have the same format and chunk_bytes
  * codebooks        host array, one codebook per tensor; tensors may share one (the pages of a K/V cache

@@ -4,8 +4,8 @@
 // with a bulk asynchronous copy (TMA, non-multicast) completing on an mbarrier.  Work proceeds in
 // rounds: every lane decodes R symbols of its own subchunk into a padded row of shared memory, then the
 // whole warp merges 32 x R symbols with the other stream and writes 16-byte vectors, fully coalesced.
-// Raw sign+mantissa bytes for a round are fetched into registers before the round's decoding, so the
-// DRAM latency hides behind the table lookups.
+// Raw sign+mantissa bytes of a round (and, for deltas, the base tensor's bytes) are prefetched into the L2 before the
+// round's decoding, so the DRAM latency hides behind the table lookups.
 #include "zc_device.cuh"
 
 #include <atomic>
