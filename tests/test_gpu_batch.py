@@ -391,6 +391,46 @@ def test_xor_delta_batched_calls():
         assert np.array_equal(out[: p.input_bytes], b[: p.input_bytes]) and (out[p.input_bytes:] == 0xEE).all()
 
 
+@pytest.mark.parametrize("fmt,chunk_bytes", [(zc.FMT_BF16, 8192), (zc.FMT_BF16, 13312), (zc.FMT_BF16, 24576), (zc.FMT_FP8_E4M3, 16384)])
+def test_batched_delta_of_tensors_that_end_in_constant_chunks_and_a_partial_batch(fmt, chunk_bytes):
+    """Chunks of several warps' tiles, both streams coded.  A constant chunk is coded without the team of warps meeting a
+    second time, and in a tensor's last batch some teams have no chunk at all: tensors of every length on both sides of a
+    batch whose chunks are constant up to the end, so that teams go from a constant chunk over a batch without one to the
+    next tensor's first chunk."""
+    G = zo.group(fmt)
+    cs = chunk_bytes // 2
+    rng = np.random.default_rng(chunk_bytes)
+    sizes, bases, curs, deltas = [], [], [], []
+    for i in range(360):
+        chunks = 1 + i % 17
+        n = (chunks * cs - (int(rng.integers(1, cs)) if i % 5 == 4 else 0)) * G
+        base = _weights(fmt, n, 3000 + i)
+        delta = np.zeros_like(base)
+        head = min(base.size, chunk_bytes * (1 + i % 3))                 # what is not constant
+        delta[:head] = rng.integers(0, 4, head, dtype=np.uint8) * (rng.random(head) < 0.3)
+        sizes.append(n); bases.append(base); curs.append(base ^ delta); deltas.append(delta)
+    plans = [zc.plan(fmt, n, chunk_bytes) for n in sizes]
+    hists = [zo.histogram(fmt, d, n) for d, n in zip(deltas, sizes)]
+    ocbs = [zo.build_codebook(h, zc.POLICY_HUFF_ALL) for h in hists]
+    d_bases, d_curs = [_to_dev(b) for b in bases], [_to_dev(c) for c in curs]
+    d_outs = [torch.empty(p.max_compressed_bytes, dtype=torch.uint8, device=DEV) for p in plans]
+    batch = zc.CompressBatch(plans, d_curs, d_outs, d_bases)
+    batch.set_codebooks([zc.build_codebook(p, h, zc.POLICY_HUFF_ALL) for p, h in zip(plans, hists)])
+    ws = torch.empty(batch.workspace_bytes, dtype=torch.uint8, device=DEV)
+    wants = [zo.compress(fmt, d, n, chunk_bytes, ocb) for d, n, ocb in zip(deltas, sizes, ocbs)]
+    for _ in range(5):
+        for o in d_outs:
+            o.fill_(0xA5)
+        got = zc.compress_batch(batch, ws)
+        for t, (want, out, nbytes) in enumerate(zip(wants, d_outs, got)):
+            assert nbytes == want.size and np.array_equal(out[:nbytes].cpu().numpy(), want), t
+    backs = [torch.full((max(p.input_bytes, 16),), 0xEE, dtype=torch.uint8, device=DEV) for p in plans]
+    zc.decompress_batch(zc.DecompressBatch(plans, d_outs, got, backs, d_bases), ws)
+    assert zc.batch_status(ws) == (zc.OK, None)
+    for p, cur, back in zip(plans, curs, backs):
+        assert np.array_equal(back[: p.input_bytes].cpu().numpy(), cur[: p.input_bytes])
+
+
 def test_batched_calls_at_bench_size_on_sampled_chunks():
     """Tensors of the size class the benchmark times (a 14336 x 4096 and a 4096 x 4096 BF16 matrix and a 1024 x 4096
     one, 4 KiB chunks, the batched calls): the oracle decodes sampled chunks one by one, properties that hold at
