@@ -602,6 +602,7 @@ __device__ __forceinline__ uint32_t run_chunks(const DecParams& P, const DecShar
         if (sliced1) staged1 = true;
         if (sliced0 || sliced1) {
             rel0 = start0; rel1 = start1;
+            org0 = org1 = 0;                                     // lanes without symbols take no slice and stay at position 0
             issue_slices(end0 > start0, end1 > start1);          // lanes that have bits at all
         }
         if (H0 && piece0 + 16 <= slot_bytes) {

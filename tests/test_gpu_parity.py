@@ -389,3 +389,28 @@ def test_decode_tables_of_every_shape_of_code(counts):
     data = v.astype(np.uint16).view(np.uint8)
     for chunk_bytes in (4096, 65536):
         _gpu_round_trip(zc.FMT_BF16, data, n, chunk_bytes, zc.POLICY_HUFF_ALL)
+
+
+@pytest.mark.parametrize("fmt", [zc.FMT_BF16, zc.FMT_FP8_E4M3])
+@pytest.mark.parametrize("chunk_kib", [40, 48, 56, 64])
+def test_ragged_large_chunk_behind_complete_ones_of_the_same_warp(fmt, chunk_kib):
+    """Both streams coded, pieces staged slice by slice, more chunks than warps: the last chunk, long enough for slices and
+    with lanes that have no symbols, is decoded by a warp that has decoded a complete one before, in the single and in the
+    batched form."""
+    cs = chunk_kib * 512
+    n = (1500 * cs + cs * 3 // 4 + 5) * zo.group(fmt)
+    g = torch.Generator(device=DEV); g.manual_seed(chunk_kib)
+    x = torch.randn(n, generator=g, device=DEV)
+    d_in = ((x * 0.02).to(torch.bfloat16) if fmt == zc.FMT_BF16 else (x * 80).clamp(-448, 448).to(torch.float8_e4m3fn)).view(torch.uint8)
+    p = zc.plan(fmt, n, chunk_kib * 1024)
+    cb = zc.build_codebook(p, zc.histogram(p, d_in).cpu().numpy(), zc.POLICY_HUFF_ALL)
+    d_out = torch.empty(p.max_compressed_bytes, dtype=torch.uint8, device=DEV)
+    ws = torch.empty(p.workspace_bytes, dtype=torch.uint8, device=DEV)
+    nbytes = zc.compress(p, cb, d_in, d_out, ws)
+    assert zc.validate_container(p, d_out[:nbytes].cpu().numpy()) == zc.OK
+    back = torch.zeros(p.input_bytes, dtype=torch.uint8, device=DEV)
+    zc.decompress(p, d_out, nbytes, back, ws)
+    assert zc.device_status(p, ws) == zc.OK and torch.equal(back, d_in)
+    back.zero_()
+    zc.decompress_batch(zc.DecompressBatch([p], [d_out], [nbytes], [back]), ws)
+    assert zc.batch_status(ws) == (zc.OK, None) and torch.equal(back, d_in)
