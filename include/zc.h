@@ -201,6 +201,8 @@ zc_status zc_histogram_batch(uint32_t n_tensors, const zc_plan_t* const* plans, 
  * Lengths are those of an optimal prefix code with maximum length 12 (leaves ordered by
  * (count, symbol); leaf before package at equal weight); codes are canonical in
  * (length, symbol) order; a stream with one active symbol gets a 1-bit code.
+ * Counts may have any value; ZC_POLICY_STATIC refuses (INVALID_ARG) a stream of 2^54 symbols or more, since it
+ * multiplies the counts by 256.
  * Host-only: needs no GPU.  Errors: INVALID_ARG, UNSUPPORTED (policy), NOMEM. */
 zc_status zc_build_codebook(const zc_plan_t* plan, const uint64_t* h_hist, zc_policy policy,
                             zc_codebook_t** out);

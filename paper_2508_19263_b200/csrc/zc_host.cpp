@@ -102,6 +102,60 @@ struct MergeScratch {
     uint16_t leaves_in[kLmax][513];                              // [r][k]: leaves among the first k items of level r
 };
 
+// Reads the code lengths off the levels: how many leaves each level's chosen prefix holds, from the last level to the first.
+// sym(i): the symbol of the i-th leaf.
+template <class Sym>
+bool chosen_lengths(const MergeScratch& scratch, const size_t* size, size_t n, uint32_t L, Sym sym, uint8_t len[256])
+{
+    uint32_t reach[257] = {0};                                   // [k]: levels whose chosen prefix holds exactly k leaves
+    size_t take = 2 * n - 2;
+    for (int r = (int)L - 1; r >= 0 && take > 0; --r) {
+        if (take > size[r]) return false;
+        const size_t leaves = scratch.leaves_in[r][take];
+        ++reach[leaves];
+        take = 2 * (take - leaves);
+    }
+    for (size_t i = n, levels = 0; i-- > 0;) {
+        levels += reach[i + 1];
+        len[sym(i)] = (uint8_t)levels;
+    }
+    return true;
+}
+
+// The quick construction below keeps a symbol beside its count in 64 bits, and sentinels above every weight (a weight of
+// level r is at most 2^r times the largest count): counts stay below this.  No tensor has as many symbols, but a caller may
+// give any histogram.
+constexpr uint64_t kQuickCounts = 1ull << 50;
+
+// limited_lengths for histograms with larger counts: the same lists, merged one item after the other.
+bool limited_lengths_any_count(const uint64_t hist[256], uint32_t L, uint8_t len[256], MergeScratch& scratch)
+{
+    int order[256];
+    size_t n = 0;
+    for (int v = 0; v < 256; ++v)
+        if (hist[v]) order[n++] = v;
+    if (n == 1) { len[order[0]] = 1; return true; }
+    if (L > kLmax || (1ull << L) < n) return false;
+    std::sort(order, order + n, [&](int a, int b) { return hist[a] != hist[b] ? hist[a] < hist[b] : a < b; });
+    size_t size[kLmax], np = 0;
+    for (uint32_t r = 0; r < L; ++r) {
+        const uint64_t* pw = scratch.w[(r + 1) & 1];
+        uint64_t* cw = scratch.w[r & 1];
+        uint16_t* in = scratch.leaves_in[r];
+        size_t a = 0, b = 0, m = 0;
+        while (a < n || b < np) {
+            const uint64_t pk = b < np ? pw[2 * b] + pw[2 * b + 1] : 0;
+            in[m] = (uint16_t)a;
+            if (b == np || (a < n && hist[order[a]] <= pk)) cw[m++] = hist[order[a++]];
+            else { cw[m++] = pk; ++b; }
+        }
+        in[m] = (uint16_t)n;
+        size[r] = m;
+        np = m / 2;
+    }
+    return chosen_lengths(scratch, size, n, L, [&](size_t i) { return order[i]; }, len);
+}
+
 // Optimal code lengths under a maximum length, by package-merge in its prefix-count form:
 // only the weights and the number of leaves in every prefix of each level's merged list are kept.  Because
 // the leaves are sorted, the leaves chosen at a level are always a prefix of the sorted list,
@@ -114,7 +168,7 @@ bool limited_lengths(const uint64_t hist[256], uint32_t L, uint8_t len[256], Mer
 {
     std::memset(len, 0, 256);
     for (int v = 0; v < 256; ++v)
-        if (hist[v] >> 55) return false;                         // the sort's keys have 64 bits, sums of 256 counts stay below 2^63
+        if (hist[v] >= kQuickCounts) return limited_lengths_any_count(hist, L, len, scratch);
     uint64_t key[256];
     const size_t n = sort_leaves(hist, key);
     if (n == 0) return true;
@@ -194,19 +248,7 @@ bool limited_lengths(const uint64_t hist[256], uint32_t L, uint8_t len[256], Mer
         in[m] = (uint16_t)n;
         size[r] = m;
     }
-    uint32_t reach[257] = {0};                                   // [k]: levels whose chosen prefix holds exactly k leaves
-    size_t take = 2 * n - 2;
-    for (int r = (int)L - 1; r >= 0 && take > 0; --r) {
-        if (take > size[r]) return false;
-        const size_t leaves = leaves_in[r][take];
-        ++reach[leaves];
-        take = 2 * (take - leaves);
-    }
-    for (size_t i = n, levels = 0; i-- > 0;) {
-        levels += reach[i + 1];
-        len[key[i] & 0xFF] = (uint8_t)levels;
-    }
-    return true;
+    return chosen_lengths(scratch, size, n, L, [&](size_t i) { return key[i] & 0xFF; }, len);
 }
 
 // Canonical assignment: walk the lengths from short to long, symbols ascending inside a length.

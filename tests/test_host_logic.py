@@ -121,6 +121,39 @@ def test_codebook_matches_oracle_on_adversarial_histograms():
             _compare_codebook(h2, policy)
 
 
+@pytest.mark.parametrize("bits", [41, 42, 47, 49, 50, 53, 54, 55, 56, 58])
+def test_codebook_takes_counts_of_any_size(bits):
+    """Counts on both sides of every power where keys, sums or smoothed counts could run out of bits; a static dictionary
+    is refused from 2^54 symbols on and nowhere below."""
+    rng = np.random.default_rng(bits)
+    p = zc.plan(zc.FMT_BF16, 16, 1024)
+    for trial in range(60):
+        n = int(rng.choice([1, 2, 3, 7, 31, 256]))
+        top = max(1, (1 << bits) // n) if trial % 2 else 1 << bits        # the sum, or the largest count, is about 2^bits
+        h2 = np.zeros((2, 256), np.uint64)
+        for s in range(2):
+            kind = (trial + s) % 4
+            if kind == 0:
+                c = [top] * n
+            elif kind == 1:
+                c = [max(1, top >> int(k)) for k in rng.integers(0, 20, n)]
+            elif kind == 2:
+                c = [max(1, top - 3 + int(k)) for k in rng.integers(0, 6, n)]
+            else:
+                c = [1 + int(k) for k in rng.integers(0, 5, n)]
+                c[0] = top
+            h2[s, rng.permutation(256)[:n]] = np.array(c, np.uint64)
+        if max(int(h2[s].astype(object).sum()) for s in range(2)) >= 1 << 60:
+            continue                                                      # the policy's own products would leave 64 bits
+        for policy in (zc.POLICY_AUTO, zc.POLICY_HUFF_ALL, zc.POLICY_STATIC):
+            if policy == zc.POLICY_STATIC and max(int(h2[s].astype(object).sum()) for s in range(2)) >= 1 << 54:
+                with pytest.raises(zc.ZcError) as e:
+                    zc.build_codebook(p, h2, policy)
+                assert e.value.status == zc.E_INVALID_ARG
+            else:
+                _compare_codebook(h2, policy)
+
+
 def test_codebook_matches_oracle_on_random_histograms():
     rng = np.random.default_rng(1)
     for trial in range(1500):
