@@ -210,11 +210,13 @@ def _quick_function(name, restype, argtypes=None):
 class Codebook:
     """zc_build_codebook result: per stream a mode, 256 code lengths and 256 canonical code values."""
 
-    __slots__ = ("_h", "_owned")
-
     def __init__(self, handle: int, owned: bool = True):
         self._h = handle
         self._owned = owned                      # a dictionary's codebook belongs to the dictionary
+
+    def __reduce_ex__(self, protocol):
+        # the handle is an address in this process with one owner: a copy would destroy it a second time
+        raise ValueError("a codebook cannot be copied or pickled")
 
     def get(self, stream_idx: int):
         mode = C.c_uint32()

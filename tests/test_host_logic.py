@@ -217,6 +217,26 @@ def test_dictionary_object_follows_the_replacement_rule():
         d.observe(0, 10)
 
 
+def test_codebook_objects_own_their_handle_and_are_ordinary_objects():
+    import copy
+    import gc
+    import pickle
+    import weakref
+    p = zc.plan(zc.FMT_BF16, 16, 1024)
+    cb = zc.build_codebook(p, np.ones((2, 256), np.uint64))
+    many = zc.build_codebooks([p, p], np.ones((2, 2, 256), np.uint64))
+    for c in [cb] + many + [zc.Dictionary(p, np.ones((2, 256), np.uint64), 0.1).codebook]:
+        for duplicate in (pickle.dumps, copy.copy, copy.deepcopy):       # two owners of one handle
+            with pytest.raises(ValueError):
+                duplicate(c)
+    cb.note = "a program's own attribute"
+    gone = weakref.ref(cb)
+    assert gone() is cb and cb.get(0)[1].max() == 8
+    del cb, c
+    gc.collect()
+    assert gone() is None
+
+
 def test_codebook_on_workload_like_histograms():
     import torch
     from paper_2508_19263_b200 import workloads as wl
