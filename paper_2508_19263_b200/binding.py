@@ -322,9 +322,13 @@ class Dictionary:
 
     # made for every page of a step: checking and converting the arguments and letting go of the GIL took 0.9 us, this 0.5 us
     def observe(self, input_bytes: int, container_bytes: int, _observe=_quick_function("zc_dict_observe", C.c_int)) -> bool:
-        self._in.value = input_bytes
-        self._out.value = container_bytes
-        status = _observe(self._h, self._in, self._out, self._flag_ref)
+        try:
+            self._in.value = input_bytes
+            self._out.value = container_bytes
+        except TypeError:                        # not a plain number: converted, or refused, argument by argument
+            status = _lib.zc_dict_observe(self._h, input_bytes, container_bytes, self._flag_ref)
+        else:
+            status = _observe(self._h, self._in, self._out, self._flag_ref)
         if status != OK:
             raise ZcError(status, "zc_dict_observe")
         return self._flag.value != 0

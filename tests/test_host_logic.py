@@ -215,6 +215,13 @@ def test_dictionary_object_follows_the_replacement_rule():
     d = zc.Dictionary(p, h, 0.1)
     with pytest.raises(zc.ZcError):
         d.observe(0, 10)
+    # sizes as a program may have them: NumPy integers, ctypes numbers; nothing else is taken for a size
+    assert not d.observe(np.int64(100), ctypes.c_uint64(50)) and not d.observe(ctypes.c_uint64(100), 55)
+    assert d.observe(ctypes.c_uint64(100), np.uint32(60)) and d.info.last_ratio == 0.6
+    for bad in ((100.0, 50), (100, "50"), (None, 1)):
+        with pytest.raises(ctypes.ArgumentError):
+            d.observe(*bad)
+    assert d.info.n_observed == 3
 
 
 def test_codebook_objects_own_their_handle_and_are_ordinary_objects():
