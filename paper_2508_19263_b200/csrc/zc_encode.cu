@@ -2,6 +2,7 @@
 #include "zc_encode.cuh"
 
 #include <atomic>
+#include <cstdlib>
 #include <cstring>
 #include <unordered_map>
 #include <vector>
@@ -133,11 +134,30 @@ BatchLayout batch_layout(uint32_t n_tensors, uint64_t total_batches)
 // it goes through a pinned staging buffer, one per calling thread, that is reused once the previous copy
 // out of it has been done (an event says so).  The buffer is never freed (a thread's last CUDA calls may come
 // after the runtime has shut down).  Without pinned memory the copy falls back to the pageable one.
+// A copy that is being captured into a graph is made anew by every replay, long after this call has returned and the
+// buffers here hold another call's lists: its source is a block of its own that the graph, and what is instantiated from it,
+// keeps.
 struct TableStage { void* ptr = nullptr; size_t cap = 0; cudaEvent_t done = nullptr; int device = -1; };
 
 cudaError_t upload_host(void* d_dst, const void* h_src, size_t bytes, cudaStream_t st)
 {
     static thread_local TableStage stage;
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    cudaGraph_t graph = nullptr;
+    cudaError_t ec = cudaStreamGetCaptureInfo_v2(st, &capture, nullptr, &graph);
+    if (ec != cudaSuccess) return ec;
+    if (capture != cudaStreamCaptureStatusNone) {
+        if (capture != cudaStreamCaptureStatusActive) return cudaErrorStreamCaptureInvalidated;
+        void* const kept = std::malloc(bytes);
+        if (!kept) return cudaErrorMemoryAllocation;
+        std::memcpy(kept, h_src, bytes);
+        cudaUserObject_t owner;
+        ec = cudaUserObjectCreate(&owner, kept, std::free, 1, cudaUserObjectNoDestructorSync);
+        if (ec != cudaSuccess) { std::free(kept); return ec; }
+        ec = cudaGraphRetainUserObject(graph, owner, 1, cudaGraphUserObjectMove);
+        if (ec != cudaSuccess) { cudaUserObjectRelease(owner, 1); return ec; }
+        return cudaMemcpyAsync(d_dst, kept, bytes, cudaMemcpyHostToDevice, st);
+    }
     if (bytes <= 48 * 1024)                      // small copies leave the caller's memory at once anyway
         return cudaMemcpyAsync(d_dst, h_src, bytes, cudaMemcpyHostToDevice, st);
     int device = -1;

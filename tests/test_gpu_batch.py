@@ -204,6 +204,39 @@ def test_batched_encoder_with_codebooks_shared_between_tensors(fmt):
         assert np.array_equal(back[: p.input_bytes].cpu().numpy(), data[: p.input_bytes])
 
 
+@pytest.mark.parametrize("count", [5, 90])
+def test_a_captured_batched_encode_keeps_its_arguments(count):
+    """A serving step with static dictionaries in a CUDA graph: replayed after other calls of the same thread, on the pages'
+    new contents, it still codes its own tensors with its own tables (few and many: small and large uploads)."""
+    fmt, chunk_bytes, n = zc.FMT_BF16, 4096, 9000
+    sizes = [n + 16 * i for i in range(count)]
+    plans = [zc.plan(fmt, m, chunk_bytes) for m in sizes]
+    hists = [zo.histogram(fmt, _weights(fmt, m, 60 + i), m) for i, m in enumerate(sizes)]
+    cbs = [zc.build_codebook(p, h, zc.POLICY_STATIC) for p, h in zip(plans, hists)]
+    ocbs = [zo.build_codebook(h, zc.POLICY_STATIC) for h in hists]
+    d_ins = [_to_dev(_weights(fmt, m, 60 + i)) for i, m in enumerate(sizes)]
+    d_outs = [torch.zeros(p.max_compressed_bytes, dtype=torch.uint8, device=DEV) for p in plans]
+    batch = zc.CompressBatch(plans, d_ins, d_outs)
+    batch.set_codebooks(cbs)
+    ws = torch.empty(batch.workspace_bytes, dtype=torch.uint8, device=DEV)
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        zc.compress_batch(batch, ws, sync=False)
+    for seed in (200, 500):
+        _, _, _, _, other, other_ws = _batch_compress(fmt, [7000 + 100 * i for i in range(2 * count)], chunk_bytes, seed, [zc.POLICY_HUFF_ALL])
+        zc.compress_batch(other, other_ws)
+        datas = [_weights(fmt, m, seed + 7 * i) for i, m in enumerate(sizes)]
+        for t, d, o in zip(d_ins, datas, d_outs):
+            t[: d.size] = torch.from_numpy(d).to(DEV)
+            o.zero_()
+        graph.replay()
+        torch.cuda.synchronize()
+        assert zc.batch_status(ws) == (zc.OK, None)
+        for m, d, ocb, o in zip(sizes, datas, ocbs, d_outs):
+            want = zo.compress(fmt, d, m, chunk_bytes, ocb)
+            assert np.array_equal(o[: want.size].cpu().numpy(), want)
+
+
 def test_batched_encoder_reports_a_symbol_without_code_and_its_tensor():
     fmt, chunk_bytes = zc.FMT_BF16, 4096
     sizes = [30000, 50000, 20000]
