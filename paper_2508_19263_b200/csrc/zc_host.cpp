@@ -396,6 +396,8 @@ zc_status zc_build_codebook(const zc_plan_t* plan, const uint64_t* h_hist, zc_po
     return ZC_OK;
 }
 
+constexpr uint32_t kOwnThreads = 16;             // most threads a batched call takes by itself
+
 zc_status zc_build_codebooks(uint32_t n_tensors, const zc_plan_t* const* plans, const uint64_t* h_hists, zc_policy policy,
                              uint32_t n_threads, zc_codebook_t** out)
 {
@@ -405,10 +407,11 @@ zc_status zc_build_codebooks(uint32_t n_tensors, const zc_plan_t* const* plans, 
     for (uint32_t t = 0; t < n_tensors; ++t) if (!plans[t]) return ZC_E_INVALID_ARG;
     if (n_threads == 0) {
         const uint32_t hw = std::max(1u, std::thread::hardware_concurrency());
-        n_threads = std::min<uint32_t>({hw, 16u, (n_tensors + 7) / 8});     // a codebook takes about ten microseconds, a thread twice that
+        n_threads = std::min<uint32_t>({hw, kOwnThreads, (n_tensors + 7) / 8});     // a codebook takes about ten microseconds, a thread twice that
     }
     n_threads = std::max<uint32_t>(1, std::min<uint32_t>(n_threads, n_tensors));
-    // The memory of all threads is the caller's: a new thread that allocates sets up an arena of its own first.
+    // The memory of all threads is the caller's: a new thread that allocates sets up an arena of its own first.  It is kept
+    // between calls for as many threads as a call uses by itself; more, for a caller who asks for more, are given back.
     static thread_local std::vector<MergeScratch> scratch;
     std::vector<zc_codebook_t*> made(n_tensors, nullptr);
     std::vector<std::thread> pool;
@@ -438,6 +441,7 @@ zc_status zc_build_codebooks(uint32_t n_tensors, const zc_plan_t* const* plans, 
     }
     if (room) work(0);
     for (auto& th : pool) th.join();
+    if (scratch.size() > kOwnThreads) std::vector<MergeScratch>().swap(scratch);
     if (first_error.load() != ZC_OK) {
         for (auto* cb : made) delete cb;
         return (zc_status)first_error.load();

@@ -365,6 +365,21 @@ def test_threaded_codebook_builder_matches_the_single_one():
     assert zc.build_codebooks([], np.zeros((0, 2, 256), np.uint64)) == []
 
 
+def test_threaded_codebook_builder_gives_the_memory_of_many_threads_back():
+    """Some 20 KB a thread: 3000 threads' worth does not stay with the calling thread."""
+    def resident():
+        return int(open("/proc/self/statm").read().split()[1]) * os.sysconf("SC_PAGE_SIZE")
+    n = 3000
+    plans = [zc.plan(zc.FMT_BF16, 16, 4096)] * n
+    hists = np.random.default_rng(1).integers(0, 1000, (n, 2, 256)).astype(np.uint64)
+    first = zc.build_codebooks(plans, hists, zc.POLICY_AUTO, 1)          # the codebooks themselves, kept on both sides
+    before = resident()
+    many = zc.build_codebooks(plans, hists, zc.POLICY_AUTO, n)
+    codebooks = n * 6000
+    assert resident() - before < codebooks + (24 << 20)
+    assert all(np.array_equal(a.get(s)[1], b.get(s)[1]) for a, b in zip(first[::97], many[::97]) for s in range(2))
+
+
 def test_codebook_builder_against_the_oracle_s_on_a_million_histograms(tmp_path):
     """tests/codebook_fuzz.c, one process per core: ties, Fibonacci, powers of two, counts near 2^33, ...
 
