@@ -665,7 +665,6 @@ encode_kernel(const __grid_constant__ EncParams P)
         uint32_t vend = 0;                                       // lane k: virtual end of the last batch it with it % 32 == k
         uint32_t bad = 0;
         bool failed = false;
-        uint32_t met = 0;                                        // batches so far in which my team met over its tiles' bit counts
         for (uint32_t it = 0;; ++it) {
             const uint32_t r = it % kEncRing;
             if (!wait_phase(&mb_info[r], (it / kEncRing) & 1u)) { failed = true; break; }
@@ -801,19 +800,15 @@ encode_kernel(const __grid_constant__ EncParams P)
 #pragma unroll
                     for (int h = 0; h < kHuff; ++h) chunk_bits[h] = (tile_bits[h] & kConstTile) ? 0u : tile_bits[h];
                 } else if (kHuff) {
-                    // Every warp of the team learns the bit counts of the chunk's tiles.  Two buffers in turn, by the batches in
-                    // which the team met: who writes a buffer again has met the team once more since, after everybody read it.
-                    // (By the number of the batch they would not do: between two batches of the same parity the team may have
-                    // had no unit, and a constant chunk is not met over a second time.)
-                    uint32_t (* const tile_counts)[kMaxW] = s_tile[met & 1u];
-                    ++met;
+                    // every warp of the team learns the bit counts of the chunk's tiles (the team meets once more before anybody
+                    // can write the same buffer again)
                     if (lane == 0)
 #pragma unroll
-                        for (int h = 0; h < kHuff; ++h) tile_counts[h][warp] = tile_bits[h];
+                        for (int h = 0; h < kHuff; ++h) s_tile[it & 1u][h][warp] = tile_bits[h];
                     if (!team_sync()) { failed = true; break; }
 #pragma unroll
                     for (int h = 0; h < kHuff; ++h) {
-                        const uint32_t v = lane < T ? tile_counts[h][my_team * T + lane] : kConstTile;
+                        const uint32_t v = lane < T ? s_tile[it & 1u][h][my_team * T + lane] : kConstTile;
                         const uint32_t a = warp_scan(v & ~kConstTile, lane);
                         const bool none = __all_sync(0xFFFFFFFFu, (v & kConstTile) != 0);
                         const uint32_t bits = __shfl_sync(0xFFFFFFFFu, a, 31);
@@ -866,9 +861,12 @@ encode_kernel(const __grid_constant__ EncParams P)
                     if (!room) { failed = true; break; }
                     // my share of the pieces starts from zero
                     for (uint32_t q = tw * 32 + lane; q < total; q += 32 * T) sts128_zero(ring_s + 16 * (piece_at + q));
-                    if (T == 1) __syncwarp();
-                    else if (!team_sync()) { failed = true; break; }
                 }
+                // The team meets for a constant chunk too, though nothing was zeroed: the next batch in which it has a chunk may
+                // be two batches on (a tensor's last batch need not have one for every team), where the tiles' bit counts go
+                // into the same buffer again, and nobody may still be reading them.
+                if (T == 1) __syncwarp();
+                else if (!team_sync()) { failed = true; break; }
                 const uint32_t c = u * unit_chunks + my_k;
 #pragma unroll
                 for (int h = 0; h < kHuff; ++h) {
