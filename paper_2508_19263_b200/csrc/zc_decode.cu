@@ -45,13 +45,13 @@ struct DecItem {
 // blocks end together although tensors, and SMs, differ in how fast they get through a range.  A range costs a block about
 // 12 us (waiting for its last warp, header, tables, first pieces), so there are few: with eight equal ones per block the
 // BF16 stack of 1.74 GB took 707 us.
-constexpr uint32_t kDecMaxRounds = 5;
+constexpr uint32_t kDecMaxRounds = 5, kDecOneRound = 64;
 constexpr uint32_t kDecBatchMax = 448;       // tensors per launch: the parameter block stays below 32 KiB
 struct DecBatchParams {
     Control* ctl;
     unsigned long long call_id;
     uint32_t cs, sub, chunk_bytes, format, group, pool_bytes;
-    uint32_t n_tensors, total_chunks, tensor_base, n_rounds;
+    uint32_t n_tensors, n_empty, tensor_base, n_rounds;   // n_empty: tensors without chunks
     uint32_t round_end[kDecMaxRounds];       // chunks of the first rounds
     uint32_t spin_limit, skip_copy, sliced;
     DecItem item[kDecBatchMax];
@@ -1203,8 +1203,8 @@ decode_split_kernel(const __grid_constant__ DecParams P)
     }
 }
 
-// Many tensors per launch: block b takes the chunks [b * total / grid, (b + 1) * total / grid) of the
-// concatenated chunk index space, tensor by tensor; it builds the tables of a tensor once for its whole share.
+// Many tensors per launch: the blocks take ranges of the concatenated chunk index space from a ticket counter (see
+// kDecMaxRounds) and go through a range tensor by tensor, building a tensor's tables once for its part of the range.
 // XOR: the launch has base tensors (delta form); a kernel of its own so that the plain form pays nothing for it.
 template <int FMT, int PPL, bool XOR>
 __global__ void __launch_bounds__(dec_block_warps<FMT, XOR>() * 32, 1)
@@ -1230,10 +1230,11 @@ decode_batch_kernel(const __grid_constant__ DecBatchParams B)
         if (err && raise_status(B.ctl, B.call_id, err)) B.ctl->failed = B.tensor_base + t + 1;
     };
 
-    // The ranges of all rounds come one after the other from a ticket counter.  Block 0 first walks over the tensors without
-    // chunks: their headers are still checked.
+    // The ranges of all rounds come one after the other from a ticket counter.  Block 0 first walks over the tensors, if there
+    // are any without chunks: their headers are still checked.  (The walk takes 0.1 us a tensor, which the block is late for its
+    // range: 64 BF16 pages of 129 chunks 37 us, without it 31 us.)
     __shared__ uint32_t s_range;
-    uint32_t empties = blockIdx.x == 0 ? 0u : B.n_tensors;      // cursor of that walk
+    uint32_t empties = blockIdx.x == 0 && B.n_empty ? 0u : B.n_tensors;      // cursor of that walk
     uint32_t t = 0, g = 0, g_hi = 0;
     bool in_range = false;
     for (;;) {
@@ -1464,6 +1465,40 @@ DecShape split_shape(const zc_plan_t* p, uint32_t n_chunks, uint32_t* groups)
     return s;
 }
 
+// Blocks of a batched launch: one per SM, or fewer.  The chunk index space is cut into equal ranges, and a range that reaches
+// over a tensor's end costs its block a second header, table and walk over a subchunk, one after the other.  A multiple of
+// the number of tensors has no such ranges when the tensors are of one size.  Taken is what is shorter for the block with the
+// longest way, in symbols of a lane's walk: a tensor's part costs kDecOpenSyms (9 us) and its chunks a walk for every round
+// over the warps.  (64 BF16 tensors of 9 chunks of 64 KiB: 135 us in 148 ranges, 77 us in 128; 36 of 64 chunks of 32 KiB: 77
+// and 52 us.)
+constexpr uint32_t kDecOpenSyms = 160, kDecChunkSyms = 16;
+uint32_t batch_grid(const DecItem* item, uint32_t n, uint32_t with_chunks, uint64_t total, uint32_t warps, uint32_t sub)
+{
+    const uint32_t most = (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>(total, (uint64_t)sm_count()));
+    const uint32_t even = with_chunks ? most / with_chunks * with_chunks : 0;
+    if (with_chunks < 2 || even == 0 || even == most || total >= (uint64_t)kDecOneRound * most * warps) return most;
+    auto longest = [&](const uint32_t ranges) {
+        const uint32_t step = (uint32_t)(total / ranges), odd = (uint32_t)(total % ranges);
+        uint32_t t = 0, g = 0, hi = 0, rest = 0, worst = 0;
+        uint64_t end = item[0].n_chunks;                         // where tensor t ends
+        for (uint32_t j = 0; j < ranges; ++j) {                  // range j ends at (j + 1) * total / ranges
+            hi += step;
+            rest += odd;
+            if (rest >= ranges) { rest -= ranges; ++hi; }
+            uint32_t way = 0;
+            while (g < hi) {
+                while (end <= g) end += item[++t].n_chunks;
+                const uint32_t part = (uint32_t)std::min<uint64_t>(hi, end) - g;
+                way += kDecOpenSyms + (part + warps - 1) / warps * (sub + kDecChunkSyms);
+                g += part;
+            }
+            worst = std::max(worst, way);
+        }
+        return worst;
+    };
+    return longest(even) < longest(most) ? even : most;
+}
+
 // no clearing of the workspace: errors are tagged with the id of the call that raised them
 unsigned long long new_call_id()
 {
@@ -1617,22 +1652,25 @@ zc_status zc_decompress_batch_xor(uint32_t n_tensors, const zc_plan_t* const* pl
             total += p->n_chunks;
             ++n;
         }
-        B.n_tensors = n; B.total_chunks = (uint32_t)total;
-        // one block per SM unless there are fewer chunks (a lane's walk over its subchunk is what a small launch takes, so
-        // its chunks are spread as far as they go)
-        const uint32_t grid = std::max<uint32_t>(1, std::min<uint32_t>((uint32_t)std::min<uint64_t>(total, 0xFFFFFFFFu), (uint32_t)sm_count()));
+        B.n_tensors = n;
         bool any_base = false;
-        for (uint32_t i = 0; i < n; ++i) any_base = any_base || B.item[i].base != nullptr;
+        B.n_empty = 0;
+        for (uint32_t i = 0; i < n; ++i) {
+            any_base = any_base || B.item[i].base != nullptr;
+            B.n_empty += B.item[i].n_chunks == 0;
+        }
+        const uint32_t grid = batch_grid(B.item, n, n - B.n_empty, total, shape.warps, B.sub);
         // Rounds: three quarters (deltas: half, since unchanged stretches take a fraction of the time) of what is left go to the
         // next one, in whole chunks per warp, until a range is down to two chunks per warp; the last one takes the rest.  With
-        // fewer than 32 chunks per warp in all, another range costs more than it evens out (FP8 at 16 KiB chunks, 9 chunks per
-        // warp: 219 us in one round, 270 us in three).
+        // fewer than kDecOneRound chunks per warp in all, another range costs more than it evens out (FP8 at 16 KiB chunks, 9
+        // chunks per warp: 219 us in one round, 270 us in three; BF16 at 1 KiB chunks, 44 per warp: 119 us in one round, 140 in
+        // four).
         const uint64_t turn = (uint64_t)grid * shape.warps;      // one chunk per warp
         uint64_t done = 0;
         B.n_rounds = 0;
         while (done < total) {
             const uint64_t left = total - done, part = (any_base ? left / 2 : left - left / 4) / turn * turn;
-            const bool last = B.n_rounds + 1 == kDecMaxRounds || total < 32 * turn || left - part < turn || part < 2 * turn;
+            const bool last = B.n_rounds + 1 == kDecMaxRounds || total < kDecOneRound * turn || left - part < turn || part < 2 * turn;
             done = last ? total : done + part;
             B.round_end[B.n_rounds++] = (uint32_t)done;
         }

@@ -555,8 +555,8 @@ def test_whole_containers_at_bench_size_equal_the_oracle_s(fmt, chunk_bytes):
 @pytest.mark.parametrize("fmt,chunk_bytes,chunks", [(zc.FMT_BF16, 4096, k) for k in (1, 31, 149, 2500, 5500)] +
                          [(zc.FMT_FP8_E4M3, 16384, k) for k in (1, 149, 700)] + [(zc.FMT_BF16, 1024, k) for k in (60000, 150000)])
 def test_batches_from_one_chunk_to_several_rounds(fmt, chunk_bytes, chunks):
-    """The batched decoder deals its chunks out in one to five rounds and the batched encoder holds one to three batches,
-    by the number of chunks: totals on both sides of those lines, in a large, a ragged and an empty tensor."""
+    """The batched encoder holds one to three batches of a block, by the number of chunks, and the batched decoder's blocks go
+    from less than a chunk to dozens per warp: totals on both sides of those lines, in a large, a ragged and an empty tensor."""
     cs = chunk_bytes // 2 * zo.group(fmt)
     a = chunks * 2 // 3
     sizes = [a * cs, 0, max((chunks - a) * cs - 3, 1)]
@@ -571,3 +571,61 @@ def test_batches_from_one_chunk_to_several_rounds(fmt, chunk_bytes, chunks):
     for p, data, back in zip(plans, datas, backs):
         back = back.cpu().numpy()
         assert np.array_equal(back[: p.input_bytes], data[: p.input_bytes]) and (back[p.input_bytes:] == 0xEE).all()
+
+
+def _encoded_batch(fmt, chunk_bytes, d_ins, sizes, d_bases=None):
+    """Containers of tensors on the device, by the library's own encoder (compared with the oracle's elsewhere)."""
+    plans = [zc.plan(fmt, n, chunk_bytes) for n in sizes]
+    d_hists = torch.zeros((len(plans), 2, 256), dtype=torch.int64, device=DEV)
+    zc.histogram_batch(zc.HistogramBatch(plans, d_ins, d_bases), d_hists)
+    d_outs = [torch.empty(p.max_compressed_bytes, dtype=torch.uint8, device=DEV) for p in plans]
+    enc = zc.CompressBatch(plans, d_ins, d_outs, d_bases)
+    enc.set_codebooks(zc.build_codebooks(plans, d_hists.cpu().numpy(), zc.POLICY_HUFF_ALL if d_bases else zc.POLICY_AUTO))
+    return plans, d_outs, zc.compress_batch(enc, torch.empty(enc.workspace_bytes, dtype=torch.uint8, device=DEV))
+
+
+@pytest.mark.parametrize("kind,chunks", [("plain", 300_000), ("plain", 750_000), ("scale", 200_000), ("delta", 200_000)])
+def test_batched_decoder_deals_chunks_out_in_several_rounds(kind, chunks):
+    """64 chunks per warp and more are dealt out in shrinking rounds, up to five (with 148 SMs: plain 4 and 5, scale 4, delta
+    5): a large tensor, an empty one, a ragged one, one without a base."""
+    fmt = zc.FMT_SCALE_U8 if kind == "scale" else zc.FMT_BF16
+    cs = 512 * zo.group(fmt)
+    sizes = [(chunks * 5 // 8) * cs, 0, (chunks // 4) * cs - 77, (chunks // 8) * cs + 1]
+    tile = torch.from_numpy(_weights(fmt, 8 << 20, chunks)).to(DEV)
+    nbytes = [zo.input_bytes(fmt, n) for n in sizes]
+    d_ins = [tile.repeat(-(-max(b, 16) // tile.numel()))[: max(b, 16)].clone() for b in nbytes]
+    d_bases = None
+    if kind == "delta":
+        g = torch.Generator(device=DEV); g.manual_seed(1)
+        d_bases = [x ^ (torch.rand(x.numel(), generator=g, device=DEV) < 0.1).to(torch.uint8) for x in d_ins]
+        d_bases[3] = None
+    plans, d_outs, got = _encoded_batch(fmt, 1024, d_ins, sizes, d_bases)
+    backs = [torch.zeros_like(x) for x in d_ins]
+    ws = torch.zeros(256, dtype=torch.uint8, device=DEV)
+    zc.decompress_batch(zc.DecompressBatch(plans, d_outs, got, backs, d_bases), ws)
+    assert zc.batch_status(ws) == (zc.OK, None)
+    for b, x, n in zip(backs, d_ins, nbytes):
+        assert torch.equal(b[:n], x[:n])
+
+
+@pytest.mark.parametrize("chunk_bytes", [4096, 32768])
+@pytest.mark.parametrize("count", [2, 20, 64, 147, 149])
+def test_batched_decoder_with_tensors_of_one_size_and_of_several(count, chunk_bytes):
+    """As many ranges as a multiple of the number of tensors, or as there are SMs, whichever is shorter for the longest
+    block: tensors of 1, 9 and 20 chunks, the last chunk ragged or not, alone and with empty and unlike tensors among them."""
+    fmt, cs = zc.FMT_FP8_E4M3, chunk_bytes
+    for chunks in (1, 9, 20):
+        n = chunks * cs - (chunks == 9) * 1000
+        for mixed in (False, True):
+            sizes = [n] * count
+            if mixed:
+                sizes[0], sizes[count // 2] = 0, 3 * n + 16
+            x = torch.from_numpy(_weights(fmt, 4 * n + 16 * count + 16, chunks)).to(DEV)
+            d_ins = [x[16 * i: 16 * i + max(m, 16)] for i, m in enumerate(sizes)]
+            plans, d_outs, got = _encoded_batch(fmt, chunk_bytes, d_ins, sizes)
+            backs = [torch.full((m + 16,), 0xEE, dtype=torch.uint8, device=DEV) for m in sizes]
+            ws = torch.zeros(256, dtype=torch.uint8, device=DEV)
+            zc.decompress_batch(zc.DecompressBatch(plans, d_outs, got, backs), ws)
+            assert zc.batch_status(ws) == (zc.OK, None)
+            for b, d, m in zip(backs, d_ins, sizes):
+                assert torch.equal(b[:m], d[:m]) and bool((b[m:] == 0xEE).all())
