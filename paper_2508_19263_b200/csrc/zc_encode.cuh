@@ -177,17 +177,25 @@ constexpr uint32_t kNoSlot = 0xFFFFFFFFu;        // "no more batches"
 constexpr uint32_t kConstTile = 0x80000000u;     // tile of nothing but the fill symbol
 constexpr int kLookWide = 4;                     // look-back rounds cover 32 * kLookWide predecessors
 
-// Kernel shapes: a chunk is one tile (4 KiB); a chunk is T whole tiles (8, 12, 16, .. KiB); everything else, with lanes of
-// 64 symbols (1 and 2 KiB: several chunks to a tile; odd sizes: the last tile is not full) or of 48 where that fills the
-// tiles better (3, 6, 9 KiB; BF16 weights at 6 KiB: 95 against 119 us); and chunks of 16 tiles with both streams coded,
-// whose team is larger than the other shapes' blocks.
-constexpr int kEncSolo = 0, kEncTeam = 1, kEncAny = 2, kEncAny48 = 3, kEncBig = 4;
-__host__ __device__ constexpr uint32_t enc_lane_syms(int shape) { return shape == kEncAny48 ? 48u : 64u; }
+// Kernel shapes:
+//   kEncSolo    a chunk is one tile (4 KiB)
+//   kEncTeam    a chunk is T whole tiles (8, 12, 16, .. KiB)
+//   kEncAny     everything else, with lanes of 64 symbols (1 and 2 KiB: several chunks to a tile; odd sizes: the last tile is
+//               not full)
+//   kEncAny48   the same with lanes of 48 where that fills the tiles better (3, 6, 9 KiB; BF16 weights at 6 KiB: 95 against 119 us)
+//   kEncBig     chunks that need more workers than the shape above has, or of which it fits twice the teams
+//   kEncSolo80, kEncSolo96, kEncSolo112   a chunk of 5, 6 or 7 KiB with one coded stream is one tile of long lanes: two tiles
+//               are a sixth to a quarter empty, and a team that meets twice per chunk is slower than a warp alone (128 MB of
+//               BF16 weights in two tiles / one, and in the encoder with lane regions that packed subchunk by subchunk: 5 KiB
+//               103 / 74 / 82 us, 6 KiB 86 / 69 / 82 us, 7 KiB 97 / 73 / 84 us)
+constexpr int kEncSolo = 0, kEncTeam = 1, kEncAny = 2, kEncAny48 = 3, kEncBig = 4, kEncSolo80 = 5, kEncSolo96 = 6, kEncSolo112 = 7;
+__host__ __device__ constexpr uint32_t enc_lane_syms(int shape) { return shape == kEncAny48 ? 48u : shape >= kEncSolo80 ? 16u * shape : 64u; }   // (these are numbered by the KiB of their chunks)
 constexpr uint32_t kMaxUnitChunks = 4;           // chunks of a unit (kEncAny)
-// Worker warps per block: the joined codes take 32 registers per lane and coded stream; with the two service warps that
-// makes 5 warps of 96 registers per scheduler with one coded stream, 4 of 128 with two.
+// Worker warps per block: the joined codes take half a register per symbol of a lane and coded stream; with the two service
+// warps that makes 5 warps of 96 registers per scheduler for 32 or fewer of them, 4 of 128 for more.  kEncAny gets the 128
+// with one coded stream too (with 18 workers it spills: BF16 weights at 1 KiB 83 -> 90 us, at 7 KiB 97 -> 106 us).
 constexpr uint32_t kServiceWarps = 2;
-__host__ __device__ constexpr uint32_t enc_max_workers(int shape, int n_huff) { return shape == kEncBig ? 16u : n_huff == 2 || shape == kEncAny ? 14u : 18u; }
+__host__ __device__ constexpr uint32_t enc_max_workers(int shape, int n_huff) { return shape == kEncBig ? 16u : n_huff == 2 || shape == kEncAny || shape >= kEncSolo80 ? 14u : 18u; }
 
 __device__ __forceinline__ uint32_t add_low_byte(uint32_t x, uint32_t acc) { return __dp4a(x, 1u, acc); }
 // Joins the table entries of two neighbouring symbols: codes behind one another in bits 31..8, length in bits 7..0.
@@ -313,7 +321,7 @@ encode_kernel(const __grid_constant__ EncParams P)
     constexpr int kHuff = (H0 ? 1 : 0) + (H1 ? 1 : 0);
     constexpr int kTabs = kHuff ? kHuff : 1;
     constexpr uint32_t kMaxW = enc_max_workers(SHAPE, kHuff);
-    constexpr bool kSolo = SHAPE == kEncSolo, kAny = SHAPE >= kEncAny;
+    constexpr bool kSolo = SHAPE == kEncSolo || SHAPE >= kEncSolo80, kAny = SHAPE >= kEncAny && SHAPE <= kEncBig;
     constexpr uint32_t kN = enc_lane_syms(SHAPE);               // symbols of a lane
     constexpr uint32_t kTileSyms = 32 * kN;
     extern __shared__ __align__(16) uint8_t smem[];

@@ -29,7 +29,14 @@ cudaError_t enc_launch_t(int shape, uint32_t grid, uint32_t threads, size_t smem
     else if (shape == kEncTeam) { ZC_ENC_CASE(kEncTeam) }
     else if (shape == kEncAny) { ZC_ENC_CASE(kEncAny) }
     else if (shape == kEncAny48) { ZC_ENC_CASE(kEncAny48) }
-    else { ZC_ENC_CASE(kEncBig) }
+    else if (shape == kEncBig) { ZC_ENC_CASE(kEncBig) }
+#undef ZC_ENC_CASE
+#define ZC_ENC_CASE(SHAPE)                                                   \
+    if (h0) launch(encode_kernel<F, true, false, SHAPE>);                   \
+    else launch(encode_kernel<F, false, true, SHAPE>);
+    else if (shape == kEncSolo80) { ZC_ENC_CASE(kEncSolo80) }                // one coded stream only (see enc_shape)
+    else if (shape == kEncSolo96) { ZC_ENC_CASE(kEncSolo96) }
+    else { ZC_ENC_CASE(kEncSolo112) }
 #undef ZC_ENC_CASE
     return e;
 }

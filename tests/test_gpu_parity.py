@@ -414,3 +414,33 @@ def test_ragged_large_chunk_behind_complete_ones_of_the_same_warp(fmt, chunk_kib
     back.zero_()
     zc.decompress_batch(zc.DecompressBatch([p], [d_out], [nbytes], [back]), ws)
     assert zc.batch_status(ws) == (zc.OK, None) and torch.equal(back, d_in)
+
+
+@pytest.mark.parametrize("fmt", FORMATS)
+@pytest.mark.parametrize("chunk_kib,chunks", [(5, 296), (5, 297), (6, 300), (7, 620), (13, 30), (19, 40), (29, 25), (30, 300), (31, 20)])
+@pytest.mark.parametrize("coded", [0, 1])
+def test_one_coded_stream_at_chunk_sizes_with_kernels_of_their_own(fmt, chunk_kib, chunks, coded):
+    """Chunks of 5 to 7 KiB that one warp codes (launches of more than two chunks per SM) and chunks of odd sizes whose teams
+    need the larger block, either stream coded and the other one raw, with and without a base tensor, a ragged end."""
+    cs = chunk_kib * 512
+    n = (chunks * cs - cs // 3 - 5) * zo.group(fmt)
+    data, base = _weights(fmt, n, chunk_kib), _weights(fmt, n, 100 + chunk_kib)
+    skewed, even = np.full((2, 256), 0, np.uint64), np.full(256, 1000, np.uint64)
+    skewed[0] = skewed[1] = (1 << 20) // (1 + np.arange(256)) ** 2 + 1
+    hist = np.stack([skewed[0], even] if coded == 0 else [even, skewed[1]])  # the AUTO rule: one stream coded, one raw
+    p = zc.plan(fmt, n, chunk_kib * 1024)
+    cb, ocb = zc.build_codebook(p, hist, zc.POLICY_STATIC), zo.build_codebook(hist, zo.POLICY_STATIC)
+    assert cb.modes == [1 - coded, coded]
+    d_base = torch.from_numpy(base).to(DEV)
+    for d_in, d_b in ((data, None), (data ^ base, d_base)):
+        d_out = torch.full((p.max_compressed_bytes + 64,), 0xA5, dtype=torch.uint8, device=DEV)
+        ws = torch.empty(p.workspace_bytes, dtype=torch.uint8, device=DEV)
+        nbytes = zc.compress(p, cb, torch.from_numpy(d_in).to(DEV), d_out[: p.max_compressed_bytes], ws, d_base=d_b)
+        want = zo.compress(fmt, data, n, chunk_kib * 1024, ocb)
+        got = d_out.cpu().numpy()
+        assert nbytes == want.size and np.array_equal(got[:nbytes], want) and (got[p.max_compressed_bytes:] == 0xA5).all()
+        back = torch.full((p.input_bytes + 32,), 0xEE, dtype=torch.uint8, device=DEV)
+        zc.decompress(p, d_out, nbytes, back, ws)
+        assert zc.device_status(p, ws) == zc.OK
+        back = back.cpu().numpy()
+        assert np.array_equal(back[: p.input_bytes], data[: p.input_bytes]) and (back[p.input_bytes:] == 0xEE).all()
