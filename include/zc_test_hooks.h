@@ -27,11 +27,12 @@ zc_status zc_test_merge16(zc_format fmt, const uint8_t* h_e8, const uint8_t* h_s
  *   zc_test_stall_encoder   zc_compress hands out its batches from this number on, so batch 0 is
  *                           never packed and every look-back waits for a word nobody posts
  *   zc_test_stall_decoder   the decoder does not start the copies of the pieces it waits for */
-/* Launch shapes (host arithmetic only, no GPU): worker warps per block the encoder would use for a plan
- * with n_coded Huffman-coded streams (0..2) in a long launch of the delta form (wide_slots: 0..2, the shape does not
- * depend on it), and warps per block of the decoder with one or both streams coded.  0 = the kernels cannot take this
- * plan.  A test checks that every chunk size zc_plan accepts gives at least one. */
-uint32_t zc_test_encoder_workers(const zc_plan_t* plan, uint32_t n_coded, uint32_t wide_slots);
+/* Launch shapes (host arithmetic only, no GPU): worker warps per block the encoder would use for a plan with n_coded
+ * Huffman-coded streams (0..2), with or without a base tensor, in a launch of total_chunks chunks, and warps per block of
+ * the decoder with one or both streams coded.  0 = the kernels cannot take this plan: more workers than the kernel is
+ * built for, more shared memory than a block has, or an output ring that does not hold a unit of 12-bit codes.  A test
+ * checks that every chunk size zc_plan accepts gives at least one. */
+uint32_t zc_test_encoder_workers(const zc_plan_t* plan, uint32_t n_coded, uint32_t any_base, uint64_t total_chunks);
 uint32_t zc_test_decoder_warps(const zc_plan_t* plan, uint32_t both_coded);
 void zc_test_set_wait_limit(uint32_t polls);
 void zc_test_stall_encoder(uint32_t first_ticket);

@@ -143,7 +143,7 @@ def _load():
     L.zc_noalloc_status.restype = C.c_int
     L.zc_noalloc_status.argtypes = [vp]
     L.zc_test_encoder_workers.restype = C.c_uint32
-    L.zc_test_encoder_workers.argtypes = [vp, C.c_uint32, C.c_uint32]
+    L.zc_test_encoder_workers.argtypes = [vp, C.c_uint32, C.c_uint32, C.c_uint64]
     L.zc_test_decoder_warps.restype = C.c_uint32
     L.zc_test_decoder_warps.argtypes = [vp, C.c_uint32]
     L.zc_test_debug_counts.restype = C.c_int
@@ -546,9 +546,9 @@ def test_debug_counts():
     return (int(out[0]), int(out[1])) if _lib.zc_test_debug_counts(out) else None
 
 
-def test_encoder_workers(p: Plan, n_coded: int, wide_slots: int) -> int:
-    """zc_test_encoder_workers; wide_slots is the slot class 0, 1 or 2."""
-    return int(_lib.zc_test_encoder_workers(p._h, n_coded, int(wide_slots)))
+def test_encoder_workers(p: Plan, n_coded: int, any_base: bool, total_chunks: int) -> int:
+    """zc_test_encoder_workers."""
+    return int(_lib.zc_test_encoder_workers(p._h, n_coded, int(any_base), total_chunks))
 
 
 def test_decoder_warps(p: Plan, both_coded: bool) -> int:

@@ -214,11 +214,13 @@ void debug_counts_encode(uint32_t out[2])
 
 extern "C" {
 
-uint32_t zc_test_encoder_workers(const zc_plan_t* p, uint32_t n_coded, uint32_t wide_slots)
+uint32_t zc_test_encoder_workers(const zc_plan_t* p, uint32_t n_coded, uint32_t any_base, uint64_t total_chunks)
 {
-    if (!p || n_coded > 2 || wide_slots > 2) return 0;
-    const EncShape sh = enc_shape(p, n_coded, true, ~0ull >> 1);
-    return sh.smem <= kEncSmem ? sh.tiles * sh.teams : 0;
+    if (!p || n_coded > 2 || any_base > 1) return 0;
+    const EncShape sh = enc_shape(p, n_coded, any_base != 0, total_chunks);
+    const uint32_t workers = sh.tiles * sh.teams, unit = n_coded * sh.unit_chunks * (uint32_t)round_up((uint64_t)p->syms_per_chunk * kLmax / 8, 16);
+    if (workers > enc_max_workers(sh.kind, (int)n_coded) || sh.smem > kEncSmem || 16 * sh.ring16 < unit) return 0;
+    return sh.tiles * 32 * enc_lane_syms(sh.kind) >= sh.unit_chunks * p->syms_per_chunk ? workers : 0;
 }
 
 zc_status zc_compress(const zc_plan_t* p, const zc_codebook_t* cb, const void* d_in, void* d_out, size_t out_capacity,

@@ -49,16 +49,19 @@ def test_plan_geometry(fmt):
 
 
 def test_every_accepted_chunk_size_has_a_launch_shape():
-    """Whatever zc_plan accepts, the encoder (any number of coded streams, every class of pack slots) and the
-    decoder (one or both streams coded) have a launch shape for; beyond the limit the plan itself is refused.
-    Half-size slots never leave room for fewer worker warps than the ordinary ones."""
+    """Whatever zc_plan accepts, the encoder (any number of coded streams, with and without a base tensor, launches of one
+    chunk to any number) has a launch shape for that fits a block, whose tiles hold its chunks and whose rings hold a unit
+    of the longest codes, and so has the decoder (one or both streams coded); beyond the limit the plan itself is refused."""
     for cb in range(1024, 65536 + 1, 1024):
         p = zc.plan(zc.FMT_BF16, 1 << 20, cb)
         for n_coded in (0, 1, 2):
-            for slots in (0, 1, 2):
-                assert zc.test_encoder_workers(p, n_coded, slots) >= 1, (cb, n_coded, slots)
-            assert zc.test_encoder_workers(p, n_coded, 2) >= zc.test_encoder_workers(p, n_coded, 0)
-            assert zc.test_encoder_workers(p, n_coded, 3) == 0
+            for any_base in (False, True):
+                few = zc.test_encoder_workers(p, n_coded, any_base, 1)
+                for total in (1, 100, 297, 1000, 5000, 1 << 32):
+                    workers = zc.test_encoder_workers(p, n_coded, any_base, total)
+                    assert workers >= 1, (cb, n_coded, any_base, total)
+                assert few <= workers <= 18                          # a launch of one chunk is one team
+        assert zc.test_encoder_workers(p, 3, False, 1) == 0
         for both in (False, True):
             assert zc.test_decoder_warps(p, both) >= 8, (cb, both)
 
