@@ -77,12 +77,6 @@ constexpr uint32_t kSliceSyms = 128;               // symbols a lane decodes fro
 constexpr uint32_t kSliceBytes = 256;              // copied per slice: 15 bytes of alignment + 128 * 12 bits + the window's look-ahead fit
 constexpr uint32_t kSliceSlot = 272;               // a lane's slot
 
-__device__ __forceinline__ void sts32_if(bool p, uint32_t addr, uint32_t v)
-{
-    if (p) ZC_DBG_SHARED(addr, 4, return);
-    asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %2, 0;\n\t@q st.shared.u32 [%0], %1;\n\t}"
-                 :: "r"(addr), "r"(v), "r"((uint32_t)p) : "memory");
-}
 __device__ __forceinline__ uint32_t lds32_if(bool p, uint32_t addr)
 {
     if (p) ZC_DBG_SHARED(addr, 4, return 0);

@@ -107,13 +107,6 @@ __device__ __forceinline__ uint4 ld_nc_v4(const void* p)
                  : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
     return v;
 }
-__device__ __forceinline__ uint2 ld_nc_v2(const void* p)
-{
-    ZC_DBG_GLOBAL(p, 8, 8, false, return make_uint2(0, 0));
-    uint2 v;
-    asm volatile("ld.global.nc.L1::no_allocate.v2.u32 {%0,%1}, [%2];" : "=r"(v.x), "=r"(v.y) : "l"(p));
-    return v;
-}
 __device__ __forceinline__ void st_cs_v4(void* p, uint4 v)
 {
     ZC_DBG_GLOBAL(p, 16, 16, true, return);
