@@ -25,18 +25,19 @@ EncShape enc_shape(const zc_plan_t* p, uint32_t n_huff, bool any_base, uint64_t 
     s.unit_chunks = 2 * cs <= full && full % cs == 0 ? std::min(kMaxUnitChunks, full / cs) : 1;
     const int solo = (int)(cs / 512);                            // the shapes of long lanes are numbered by the chunk's KiB
     if (cs == full) s.kind = kEncSolo;
+    else if (s.unit_chunks > 1) s.kind = kEncUnit;
     // (a launch of few chunks takes a warp's way through one, which is shorter in two tiles: 205 chunks of 5 KiB 16.2 against
     // 16.8 us; from about two chunks per SM on one tile is faster: 1184 chunks of 7 KiB 20.7 against 19.0 us)
     else if (n_huff == 1 && solo >= kEncSolo80 && solo <= kEncSolo112 && total_chunks > 2ull * sm_count()) s.kind = solo;
     else if (cs % full == 0) s.kind = kEncTeam;
-    else if (s.unit_chunks == 1 && tiles(small) * small < tiles(full) * full && tiles(small) <= enc_max_workers(kEncAny48, (int)n_huff)) s.kind = kEncAny48;
+    else if (tiles(small) * small < tiles(full) * full && tiles(small) <= enc_max_workers(kEncAny48, (int)n_huff)) s.kind = kEncAny48;
     else s.kind = kEncAny;
     s.tiles = tiles(32 * enc_lane_syms(s.kind));
     // kEncBig has the workers for 16 tiles, or with one coded stream for half as many teams again (29 to 31 KiB: two teams
     // instead of one, 128 MB of BF16 weights 124 -> 102 us; 19 KiB: three instead of two, 111 -> 102 us; not 13 and 14 KiB,
     // four instead of three: +2 %)
     const uint32_t workers = enc_max_workers(s.kind, (int)n_huff), big_teams = enc_max_workers(kEncBig, (int)n_huff) / tiles(full);
-    if (s.tiles > workers || (n_huff == 1 && s.kind >= kEncAny && s.kind < kEncBig && s.unit_chunks == 1 && 2 * big_teams >= 3 * (workers / s.tiles))) {
+    if (s.tiles > workers || (n_huff == 1 && (s.kind == kEncAny || s.kind == kEncAny48) && 2 * big_teams >= 3 * (workers / s.tiles))) {
         s.kind = kEncBig;
         s.tiles = tiles(full);
     }

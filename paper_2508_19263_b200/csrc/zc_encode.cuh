@@ -180,17 +180,18 @@ constexpr int kLookWide = 4;                     // look-back rounds cover 32 * 
 // Kernel shapes:
 //   kEncSolo    a chunk is one tile (4 KiB)
 //   kEncTeam    a chunk is T whole tiles (8, 12, 16, .. KiB)
-//   kEncAny     everything else, with lanes of 64 symbols (1 and 2 KiB: several chunks to a tile; odd sizes: the last tile is
-//               not full)
+//   kEncUnit    a tile is several whole chunks (1 and 2 KiB); in one kernel with the odd sizes both streams' codes did not fit
+//               the registers (96 MB at 2 KiB, both streams coded: FP8 152 -> 127 us, scale bytes 122 -> 96 us)
+//   kEncAny     everything else, with lanes of 64 symbols (the last tile is not full)
 //   kEncAny48   the same with lanes of 48 where that fills the tiles better (3, 6, 9 KiB; BF16 weights at 6 KiB: 95 against 119 us)
 //   kEncBig     chunks that need more workers than the shape above has, or of which it fits twice the teams
 //   kEncSolo80, kEncSolo96, kEncSolo112   a chunk of 5, 6 or 7 KiB with one coded stream is one tile of long lanes: two tiles
 //               are a sixth to a quarter empty, and a team that meets twice per chunk is slower than a warp alone (128 MB of
 //               BF16 weights in two tiles / one, and in the encoder with lane regions that packed subchunk by subchunk: 5 KiB
 //               103 / 74 / 82 us, 6 KiB 86 / 69 / 82 us, 7 KiB 97 / 73 / 84 us)
-constexpr int kEncSolo = 0, kEncTeam = 1, kEncAny = 2, kEncAny48 = 3, kEncBig = 4, kEncSolo80 = 5, kEncSolo96 = 6, kEncSolo112 = 7;
-__host__ __device__ constexpr uint32_t enc_lane_syms(int shape) { return shape == kEncAny48 ? 48u : shape >= kEncSolo80 ? 16u * shape : 64u; }   // (these are numbered by the KiB of their chunks)
-constexpr uint32_t kMaxUnitChunks = 4;           // chunks of a unit (kEncAny)
+constexpr int kEncSolo = 0, kEncTeam = 1, kEncAny = 2, kEncAny48 = 3, kEncBig = 4, kEncSolo80 = 5, kEncSolo96 = 6, kEncSolo112 = 7, kEncUnit = 8;
+__host__ __device__ constexpr uint32_t enc_lane_syms(int shape) { return shape == kEncAny48 ? 48u : shape >= kEncSolo80 && shape <= kEncSolo112 ? 16u * shape : 64u; }   // (these are numbered by the KiB of their chunks)
+constexpr uint32_t kMaxUnitChunks = 4;           // chunks of a unit (kEncUnit)
 // Worker warps per block: the joined codes take half a register per symbol of a lane and coded stream; with the two service
 // warps that makes 5 warps of 96 registers per scheduler for 32 or fewer of them, 4 of 128 for more.  kEncAny gets the 128
 // with one coded stream too (with 18 workers it spills: BF16 weights at 1 KiB 83 -> 90 us, at 7 KiB 97 -> 106 us).
@@ -321,14 +322,15 @@ encode_kernel(const __grid_constant__ EncParams P)
     constexpr int kHuff = (H0 ? 1 : 0) + (H1 ? 1 : 0);
     constexpr int kTabs = kHuff ? kHuff : 1;
     constexpr uint32_t kMaxW = enc_max_workers(SHAPE, kHuff);
-    constexpr bool kSolo = SHAPE == kEncSolo || SHAPE >= kEncSolo80, kAny = SHAPE >= kEncAny && SHAPE <= kEncBig;
+    constexpr bool kUnit = SHAPE == kEncUnit, kSolo = SHAPE == kEncSolo || SHAPE >= kEncSolo80;   // kSolo: a unit is one full tile
+    constexpr bool kAny = SHAPE >= kEncAny && SHAPE <= kEncBig;
     constexpr uint32_t kN = enc_lane_syms(SHAPE);               // symbols of a lane
     constexpr uint32_t kTileSyms = 32 * kN;
     extern __shared__ __align__(16) uint8_t smem[];
     const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const uint32_t n_workers = (blockDim.x >> 5) - kServiceWarps;
     const uint32_t T = kSolo ? 1u : P.tiles, teams = kSolo ? n_workers : P.teams;
-    const uint32_t unit_syms = kSolo ? kTileSyms : P.unit_syms, unit_chunks = SHAPE == kEncAny ? P.unit_chunks : 1u;
+    const uint32_t unit_syms = kSolo ? kTileSyms : P.unit_syms, unit_chunks = kUnit ? P.unit_chunks : 1u;
 
     // shared: rings[teams] | input buffers[workers] | tables[kTabSlots][kTabs][256]
     const uint32_t rings_s = smem_u32(smem);
@@ -338,7 +340,7 @@ encode_kernel(const __grid_constant__ EncParams P)
     __shared__ EncItem s_item[kTabSlots];
     __shared__ uint32_t s_fill[kTabSlots][2];
     __shared__ uint32_t s_slot[kEncRing], s_c0[kEncRing], s_ticket[kEncRing], s_tensor[kEncRing], s_tot[kEncRing];
-    __shared__ uint32_t s_bits[kEncRing][kTabs][kMaxW * (SHAPE == kEncAny ? kMaxUnitChunks : 1)], s_src[kEncRing][kMaxW];
+    __shared__ uint32_t s_bits[kEncRing][kTabs][kMaxW * (kUnit ? kMaxUnitChunks : 1)], s_src[kEncRing][kMaxW];
     __shared__ uint32_t s_tile[2][kTabs][kMaxW];
     __shared__ uint32_t s_freed_seq, s_end, s_fail;
     __shared__ uint64_t mb_in[kMaxW], mb_team[kMaxW], mb_info[kEncRing], mb_size[kEncRing], mb_posted[kEncRing], mb_done[kEncRing];
@@ -650,7 +652,11 @@ encode_kernel(const __grid_constant__ EncParams P)
         const uint32_t at0 = kN == 64 ? (lane >> 3) * 64 + ((((lane & 7) >> 1) ^ (lane >> 4)) << 4) + 8 * (lane & 1u) : 8 * lane;
         auto stage_at = [&](const uint32_t i) { return (kN == 64 ? at0 ^ ((i & 1u) << 5) : at0) + 256 * i; };
         // several chunks in a unit: the lanes of my chunk
-        const uint32_t chunk_lanes = (SHAPE == kEncAny && unit_chunks > 1) ? P.cs / kN : 32u, my_k = kAny ? lane / chunk_lanes : 0u, k_lane = my_k * chunk_lanes;
+        const uint32_t chunk_lanes = kUnit ? P.cs / kN : 32u, my_k = kUnit ? lane / chunk_lanes : 0u;
+        uint32_t k_lane = my_k * chunk_lanes;
+        // (Knowing that it is 0, the compiler keeps more over the loop than the kernels of two coded streams have registers
+        // for: 144 bytes of spills against 74.)
+        if (kAny) asm("" : "+r"(k_lane));
 
         bool loaded = false;                                     // the next tile's input has been requested
         uint32_t ph_in = 0;
@@ -754,7 +760,7 @@ encode_kernel(const __grid_constant__ EncParams P)
 
                 // ---- phase B ----
                 const uint32_t n_my = t_syms > kN * lane ? min(kN, t_syms - kN * lane) : 0u;
-                const uint32_t k_syms = (SHAPE == kEncAny && unit_chunks > 1) ? (t_syms > my_k * P.cs ? min(P.cs, t_syms - my_k * P.cs) : 0u) : t_syms;   // of my chunk in the tile
+                const uint32_t k_syms = kUnit ? (t_syms > my_k * P.cs ? min(P.cs, t_syms - my_k * P.cs) : 0u) : t_syms;   // of my chunk in the tile
                 uint32_t tile_bits[kTabs];
 #pragma unroll
                 for (int h = 0; h < kHuff; ++h) {
@@ -788,7 +794,7 @@ encode_kernel(const __grid_constant__ EncParams P)
                     }
                     const uint32_t inc = warp_scan(mine[h], lane);
                     uint32_t bits = __shfl_sync(0xFFFFFFFFu, inc, 31), lead = 0;         // of my chunk in the tile; of the chunks before it
-                    if (SHAPE == kEncAny && unit_chunks > 1) {
+                    if (kUnit) {
                         lead = __shfl_sync(0xFFFFFFFFu, inc, k_lane ? k_lane - 1 : 0);
                         if (k_lane == 0) lead = 0;
                         bits = __shfl_sync(0xFFFFFFFFu, inc, k_lane + chunk_lanes - 1) - lead;
@@ -830,7 +836,7 @@ encode_kernel(const __grid_constant__ EncParams P)
             uint32_t p16[kTabs], total = 0, my_at = 0;           // my chunk's pieces; the unit's; where mine start among them
 #pragma unroll
             for (int h = 0; h < kHuff; ++h) { p16[h] = (chunk_bits[h] + 127) >> 7; total += p16[h]; }
-            if (SHAPE == kEncAny && unit_chunks > 1) {
+            if (kUnit) {
                 const uint32_t own = total;
                 total = 0;
                 for (uint32_t k = 0; k < unit_chunks; ++k) {
@@ -849,7 +855,7 @@ encode_kernel(const __grid_constant__ EncParams P)
 #pragma unroll
                     for (int h = 0; h < kHuff; ++h) s_bits[r][h][my_team * unit_chunks + my_k] = chunk_bits[h];
                 }
-                if (kAny) __syncwarp();
+                if (kUnit) __syncwarp();
                 if (lane == 0) {
                     s_src[r][my_team] = piece_at;
                     mbar_arrive(&mb_size[r]);
@@ -884,22 +890,32 @@ encode_kernel(const __grid_constant__ EncParams P)
                         if (kSolo || P.sub_width == 2) reinterpret_cast<uint16_t*>(tab)[i] = (uint16_t)at;
                         else reinterpret_cast<uint32_t*>(tab)[i] = at;
                     };
-                    if (kAny) {
+                    if (kUnit) {
+                        // subchunks are 16 or 32 symbols: a lane ends four, or two
+                        uint32_t at = end[h] - mine[h];
+                        const uint32_t two = P.sub >> 5;
+#pragma unroll
+                        for (uint32_t p = 0; p < kN / 16; ++p) {
+#pragma unroll
+                            for (uint32_t i = 0; i < 8; ++i) at = add_low_byte(e[h][8 * p + i], at);
+                            if (c < I.n_chunks && !(two & ~p)) put_end(((4 * (lane - k_lane) + p + 1) >> two) - 1, chunk_bits[h] ? at : 0u);
+                        }
+                    } else if (kAny) {
                         // subchunks end where a lane has added up a multiple of 16 symbols
                         uint32_t at = end[h] - mine[h];
 #pragma unroll
                         for (uint32_t p = 0; p < kN / 16; ++p) {
 #pragma unroll
                             for (uint32_t i = 0; i < 8; ++i) at = add_low_byte(e[h][8 * p + i], at);
-                            const uint32_t k = t_lo + kN * (lane - k_lane) + 16 * (p + 1), i = __umulhi(k, P.sub_magic);
-                            if (c < I.n_chunks && k <= P.cs && i * P.sub == k) put_end(i - 1, chunk_bits[h] ? at : 0u);
+                            const uint32_t k = t_lo + kN * lane + 16 * (p + 1), i = __umulhi(k, P.sub_magic);
+                            if (k <= P.cs && i * P.sub == k) put_end(i - 1, chunk_bits[h] ? at : 0u);
                         }
                     } else {
                         // T lanes are a subchunk: lane g of the chunk (counting through its tiles) ends subchunk (g + 1) / T - 1 if T divides g + 1
                         const uint32_t g1 = tw * 32 + lane + 1, i = kSolo ? g1 : g1 / T;
                         if (i * T == g1) put_end(i - 1, chunk_bits[h] ? end[h] : 0u);
                     }
-                    if (chunk_bits[h] && (!kAny || mine[h])) {
+                    if (chunk_bits[h] && (!(kAny || kUnit) || mine[h])) {
                         const uint32_t piece_s = ring_s + 16 * (piece_at + my_at + (h ? p16[0] : 0u));
                         if (longer[h] == 0) emit_codes<true>(e[h], piece_s, end[h] - mine[h]);
                         else emit_codes<false>(e[h], piece_s, end[h] - mine[h]);

@@ -30,6 +30,7 @@ cudaError_t enc_launch_t(int shape, uint32_t grid, uint32_t threads, size_t smem
     else if (shape == kEncAny) { ZC_ENC_CASE(kEncAny) }
     else if (shape == kEncAny48) { ZC_ENC_CASE(kEncAny48) }
     else if (shape == kEncBig) { ZC_ENC_CASE(kEncBig) }
+    else if (shape == kEncUnit) { ZC_ENC_CASE(kEncUnit) }
 #undef ZC_ENC_CASE
 #define ZC_ENC_CASE(SHAPE)                                                   \
     if (h0) launch(encode_kernel<F, true, false, SHAPE>);                   \
