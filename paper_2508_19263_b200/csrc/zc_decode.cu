@@ -1011,8 +1011,14 @@ __device__ __forceinline__ uint32_t split_code(SplitBits& B, uint32_t lut_s, uin
 }
 
 constexpr uint32_t kSplitThreads = 512;
-// Shortest subchunk it is used for (chunks from 32 KiB on).  With one coded stream, 16 chunks of BF16 weights, here against
-// decode_kernel: 16 KiB 24.6 / 18.4 us, 32 KiB 25.4 / 30.6 us, 64 KiB 26.6 / 51 us.
+// Shortest subchunk it is used for (chunks from 32 KiB on).  16 chunks of 16 KiB of BF16 weights, one stream coded, 24.6 us
+// here, 18.4 us in decode_kernel; device times of longer ones, here / decode_kernel (few chunks) in us:
+//                                  32 KiB, 16    32 KiB, 148   64 KiB, 16    64 KiB, 74    64 KiB, 148 chunks
+//   BF16, one stream coded         20 / 24       22 / 25       21 / 43       23 / 44       26 / 43
+//   scale bytes, both coded        25 / 33       28 / 36       25 / 59       28 / 61       45 / 62
+//   FP8 weights, both coded        39 / 32       46 / 32       43 / 55       51 / 56       62 / 56
+// The last kind's sign+mantissa code is nearly uniform and falls back into step late.  The host does not know the codes of
+// the container, so the line is drawn for the others.
 constexpr uint32_t kSplitMinSub = 512;
 
 template <int FMT>
@@ -1550,8 +1556,8 @@ zc_status zc_decompress_chunks(const zc_plan_t* p, const void* d_comp, size_t co
     DecShape shape;
     uint32_t active = 0;
     uint32_t groups = 1;
-    // decode_split_kernel's rounds cost more than a lane's walk where subchunks are short, and more than other warps' walks
-    // where a block would have several chunks.
+    // decode_split_kernel's rounds cost more than a lane's walk where subchunks are short (see kSplitMinSub), and more than
+    // other warps' walks where a block would have several chunks.
     const int kind = p->syms_per_sub >= kSplitMinSub && n_chunks <= (uint32_t)sm_count() ? kDecSplit
                      : n_chunks <= kDecFewActive * (uint32_t)sm_count() ? kDecFew : kDecMany;
     if (kind == kDecSplit) {

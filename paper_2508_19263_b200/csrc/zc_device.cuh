@@ -68,15 +68,21 @@ __device__ __forceinline__ bool dbg_global(const void* p, uint32_t bytes, uint32
 }
 #define ZC_DBG_SHARED(addr, bytes, fail) do { if (!dbg_shared((addr), (bytes))) { fail; } } while (0)
 #define ZC_DBG_GLOBAL(p, bytes, align, store, fail) do { if (!dbg_global((p), (bytes), (align), (store))) { fail; } } while (0)
-// host: the address ranges of the launch that follows on `st` (pairs of first byte and byte count)
+// host: the address ranges of the launch that follows on `st` (pairs of first byte and byte count); by a kernel, so that a
+// captured launch keeps its ranges
+struct DebugRanges { unsigned long long lo[3], hi[3]; };
+static __global__ void dbg_set_ranges_kernel(const DebugRanges r)
+{
+    for (int k = 0; k < 3; ++k) { g_debug.lo[k] = r.lo[k]; g_debug.hi[k] = r.hi[k]; }
+}
 inline void dbg_set_ranges(cudaStream_t st, const void* in, size_t in_bytes, const void* out, size_t out_bytes,
                            const void* ws, size_t ws_bytes)
 {
-    DebugState h{};
+    DebugRanges r{};
     const void* lo[3] = {in, out, ws};
     const size_t n[3] = {in_bytes, out_bytes, ws_bytes};
-    for (int k = 0; k < 3; ++k) { h.lo[k] = (unsigned long long)lo[k]; h.hi[k] = h.lo[k] + n[k]; }
-    cudaMemcpyToSymbolAsync(g_debug, &h, 6 * sizeof(unsigned long long), 0, cudaMemcpyHostToDevice, st);
+    for (int k = 0; k < 3; ++k) { r.lo[k] = (unsigned long long)lo[k]; r.hi[k] = r.lo[k] + n[k]; }
+    dbg_set_ranges_kernel<<<1, 1, 0, st>>>(r);
 }
 inline void dbg_read_counts(uint32_t out[2])
 {
