@@ -226,17 +226,25 @@ static __device__ bool build_lut(uint32_t my_len, uint32_t* lut, uint16_t* singl
         sts128(single_s + 2 * idx, w[0], w[1], w[2], w[3]);
     }
     __syncthreads();
-    // The entries one at a time: neighbouring lanes then look up the second codes of neighbouring windows.  (With eight
-    // neighbouring windows to a lane those lookups were up to 16-way bank conflicts: 16 BF16 chunks of 4 KiB 8.7 against 7.8 us,
-    // 300 BF16 tensors of 16 chunks in a batch 55.6 against 51.3 us.)
-    for (uint32_t idx = tid; idx < kLutEntries; idx += blockDim.x) {
-        const uint32_t e1 = lds16(single_s + 2 * idx), l1 = e1 >> 8, s1 = e1 & 0xFF;
-        uint32_t e = l1 | (s1 << 24);                             // one-symbol mode: length | symbol << 24
-        if (mode == 2) {
+    if (mode == 2) {
+        // Neighbouring lanes look up the second codes of neighbouring windows.  (With eight windows to a lane those lookups
+        // were up to 16-way bank conflicts: 16 BF16 chunks of 4 KiB 8.7 against 7.8 us, 300 BF16 tensors of 16 chunks in a
+        // batch 55.6 against 51.3 us.)
+        for (uint32_t idx = tid; idx < kLutEntries; idx += blockDim.x) {
+            const uint32_t e1 = lds16(single_s + 2 * idx), l1 = e1 >> 8, s1 = e1 & 0xFF;
             const uint32_t e2 = lds16(single_s + 2 * ((idx << l1) & (kLutEntries - 1))), l2 = e2 >> 8, s2 = e2 & 0xFF;
-            e = l1 + l2 <= kLmax ? (l1 + l2) | (s1 << 8) | (s2 << 16) | (l1 << 24) : l1 | (s1 << 8) | (l1 << 24) | 0x80000000u;
+            sts32(lut_s + 4 * idx, l1 + l2 <= kLmax ? (l1 + l2) | (s1 << 8) | (s2 << 16) | (l1 << 24) : l1 | (s1 << 8) | (l1 << 24) | 0x80000000u);
         }
-        sts32(lut_s + 4 * idx, e);
+    } else {
+        for (uint32_t idx = 8 * tid; idx < kLutEntries; idx += 8 * blockDim.x) {
+            const uint4 v = lds128(single_s + 2 * idx);
+            const uint32_t w[4] = {v.x, v.y, v.z, v.w};          // two first codes each: length << 8 | symbol
+            uint32_t e[8];
+#pragma unroll
+            for (uint32_t i = 0; i < 8; ++i) e[i] = __byte_perm(w[i / 2], 0, i & 1u ? 0x2443 : 0x0441);
+            sts128(lut_s + 4 * idx, e[0], e[1], e[2], e[3]);
+            sts128(lut_s + 4 * idx + 16, e[4], e[5], e[6], e[7]);
+        }
     }
     __syncthreads();
     if (tid == 0) *per_lookup = mode;
