@@ -56,7 +56,7 @@
  *   payload area: for chunk 0, 1, ...: for each HUFF stream (stream order) the
  *      chunk's bits, zero padded to a multiple of 16 bytes
  *   16 zero guard bytes when at least one stream is HUFF
- *   Constant chunks: when both streams are HUFF, a chunk of a stream whose symbols are all the
+ *   Constant chunks: a chunk of a HUFF stream (whatever the other stream's mode) whose symbols are all the
  *      stream's fill symbol (the first symbol in (length, symbol) order, whose code is all zeros)
  *      has no payload at all: its 32 sub_end entries are 0, its piece is empty and its chunk_off16
  *      equals that of the piece that follows.  A chunk that holds symbols and has 0 bits can be
