@@ -72,7 +72,13 @@ constexpr uint32_t dec_block_warps() { return (XOR || FMT == ZC_FMT_SCALE_U8) ? 
 // one block that staged slices.
 constexpr uint32_t kDecFewWarps = 16, kDecFewActive = 8;
 constexpr int kDecMany = 0, kDecFew = 1, kDecSplit = 2;   // kernels of a single-tensor launch
-constexpr uint32_t kDecFixedSmem = 2 * kLutBytes + kScratchBytes;
+constexpr uint32_t kDecStaticSmem = 2 * kLutBytes + 512;      // the decode tables (block_luts), and the kernels' variables
+// The block's decode tables.  They are static shared memory: their addresses are constants and no register holds them.
+__device__ __forceinline__ uint32_t* block_luts()
+{
+    __shared__ __align__(16) uint32_t s_lut[2 * kLutEntries];
+    return s_lut;
+}
 constexpr uint32_t kSliceSyms = 128;               // symbols a lane decodes from one slice of its subchunk
 constexpr uint32_t kSliceBytes = 256;              // copied per slice: 15 bytes of alignment + 128 * 12 bits + the window's look-ahead fit
 constexpr uint32_t kSliceSlot = 272;               // a lane's slot
@@ -272,39 +278,45 @@ __device__ __forceinline__ uint32_t load_sub_end(const uint8_t* tab, uint32_t wi
 // slot.  With a valid container a lane reads at most 16 bytes past its piece (covered by the copy); with a
 // damaged payload it decodes garbage in bounds and the consumed-bits check after the chunk reports the damage.
 
-// The two payload words a lane's windows come from, kept in registers between lookups: w0, w1 = the aligned
-// words that hold bits [32 i, 32 i + 64) of shared memory, next = 32 (i + 1), with i = pos / 32.  A lane consumes at
-// most 24 bits between two windows, so pos crosses at most one word boundary: then w1 moves to w0 and one word
-// is loaded (a predicated load in which only the lanes that crossed take part: about one word per 32 bits of
-// payload instead of two words per window).
-#define ZC_LANE_BITS uint32_t &pos, uint32_t &w0, uint32_t &w1, uint32_t &next
-#define ZC_LANE_ARGS pos, w0, w1, next
+// A lane's bit reader.  w0, w1 = the aligned words that hold bits [32 i, 32 i + 64) of shared memory with i = pos / 32, w2 = the
+// word behind them, addr = the address of the one after that.  A lane consumes at most 24 bits between two windows, so pos
+// crosses at most one word boundary: then the words move up and the next one is requested (a predicated load in which only
+// the lanes that crossed take part), a word ahead, so that no window waits for it.
+struct LaneBits { uint32_t pos, w0, w1, w2, addr; };
 
-__device__ __forceinline__ void lane_start(ZC_LANE_BITS, uint32_t at)
+__device__ __forceinline__ void lane_start(LaneBits& L, const uint32_t at)
 {
-    ZC_DBG_SHARED((at >> 3) & ~3u, 4, return); ZC_DBG_SHARED(((at >> 3) & ~3u) + 4, 4, return);
     const uint32_t a = (at >> 3) & ~3u;
-    pos = at;
-    asm volatile("ld.shared.u32 %0, [%2];\n\tld.shared.u32 %1, [%2+4];" : "=r"(w0), "=r"(w1) : "r"(a));
-    next = (at & ~31u) + 32;
+    ZC_DBG_SHARED(a, 4, return); ZC_DBG_SHARED(a + 8, 4, return);
+    L.pos = at;
+    L.addr = a + 12;
+    asm volatile("ld.shared.u32 %0, [%3];\n\tld.shared.u32 %1, [%3+4];\n\tld.shared.u32 %2, [%3+8];" : "=r"(L.w0), "=r"(L.w1), "=r"(L.w2) : "r"(a));
 }
-__device__ __forceinline__ uint32_t window_s(ZC_LANE_BITS)
+__device__ __forceinline__ uint32_t window_s(const LaneBits& L)
 {
-    const bool cross = pos >= next;
-    const uint32_t w2 = lds32_if(cross, (next >> 3) + 4);
-    w0 = cross ? w1 : w0;
-    w1 = cross ? w2 : w1;
-    next += cross ? 32u : 0u;
-    return __funnelshift_l(w1, w0, pos);                        // the shift takes the low 5 bits of pos
+    return __funnelshift_l(L.w1, L.w0, L.pos);                  // the shift takes the low 5 bits of pos
+}
+// pos moves on to `to` (at most 32 bits further)
+__device__ __forceinline__ void lane_advance(LaneBits& L, const uint32_t to)
+{
+    const uint32_t cross = (L.pos ^ to) & 32u;
+    L.pos = to;
+    if (cross) ZC_DBG_SHARED(L.addr, 4, return);
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %4, 0;\n\t@p mov.u32 %0, %1;\n\t@p mov.u32 %1, %2;\n\t"
+                 "@p ld.shared.u32 %2, [%3];\n\t@p add.u32 %3, %3, 4;\n\t}"
+                 : "+r"(L.w0), "+r"(L.w1), "+r"(L.w2), "+r"(L.addr) : "r"(cross));
 }
 __device__ __forceinline__ uint32_t window_g(const uint32_t* __restrict__ pay, uint32_t pos, uint32_t lim)
 {
     const uint32_t w = min(pos >> 5, lim);
     return __funnelshift_l(__ldg(pay + w + 1), __ldg(pay + w), pos);
 }
+// window = top 12 bits; the address by a multiply-add, off the integer ALU pipe
 __device__ __forceinline__ uint32_t lut_peek(uint32_t win, uint32_t lut_s)
 {
-    return lds32(lut_s + 4u * (win >> (32 - kLmax)));           // window = top 12 bits; scaled by the address add
+    uint32_t addr;
+    asm("mad.lo.u32 %0, %1, 4, %2;" : "=r"(addr) : "r"(win >> (32 - kLmax)), "r"(lut_s));
+    return lds32(addr);
 }
 // pos + low byte of x, in one multiply-add-like instruction off the integer ALU pipe
 __device__ __forceinline__ uint32_t add_low_byte(uint32_t pos, uint32_t x) { return __dp4a(x, 1u, pos); }
@@ -317,36 +329,49 @@ __device__ __forceinline__ uint32_t add_low_byte(uint32_t pos, uint32_t x) { ret
 // carry the flag); the missing symbols come from a fresh window.
 // One-symbol mode: entry = length | symbol << 24, so that `pos += entry` advances the position and leaves the
 // symbol in bits the position does not use.
-template <int K>
-__device__ __forceinline__ uint32_t decode_word(ZC_LANE_BITS, uint32_t lut_s)
+// word_first makes the window and the two lookups that every word needs; word_second finishes the word: two more lookups
+// from a second window in one-symbol mode, the rare extra lookups of short pair entries in two-symbol mode.  WARP: the whole
+// warp is here, so that one vote decides whether anybody has a short entry and the others' way has no divergent branch.
+__device__ __forceinline__ void word_first(LaneBits& L, const uint32_t lut_s, uint32_t& x, uint32_t& y)
 {
-    uint32_t win = window_s(ZC_LANE_ARGS);
+    const uint32_t win = window_s(L);
+    x = lut_peek(win, lut_s);
+    y = lut_peek(__funnelshift_l(0, win, x), lut_s);            // consume: low 5 bits of the entry
+    lane_advance(L, add_low_byte(add_low_byte(L.pos, x), y));
+}
+template <int K, bool WARP>
+__device__ __forceinline__ uint32_t word_second(LaneBits& L, const uint32_t lut_s, const uint32_t e0, const uint32_t e1)
+{
     if (K == 2) {
-        const uint32_t e0 = lut_peek(win, lut_s);
-        const uint32_t e1 = lut_peek(__funnelshift_l(0, win, e0), lut_s);   // consume: low 5 bits of the entry
-        pos = add_low_byte(pos, e0 + e1);                    // the sum of two bit counts stays below 256
-        if ((int)(e0 | e1) < 0) {
-            win = window_s(ZC_LANE_ARGS);
-            const uint32_t f = lut_peek(win, lut_s), lf = (f >> 24) & 15;
-            pos += lf;
-            if ((int)(e0 & e1) < 0) {                            // both: first symbols of e0, e1, f and of one more lookup
-                const uint32_t g = lut_peek(__funnelshift_l(0, win, lf), lut_s);
-                pos += (g >> 24) & 15;
-                return __byte_perm(__byte_perm(e0, e1, 0x0051), __byte_perm(f, g, 0x0051), 0x5410);
+        uint32_t word = __byte_perm(e0, e1, 0x6521);
+        const bool mine = (int)(e0 | e1) < 0;
+        if (WARP ? __any_sync(0xFFFFFFFFu, mine) : mine) {
+            if (mine) {
+                const uint32_t win = window_s(L);
+                const uint32_t f = lut_peek(win, lut_s), lf = (f >> 24) & 15;
+                uint32_t to = L.pos + lf;
+                if ((int)(e0 & e1) < 0) {                        // both: first symbols of e0, e1, f and of one more lookup
+                    const uint32_t g = lut_peek(__funnelshift_l(0, win, lf), lut_s);
+                    to += (g >> 24) & 15;
+                    word = __byte_perm(__byte_perm(e0, e1, 0x0051), __byte_perm(f, g, 0x0051), 0x5410);
+                } else {                                         // e0 short: e0's first, e1's two; e1 short: e0's two, e1's first; then f's first
+                    word = __byte_perm(__byte_perm(e0, e1, (int)e0 < 0 ? 0x0651 : 0x0521), f, 0x5210);
+                }
+                lane_advance(L, to);
             }
-            // e0 short: e0's first, e1's two; e1 short: e0's two, e1's first; then f's first
-            return __byte_perm(__byte_perm(e0, e1, (int)e0 < 0 ? 0x0651 : 0x0521), f, 0x5210);
         }
-        return __byte_perm(e0, e1, 0x6521);
+        return word;
     }
-    const uint32_t a = lut_peek(win, lut_s);
-    const uint32_t bb = lut_peek(__funnelshift_l(0, win, a), lut_s);
-    pos = add_low_byte(pos, a + bb);
-    win = window_s(ZC_LANE_ARGS);
-    const uint32_t c = lut_peek(win, lut_s);
-    const uint32_t d = lut_peek(__funnelshift_l(0, win, c), lut_s);
-    pos = add_low_byte(pos, c + d);
-    return __byte_perm(__byte_perm(a, bb, 0x0073), __byte_perm(c, d, 0x0073), 0x5410);
+    uint32_t c, d;
+    word_first(L, lut_s, c, d);
+    return __byte_perm(__byte_perm(e0, e1, 0x0073), __byte_perm(c, d, 0x0073), 0x5410);
+}
+template <int K, bool WARP>
+__device__ __forceinline__ uint32_t decode_word(LaneBits& L, const uint32_t lut_s)
+{
+    uint32_t x, y;
+    word_first(L, lut_s, x, y);
+    return word_second<K, WARP>(L, lut_s, x, y);
 }
 
 // Decoded symbols of a round, per coded stream and warp: lane L owns PPL quads (16 symbols = 16 bytes each);
@@ -355,58 +380,24 @@ __device__ __forceinline__ uint32_t decode_word(ZC_LANE_BITS, uint32_t lut_s)
 // reads quad l % PPL of row l / PPL + i * 32 / PPL) touch eight different 16-byte bank groups per quarter warp:
 // no bank conflicts on either side, one store per 16 symbols and one load per merged part.
 template <int K, int PPL, bool FULL>
-__device__ __forceinline__ void decode_round(ZC_LANE_BITS, uint32_t lut_s, uint32_t wr_s, uint32_t fw, uint32_t n_quads)
+__device__ __forceinline__ void decode_round(LaneBits& L, const uint32_t lut_s, uint32_t wr_s, uint32_t fw, uint32_t n_quads)
 {
 #pragma unroll
     for (int q = 0; q < PPL; ++q) {
         if (!FULL && (uint32_t)q >= n_quads) break;
-        const uint32_t s0 = decode_word<K>(ZC_LANE_ARGS, lut_s);
-        const uint32_t s1 = decode_word<K>(ZC_LANE_ARGS, lut_s);
-        const uint32_t s2 = decode_word<K>(ZC_LANE_ARGS, lut_s);
-        const uint32_t s3 = decode_word<K>(ZC_LANE_ARGS, lut_s);
+        const uint32_t s0 = decode_word<K, FULL>(L, lut_s);
+        const uint32_t s1 = decode_word<K, FULL>(L, lut_s);
+        const uint32_t s2 = decode_word<K, FULL>(L, lut_s);
+        const uint32_t s3 = decode_word<K, FULL>(L, lut_s);
         sts128(wr_s + 16 * ((uint32_t)q ^ fw), s0, s1, s2, s3);
     }
 }
 
 // Two coded streams: the same words, decoded for both streams side by side.  A lane's two bit readers are independent
 // chains of dependent operations (window -> lookup -> shift -> lookup); issued alternately, one chain's shared-memory
-// latency is covered by the other's arithmetic.  word_first makes the window and the two lookups that every word
-// needs; word_second finishes the word: two more lookups from a second window in one-symbol mode, the rare extra
-// lookups of short pair entries in two-symbol mode.  Together they compute exactly what decode_word computes.
-template <int K>
-__device__ __forceinline__ void word_first(ZC_LANE_BITS, uint32_t lut_s, uint32_t& x, uint32_t& y)
-{
-    const uint32_t win = window_s(ZC_LANE_ARGS);
-    x = lut_peek(win, lut_s);
-    y = lut_peek(__funnelshift_l(0, win, x), lut_s);
-    pos = add_low_byte(pos, x + y);
-}
-template <int K>
-__device__ __forceinline__ uint32_t word_second(ZC_LANE_BITS, uint32_t lut_s, const uint32_t e0, const uint32_t e1)
-{
-    if (K == 2) {
-        if ((int)(e0 | e1) < 0) {
-            const uint32_t win = window_s(ZC_LANE_ARGS);
-            const uint32_t f = lut_peek(win, lut_s), lf = (f >> 24) & 15;
-            pos += lf;
-            if ((int)(e0 & e1) < 0) {
-                const uint32_t g = lut_peek(__funnelshift_l(0, win, lf), lut_s);
-                pos += (g >> 24) & 15;
-                return __byte_perm(__byte_perm(e0, e1, 0x0051), __byte_perm(f, g, 0x0051), 0x5410);
-            }
-            return __byte_perm(__byte_perm(e0, e1, (int)e0 < 0 ? 0x0651 : 0x0521), f, 0x5210);
-        }
-        return __byte_perm(e0, e1, 0x6521);
-    }
-    const uint32_t win = window_s(ZC_LANE_ARGS);
-    const uint32_t c = lut_peek(win, lut_s);
-    const uint32_t d = lut_peek(__funnelshift_l(0, win, c), lut_s);
-    pos = add_low_byte(pos, c + d);
-    return __byte_perm(__byte_perm(e0, e1, 0x0073), __byte_perm(c, d, 0x0073), 0x5410);
-}
+// latency is covered by the other's arithmetic.
 template <int K0, int K1, int PPL, bool FULL>
-__device__ __forceinline__ void decode_round2(uint32_t& posa, uint32_t& wa0, uint32_t& wa1, uint32_t& nexta, uint32_t luta_s, uint32_t wra_s,
-                                              uint32_t& posb, uint32_t& wb0, uint32_t& wb1, uint32_t& nextb, uint32_t lutb_s, uint32_t wrb_s,
+__device__ __forceinline__ void decode_round2(LaneBits& A, const uint32_t luta_s, uint32_t wra_s, LaneBits& B, const uint32_t lutb_s, uint32_t wrb_s,
                                               uint32_t fw, uint32_t n_quads)
 {
 #pragma unroll
@@ -416,10 +407,10 @@ __device__ __forceinline__ void decode_round2(uint32_t& posa, uint32_t& wa0, uin
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
             uint32_t ax, ay, bx, by;
-            word_first<K0>(posa, wa0, wa1, nexta, luta_s, ax, ay);
-            word_first<K1>(posb, wb0, wb1, nextb, lutb_s, bx, by);
-            a[j] = word_second<K0>(posa, wa0, wa1, nexta, luta_s, ax, ay);
-            b[j] = word_second<K1>(posb, wb0, wb1, nextb, lutb_s, bx, by);
+            word_first(A, luta_s, ax, ay);
+            word_first(B, lutb_s, bx, by);
+            a[j] = word_second<K0, FULL>(A, luta_s, ax, ay);
+            b[j] = word_second<K1, FULL>(B, lutb_s, bx, by);
         }
         sts128(wra_s + 16 * ((uint32_t)q ^ fw), a[0], a[1], a[2], a[3]);
         sts128(wrb_s + 16 * ((uint32_t)q ^ fw), b[0], b[1], b[2], b[3]);
@@ -463,7 +454,6 @@ static __device__ __noinline__ uint32_t decode_quads_global(uint32_t pos, const 
 // ------------------------------------------------------------------------------------------------
 
 struct DecShared {                   // what the block's prologue leaves for the chunk loop
-    uint32_t lut0_s, lut1_s;         // shared addresses of the decode tables
     uint32_t pairs0, pairs1;         // the stream's table yields two symbols per lookup
     unsigned long long sec0, sec1;   // byte offsets of the streams' sections
     unsigned long long payload_off, payload_bytes;
@@ -489,6 +479,7 @@ __device__ __forceinline__ uint32_t run_chunks(const DecParams& P, const DecShar
     const uint64_t tab_chunk = 256, tab_sub = 256 + (((uint64_t)4 * P.n_chunks + 15) & ~15ull);
     const uint8_t* sec0 = P.comp + S.sec0;
     const uint8_t* sec1 = P.comp + S.sec1;
+    const uint32_t lut0_s = smem_u32(block_luts()), lut1_s = lut0_s + kLutBytes;
     const uint8_t* payload = P.comp + S.payload_off;
     const uint64_t payload16 = S.payload_bytes >> 4;
 
@@ -640,7 +631,7 @@ __device__ __forceinline__ uint32_t run_chunks(const DecParams& P, const DecShar
             const uint8_t* raw0 = sec0 + c_lo + k_lane;             // my first part's bytes in a raw stream
             const uint8_t* raw1 = sec1 + c_lo + k_lane;
             uint8_t* dst_lane = P.out + 2 * c_lo + 2 * k_lane;      // two element bytes per symbol in every format
-            uint32_t pos0 = 0, pos1 = 0, w00 = 0, w01 = 0, w10 = 0, w11 = 0, next0 = 0, next1 = 0;
+            LaneBits L0{}, L1{};                                 // (.pos also where the piece is read from global memory)
             uint32_t lim0 = 0, lim1 = 0;
             for (uint32_t r = 0; r <= last_r; ++r) {
                 // ---- what this round is merged with (raw stream, base tensor) travels to the L2 while it is decoded ----
@@ -657,8 +648,8 @@ __device__ __forceinline__ uint32_t run_chunks(const DecParams& P, const DecShar
                     if (tot0) { if (mbar_wait(&bar[0], parity0, P.spin_limit)) { parity0 ^= 1; flying0 = false; } else err = ZC_E_DEVICE_TIMEOUT; }
                     if (tot1) { if (mbar_wait(&bar[1], parity1, P.spin_limit)) { parity1 ^= 1; flying1 = false; } else err = ZC_E_DEVICE_TIMEOUT; }
                     if (__any_sync(0xFFFFFFFFu, err == ZC_E_DEVICE_TIMEOUT)) { err = ZC_E_DEVICE_TIMEOUT; return; }
-                    if (by0) { org0 = 8 * slot0_s + min(rel0 - 8 * at0, 127u); lane_start(pos0, w00, w01, next0, org0); }
-                    if (by1) { org1 = 8 * slot1_s + min(rel1 - 8 * at1, 127u); lane_start(pos1, w10, w11, next1, org1); }
+                    if (by0) { org0 = 8 * slot0_s + min(rel0 - 8 * at0, 127u); lane_start(L0, org0); }
+                    if (by1) { org1 = 8 * slot1_s + min(rel1 - 8 * at1, 127u); lane_start(L1, org1); }
                     tot0 = tot1 = 0;
                 }
                 if (kHuff && r == 0) {
@@ -673,8 +664,8 @@ __device__ __forceinline__ uint32_t run_chunks(const DecParams& P, const DecShar
                     if (!sliced1) flying1 = false;
                     // staged: positions count from shared address 0; from global memory: from the piece, and the last
                     // readable word pair ends with the guard (piece + 16 bytes)
-                    if (H0 && !sliced0) { if (staged0) lane_start(pos0, w00, w01, next0, 8 * slot0_s + start0); else pos0 = start0; lim0 = piece0 / 4 + 2; }
-                    if (H1 && !sliced1) { if (staged1) lane_start(pos1, w10, w11, next1, 8 * slot1_s + start1); else pos1 = start1; lim1 = piece1 / 4 + 2; }
+                    if (H0 && !sliced0) { if (staged0) lane_start(L0, 8 * slot0_s + start0); else L0.pos = start0; lim0 = piece0 / 4 + 2; }
+                    if (H1 && !sliced1) { if (staged1) lane_start(L1, 8 * slot1_s + start1); else L1.pos = start1; lim1 = piece1 / 4 + 2; }
                 }
                 // ---- every lane decodes R symbols of its subchunk ----
                 if (kHuff) {
@@ -687,32 +678,32 @@ __device__ __forceinline__ uint32_t run_chunks(const DecParams& P, const DecShar
                         // both streams come from staged pieces: their words are decoded side by side
                         const uint32_t wra_s = rows0_s + wr_off, wrb_s = rows1_s + wr_off;
                         if (S.pairs0) {
-                            if (S.pairs1) decode_round2<2, 2, PPL, FULL>(pos0, w00, w01, next0, S.lut0_s, wra_s, pos1, w10, w11, next1, S.lut1_s, wrb_s, fw, n_quads);
-                            else decode_round2<2, 1, PPL, FULL>(pos0, w00, w01, next0, S.lut0_s, wra_s, pos1, w10, w11, next1, S.lut1_s, wrb_s, fw, n_quads);
+                            if (S.pairs1) decode_round2<2, 2, PPL, FULL>(L0, lut0_s, wra_s, L1, lut1_s, wrb_s, fw, n_quads);
+                            else decode_round2<2, 1, PPL, FULL>(L0, lut0_s, wra_s, L1, lut1_s, wrb_s, fw, n_quads);
                         } else {
-                            if (S.pairs1) decode_round2<1, 2, PPL, FULL>(pos0, w00, w01, next0, S.lut0_s, wra_s, pos1, w10, w11, next1, S.lut1_s, wrb_s, fw, n_quads);
-                            else decode_round2<1, 1, PPL, FULL>(pos0, w00, w01, next0, S.lut0_s, wra_s, pos1, w10, w11, next1, S.lut1_s, wrb_s, fw, n_quads);
+                            if (S.pairs1) decode_round2<1, 2, PPL, FULL>(L0, lut0_s, wra_s, L1, lut1_s, wrb_s, fw, n_quads);
+                            else decode_round2<1, 1, PPL, FULL>(L0, lut0_s, wra_s, L1, lut1_s, wrb_s, fw, n_quads);
                         }
                     } else if (n_quads) {
                         if (H0) {
                             const uint32_t wr_s = rows0_s + wr_off;
-                            if (piece0 == 0) fill_quads(S.lut0_s, S.pairs0, wr_s, fw, n_quads);   // a chunk without bits: nothing but the fill symbol
-                            else if (!staged0) pos0 = decode_quads_global(pos0, pay0_g, S.lut0_s, S.pairs0, wr_s, fw, n_quads, lim0);
-                            else if (S.pairs0) decode_round<2, PPL, FULL>(pos0, w00, w01, next0, S.lut0_s, wr_s, fw, n_quads);
-                            else decode_round<1, PPL, FULL>(pos0, w00, w01, next0, S.lut0_s, wr_s, fw, n_quads);
+                            if (piece0 == 0) fill_quads(lut0_s, S.pairs0, wr_s, fw, n_quads);   // a chunk without bits: nothing but the fill symbol
+                            else if (!staged0) L0.pos = decode_quads_global(L0.pos, pay0_g, lut0_s, S.pairs0, wr_s, fw, n_quads, lim0);
+                            else if (S.pairs0) decode_round<2, PPL, FULL>(L0, lut0_s, wr_s, fw, n_quads);
+                            else decode_round<1, PPL, FULL>(L0, lut0_s, wr_s, fw, n_quads);
                         }
                         if (H1) {
                             const uint32_t wr_s = rows1_s + wr_off;
-                            if (piece1 == 0) fill_quads(S.lut1_s, S.pairs1, wr_s, fw, n_quads);
-                            else if (!staged1) pos1 = decode_quads_global(pos1, pay1_g, S.lut1_s, S.pairs1, wr_s, fw, n_quads, lim1);
-                            else if (S.pairs1) decode_round<2, PPL, FULL>(pos1, w10, w11, next1, S.lut1_s, wr_s, fw, n_quads);
-                            else decode_round<1, PPL, FULL>(pos1, w10, w11, next1, S.lut1_s, wr_s, fw, n_quads);
+                            if (piece1 == 0) fill_quads(lut1_s, S.pairs1, wr_s, fw, n_quads);
+                            else if (!staged1) L1.pos = decode_quads_global(L1.pos, pay1_g, lut1_s, S.pairs1, wr_s, fw, n_quads, lim1);
+                            else if (S.pairs1) decode_round<2, PPL, FULL>(L1, lut1_s, wr_s, fw, n_quads);
+                            else decode_round<1, PPL, FULL>(L1, lut1_s, wr_s, fw, n_quads);
                         }
                     }
                     __syncwarp();
                     if ((sliced0 || sliced1) && (r + 1) % kRoundsPerSlice == 0 && r < last_r) {
-                        if (sliced0) { rel0 += pos0 - org0; org0 = pos0; }
-                        if (sliced1) { rel1 += pos1 - org1; org1 = pos1; }
+                        if (sliced0) { rel0 += L0.pos - org0; org0 = L0.pos; }
+                        if (sliced1) { rel1 += L1.pos - org1; org1 = L1.pos; }
                         issue_slices(n_my > (r + 1) * R, n_my > (r + 1) * R);
                     }
                     if (r == last_r) {
@@ -722,11 +713,11 @@ __device__ __forceinline__ uint32_t run_chunks(const DecParams& P, const DecShar
                         // symbols a slice origin of their own took a register of the chunk loop: 15 GB of BF16 5.05 -> 5.27 ms.)
                         bool good = true;
                         if (H0) {
-                            const uint32_t used = sliced0 ? rel0 + pos0 - org0 : pos0 - (staged0 ? 8 * slot0_s : 0u);
+                            const uint32_t used = sliced0 ? rel0 + L0.pos - org0 : L0.pos - (staged0 ? 8 * slot0_s : 0u);
                             good = good && (FULL ? used == end0 : n_my ? used - end0 <= 15 * kLmax : start0 == end0);
                         }
                         if (H1) {
-                            const uint32_t used = sliced1 ? rel1 + pos1 - org1 : pos1 - (staged1 ? 8 * slot1_s : 0u);
+                            const uint32_t used = sliced1 ? rel1 + L1.pos - org1 : L1.pos - (staged1 ? 8 * slot1_s : 0u);
                             good = good && (FULL ? used == end1 : n_my ? used - end1 <= 15 * kLmax : start1 == end1);
                         }
                         if (!__all_sync(0xFFFFFFFFu, good)) err = ZC_E_CORRUPT;
@@ -790,11 +781,268 @@ __device__ __forceinline__ uint32_t run_chunks(const DecParams& P, const DecShar
 }
 
 // ------------------------------------------------------------------------------------------------
+// the same for chunks of up to 4 KiB
+// ------------------------------------------------------------------------------------------------
+constexpr uint32_t kSmallChunk = 4096;
+
+// What the chunk loop has to know of the tensor, in shared memory: read where it is needed (a chunk needs each value once or
+// twice), so that it takes no registers over the loop.
+struct DecView {
+    const uint8_t* sec[2];           // the streams' sections: tables of a coded one, bytes of a raw one
+    const uint8_t* payload;
+    const uint8_t* base;
+    uint8_t* out;
+    unsigned long long payload16;    // payload bytes / 16
+    unsigned long long tab_sub;      // where a section's subchunk ends start
+    unsigned long long n_syms, input_bytes;
+    uint32_t n_full;                 // complete chunks (every lane has a whole subchunk)
+};
+
+// Chunks of up to 4 KiB are decoded as run_chunks does it, but everything a chunk needs comes by bulk copies: its pieces,
+// staged whole, and the bytes of a raw stream, so that the merge reads both streams from shared memory.  Both are requested as
+// soon as the chunk before has been decoded; the raw bytes of 4 KiB chunks, for which the block's memory has one buffer per
+// warp, when that has been written.  Subchunks of 32 and 64 symbols are one round, their addresses immediates.  What bounds
+// it is the chain window -> lookup -> shift of every lane at 7 warps per scheduler.  872 MB of BF16 weights in 4 KiB chunks
+// 329 -> 312 us, of FP8 weights 410 -> 383 us, 300 MB of BF16 in 3 KiB chunks 77 -> 70 us, block scales 60.6 -> 54.3 us; FP8
+// weights with both streams coded 396 -> 228 us (their pieces did not fit the slots of 28 warps and were read from global
+// memory; 20 warps stage them).
+__host__ __device__ constexpr uint32_t small_raw_buffers(uint32_t ppl) { return ppl == 4 ? 1u : 2u; }   // (ppl 4: 4 KiB)
+
+template <int FMT, int PPL, bool H0, bool H1, bool XOR, bool SIDE>
+__device__ __forceinline__ uint32_t run_small(const DecParams& P, const volatile DecView& V, const uint32_t pairs0, const uint32_t pairs1,
+                                              uint8_t* const pool, const uint32_t pool_bytes, uint64_t* const bar,
+                                              uint32_t nx_end0, uint32_t nx_off0,
+                                              uint32_t c, const uint32_t c_end, const uint32_t step,
+                                              uint32_t& parity0, uint32_t& parity1)
+{
+    constexpr uint32_t R = 16 * PPL;
+    constexpr uint32_t kLog = PPL == 4 ? 2 : PPL == 2 ? 1 : 0;
+    constexpr uint32_t kRowsBytes = 512 * PPL;
+    constexpr uint32_t kHuff = (H0 ? 1u : 0u) + (H1 ? 1u : 0u);
+    constexpr bool kCopyRaw = kHuff == 1;                        // one coded stream, one raw
+    constexpr int kRaw = H0 ? 1 : 0;                             // the raw one, and its mbarrier
+    constexpr uint32_t kRawBufs = small_raw_buffers(PPL);
+    const uint32_t lane = threadIdx.x & 31;
+    const uint32_t sub = PPL > 1 ? R : P.sub, cs = 32 * sub, chunk_bytes = 2 * cs, n_rounds = PPL > 1 ? 1u : sub / R;
+    const uint32_t lut0_s = smem_u32(block_luts()), lut1_s = lut0_s + kLutBytes;
+
+    // pool: symbols of stream 0 (if coded), of stream 1 (if coded), raw bytes of a chunk, one staging slot per coded stream
+    constexpr uint32_t rows1_off = H0 ? kRowsBytes : 0, raw_off = kHuff * kRowsBytes;
+    const uint32_t slots_off = raw_off + (kCopyRaw ? kRawBufs * cs : 0u);
+    const uint32_t slot_bytes = kHuff ? ((pool_bytes - slots_off) / (kHuff ? kHuff : 1)) & ~15u : 0u;
+    const uint32_t rows0_s = smem_u32(pool), rows1_s = rows0_s + rows1_off;
+    uint32_t raw_s = rows0_s + raw_off;                          // of the chunk that is merged next
+    const uint32_t slot0_s = rows0_s + slots_off, slot1_s = slot0_s + (H0 ? slot_bytes : 0u);
+    // where this lane writes its quads and reads the parts it merges (see decode_round)
+    const uint32_t fw = (lane >> (3 - kLog)) & (PPL - 1);
+    const uint32_t wr_off = 16 * PPL * lane;
+    const uint32_t rl = lane / PPL, rq = lane % PPL;
+    const uint32_t rd_off = 16 * (rl * PPL + (rq ^ ((rl >> (3 - kLog)) & (PPL - 1))));   // part i: + 512 * i
+    const uint32_t k_lane = rl * sub + rq * 16, k_step = (32 / PPL) * sub;
+    const bool out32 = ((uintptr_t)V.out & 16) == 0;
+
+    uint32_t err = 0, nx_end1 = 0, nx_off1 = 0;
+    // the chunk whose pieces are in the slots or on their way
+    uint32_t end0 = 0, end1 = 0, start0 = 0, start1 = 0, piece0 = 0, piece1 = 0, off0 = 0, off1 = 0;
+    bool staged0 = false, staged1 = false, flying0 = false, flying1 = false;
+    auto load_tables = [&](const int s, const uint32_t cc, uint32_t& end, uint32_t& off) {
+        const uint8_t* const sec = V.sec[s];
+        end = reinterpret_cast<const uint16_t*>(sec + V.tab_sub + 64ull * cc)[lane];
+        off = reinterpret_cast<const uint32_t*>(sec + 256)[cc];
+    };
+    auto copy = [&](const uint32_t dst_s, const uint8_t* src, const uint32_t bytes, uint64_t* b) {   // one lane calls it
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        mbar_expect_tx(b, bytes);
+        bulk_g2s_addr(dst_s, src, bytes, b);
+    };
+    // the raw bytes of a chunk (a raw section is padded to 16 bytes)
+    auto copy_raw = [&](const uint32_t dst_s, const uint32_t cc) {
+        const uint64_t lo = (uint64_t)cc * cs;
+        const uint32_t n = cc < V.n_full ? cs : ((uint32_t)min((unsigned long long)cs, V.n_syms - lo) + 15u) & ~15u;
+        if (kRaw == 1) flying1 = true; else flying0 = true;
+        if (lane == 0 && !P.skip_copy) copy(dst_s, V.sec[kRaw] + lo, n, &bar[kRaw]);
+    };
+    auto check = [&](const uint32_t end, const uint32_t off, uint32_t& start, uint32_t& piece) -> bool {
+        start = __shfl_up_sync(0xFFFFFFFFu, end, 1);
+        if (lane == 0) start = 0;
+        piece = (__shfl_sync(0xFFFFFFFFu, end, 31) + 127) / 128 * 16;
+        return start <= end && end - start <= sub * kLmax && (uint64_t)off + piece / 16 <= V.payload16;
+    };
+    // Takes the table entries in nx_* (of chunk cc), checks them, starts the copies, and requests the entries of the chunk
+    // after it.  A copy takes 16 bytes more than the piece (the next piece or the guard), for the windows' look-ahead.
+    auto prepare = [&](const uint32_t cc) {
+        bool ok = true;
+        if (H0) { end0 = nx_end0; off0 = nx_off0; ok = check(end0, off0, start0, piece0); }
+        if (H1) { end1 = nx_end1; off1 = nx_off1; ok = check(end1, off1, start1, piece1) && ok; }
+        staged0 = staged1 = false;
+        if (kHuff && !__all_sync(0xFFFFFFFFu, ok)) { err = ZC_E_CORRUPT; return; }
+        if (H0 && piece0 + 16 <= slot_bytes) {
+            staged0 = flying0 = true;
+            if (lane == 0 && !P.skip_copy) copy(slot0_s, V.payload + 16ull * off0, piece0 + 16, &bar[0]);
+        }
+        if (H1 && piece1 + 16 <= slot_bytes) {
+            staged1 = flying1 = true;
+            if (lane == 0 && !P.skip_copy) copy(slot1_s, V.payload + 16ull * off1, piece1 + 16, &bar[1]);
+        }
+        if (XOR) {                                               // the base tensor's bytes travel to the L2
+            const uint8_t* const base = V.base;
+            const uint32_t n = cc < V.n_full ? chunk_bytes : (uint32_t)min((unsigned long long)chunk_bytes, V.input_bytes - (uint64_t)cc * chunk_bytes) & ~15u;
+            if (lane == 0 && base && n)
+                asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" :: "l"(base + (uint64_t)cc * chunk_bytes), "r"(n) : "memory");
+        }
+        if (cc + step < c_end) {
+            if (H0) load_tables(0, cc + step, nx_end0, nx_off0);
+            if (H1) load_tables(1, cc + step, nx_end1, nx_off1);
+        }
+    };
+    auto other_raw = [&]() { return rows0_s + raw_off + (raw_s == rows0_s + raw_off ? cs : 0u); };
+    auto wait_raw = [&]() -> bool {
+        uint32_t& parity = kRaw == 1 ? parity1 : parity0;
+        const bool here = mbar_wait(&bar[kRaw], parity, P.spin_limit);
+        if (!__all_sync(0xFFFFFFFFu, here)) { err = ZC_E_DEVICE_TIMEOUT; return false; }
+        parity ^= 1;
+        if (kRaw == 1) flying1 = false; else flying0 = false;
+        return true;
+    };
+    if (c < c_end) {
+        if (H1) load_tables(1, c, nx_end1, nx_off1);
+        if (kCopyRaw) copy_raw(raw_s, c);
+        prepare(c);
+    }
+
+    for (; c < c_end && !err; c += step) {
+        // ---- the chunk; FULL: a complete chunk, every lane has `sub` symbols ----
+        auto body = [&](auto full_tag) {
+            constexpr bool FULL = decltype(full_tag)::value;
+            const uint64_t c_lo = (uint64_t)c * cs;
+            const uint32_t c_syms = FULL ? cs : (uint32_t)min((unsigned long long)cs, V.n_syms - c_lo);
+            const uint32_t out_bytes = FULL ? chunk_bytes : (uint32_t)min((unsigned long long)chunk_bytes, V.input_bytes - 2 * c_lo);
+            const uint32_t lo_sym = lane * sub;
+            const uint32_t n_my = FULL ? sub : (lo_sym < c_syms ? min(sub, c_syms - lo_sym) : 0u);
+            const uint32_t last_r = FULL ? n_rounds - 1 : (min(c_syms, sub) - 1) / R;         // lane 0 has the most symbols
+            LaneBits L0{}, L1{};                                 // (.pos also where the piece is read from global memory)
+            for (uint32_t r = 0; r <= last_r; ++r) {
+                if (kHuff && r == 0) {
+                    if (H0 && staged0) { if (mbar_wait(&bar[0], parity0, P.spin_limit)) parity0 ^= 1; else err = ZC_E_DEVICE_TIMEOUT; }
+                    if (H1 && staged1) { if (mbar_wait(&bar[1], parity1, P.spin_limit)) parity1 ^= 1; else err = ZC_E_DEVICE_TIMEOUT; }
+                    if (__any_sync(0xFFFFFFFFu, err == ZC_E_DEVICE_TIMEOUT)) { err = ZC_E_DEVICE_TIMEOUT; return; }
+                    if (H0) flying0 = false;
+                    if (H1) flying1 = false;
+                    if (H0) { if (staged0) lane_start(L0, 8 * slot0_s + start0); else L0.pos = start0; }
+                    if (H1) { if (staged1) lane_start(L1, 8 * slot1_s + start1); else L1.pos = start1; }
+                }
+                // ---- every lane decodes R symbols of its subchunk ----
+                if (kHuff) {
+                    const uint32_t done = r * R;
+                    // a ragged end decodes up to 15 symbols too many (from the bits that follow); they are not used
+                    const uint32_t n_quads = FULL ? (uint32_t)PPL : (n_my > done ? (min(R, n_my - done) + 15) / 16 : 0u);
+                    constexpr bool kSideBySide = H0 && H1 && SIDE;           // (only in the kernels that have the registers for it)
+                    const uint32_t wr0_s = rows0_s + wr_off, wr1_s = rows1_s + wr_off;
+                    if (kSideBySide && n_quads && staged0 && staged1 && piece0 != 0 && piece1 != 0) {
+                        if (pairs0) {
+                            if (pairs1) decode_round2<2, 2, PPL, FULL>(L0, lut0_s, wr0_s, L1, lut1_s, wr1_s, fw, n_quads);
+                            else decode_round2<2, 1, PPL, FULL>(L0, lut0_s, wr0_s, L1, lut1_s, wr1_s, fw, n_quads);
+                        } else {
+                            if (pairs1) decode_round2<1, 2, PPL, FULL>(L0, lut0_s, wr0_s, L1, lut1_s, wr1_s, fw, n_quads);
+                            else decode_round2<1, 1, PPL, FULL>(L0, lut0_s, wr0_s, L1, lut1_s, wr1_s, fw, n_quads);
+                        }
+                    } else if (n_quads) {
+                        // (the last word pair that may be read from global memory ends with the guard, 16 bytes behind the piece)
+                        if (H0) {
+                            if (piece0 == 0) fill_quads(lut0_s, pairs0, wr0_s, fw, n_quads);   // a chunk without bits: nothing but the fill symbol
+                            else if (!staged0) L0.pos = decode_quads_global(L0.pos, reinterpret_cast<const uint32_t*>(V.payload + 16ull * off0), lut0_s, pairs0, wr0_s, fw, n_quads, piece0 / 4 + 2);
+                            else if (pairs0) decode_round<2, PPL, FULL>(L0, lut0_s, wr0_s, fw, n_quads);
+                            else decode_round<1, PPL, FULL>(L0, lut0_s, wr0_s, fw, n_quads);
+                        }
+                        if (H1) {
+                            if (piece1 == 0) fill_quads(lut1_s, pairs1, wr1_s, fw, n_quads);
+                            else if (!staged1) L1.pos = decode_quads_global(L1.pos, reinterpret_cast<const uint32_t*>(V.payload + 16ull * off1), lut1_s, pairs1, wr1_s, fw, n_quads, piece1 / 4 + 2);
+                            else if (pairs1) decode_round<2, PPL, FULL>(L1, lut1_s, wr1_s, fw, n_quads);
+                            else decode_round<1, PPL, FULL>(L1, lut1_s, wr1_s, fw, n_quads);
+                        }
+                    }
+                    __syncwarp();
+                    if (kCopyRaw && kRawBufs == 2 && r == 0 && !wait_raw()) return;
+                    if (r == last_r) {
+                        // Every lane must have consumed exactly the bits of its subchunk (a ragged end decodes up to fifteen
+                        // symbols too many).  Anything else means the payload does not belong to the tables.
+                        bool good = true;
+                        if (H0) {
+                            const uint32_t used = L0.pos - (staged0 ? 8 * slot0_s : 0u);
+                            good = good && (FULL ? used == end0 : n_my ? used - end0 <= 15 * kLmax : start0 == end0);
+                        }
+                        if (H1) {
+                            const uint32_t used = L1.pos - (staged1 ? 8 * slot1_s : 0u);
+                            good = good && (FULL ? used == end1 : n_my ? used - end1 <= 15 * kLmax : start1 == end1);
+                        }
+                        if (!__all_sync(0xFFFFFFFFu, good)) err = ZC_E_CORRUPT;
+                        // the slots are free: the next chunk's pieces travel while this round is merged and written
+                        if (!err && c + step < c_end) {
+                            prepare(c + step);
+                            if (kCopyRaw && kRawBufs == 2) copy_raw(other_raw(), c + step);
+                        }
+                    }
+                }
+                if (kCopyRaw && kRawBufs == 1 && r == 0 && !wait_raw()) return;
+                // ---- cooperative merge: a part covers 16 symbols = 32 output bytes ----
+                uint8_t* const dst0 = V.out + 2 * c_lo + 2 * (k_lane + r * R);   // two element bytes per symbol in every format
+#pragma unroll
+                for (int i = 0; i < PPL; ++i) {
+                    const uint32_t k = k_lane + i * k_step + r * R;
+                    if ((!FULL && k >= c_syms)) continue;
+                    uint32_t e[4], m[4];
+                    {
+                        const uint4 v = H0 ? lds128(rows0_s + rd_off + 512 * i) : kCopyRaw ? lds128(raw_s + k) : ld_nc_v4(V.sec[0] + c_lo + k);
+                        e[0] = v.x; e[1] = v.y; e[2] = v.z; e[3] = v.w;
+                    }
+                    {
+                        const uint4 v = H1 ? lds128(rows1_s + rd_off + 512 * i) : kCopyRaw ? lds128(raw_s + k) : ld_nc_v4(V.sec[1] + c_lo + k);
+                        m[0] = v.x; m[1] = v.y; m[2] = v.z; m[3] = v.w;
+                    }
+                    uint32_t o[8];
+                    merge16<FMT>(e, m, o);
+                    merge16<FMT>(e + 2, m + 2, o + 4);
+                    uint8_t* const dst = dst0 + 2 * (i * k_step);
+                    if (XOR && V.base) {                              // delta form: XOR the base tensor back in
+                        const uint8_t* const base = V.base;
+                        const uint64_t off = 2 * (c_lo + k);
+                        const uint4 b0 = FULL ? ld_nc_v4(base + off) : load16_guarded(base, off, V.input_bytes);
+                        const uint4 b1 = FULL ? ld_nc_v4(base + off + 16) : load16_guarded(base, off + 16, V.input_bytes);
+                        o[0] ^= b0.x; o[1] ^= b0.y; o[2] ^= b0.z; o[3] ^= b0.w;
+                        o[4] ^= b1.x; o[5] ^= b1.y; o[6] ^= b1.z; o[7] ^= b1.w;
+                    }
+                    if (FULL || 2 * k + 32 <= out_bytes) {
+                        if (out32) {
+                            st_cs_v8(dst, o);
+                        } else {                                 // an output that is aligned to 16 bytes only
+                            st_cs_v4(dst, make_uint4(o[0], o[1], o[2], o[3]));
+                            st_cs_v4(dst + 16, make_uint4(o[4], o[5], o[6], o[7]));
+                        }
+                    } else {
+#pragma unroll
+                        for (int t = 0; t < 32; ++t)
+                            if (2 * k + t < out_bytes) dst[t] = (uint8_t)(o[t >> 2] >> (8 * (t & 3)));
+                    }
+                }
+                if (kHuff) __syncwarp();
+            }
+            if (kCopyRaw && kRawBufs == 1 && !err && c + step < c_end) copy_raw(raw_s, c + step);   // everybody has read this chunk's
+            if (kCopyRaw && kRawBufs == 2) raw_s = other_raw();
+        };
+        if (c < V.n_full) body(BoolTag<true>{}); else body(BoolTag<false>{});
+    }
+    // a copy that was started and not waited for (the loop ended early) must land before the block may leave
+    if (flying0 && !P.skip_copy) mbar_wait(&bar[0], parity0, P.spin_limit);
+    if (flying1 && !P.skip_copy) mbar_wait(&bar[1], parity1, P.spin_limit);
+    return err;
+}
+
+// ------------------------------------------------------------------------------------------------
 // the kernel
 // ------------------------------------------------------------------------------------------------
 // PPL = 16-symbol parts each lane merges per round = R / 16, R in {16, 32, 64}.
 
-struct DecSmem {                     // the block's dynamic shared memory, carved up once per kernel
+struct DecSmem {                     // the block's shared memory, carved up once per kernel
     uint32_t* lut0;                  // decode table of stream 0
     uint32_t* lut1;                  // decode table of stream 1
     uint32_t* scratch;
@@ -807,10 +1055,10 @@ __device__ __forceinline__ DecSmem carve_smem(uint8_t* smem, uint32_t pool_bytes
 {
     const uint32_t warp = threadIdx.x >> 5, n_warps = blockDim.x >> 5;
     DecSmem m;
-    m.lut0 = reinterpret_cast<uint32_t*>(smem);
-    m.lut1 = reinterpret_cast<uint32_t*>(smem + kLutBytes);
-    m.scratch = reinterpret_cast<uint32_t*>(smem + 2 * kLutBytes);
-    uint64_t* bars = reinterpret_cast<uint64_t*>(smem + kDecFixedSmem);
+    m.lut0 = block_luts();
+    m.lut1 = m.lut0 + kLutEntries;
+    m.scratch = reinterpret_cast<uint32_t*>(smem);
+    uint64_t* bars = reinterpret_cast<uint64_t*>(smem + kScratchBytes);
     m.pools = reinterpret_cast<uint8_t*>(bars + 2 * n_warps);
     m.pool = m.pools + (size_t)min(warp, active - 1) * pool_bytes;
     m.bar = bars + 2 * warp;
@@ -897,7 +1145,6 @@ __device__ __forceinline__ uint32_t open_container(const DecParams& P, const Dec
         if (!tables_ok) return ZC_E_CORRUPT;
     }
     H.S.pool_bytes = P.pool_bytes;
-    H.S.lut0_s = smem_u32(M.lut0); H.S.lut1_s = smem_u32(M.lut1);
     H.S.pairs0 = H.huff0 && s_per_lookup[0] == 2;
     H.S.pairs1 = H.huff1 && s_per_lookup[1] == 2;
     H.S.sec0 = s_sec[0]; H.S.sec1 = s_sec[1];
@@ -908,7 +1155,7 @@ __device__ __forceinline__ uint32_t open_container(const DecParams& P, const Dec
 // Decodes the chunks c0, c0 + step, ... (< c_end) of one tensor with this warp; the whole block calls it
 // together (the header check and the table build are block-wide).  Returns a zc_status, the same in every
 // thread for the block-wide checks.
-template <int FMT, int PPL, bool XOR, bool SIDE>
+template <int FMT, int PPL, bool XOR, bool SIDE, bool SMALL>
 __device__ __forceinline__ uint32_t decode_one(const DecParams& P, const DecSmem& M, const uint32_t chunk_base, const uint32_t c_end,
                                                const uint32_t block_index, const uint32_t n_blocks, uint32_t& parity0, uint32_t& parity1)
 {
@@ -928,13 +1175,12 @@ __device__ __forceinline__ uint32_t decode_one(const DecParams& P, const DecSmem
     if (opened != ZC_OK) return opened;
     const bool huff0 = H.huff0, huff1 = H.huff1;
     DecShared& S = H.S;
-    // Large chunks with both streams coded: a warp's pool was sized for one coded stream's lane slots (the plan
-    // does not say how many streams a container codes); fewer warps then share the block's pools, each with room
-    // for both, and the chunks are dealt to those warps only.
+    // Both streams coded where a warp's pool was sized for one of them (the plan does not say how many streams a container
+    // codes): fewer warps then share the block's pools, each with room for both, and the chunks are dealt to those warps only.
     uint8_t* pool = M.pool;
     uint32_t pool_bytes = P.pool_bytes;
-    if (P.sliced && huff0 && huff1) {
-        const uint32_t need = 2 * (512 * PPL + 32 * kSliceSlot);
+    if ((SMALL || P.sliced) && huff0 && huff1) {
+        const uint32_t need = 2 * (512 * PPL + (SMALL ? P.cs + 32 : 32 * kSliceSlot));
         if (need > P.pool_bytes) {
             const uint32_t active = max(1u, P.active * P.pool_bytes / need);
             pool = M.pools + (size_t)min(warp, active - 1) * need;
@@ -954,14 +1200,36 @@ __device__ __forceinline__ uint32_t decode_one(const DecParams& P, const DecSmem
         first_end0 = load_sub_end(P.comp + S.sec0 + tab_sub, sub_w, c0, lane);
         first_off0 = reinterpret_cast<const uint32_t*>(P.comp + S.sec0 + tab_chunk)[c0];
     }
-    if (huff0 && !huff1) return run_chunks<FMT, PPL, true, false, XOR, SIDE>(P, S, pool, M.bar, first_end0, first_off0, c0, c_end, step, parity0, parity1);
-    if (!huff0 && !huff1) return run_chunks<FMT, PPL, false, false, XOR, SIDE>(P, S, pool, M.bar, 0, 0, c0, c_end, step, parity0, parity1);
-    if (huff0) return run_chunks<FMT, PPL, true, true, XOR, SIDE>(P, S, pool, M.bar, first_end0, first_off0, c0, c_end, step, parity0, parity1);
-    return run_chunks<FMT, PPL, false, true, XOR, SIDE>(P, S, pool, M.bar, 0, 0, c0, c_end, step, parity0, parity1);
+    if constexpr (SMALL) {
+        __shared__ DecView s_view;
+        if (threadIdx.x == 0) {
+            s_view.sec[0] = P.comp + S.sec0;
+            s_view.sec[1] = P.comp + S.sec1;
+            s_view.payload = P.comp + S.payload_off;
+            s_view.base = XOR ? P.base : nullptr;
+            s_view.out = P.out;
+            s_view.payload16 = S.payload_bytes >> 4;
+            s_view.tab_sub = tab_sub;
+            s_view.n_syms = P.n_syms;
+            s_view.input_bytes = P.input_bytes;
+            s_view.n_full = (uint64_t)P.n_chunks * P.cs == P.n_syms && (uint64_t)P.n_chunks * P.chunk_bytes == P.input_bytes ? P.n_chunks : P.n_chunks - 1;
+        }
+        __syncthreads();
+        const volatile DecView& V = s_view;
+        if (huff0 && !huff1) return run_small<FMT, PPL, true, false, XOR, SIDE>(P, V, S.pairs0, 0, pool, pool_bytes, M.bar, first_end0, first_off0, c0, c_end, step, parity0, parity1);
+        if (!huff0 && !huff1) return run_small<FMT, PPL, false, false, XOR, SIDE>(P, V, 0, 0, pool, pool_bytes, M.bar, 0, 0, c0, c_end, step, parity0, parity1);
+        if (huff0) return run_small<FMT, PPL, true, true, XOR, SIDE>(P, V, S.pairs0, S.pairs1, pool, pool_bytes, M.bar, first_end0, first_off0, c0, c_end, step, parity0, parity1);
+        return run_small<FMT, PPL, false, true, XOR, SIDE>(P, V, 0, S.pairs1, pool, pool_bytes, M.bar, 0, 0, c0, c_end, step, parity0, parity1);
+    } else {
+        if (huff0 && !huff1) return run_chunks<FMT, PPL, true, false, XOR, SIDE>(P, S, pool, M.bar, first_end0, first_off0, c0, c_end, step, parity0, parity1);
+        if (!huff0 && !huff1) return run_chunks<FMT, PPL, false, false, XOR, SIDE>(P, S, pool, M.bar, 0, 0, c0, c_end, step, parity0, parity1);
+        if (huff0) return run_chunks<FMT, PPL, true, true, XOR, SIDE>(P, S, pool, M.bar, first_end0, first_off0, c0, c_end, step, parity0, parity1);
+        return run_chunks<FMT, PPL, false, true, XOR, SIDE>(P, S, pool, M.bar, 0, 0, c0, c_end, step, parity0, parity1);
+    }
 }
 
 // One tensor per launch: the warps of all blocks take the chunks in turn.  FEW: see kDecFewWarps.
-template <int FMT, int PPL, bool FEW>
+template <int FMT, int PPL, bool FEW, bool SMALL>
 __global__ void __launch_bounds__((FEW ? kDecFewWarps : dec_block_warps<FMT, false>()) * 32, 1)
 decode_kernel(const __grid_constant__ DecParams P)
 {
@@ -969,7 +1237,7 @@ decode_kernel(const __grid_constant__ DecParams P)
     const DecSmem M = carve_smem(smem, P.pool_bytes, P.active);
     if (P.ctl && blockIdx.x == 0 && threadIdx.x == 0) P.ctl->call_id = P.call_id;
     uint32_t parity0 = 0, parity1 = 0;
-    const uint32_t err = decode_one<FMT, PPL, false, FEW || FMT == ZC_FMT_SCALE_U8>(P, M, P.c_begin, P.c_end, blockIdx.x, gridDim.x, parity0, parity1);
+    const uint32_t err = decode_one<FMT, PPL, false, FEW || FMT == ZC_FMT_SCALE_U8, SMALL>(P, M, P.c_begin, P.c_end, blockIdx.x, gridDim.x, parity0, parity1);
     if (err) raise_status(P.ctl, P.call_id, err);
 }
 
@@ -1106,7 +1374,7 @@ decode_split_kernel(const __grid_constant__ DecParams P)
     if ((H.huff0 || H.huff1) && bits[st]) {
         const bool on = q < g_subs * parts;
         const uint32_t sub = g_lo + (on ? q / parts : 0u), part = q % parts;
-        const uint32_t lut_s = st ? S.lut1_s : S.lut0_s, pairs = st ? S.pairs1 : S.pairs0;
+        const uint32_t lut_s = smem_u32(st ? M.lut1 : M.lut0), pairs = st ? S.pairs1 : S.pairs0;
         const uint32_t len_shift = pairs ? 24u : 0u, sym_shift = pairs ? 8u : 24u;   // of an entry's first code
         const uint32_t piece_s = pieces_s + st * piece_room, base = 8 * from_byte[st];
         const uint32_t lo = (sub ? s_end[st][sub - 1] : 0u) - base, end_bit = s_end[st][sub] - base, len = end_bit - lo;
@@ -1183,7 +1451,7 @@ decode_split_kernel(const __grid_constant__ DecParams P)
     uint32_t fill4[2];                                           // a chunk without bits: nothing but the fill symbol
 #pragma unroll
     for (int s = 0; s < 2; ++s) {
-        const uint32_t e = lds32(s ? S.lut1_s : S.lut0_s);
+        const uint32_t e = lds32(smem_u32(s ? M.lut1 : M.lut0));
         fill4[s] = ((s ? S.pairs1 : S.pairs0) ? (e >> 8) & 0xFFu : e >> 24) * 0x01010101u;
     }
     const uint32_t k_lo = g_lo * P.sub, k_hi = min(c_syms, k_lo + g_syms);
@@ -1215,7 +1483,7 @@ decode_split_kernel(const __grid_constant__ DecParams P)
 // Many tensors per launch: the blocks take ranges of the concatenated chunk index space from a ticket counter (see
 // kDecMaxRounds) and go through a range tensor by tensor, building a tensor's tables once for its part of the range.
 // XOR: the launch has base tensors (delta form); a kernel of its own so that the plain form pays nothing for it.
-template <int FMT, int PPL, bool XOR>
+template <int FMT, int PPL, bool XOR, bool SMALL>
 __global__ void __launch_bounds__(dec_block_warps<FMT, XOR>() * 32, 1)
 decode_batch_kernel(const __grid_constant__ DecBatchParams B)
 {
@@ -1235,7 +1503,7 @@ decode_batch_kernel(const __grid_constant__ DecBatchParams B)
         const uint64_t tables = 256 + (((uint64_t)4 * P.n_chunks + 15) & ~15ull) + 32ull * (P.chunk_bytes <= 8192 ? 2u : 4u) * P.n_chunks;
         P.spec = P.comp_bytes >= kHeaderBytes + tables ? 1u : 0u;
         __syncthreads();                                         // everybody is done with the previous tensor's tables
-        const uint32_t err = decode_one<FMT, PPL, XOR, XOR || FMT == ZC_FMT_SCALE_U8>(P, M, seg_lo, seg_hi, 0, 1, parity0, parity1);
+        const uint32_t err = decode_one<FMT, PPL, XOR, XOR || FMT == ZC_FMT_SCALE_U8, SMALL>(P, M, seg_lo, seg_hi, 0, 1, parity0, parity1);
         if (err && raise_status(B.ctl, B.call_id, err)) B.ctl->failed = B.tensor_base + t + 1;
     };
 
@@ -1314,13 +1582,17 @@ cudaError_t dec_launch_single_t(uint32_t ppl, int kind, uint32_t grid, uint32_t 
     if (kind == kDecSplit) {
         launch(decode_split_kernel<F>);
     } else if (kind == kDecFew) {
-        if (ppl == 4) launch(decode_kernel<F, 4, true>);
-        else if (ppl == 2) launch(decode_kernel<F, 2, true>);
-        else launch(decode_kernel<F, 1, true>);
+        if (ppl == 4) launch(decode_kernel<F, 4, true, false>);
+        else if (ppl == 2) launch(decode_kernel<F, 2, true, false>);
+        else launch(decode_kernel<F, 1, true, false>);
+    } else if (P.chunk_bytes <= kSmallChunk) {
+        if (ppl == 4) launch(decode_kernel<F, 4, false, true>);
+        else if (ppl == 2) launch(decode_kernel<F, 2, false, true>);
+        else launch(decode_kernel<F, 1, false, true>);
     } else {
-        if (ppl == 4) launch(decode_kernel<F, 4, false>);
-        else if (ppl == 2) launch(decode_kernel<F, 2, false>);
-        else launch(decode_kernel<F, 1, false>);
+        if (ppl == 4) launch(decode_kernel<F, 4, false, false>);
+        else if (ppl == 2) launch(decode_kernel<F, 2, false, false>);
+        else launch(decode_kernel<F, 1, false, false>);
     }
     return e;
 }
@@ -1341,15 +1613,15 @@ cudaError_t dec_launch_batch_t(uint32_t ppl, bool any_base, uint32_t grid, uint3
         kern<<<grid, threads, smem, st>>>(B);
         e = cudaGetLastError();
     };
-    if (any_base) {
-        if (ppl == 4) launch(decode_batch_kernel<F, 4, true>);
-        else if (ppl == 2) launch(decode_batch_kernel<F, 2, true>);
-        else launch(decode_batch_kernel<F, 1, true>);
-    } else {
-        if (ppl == 4) launch(decode_batch_kernel<F, 4, false>);
-        else if (ppl == 2) launch(decode_batch_kernel<F, 2, false>);
-        else launch(decode_batch_kernel<F, 1, false>);
-    }
+    auto pick = [&](auto xor_tag, auto small_tag) {
+        constexpr bool XOR = decltype(xor_tag)::value, SMALL = decltype(small_tag)::value;
+        if (ppl == 4) launch(decode_batch_kernel<F, 4, XOR, SMALL>);
+        else if (ppl == 2) launch(decode_batch_kernel<F, 2, XOR, SMALL>);
+        else launch(decode_batch_kernel<F, 1, XOR, SMALL>);
+    };
+    const bool small = B.chunk_bytes <= kSmallChunk;
+    if (any_base) { if (small) pick(BoolTag<true>{}, BoolTag<true>{}); else pick(BoolTag<true>{}, BoolTag<false>{}); }
+    else { if (small) pick(BoolTag<false>{}, BoolTag<true>{}); else pick(BoolTag<false>{}, BoolTag<false>{}); }
     return e;
 }
 
@@ -1418,12 +1690,14 @@ zc_status dec_shape(const zc_plan_t* p, bool both_coded, DecShape* out)
     // stream; pieces that do not fit (or chunks above 16 KiB of symbols) are read from global memory instead
     s.sliced = p->syms_per_sub % kSliceSyms == 0 ? 1u : 0u;   // pieces beyond their slot can be staged slice by slice
     s.pool_bytes = std::max<uint32_t>(coded * (rows_bytes + std::min<uint32_t>(p->syms_per_chunk, 16384) + 32), 2 * rows_bytes);
+    // up to 4 KiB: room for the bytes of a raw stream too (see run_small)
+    if (p->chunk_bytes <= kSmallChunk) s.pool_bytes = std::max(s.pool_bytes, rows_bytes + p->syms_per_chunk + 32 + small_raw_buffers(s.ppl) * p->syms_per_chunk);
     // chunks above 16 KiB: whole pieces would leave room for a dozen warps at most; lane slots for sliced pieces
     // are enough, and more warps decode
     if (s.sliced && p->syms_per_chunk > 8192) s.pool_bytes = std::max<uint32_t>(coded * (rows_bytes + 32 * kSliceSlot), 2 * rows_bytes);
     // slack behind the last slot: what a lane can read past its piece when the payload is damaged (see window_s)
     const size_t slack = (size_t)round_up(p->syms_per_sub + p->syms_per_sub / 2 + 16, 16);
-    const size_t fixed = kDecFixedSmem + 512 /* static shared */ + slack;
+    const size_t fixed = kDecStaticSmem + kScratchBytes + slack;
     size_t per_warp = 16 + s.pool_bytes;
     const size_t max_warps = coded == 2 ? kDecMaxWarpsBoth : kDecMaxWarps;     // the kernels' launch bounds
     s.warps = (uint32_t)std::min<size_t>(max_warps, (kMaxSmem - fixed - 1024) / per_warp);
@@ -1435,7 +1709,7 @@ zc_status dec_shape(const zc_plan_t* p, bool both_coded, DecShape* out)
     // the table build uses 8 KiB of the pools and 256 threads
     while (s.warps * (size_t)s.pool_bytes < 8192) ++s.warps;
     if (s.warps < 8 || s.warps > max_warps) return ZC_E_UNSUPPORTED;
-    s.smem = kDecFixedSmem + s.warps * per_warp + slack;
+    s.smem = kScratchBytes + s.warps * per_warp + slack;
     *out = s;
     return ZC_OK;
 }
@@ -1447,7 +1721,7 @@ DecShape few_shape(const zc_plan_t* p, uint32_t n_chunks, uint32_t* active)
     s.ppl = (p->syms_per_sub % 64 == 0) ? 4 : (p->syms_per_sub % 32 == 0) ? 2 : 1;
     s.warps = kDecFewWarps;
     const size_t slack = (size_t)round_up(p->syms_per_sub + p->syms_per_sub / 2 + 16, 16);
-    const size_t room = kMaxSmem - 1024 - kDecFixedSmem - 512 - 16 * s.warps - slack;
+    const size_t room = kMaxSmem - 1024 - kDecStaticSmem - kScratchBytes - 16 * s.warps - slack;
     *active = std::max<uint32_t>(1, (n_chunks + sm_count() - 1) / sm_count());
     // rows of both streams and room for whole pieces of 12-bit codes (less when the warps' shares are smaller: slices then)
     const uint32_t most = 2 * (512 * s.ppl + (uint32_t)round_up((uint64_t)p->syms_per_chunk * kLmax / 8, 16) + 32);
@@ -1456,7 +1730,7 @@ DecShape few_shape(const zc_plan_t* p, uint32_t n_chunks, uint32_t* active)
     // slices only where whole pieces might not fit (then the pools fill the block's memory, as decode_one's sharing of them
     // among fewer warps expects)
     s.sliced = share < most && p->syms_per_sub % kSliceSyms == 0 ? 1u : 0u;
-    s.smem = kDecFixedSmem + 16 * s.warps + (size_t)*active * s.pool_bytes + slack;
+    s.smem = kScratchBytes + 16 * s.warps + (size_t)*active * s.pool_bytes + slack;
     return s;
 }
 
@@ -1470,7 +1744,7 @@ DecShape split_shape(const zc_plan_t* p, uint32_t n_chunks, uint32_t* groups)
     while (*groups < 8 && 2ull * *groups * n_chunks <= (uint64_t)sm_count()) *groups *= 2;
     const uint32_t syms = p->syms_per_chunk / *groups;
     s.pool_bytes = std::max<uint32_t>(2 * syms + 2 * ((uint32_t)round_up((uint64_t)syms * kLmax / 8, 16) + 48), 8192);
-    s.smem = kDecFixedSmem + 16 * s.warps + s.pool_bytes + 64;   // the bit readers look a few words past a piece's copy
+    s.smem = kScratchBytes + 16 * s.warps + s.pool_bytes + 64;   // the bit readers look a few words past a piece's copy
     return s;
 }
 
