@@ -32,7 +32,7 @@ struct DecParams {
 };
 
 // One tensor of a batch, and the parameters of a batched launch.  The tensors share format and chunk size;
-// the chunks of all of them form one index space that is cut into contiguous ranges (see kDecMaxRounds).
+// the chunks of all of them form one index space that is cut into contiguous ranges (see kDecMaxPieces).
 struct DecItem {
     const uint8_t* comp;
     const uint8_t* base;
@@ -40,19 +40,25 @@ struct DecItem {
     uint64_t comp_bytes, input_bytes, n_syms, n_elems;
     uint32_t n_chunks, first_chunk;          // first_chunk = chunks of all earlier tensors of the launch
 };
-// The chunk index space of a batched launch is dealt out in rounds, every round in as many equal contiguous ranges as there
-// are blocks; the blocks take ranges from a ticket counter.  The first round is most of it and the others shrink, so that
-// blocks end together although tensors, and SMs, differ in how fast they get through a range.  A range costs a block about
-// 12 us (waiting for its last warp, header, tables, first pieces), so there are few: with eight equal ones per block the
-// BF16 stack of 1.74 GB took 707 us.
-constexpr uint32_t kDecMaxRounds = 5, kDecOneRound = 64;
+// The chunk index space of a batched launch is cut into as many equal slices as there are blocks, and a slice into pieces that
+// shrink.  A block takes the pieces of its own slice one after the other; when it is through, it takes pieces that the slices'
+// owners have not come to yet, largest first, so that blocks end together although tensors, and SMs, differ in how fast they
+// get through a piece.  Who takes a piece sets its bit in the control block (nobody else takes a slice's first piece).  The next
+// piece of one's own slice is nearly always of the same tensor, whose tables are kept; another one costs about 12 us (waiting for
+// the block's last warp, header, tables, first pieces).  (Dealt out in rounds over the whole index space by a ticket counter, every
+// piece of a block was of another tensor: 1.74 GB of BF16 weights 621 us, now 612; their delta of 872 MB 550 and 524; 18 tensors of
+// 66 MB in all 58 and 53.  In one piece each, the delta takes 659 us.)
+constexpr uint32_t kDecMaxPieces = 5, kDecOneRound = 64;
+constexpr uint32_t kDecMaxBlocks = 160, kDecClaimWords = kDecMaxBlocks / 32;
+constexpr size_t kDecClaims = 128;           // where the bits are in the control block: [piece - 1][kDecClaimWords]
+static_assert(sizeof(Control) <= kDecClaims && kDecClaims + 4 * (kDecMaxPieces - 1) * kDecClaimWords <= kControlBytes, "control block");
 constexpr uint32_t kDecBatchMax = 448;       // tensors per launch: the parameter block stays below 32 KiB
 struct DecBatchParams {
     Control* ctl;
     unsigned long long call_id;
     uint32_t cs, sub, chunk_bytes, format, group, pool_bytes;
-    uint32_t n_tensors, n_empty, tensor_base, n_rounds;   // n_empty: tensors without chunks
-    uint32_t round_end[kDecMaxRounds];       // chunks of the first rounds
+    uint32_t n_tensors, n_empty, tensor_base, total;      // n_empty: tensors without chunks; total: chunks
+    uint32_t n_pieces, piece_end[kDecMaxPieces];          // where a slice's pieces end, in 65536ths of it
     uint32_t spin_limit, skip_copy, sliced;
     DecItem item[kDecBatchMax];
 };
@@ -278,10 +284,10 @@ __device__ __forceinline__ uint32_t load_sub_end(const uint8_t* tab, uint32_t wi
 // slot.  With a valid container a lane reads at most 16 bytes past its piece (covered by the copy); with a
 // damaged payload it decodes garbage in bounds and the consumed-bits check after the chunk reports the damage.
 
-// A lane's bit reader.  w0, w1 = the aligned words that hold bits [32 i, 32 i + 64) of shared memory with i = pos / 32, w2 = the
-// word behind them, addr = the address of the one after that.  A lane consumes at most 24 bits between two windows, so pos
-// crosses at most one word boundary: then the words move up and the next one is requested (a predicated load in which only
-// the lanes that crossed take part), a word ahead, so that no window waits for it.
+// A lane's bit reader.  w0, w1 = the aligned words that hold bits [32 i, 32 i + 64) of shared memory with i = pos / 32; with the
+// look-ahead (see word_first) also w2 = the word behind them, addr = the address of the one after that.  A lane consumes at
+// most 24 bits between two windows, so pos crosses at most one word boundary: then the words move up and one is loaded, in a
+// predicated load in which only the lanes that crossed take part.
 struct LaneBits { uint32_t pos, w0, w1, w2, addr; };
 
 __device__ __forceinline__ void lane_start(LaneBits& L, const uint32_t at)
@@ -296,15 +302,24 @@ __device__ __forceinline__ uint32_t window_s(const LaneBits& L)
 {
     return __funnelshift_l(L.w1, L.w0, L.pos);                  // the shift takes the low 5 bits of pos
 }
-// pos moves on to `to` (at most 32 bits further)
+// pos moves on to `to` (at most 32 bits further).  AHEAD: the word behind the window's is in a register already and the next one
+// is requested; otherwise the window's second word is loaded when it is needed.
+template <bool AHEAD>
 __device__ __forceinline__ void lane_advance(LaneBits& L, const uint32_t to)
 {
     const uint32_t cross = (L.pos ^ to) & 32u;
     L.pos = to;
-    if (cross) ZC_DBG_SHARED(L.addr, 4, return);
-    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %4, 0;\n\t@p mov.u32 %0, %1;\n\t@p mov.u32 %1, %2;\n\t"
-                 "@p ld.shared.u32 %2, [%3];\n\t@p add.u32 %3, %3, 4;\n\t}"
-                 : "+r"(L.w0), "+r"(L.w1), "+r"(L.w2), "+r"(L.addr) : "r"(cross));
+    if (AHEAD) {
+        if (cross) ZC_DBG_SHARED(L.addr, 4, return);
+        asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %4, 0;\n\t@p mov.u32 %0, %1;\n\t@p mov.u32 %1, %2;\n\t"
+                     "@p ld.shared.u32 %2, [%3];\n\t@p add.u32 %3, %3, 4;\n\t}"
+                     : "+r"(L.w0), "+r"(L.w1), "+r"(L.w2), "+r"(L.addr) : "r"(cross));
+    } else {
+        const uint32_t a = ((to >> 3) & ~3u) + 4;
+        if (cross) ZC_DBG_SHARED(a, 4, return);
+        L.w0 = cross ? L.w1 : L.w0;
+        asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %2, 0;\n\t@p ld.shared.u32 %0, [%1];\n\t}" : "+r"(L.w1) : "r"(a), "r"(cross));
+    }
 }
 __device__ __forceinline__ uint32_t window_g(const uint32_t* __restrict__ pay, uint32_t pos, uint32_t lim)
 {
@@ -330,48 +345,46 @@ __device__ __forceinline__ uint32_t add_low_byte(uint32_t pos, uint32_t x) { ret
 // One-symbol mode: entry = length | symbol << 24, so that `pos += entry` advances the position and leaves the
 // symbol in bits the position does not use.
 // word_first makes the window and the two lookups that every word needs; word_second finishes the word: two more lookups
-// from a second window in one-symbol mode, the rare extra lookups of short pair entries in two-symbol mode.  WARP: the whole
-// warp is here, so that one vote decides whether anybody has a short entry and the others' way has no divergent branch.
+// from a second window in one-symbol mode, the rare extra lookups of short pair entries in two-symbol mode.
+// The one-symbol mode keeps a word in flight ahead of its windows, of which it has twice as many: without it 436 MB of FP8
+// weights at 16 KiB take 200 instead of 193 us.  The two-symbol mode is bound by its instructions, and the look-ahead costs
+// three registers to move at every window: 872 MB of BF16 weights 307 us with it, 301 us without.
+template <int K>
 __device__ __forceinline__ void word_first(LaneBits& L, const uint32_t lut_s, uint32_t& x, uint32_t& y)
 {
     const uint32_t win = window_s(L);
     x = lut_peek(win, lut_s);
     y = lut_peek(__funnelshift_l(0, win, x), lut_s);            // consume: low 5 bits of the entry
-    lane_advance(L, add_low_byte(add_low_byte(L.pos, x), y));
+    lane_advance<K == 1>(L, add_low_byte(add_low_byte(L.pos, x), y));
 }
-template <int K, bool WARP>
+template <int K>
 __device__ __forceinline__ uint32_t word_second(LaneBits& L, const uint32_t lut_s, const uint32_t e0, const uint32_t e1)
 {
     if (K == 2) {
-        uint32_t word = __byte_perm(e0, e1, 0x6521);
-        const bool mine = (int)(e0 | e1) < 0;
-        if (WARP ? __any_sync(0xFFFFFFFFu, mine) : mine) {
-            if (mine) {
-                const uint32_t win = window_s(L);
-                const uint32_t f = lut_peek(win, lut_s), lf = (f >> 24) & 15;
-                uint32_t to = L.pos + lf;
-                if ((int)(e0 & e1) < 0) {                        // both: first symbols of e0, e1, f and of one more lookup
-                    const uint32_t g = lut_peek(__funnelshift_l(0, win, lf), lut_s);
-                    to += (g >> 24) & 15;
-                    word = __byte_perm(__byte_perm(e0, e1, 0x0051), __byte_perm(f, g, 0x0051), 0x5410);
-                } else {                                         // e0 short: e0's first, e1's two; e1 short: e0's two, e1's first; then f's first
-                    word = __byte_perm(__byte_perm(e0, e1, (int)e0 < 0 ? 0x0651 : 0x0521), f, 0x5210);
-                }
-                lane_advance(L, to);
+        if ((int)(e0 | e1) < 0) {
+            const uint32_t win = window_s(L);
+            const uint32_t f = lut_peek(win, lut_s), lf = (f >> 24) & 15;
+            if ((int)(e0 & e1) < 0) {                            // both: first symbols of e0, e1, f and of one more lookup
+                const uint32_t g = lut_peek(__funnelshift_l(0, win, lf), lut_s);
+                lane_advance<false>(L, L.pos + lf + ((g >> 24) & 15));
+                return __byte_perm(__byte_perm(e0, e1, 0x0051), __byte_perm(f, g, 0x0051), 0x5410);
             }
+            lane_advance<false>(L, L.pos + lf);
+            // e0 short: e0's first, e1's two; e1 short: e0's two, e1's first; then f's first
+            return __byte_perm(__byte_perm(e0, e1, (int)e0 < 0 ? 0x0651 : 0x0521), f, 0x5210);
         }
-        return word;
+        return __byte_perm(e0, e1, 0x6521);
     }
     uint32_t c, d;
-    word_first(L, lut_s, c, d);
+    word_first<1>(L, lut_s, c, d);
     return __byte_perm(__byte_perm(e0, e1, 0x0073), __byte_perm(c, d, 0x0073), 0x5410);
 }
-template <int K, bool WARP>
+template <int K>
 __device__ __forceinline__ uint32_t decode_word(LaneBits& L, const uint32_t lut_s)
 {
     uint32_t x, y;
-    word_first(L, lut_s, x, y);
-    return word_second<K, WARP>(L, lut_s, x, y);
+    word_first<K>(L, lut_s, x, y);
+    return word_second<K>(L, lut_s, x, y);
 }
 
 // Decoded symbols of a round, per coded stream and warp: lane L owns PPL quads (16 symbols = 16 bytes each);
@@ -385,10 +398,10 @@ __device__ __forceinline__ void decode_round(LaneBits& L, const uint32_t lut_s, 
 #pragma unroll
     for (int q = 0; q < PPL; ++q) {
         if (!FULL && (uint32_t)q >= n_quads) break;
-        const uint32_t s0 = decode_word<K, FULL>(L, lut_s);
-        const uint32_t s1 = decode_word<K, FULL>(L, lut_s);
-        const uint32_t s2 = decode_word<K, FULL>(L, lut_s);
-        const uint32_t s3 = decode_word<K, FULL>(L, lut_s);
+        const uint32_t s0 = decode_word<K>(L, lut_s);
+        const uint32_t s1 = decode_word<K>(L, lut_s);
+        const uint32_t s2 = decode_word<K>(L, lut_s);
+        const uint32_t s3 = decode_word<K>(L, lut_s);
         sts128(wr_s + 16 * ((uint32_t)q ^ fw), s0, s1, s2, s3);
     }
 }
@@ -407,10 +420,10 @@ __device__ __forceinline__ void decode_round2(LaneBits& A, const uint32_t luta_s
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
             uint32_t ax, ay, bx, by;
-            word_first(A, luta_s, ax, ay);
-            word_first(B, lutb_s, bx, by);
-            a[j] = word_second<K0, FULL>(A, luta_s, ax, ay);
-            b[j] = word_second<K1, FULL>(B, lutb_s, bx, by);
+            word_first<K0>(A, luta_s, ax, ay);
+            word_first<K1>(B, lutb_s, bx, by);
+            a[j] = word_second<K0>(A, luta_s, ax, ay);
+            b[j] = word_second<K1>(B, lutb_s, bx, by);
         }
         sts128(wra_s + 16 * ((uint32_t)q ^ fw), a[0], a[1], a[2], a[3]);
         sts128(wrb_s + 16 * ((uint32_t)q ^ fw), b[0], b[1], b[2], b[3]);
@@ -801,11 +814,7 @@ struct DecView {
 // Chunks of up to 4 KiB are decoded as run_chunks does it, but everything a chunk needs comes by bulk copies: its pieces,
 // staged whole, and the bytes of a raw stream, so that the merge reads both streams from shared memory.  Both are requested as
 // soon as the chunk before has been decoded; the raw bytes of 4 KiB chunks, for which the block's memory has one buffer per
-// warp, when that has been written.  Subchunks of 32 and 64 symbols are one round, their addresses immediates.  What bounds
-// it is the chain window -> lookup -> shift of every lane at 7 warps per scheduler.  872 MB of BF16 weights in 4 KiB chunks
-// 329 -> 312 us, of FP8 weights 410 -> 383 us, 300 MB of BF16 in 3 KiB chunks 77 -> 70 us, block scales 60.6 -> 54.3 us; FP8
-// weights with both streams coded 396 -> 228 us (their pieces did not fit the slots of 28 warps and were read from global
-// memory; 20 warps stage them).
+// warp, when that has been written.  Subchunks of 32 and 64 symbols are one round, their addresses immediates.
 __host__ __device__ constexpr uint32_t small_raw_buffers(uint32_t ppl) { return ppl == 4 ? 1u : 2u; }   // (ppl 4: 4 KiB)
 
 template <int FMT, int PPL, bool H0, bool H1, bool XOR, bool SIDE>
@@ -895,6 +904,17 @@ __device__ __forceinline__ uint32_t run_small(const DecParams& P, const volatile
             if (H1) load_tables(1, cc + step, nx_end1, nx_off1);
         }
     };
+    // One-symbol tables: the next chunk's pieces travel to the L2 while a chunk is decoded (their table entries are in nx_*), so that
+    // the copies are quicker than the merge they hide behind (872 MB of FP8 weights 382 -> 372 us; with two-symbol tables it is
+    // more instructions than it saves: BF16 297 -> 302 us).
+    auto prefetch_next = [&]() {
+        if (lane != 31) return;                                  // its subchunk's end is the piece's
+        const uint32_t n0 = (nx_end0 + 127) / 128, n1 = (nx_end1 + 127) / 128;
+        if (H0 && n0 && (uint64_t)nx_off0 + n0 <= V.payload16)
+            asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" :: "l"(V.payload + 16ull * nx_off0), "r"(16 * n0) : "memory");
+        if (H1 && n1 && (uint64_t)nx_off1 + n1 <= V.payload16)
+            asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" :: "l"(V.payload + 16ull * nx_off1), "r"(16 * n1) : "memory");
+    };
     auto other_raw = [&]() { return rows0_s + raw_off + (raw_s == rows0_s + raw_off ? cs : 0u); };
     auto wait_raw = [&]() -> bool {
         uint32_t& parity = kRaw == 1 ? parity1 : parity0;
@@ -906,8 +926,8 @@ __device__ __forceinline__ uint32_t run_small(const DecParams& P, const volatile
     };
     if (c < c_end) {
         if (H1) load_tables(1, c, nx_end1, nx_off1);
-        if (kCopyRaw) copy_raw(raw_s, c);
         prepare(c);
+        if (kCopyRaw) copy_raw(raw_s, c);
     }
 
     for (; c < c_end && !err; c += step) {
@@ -930,6 +950,7 @@ __device__ __forceinline__ uint32_t run_small(const DecParams& P, const volatile
                     if (H1) flying1 = false;
                     if (H0) { if (staged0) lane_start(L0, 8 * slot0_s + start0); else L0.pos = start0; }
                     if (H1) { if (staged1) lane_start(L1, 8 * slot1_s + start1); else L1.pos = start1; }
+                    if (((H0 && !pairs0) || (H1 && !pairs1)) && c + step < c_end) prefetch_next();
                 }
                 // ---- every lane decodes R symbols of its subchunk ----
                 if (kHuff) {
@@ -1073,6 +1094,26 @@ struct DecOpened {                   // what open_container leaves
     bool huff0, huff1;
 };
 
+struct DecHeader {                   // of the tensor whose tables the block has built, in shared memory
+    uint32_t mode[2], per_lookup[2], ok;
+    unsigned long long payload_off, payload_bytes, sec[2];
+};
+__device__ __forceinline__ DecHeader& block_header()
+{
+    __shared__ DecHeader s_header;
+    return s_header;
+}
+__device__ __forceinline__ void opened_container(const DecParams& P, DecOpened& H)
+{
+    const DecHeader& T = block_header();
+    H.huff0 = T.mode[0] == ZC_MODE_HUFF; H.huff1 = T.mode[1] == ZC_MODE_HUFF;
+    H.S.pool_bytes = P.pool_bytes;
+    H.S.pairs0 = H.huff0 && T.per_lookup[0] == 2;
+    H.S.pairs1 = H.huff1 && T.per_lookup[1] == 2;
+    H.S.sec0 = T.sec[0]; H.S.sec1 = T.sec[1];
+    H.S.payload_off = T.payload_off; H.S.payload_bytes = T.payload_bytes;
+}
+
 // Checks the header against the plan and builds the decode tables of the coded streams; the whole block calls it.  Returns a
 // zc_status, the same in every thread.
 __device__ __forceinline__ uint32_t open_container(const DecParams& P, const DecSmem& M, DecOpened& H)
@@ -1084,10 +1125,8 @@ __device__ __forceinline__ uint32_t open_container(const DecParams& P, const Dec
     uint32_t spec_len = 0;
     if (P.spec && threadIdx.x < 256) spec_len = P.comp[kHeaderBytes + threadIdx.x];
     // ---- header check against the plan ----
-    __shared__ uint32_t s_mode[2], s_per_lookup[2];
-    __shared__ uint32_t s_ok;
-    __shared__ unsigned long long s_payload_off, s_payload_bytes, s_sec[2];
     __shared__ __align__(16) uint32_t s_hdr[32];
+    DecHeader& T = block_header();
     if (warp == 0) {
         s_hdr[lane] = reinterpret_cast<const uint32_t*>(P.comp)[lane];      // the 128-byte header in one request
         __syncwarp();
@@ -1117,47 +1156,44 @@ __device__ __forceinline__ uint32_t open_container(const DecParams& P, const Dec
             ok = poff == off && (pbytes & 15) == 0 && total == poff + pbytes + (any_huff ? 16 : 0) && total <= P.comp_bytes;
             for (int s = 0; s < 2 && ok; ++s)
                 ok = reinterpret_cast<const unsigned long long*>(h + kHdrStream0 + kHdrStreamStride * s)[3] == sec[s];
-            s_mode[0] = mode[0]; s_mode[1] = mode[1];
-            s_sec[0] = sec[0]; s_sec[1] = sec[1];
-            s_payload_off = poff; s_payload_bytes = pbytes;
+            T.mode[0] = mode[0]; T.mode[1] = mode[1];
+            T.sec[0] = sec[0]; T.sec[1] = sec[1];
+            T.payload_off = poff; T.payload_bytes = pbytes;
         }
-        s_ok = ok ? 1u : 0u;
+        T.ok = ok ? 1u : 0u;
     }
     __syncthreads();
-    if (!s_ok) return ZC_E_CORRUPT;
+    if (!T.ok) return ZC_E_CORRUPT;
 
-    H.huff0 = s_mode[0] == ZC_MODE_HUFF; H.huff1 = s_mode[1] == ZC_MODE_HUFF;
+    const bool huff0 = T.mode[0] == ZC_MODE_HUFF, huff1 = T.mode[1] == ZC_MODE_HUFF;
     {
         // the warps' pools are free until the chunk loop: 8 KiB of them hold the one-symbol scratch table
         uint16_t* single = reinterpret_cast<uint16_t*>(M.pools);
         bool tables_ok = true;
-        if (H.huff0) {
+        if (huff0) {
             uint32_t len = spec_len;                             // stream 0's section always starts behind the header
-            if (!P.spec && threadIdx.x < 256) len = P.comp[s_sec[0] + threadIdx.x];
-            tables_ok = build_lut(len, M.lut0, single, M.scratch, &s_per_lookup[0]) && tables_ok;
+            if (!P.spec && threadIdx.x < 256) len = P.comp[T.sec[0] + threadIdx.x];
+            tables_ok = build_lut(len, M.lut0, single, M.scratch, &T.per_lookup[0]) && tables_ok;
         }
-        if (H.huff1) {
+        if (huff1) {
             uint32_t len = 0;
-            if (threadIdx.x < 256) len = P.comp[s_sec[1] + threadIdx.x];
-            tables_ok = build_lut(len, M.lut1, single, M.scratch, &s_per_lookup[1]) && tables_ok;
+            if (threadIdx.x < 256) len = P.comp[T.sec[1] + threadIdx.x];
+            tables_ok = build_lut(len, M.lut1, single, M.scratch, &T.per_lookup[1]) && tables_ok;
         }
         __syncthreads();
         if (!tables_ok) return ZC_E_CORRUPT;
     }
-    H.S.pool_bytes = P.pool_bytes;
-    H.S.pairs0 = H.huff0 && s_per_lookup[0] == 2;
-    H.S.pairs1 = H.huff1 && s_per_lookup[1] == 2;
-    H.S.sec0 = s_sec[0]; H.S.sec1 = s_sec[1];
-    H.S.payload_off = s_payload_off; H.S.payload_bytes = s_payload_bytes;
+    opened_container(P, H);
     return ZC_OK;
 }
 
 // Decodes the chunks c0, c0 + step, ... (< c_end) of one tensor with this warp; the whole block calls it
-// together (the header check and the table build are block-wide).  Returns a zc_status, the same in every
-// thread for the block-wide checks.
+// together (the header check and the table build are block-wide).  opened_before: the block has the tensor's tables already.
+// Returns a zc_status, the same in every thread for the block-wide checks.
 template <int FMT, int PPL, bool XOR, bool SIDE, bool SMALL>
 __device__ __forceinline__ uint32_t decode_one(const DecParams& P, const DecSmem& M, const uint32_t chunk_base, const uint32_t c_end,
-                                               const uint32_t block_index, const uint32_t n_blocks, uint32_t& parity0, uint32_t& parity1)
+                                               const uint32_t block_index, const uint32_t n_blocks, const bool opened_before,
+                                               uint32_t& parity0, uint32_t& parity1)
 {
     const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     // chunk chunk_base + k goes to block k % n_blocks, warp (k / n_blocks) % P.active
@@ -1171,8 +1207,12 @@ __device__ __forceinline__ uint32_t decode_one(const DecParams& P, const DecSmem
         spec_off = reinterpret_cast<const uint32_t*>(P.comp + kHeaderBytes + tab_chunk)[c0];
     }
     DecOpened H;
-    const uint32_t opened = open_container(P, M, H);
-    if (opened != ZC_OK) return opened;
+    if (opened_before) {
+        opened_container(P, H);
+    } else {
+        const uint32_t opened = open_container(P, M, H);
+        if (opened != ZC_OK) return opened;
+    }
     const bool huff0 = H.huff0, huff1 = H.huff1;
     DecShared& S = H.S;
     // Both streams coded where a warp's pool was sized for one of them (the plan does not say how many streams a container
@@ -1237,7 +1277,7 @@ decode_kernel(const __grid_constant__ DecParams P)
     const DecSmem M = carve_smem(smem, P.pool_bytes, P.active);
     if (P.ctl && blockIdx.x == 0 && threadIdx.x == 0) P.ctl->call_id = P.call_id;
     uint32_t parity0 = 0, parity1 = 0;
-    const uint32_t err = decode_one<FMT, PPL, false, FEW || FMT == ZC_FMT_SCALE_U8, SMALL>(P, M, P.c_begin, P.c_end, blockIdx.x, gridDim.x, parity0, parity1);
+    const uint32_t err = decode_one<FMT, PPL, false, FEW || FMT == ZC_FMT_SCALE_U8, SMALL>(P, M, P.c_begin, P.c_end, blockIdx.x, gridDim.x, false, parity0, parity1);
     if (err) raise_status(P.ctl, P.call_id, err);
 }
 
@@ -1480,8 +1520,8 @@ decode_split_kernel(const __grid_constant__ DecParams P)
     }
 }
 
-// Many tensors per launch: the blocks take ranges of the concatenated chunk index space from a ticket counter (see
-// kDecMaxRounds) and go through a range tensor by tensor, building a tensor's tables once for its part of the range.
+// Many tensors per launch: the blocks take pieces of the concatenated chunk index space (see kDecMaxPieces) and go through a
+// piece tensor by tensor, building a tensor's tables once for its part of it.
 // XOR: the launch has base tensors (delta form); a kernel of its own so that the plain form pays nothing for it.
 template <int FMT, int PPL, bool XOR, bool SMALL>
 __global__ void __launch_bounds__(dec_block_warps<FMT, XOR>() * 32, 1)
@@ -1492,7 +1532,103 @@ decode_batch_kernel(const __grid_constant__ DecBatchParams B)
     if (blockIdx.x == 0 && threadIdx.x == 0 && B.tensor_base == 0) B.ctl->call_id = B.call_id;
     uint32_t parity0 = 0, parity1 = 0;
 
-    auto run = [&](const uint32_t t, const uint32_t seg_lo, const uint32_t seg_hi) {
+    // Where the block is, in shared memory (the first warp's business; nobody keeps it in registers while decoding).
+    constexpr uint32_t kNone = 0xFFFFFFFFu;
+    __shared__ uint32_t s_t, s_lo, s_hi;                         // the part to decode next: chunks [s_lo, s_hi) of tensor s_t
+    __shared__ uint32_t s_opened;                                // the tensor whose tables the block has
+    __shared__ uint32_t s_empty, s_piece, s_g, s_g_hi, s_g_t;    // tensor to look at for an empty one; pieces taken of my slice; the rest of a piece
+    if (threadIdx.x == 0) {
+        s_opened = kNone;
+        // Block 0 first walks over the tensors, if there are any without chunks: their headers are still checked.  (The walk takes
+        // 0.1 us a tensor, which the block is late for its slice: 64 BF16 pages of 129 chunks 37 us, without it 31 us.)
+        s_empty = blockIdx.x == 0 && B.n_empty ? 0u : B.n_tensors;
+        s_piece = s_g = s_g_hi = s_g_t = 0;
+    }
+    // The first warp: piece p of slice j is the block's now.
+    auto enter = [&](const uint32_t p, const uint32_t j) {
+        const uint32_t from = (uint32_t)((uint64_t)j * B.total / gridDim.x), len = (uint32_t)((uint64_t)(j + 1) * B.total / gridDim.x) - from;
+        const uint32_t warps = blockDim.x >> 5;
+        auto cut = [&](const uint32_t k) -> uint32_t {           // pieces are whole turns of the warps
+            return k == B.n_pieces ? len : (uint32_t)((uint64_t)len * (k ? B.piece_end[k - 1] : 0u) >> 16) / warps * warps;
+        };
+        const uint32_t g = from + cut(p);
+        // the last tensor that starts at or before g (tensors without chunks share their start with the next one)
+        uint32_t lo = 0, hi = B.n_tensors;
+        while (hi - lo > 1) {
+            const uint32_t mid = (lo + hi) / 2;
+            if (B.item[mid].first_chunk <= g) lo = mid; else hi = mid;
+        }
+        if (threadIdx.x == 0) { s_g = g; s_g_hi = from + cut(p + 1); s_g_t = lo; }
+        __syncwarp();
+    };
+    uint32_t* const claims = reinterpret_cast<uint32_t*>(reinterpret_cast<uint8_t*>(B.ctl) + kDecClaims);
+    auto claim = [&](const uint32_t p, const uint32_t j) -> bool {
+        const uint32_t bit = 1u << (j % 32);
+        return (atomicOr(&claims[(p - 1) * kDecClaimWords + j / 32], bit) & bit) == 0;
+    };
+    // The first warp: looks for another piece; false when none is left.
+    auto next_piece = [&]() -> bool {
+        const uint32_t lane = threadIdx.x & 31, p = s_piece;
+        if (p < B.n_pieces) {
+            bool got = p == 0;
+            if (p && lane == 0) got = claim(p, blockIdx.x);
+            got = __shfl_sync(0xFFFFFFFFu, got, 0);
+            __syncwarp();
+            if (lane == 0) s_piece = got ? p + 1 : B.n_pieces;
+            if (got) { enter(p, blockIdx.x); return true; }
+        }
+        // Lane l looks at word l of the bits, starting behind the block's own place, so that blocks do not all try the same one.
+        const uint32_t q = lane / kDecClaimWords + 1, w = (lane + blockIdx.x / 32) % kDecClaimWords;
+        const uint32_t in_word = gridDim.x > 32 * w ? min(32u, gridDim.x - 32 * w) : 0u;
+        for (uint32_t tries = 0; tries < kDecMaxPieces * kDecMaxBlocks; ++tries) {
+            uint32_t open = 0;
+            if (q < B.n_pieces && lane < (kDecMaxPieces - 1) * kDecClaimWords && in_word)
+                open = ~*reinterpret_cast<volatile uint32_t*>(&claims[(q - 1) * kDecClaimWords + w]) & (0xFFFFFFFFu >> (32 - in_word));
+            const uint32_t have = __ballot_sync(0xFFFFFFFFu, open != 0);
+            if (!have) return false;
+            const uint32_t who = __ffs(have) - 1;
+            const uint32_t behind = open & (0xFFFFFFFFu << (blockIdx.x % 32));
+            const uint32_t j = 32 * w + __ffs(behind ? behind : open) - 1;
+            bool got = false;
+            if (lane == who) got = claim(q, j);
+            if (__shfl_sync(0xFFFFFFFFu, got, who)) {
+                enter(__shfl_sync(0xFFFFFFFFu, q, who), __shfl_sync(0xFFFFFFFFu, j, who));
+                return true;
+            }
+        }
+        return false;
+    };
+    // The first warp: the next part.
+    auto next_part = [&]() {
+        uint32_t t = kNone, lo = 0, hi = 0, e = s_empty;
+        while (e < B.n_tensors && B.item[e].n_chunks != 0) ++e;
+        if (e < B.n_tensors) {
+            t = e++;
+        } else {
+            bool more = true;
+            while (s_g >= s_g_hi && more) more = next_piece();
+            if (more) {
+                const uint32_t g = s_g;
+                t = s_g_t;
+                while (g >= B.item[t].first_chunk + B.item[t].n_chunks) ++t;
+                lo = g - B.item[t].first_chunk;
+                hi = min(s_g_hi - B.item[t].first_chunk, B.item[t].n_chunks);
+            }
+        }
+        __syncwarp();
+        if (threadIdx.x == 0) {
+            s_empty = e;
+            s_t = t; s_lo = lo; s_hi = hi;
+            if (hi > lo) { s_g += hi - lo; s_g_t = t; }
+        }
+    };
+    for (;;) {
+        __syncthreads();                                         // everybody is done with the previous part
+        if (threadIdx.x < 32) next_part();
+        __syncthreads();
+        const uint32_t t = s_t;
+        if (t == kNone) break;
+        const bool opened_before = s_opened == t;
         DecParams P;
         P.comp = B.item[t].comp; P.base = XOR ? B.item[t].base : nullptr; P.out = B.item[t].out; P.ctl = B.ctl;
         P.comp_bytes = B.item[t].comp_bytes; P.input_bytes = B.item[t].input_bytes;
@@ -1502,52 +1638,10 @@ decode_batch_kernel(const __grid_constant__ DecBatchParams B)
         P.spin_limit = B.spin_limit; P.skip_copy = B.skip_copy; P.sliced = B.sliced; P.active = blockDim.x >> 5;
         const uint64_t tables = 256 + (((uint64_t)4 * P.n_chunks + 15) & ~15ull) + 32ull * (P.chunk_bytes <= 8192 ? 2u : 4u) * P.n_chunks;
         P.spec = P.comp_bytes >= kHeaderBytes + tables ? 1u : 0u;
-        __syncthreads();                                         // everybody is done with the previous tensor's tables
-        const uint32_t err = decode_one<FMT, PPL, XOR, XOR || FMT == ZC_FMT_SCALE_U8, SMALL>(P, M, seg_lo, seg_hi, 0, 1, parity0, parity1);
-        if (err && raise_status(B.ctl, B.call_id, err)) B.ctl->failed = B.tensor_base + t + 1;
-    };
-
-    // The ranges of all rounds come one after the other from a ticket counter.  Block 0 first walks over the tensors, if there
-    // are any without chunks: their headers are still checked.  (The walk takes 0.1 us a tensor, which the block is late for its
-    // range: 64 BF16 pages of 129 chunks 37 us, without it 31 us.)
-    __shared__ uint32_t s_range;
-    uint32_t empties = blockIdx.x == 0 && B.n_empty ? 0u : B.n_tensors;      // cursor of that walk
-    uint32_t t = 0, g = 0, g_hi = 0;
-    bool in_range = false;
-    for (;;) {
-        uint32_t tt, seg_lo, seg_hi;
-        if (empties < B.n_tensors) {
-            if (B.item[empties].n_chunks != 0) { ++empties; continue; }
-            tt = empties++; seg_lo = 0; seg_hi = 0;
-        } else {
-            if (!in_range) {
-                __syncthreads();
-                if (threadIdx.x == 0) s_range = atomicAdd(&B.ctl->ticket, 1u);
-                __syncthreads();
-                const uint32_t r = s_range;
-                const uint32_t round = r / gridDim.x, j = r % gridDim.x;
-                if (round >= B.n_rounds) break;
-                const uint32_t lo_c = round ? B.round_end[round - 1] : 0u, n_c = B.round_end[round] - lo_c;
-                g = lo_c + (uint32_t)((uint64_t)j * n_c / gridDim.x);
-                g_hi = lo_c + (uint32_t)((uint64_t)(j + 1) * n_c / gridDim.x);
-                // the last tensor that starts at or before g (tensors without chunks share their start with the next one)
-                uint32_t lo = 0, hi = B.n_tensors;
-                while (hi - lo > 1) {
-                    const uint32_t mid = (lo + hi) / 2;
-                    if (B.item[mid].first_chunk <= g) lo = mid; else hi = mid;
-                }
-                t = lo;
-                in_range = true;
-            }
-            if (g >= g_hi || t >= B.n_tensors) { in_range = false; continue; }
-            const uint32_t first = B.item[t].first_chunk, n = B.item[t].n_chunks;
-            if (g >= first + n) { ++t; continue; }
-            seg_hi = min(g_hi, first + n) - first;
-            seg_lo = g - first;
-            tt = t++;
-            g = first + seg_hi;
-        }
-        run(tt, seg_lo, seg_hi);
+        const uint32_t err = decode_one<FMT, PPL, XOR, XOR || FMT == ZC_FMT_SCALE_U8, SMALL>(P, M, s_lo, s_hi, 0, 1, opened_before, parity0, parity1);
+        if (err && raise_status(B.ctl, B.call_id, err)) B.ctl->failed = B.tensor_base + s_t + 1;
+        // (a tensor that could not be opened is opened again, and refused again, in every part)
+        if (!opened_before && threadIdx.x == 0) s_opened = err ? kNone : t;
     }
 }
 
@@ -1748,7 +1842,7 @@ DecShape split_shape(const zc_plan_t* p, uint32_t n_chunks, uint32_t* groups)
     return s;
 }
 
-// Blocks of a batched launch: one per SM, or fewer.  The chunk index space is cut into equal ranges, and a range that reaches
+// Blocks of a batched launch: one per SM, or fewer.  The chunk index space is cut into equal slices, and a slice that reaches
 // over a tensor's end costs its block a second header, table and walk over a subchunk, one after the other.  A multiple of
 // the number of tensors has no such ranges when the tensors are of one size.  Taken is what is shorter for the block with the
 // longest way, in symbols of a lane's walk: a tensor's part costs kDecOpenSyms (9 us) and its chunks a walk for every round
@@ -1757,7 +1851,7 @@ DecShape split_shape(const zc_plan_t* p, uint32_t n_chunks, uint32_t* groups)
 constexpr uint32_t kDecOpenSyms = 160, kDecChunkSyms = 16;
 uint32_t batch_grid(const DecItem* item, uint32_t n, uint32_t with_chunks, uint64_t total, uint32_t warps, uint32_t sub)
 {
-    const uint32_t most = (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>(total, (uint64_t)sm_count()));
+    const uint32_t most = (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>({total, (uint64_t)sm_count(), kDecMaxBlocks}));
     const uint32_t even = with_chunks ? most / with_chunks * with_chunks : 0;
     if (with_chunks < 2 || even == 0 || even == most || total >= (uint64_t)kDecOneRound * most * warps) return most;
     auto longest = [&](const uint32_t ranges) {
@@ -1943,22 +2037,20 @@ zc_status zc_decompress_batch_xor(uint32_t n_tensors, const zc_plan_t* const* pl
             B.n_empty += B.item[i].n_chunks == 0;
         }
         const uint32_t grid = batch_grid(B.item, n, n - B.n_empty, total, shape.warps, B.sub);
-        // Rounds: three quarters (deltas: half, since unchanged stretches take a fraction of the time) of what is left go to the
-        // next one, in whole chunks per warp, until a range is down to two chunks per warp; the last one takes the rest.  With
-        // fewer than kDecOneRound chunks per warp in all, another range costs more than it evens out (FP8 at 16 KiB chunks, 9
-        // chunks per warp: 219 us in one round, 270 us in three; BF16 at 1 KiB chunks, 44 per warp: 119 us in one round, 140 in
-        // four).
+        // Pieces of a slice: seven eighths (deltas: half, since unchanged stretches take a fraction of the time) of what is left, until
+        // one is down to two chunks per warp; the last one is the rest.  With fewer than kDecOneRound chunks per warp in all, another
+        // piece costs more than it evens out (FP8 at 16 KiB chunks, 9 chunks per warp: 219 us in one round, 270 us in three; BF16 at
+        // 1 KiB chunks, 44 per warp: 119 us in one round, 140 in four).
         const uint64_t turn = (uint64_t)grid * shape.warps;      // one chunk per warp
-        uint64_t done = 0;
-        B.n_rounds = 0;
-        while (done < total) {
-            const uint64_t left = total - done, part = (any_base ? left / 2 : left - left / 4) / turn * turn;
-            const bool last = B.n_rounds + 1 == kDecMaxRounds || total < kDecOneRound * turn || left - part < turn || part < 2 * turn;
-            done = last ? total : done + part;
-            B.round_end[B.n_rounds++] = (uint32_t)done;
+        B.total = (uint32_t)total;
+        B.n_pieces = 0;
+        for (uint64_t done = 0; done < 65536;) {
+            const uint64_t left = 65536 - done, part = any_base ? left / 2 : left - left / 8;
+            const bool last = B.n_pieces + 1 == kDecMaxPieces || total < kDecOneRound * turn || (left - part) * total < 2 * turn * 65536;
+            done = last ? 65536 : done + part;
+            B.piece_end[B.n_pieces++] = (uint32_t)done;
         }
-        // the ranges are handed out through the ticket word of the control block
-        if (cudaMemsetAsync(&B.ctl->ticket, 0, sizeof(uint32_t), st) != cudaSuccess) return ZC_E_CUDA;
+        if (B.n_pieces > 1 && cudaMemsetAsync((uint8_t*)d_workspace + kDecClaims, 0, 4 * (kDecMaxPieces - 1) * kDecClaimWords, st) != cudaSuccess) return ZC_E_CUDA;
         DecRanges R{nullptr, 0, nullptr, 0, d_workspace, sizeof(Control)};
 #if ZC_DEBUG_CHECKS
         DbgHull rd, wr;

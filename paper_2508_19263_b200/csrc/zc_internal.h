@@ -103,7 +103,7 @@ struct Control {
     unsigned long long status;   // (call id << 8) | zc_status raised on the device; first error of a call wins
     unsigned long long call_id;  // id of the call that last used the block; a status with another id is stale.
                                  // The compress calls clear the whole block and use id 0.
-    uint32_t ticket;             // next batch of chunks (encoder) or range of chunks (batched decoder) to hand out
+    uint32_t ticket;             // next batch of chunks the encoder hands out
     uint32_t failed;             // batched calls: 1 + index of the tensor the recorded error belongs to
     TensorCounters tc;           // zc_compress: the counters of its one tensor
     uint32_t pad[4];

@@ -629,3 +629,30 @@ def test_batched_decoder_with_tensors_of_one_size_and_of_several(count, chunk_by
             assert zc.batch_status(ws) == (zc.OK, None)
             for b, d, m in zip(backs, d_ins, sizes):
                 assert torch.equal(b[:m], d[:m]) and bool((b[m:] == 0xEE).all())
+
+
+@pytest.mark.parametrize("fmt", FORMATS)
+@pytest.mark.parametrize("chunk_bytes", [1024, 2048, 3072, 4096, 5120])
+def test_decoder_of_small_chunks_with_one_and_two_coded_streams(fmt, chunk_bytes):
+    """Chunks up to 4 KiB have a loop of their own (one or two buffers for raw bytes), in which a container with both streams
+    coded goes to fewer warps: tensors of either kind in turn, from one symbol to more chunks than the kernel for few chunks
+    takes, ragged and complete, in one batched call and each on its own."""
+    cs = chunk_bytes // 2 * zo.group(fmt)
+    sizes = [1300 * cs, 2, 0, 1300 * cs - 2, 40 * cs + 8 * zo.group(fmt), cs, cs - 4 * zo.group(fmt), 29 * cs + 2]
+    datas, plans, ocbs, d_outs, batch, ws = _batch_compress(fmt, sizes, chunk_bytes, 70, [zc.POLICY_AUTO, zc.POLICY_HUFF_ALL])
+    got_sizes = zc.compress_batch(batch, ws)
+    backs = [torch.full((p.input_bytes + 16,), 0xEE, dtype=torch.uint8, device=DEV) for p in plans]
+
+    def check():
+        for p, data, back in zip(plans, datas, backs):
+            back = back.cpu().numpy()
+            assert np.array_equal(back[: p.input_bytes], data[: p.input_bytes]) and (back[p.input_bytes:] == 0xEE).all()
+
+    zc.decompress_batch(zc.DecompressBatch(plans, d_outs, got_sizes, backs), ws)
+    assert zc.batch_status(ws) == (zc.OK, None)
+    check()
+    for p, out, nbytes, back in zip(plans, d_outs, got_sizes, backs):
+        back.fill_(0xEE)
+        zc.decompress(p, out, nbytes, back, ws)
+        assert zc.device_status(p, ws) == zc.OK
+    check()
