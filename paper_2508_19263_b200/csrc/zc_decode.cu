@@ -831,6 +831,11 @@ __device__ __forceinline__ uint32_t run_small(const DecParams& P, const volatile
     constexpr bool kCopyRaw = kHuff == 1;                        // one coded stream, one raw
     constexpr int kRaw = H0 ? 1 : 0;                             // the raw one, and its mbarrier
     constexpr uint32_t kRawBufs = small_raw_buffers(PPL);
+    // 4 KiB chunks with one coded stream look ahead: the next chunk's table entries are taken and checked before a chunk is decoded,
+    // and where both pieces fit half a slot they lie side by side and the next one's copy is requested then, too, not when the
+    // slot is free.  (872 MB of BF16 weights 303 -> 291 us, of FP8 weights 372 -> 365 us.  With both streams coded the registers
+    // for two more pieces spill: 436 MB of deltas 345 -> 356 us; chunks up to 3 KiB gain nothing.)
+    constexpr bool kAhead = kHuff == 1 && PPL == 4;
     const uint32_t lane = threadIdx.x & 31;
     const uint32_t sub = PPL > 1 ? R : P.sub, cs = 32 * sub, chunk_bytes = 2 * cs, n_rounds = PPL > 1 ? 1u : sub / R;
     const uint32_t lut0_s = smem_u32(block_luts()), lut1_s = lut0_s + kLutBytes;
@@ -879,6 +884,12 @@ __device__ __forceinline__ uint32_t run_small(const DecParams& P, const volatile
     };
     // Takes the table entries in nx_* (of chunk cc), checks them, starts the copies, and requests the entries of the chunk
     // after it.  A copy takes 16 bytes more than the piece (the next piece or the guard), for the windows' look-ahead.
+    auto prefetch_base = [&](const uint32_t cc) {                // the base tensor's bytes travel to the L2
+        const uint8_t* const base = V.base;
+        const uint32_t n = cc < V.n_full ? chunk_bytes : (uint32_t)min((unsigned long long)chunk_bytes, V.input_bytes - (uint64_t)cc * chunk_bytes) & ~15u;
+        if (lane == 0 && base && n)
+            asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" :: "l"(base + (uint64_t)cc * chunk_bytes), "r"(n) : "memory");
+    };
     auto prepare = [&](const uint32_t cc) {
         bool ok = true;
         if (H0) { end0 = nx_end0; off0 = nx_off0; ok = check(end0, off0, start0, piece0); }
@@ -893,20 +904,45 @@ __device__ __forceinline__ uint32_t run_small(const DecParams& P, const volatile
             staged1 = flying1 = true;
             if (lane == 0 && !P.skip_copy) copy(slot1_s, V.payload + 16ull * off1, piece1 + 16, &bar[1]);
         }
-        if (XOR) {                                               // the base tensor's bytes travel to the L2
-            const uint8_t* const base = V.base;
-            const uint32_t n = cc < V.n_full ? chunk_bytes : (uint32_t)min((unsigned long long)chunk_bytes, V.input_bytes - (uint64_t)cc * chunk_bytes) & ~15u;
-            if (lane == 0 && base && n)
-                asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" :: "l"(base + (uint64_t)cc * chunk_bytes), "r"(n) : "memory");
-        }
+        if (XOR) prefetch_base(cc);
         if (cc + step < c_end) {
             if (H0) load_tables(0, cc + step, nx_end0, nx_off0);
             if (H1) load_tables(1, cc + step, nx_end1, nx_off1);
         }
     };
+    // kAhead: the coded stream's next piece (see prepare for the present one), where it lies, and where the present one does
+    uint32_t ne_end = 0, ne_off = 0, ne_at = 0, at_s = H0 ? slot0_s : slot1_s;
+    auto ask_next = [&](const uint32_t dst_s, const uint32_t bytes) {
+        ne_at = dst_s;
+        if (H0) flying0 = true; else flying1 = true;
+        if (lane == 0 && !P.skip_copy) copy(dst_s, V.payload + 16ull * ne_off, bytes + 16, &bar[H0 ? 0 : 1]);
+    };
+    auto look_ahead = [&](const uint32_t cc) {
+        uint32_t start, bytes;
+        ne_end = H0 ? nx_end0 : nx_end1; ne_off = H0 ? nx_off0 : nx_off1; ne_at = 0;
+        const bool ok = check(ne_end, ne_off, start, bytes);
+        if (!__all_sync(0xFFFFFFFFu, ok)) { err = ZC_E_CORRUPT; return; }
+        const uint32_t half = slot_bytes / 2 & ~15u, first_s = H0 ? slot0_s : slot1_s;
+        if (bytes + 16 <= half && (H0 ? piece0 : piece1) + 16 <= half) ask_next(at_s == first_s ? first_s + half : first_s, bytes);
+        if (XOR) prefetch_base(cc);
+        if (cc + step < c_end) {
+            if (H0) load_tables(0, cc + step, nx_end0, nx_off0);
+            if (H1) load_tables(1, cc + step, nx_end1, nx_off1);
+        }
+    };
+    // the next piece's copy, if it had to wait for the slot; and it becomes the present one (ne_at 0: it is not staged)
+    auto ask_late = [&]() {
+        const uint32_t bytes = (__shfl_sync(0xFFFFFFFFu, ne_end, 31) + 127) / 128 * 16;
+        if (!ne_at && bytes + 16 <= slot_bytes) ask_next(H0 ? slot0_s : slot1_s, bytes);
+    };
+    auto adopt = [&]() {
+        if (H0) { end0 = ne_end; off0 = ne_off; check(end0, off0, start0, piece0); staged0 = ne_at != 0; }
+        if (H1) { end1 = ne_end; off1 = ne_off; check(end1, off1, start1, piece1); staged1 = ne_at != 0; }
+        if (ne_at) at_s = ne_at;
+    };
     // One-symbol tables: the next chunk's pieces travel to the L2 while a chunk is decoded (their table entries are in nx_*), so that
-    // the copies are quicker than the merge they hide behind (872 MB of FP8 weights 382 -> 372 us; with two-symbol tables it is
-    // more instructions than it saves: BF16 297 -> 302 us).
+    // the copies are quicker than the merge they hide behind (436 MB of deltas 350 -> 345 us; with two-symbol tables it is more
+    // instructions than it saves: BF16 weights 297 -> 302 us).
     auto prefetch_next = [&]() {
         if (lane != 31) return;                                  // its subchunk's end is the piece's
         const uint32_t n0 = (nx_end0 + 127) / 128, n1 = (nx_end1 + 127) / 128;
@@ -948,9 +984,10 @@ __device__ __forceinline__ uint32_t run_small(const DecParams& P, const volatile
                     if (__any_sync(0xFFFFFFFFu, err == ZC_E_DEVICE_TIMEOUT)) { err = ZC_E_DEVICE_TIMEOUT; return; }
                     if (H0) flying0 = false;
                     if (H1) flying1 = false;
-                    if (H0) { if (staged0) lane_start(L0, 8 * slot0_s + start0); else L0.pos = start0; }
-                    if (H1) { if (staged1) lane_start(L1, 8 * slot1_s + start1); else L1.pos = start1; }
-                    if (((H0 && !pairs0) || (H1 && !pairs1)) && c + step < c_end) prefetch_next();
+                    if (H0) { if (staged0) lane_start(L0, 8 * (kAhead ? at_s : slot0_s) + start0); else L0.pos = start0; }
+                    if (H1) { if (staged1) lane_start(L1, 8 * (kAhead ? at_s : slot1_s) + start1); else L1.pos = start1; }
+                    if (kAhead && c + step < c_end) look_ahead(c + step);
+                    if (!kAhead && ((H0 && !pairs0) || (H1 && !pairs1)) && c + step < c_end) prefetch_next();
                 }
                 // ---- every lane decodes R symbols of its subchunk ----
                 if (kHuff) {
@@ -989,17 +1026,17 @@ __device__ __forceinline__ uint32_t run_small(const DecParams& P, const volatile
                         // symbols too many).  Anything else means the payload does not belong to the tables.
                         bool good = true;
                         if (H0) {
-                            const uint32_t used = L0.pos - (staged0 ? 8 * slot0_s : 0u);
+                            const uint32_t used = L0.pos - (staged0 ? 8 * (kAhead ? at_s : slot0_s) : 0u);
                             good = good && (FULL ? used == end0 : n_my ? used - end0 <= 15 * kLmax : start0 == end0);
                         }
                         if (H1) {
-                            const uint32_t used = L1.pos - (staged1 ? 8 * slot1_s : 0u);
+                            const uint32_t used = L1.pos - (staged1 ? 8 * (kAhead ? at_s : slot1_s) : 0u);
                             good = good && (FULL ? used == end1 : n_my ? used - end1 <= 15 * kLmax : start1 == end1);
                         }
                         if (!__all_sync(0xFFFFFFFFu, good)) err = ZC_E_CORRUPT;
                         // the slots are free: the next chunk's pieces travel while this round is merged and written
                         if (!err && c + step < c_end) {
-                            prepare(c + step);
+                            if (kAhead) ask_late(); else prepare(c + step);
                             if (kCopyRaw && kRawBufs == 2) copy_raw(other_raw(), c + step);
                         }
                     }
@@ -1049,6 +1086,7 @@ __device__ __forceinline__ uint32_t run_small(const DecParams& P, const volatile
             }
             if (kCopyRaw && kRawBufs == 1 && !err && c + step < c_end) copy_raw(raw_s, c + step);   // everybody has read this chunk's
             if (kCopyRaw && kRawBufs == 2) raw_s = other_raw();
+            if (kAhead && !err && c + step < c_end) adopt();
         };
         if (c < V.n_full) body(BoolTag<true>{}); else body(BoolTag<false>{});
     }
