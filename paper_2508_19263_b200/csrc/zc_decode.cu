@@ -833,7 +833,7 @@ __device__ __forceinline__ uint32_t run_small(const DecParams& P, const volatile
     constexpr uint32_t kRawBufs = small_raw_buffers(PPL);
     // 4 KiB chunks with one coded stream look ahead: the next chunk's table entries are taken and checked before a chunk is decoded,
     // and where both pieces fit half a slot they lie side by side and the next one's copy is requested then, too, not when the
-    // slot is free.  (872 MB of BF16 weights 303 -> 291 us, of FP8 weights 372 -> 365 us.  With both streams coded the registers
+    // slot is free.  (872 MB of BF16 weights 303 -> 283 us, of FP8 weights 372 -> 359 us.  With both streams coded the registers
     // for two more pieces spill: 436 MB of deltas 345 -> 356 us; chunks up to 3 KiB gain nothing.)
     constexpr bool kAhead = kHuff == 1 && PPL == 4;
     const uint32_t lane = threadIdx.x & 31;
@@ -911,19 +911,18 @@ __device__ __forceinline__ uint32_t run_small(const DecParams& P, const volatile
         }
     };
     // kAhead: the coded stream's next piece (see prepare for the present one), where it lies, and where the present one does
-    uint32_t ne_end = 0, ne_off = 0, ne_at = 0, at_s = H0 ? slot0_s : slot1_s;
-    auto ask_next = [&](const uint32_t dst_s, const uint32_t bytes) {
+    uint32_t ne_start = 0, ne_end = 0, ne_bytes = 0, ne_off = 0, ne_at = 0, at_s = H0 ? slot0_s : slot1_s;
+    auto ask_next = [&](const uint32_t dst_s) {
         ne_at = dst_s;
         if (H0) flying0 = true; else flying1 = true;
-        if (lane == 0 && !P.skip_copy) copy(dst_s, V.payload + 16ull * ne_off, bytes + 16, &bar[H0 ? 0 : 1]);
+        if (lane == 0 && !P.skip_copy) copy(dst_s, V.payload + 16ull * ne_off, ne_bytes + 16, &bar[H0 ? 0 : 1]);
     };
     auto look_ahead = [&](const uint32_t cc) {
-        uint32_t start, bytes;
         ne_end = H0 ? nx_end0 : nx_end1; ne_off = H0 ? nx_off0 : nx_off1; ne_at = 0;
-        const bool ok = check(ne_end, ne_off, start, bytes);
+        const bool ok = check(ne_end, ne_off, ne_start, ne_bytes);
         if (!__all_sync(0xFFFFFFFFu, ok)) { err = ZC_E_CORRUPT; return; }
         const uint32_t half = slot_bytes / 2 & ~15u, first_s = H0 ? slot0_s : slot1_s;
-        if (bytes + 16 <= half && (H0 ? piece0 : piece1) + 16 <= half) ask_next(at_s == first_s ? first_s + half : first_s, bytes);
+        if (ne_bytes + 16 <= half && (H0 ? piece0 : piece1) + 16 <= half) ask_next(at_s == first_s ? first_s + half : first_s);
         if (XOR) prefetch_base(cc);
         if (cc + step < c_end) {
             if (H0) load_tables(0, cc + step, nx_end0, nx_off0);
@@ -932,12 +931,11 @@ __device__ __forceinline__ uint32_t run_small(const DecParams& P, const volatile
     };
     // the next piece's copy, if it had to wait for the slot; and it becomes the present one (ne_at 0: it is not staged)
     auto ask_late = [&]() {
-        const uint32_t bytes = (__shfl_sync(0xFFFFFFFFu, ne_end, 31) + 127) / 128 * 16;
-        if (!ne_at && bytes + 16 <= slot_bytes) ask_next(H0 ? slot0_s : slot1_s, bytes);
+        if (!ne_at && ne_bytes + 16 <= slot_bytes) ask_next(H0 ? slot0_s : slot1_s);
     };
     auto adopt = [&]() {
-        if (H0) { end0 = ne_end; off0 = ne_off; check(end0, off0, start0, piece0); staged0 = ne_at != 0; }
-        if (H1) { end1 = ne_end; off1 = ne_off; check(end1, off1, start1, piece1); staged1 = ne_at != 0; }
+        if (H0) { start0 = ne_start; end0 = ne_end; piece0 = ne_bytes; off0 = ne_off; staged0 = ne_at != 0; }
+        if (H1) { start1 = ne_start; end1 = ne_end; piece1 = ne_bytes; off1 = ne_off; staged1 = ne_at != 0; }
         if (ne_at) at_s = ne_at;
     };
     // One-symbol tables: the next chunk's pieces travel to the L2 while a chunk is decoded (their table entries are in nx_*), so that
