@@ -475,6 +475,37 @@ struct DecShared {                   // what the block's prologue leaves for the
 
 template <bool V> struct BoolTag { static constexpr bool value = V; };
 
+// The warp waits for the copies on its two mbarriers (those it has on the way); false when a wait gave up.  The phases count only
+// where every lane has seen the copies land: all lanes keep the same parity.
+__device__ __forceinline__ bool pieces_here(const bool on0, const bool on1, uint64_t* const bar, uint32_t& parity0, uint32_t& parity1, const uint32_t spin_limit)
+{
+    bool late = false;
+    if (on0) late = !mbar_wait(&bar[0], parity0, spin_limit);
+    if (on1) late = !mbar_wait(&bar[1], parity1, spin_limit) || late;
+    if (__any_sync(0xFFFFFFFFu, late)) return false;
+    if (on0) parity0 ^= 1;
+    if (on1) parity1 ^= 1;
+    return true;
+}
+
+// Whether one of the block's copies did not land within the limit.  The block then takes no more parts: the copy may still write into
+// the pools, and the phases of its mbarrier are not known any more.
+__device__ __forceinline__ uint32_t& block_lost()
+{
+    __shared__ uint32_t s_lost;
+    return s_lost;
+}
+// A copy that was started and not waited for (the warp's loop ended early, on damage or on a wait that gave up) must land before the
+// block goes on or leaves, and its phase counts: the warp's next wait on the mbarrier is for the next phase.  False when it did not land.
+__device__ __forceinline__ bool settle(const bool flying, uint64_t* const bar, uint32_t& parity, const uint32_t spin_limit)
+{
+    if (!flying) return true;                                    // (the same in every lane)
+    const bool landed = mbar_wait(bar, parity, spin_limit);
+    if (__all_sync(0xFFFFFFFFu, landed)) { parity ^= 1; return true; }
+    if ((threadIdx.x & 31) == 0) block_lost() = 1;
+    return false;
+}
+
 // PPL = 16-symbol parts each lane merges per round = R / 16, R in {16, 32, 64}.
 // SIDE: the streams of chunks with both streams coded are decoded side by side.
 template <int FMT, int PPL, bool H0, bool H1, bool XOR, bool SIDE>
@@ -658,21 +689,15 @@ __device__ __forceinline__ uint32_t run_chunks(const DecParams& P, const DecShar
                 if (kHuff && (sliced0 || sliced1) && r % kRoundsPerSlice == 0) {
                     // the slice requested after the previous one was used up (or, for the chunk's first one, while
                     // the chunk before was merged) is needed now
-                    if (tot0) { if (mbar_wait(&bar[0], parity0, P.spin_limit)) { parity0 ^= 1; flying0 = false; } else err = ZC_E_DEVICE_TIMEOUT; }
-                    if (tot1) { if (mbar_wait(&bar[1], parity1, P.spin_limit)) { parity1 ^= 1; flying1 = false; } else err = ZC_E_DEVICE_TIMEOUT; }
-                    if (__any_sync(0xFFFFFFFFu, err == ZC_E_DEVICE_TIMEOUT)) { err = ZC_E_DEVICE_TIMEOUT; return; }
+                    if (!pieces_here(tot0 != 0, tot1 != 0, bar, parity0, parity1, P.spin_limit)) { err = ZC_E_DEVICE_TIMEOUT; return; }
+                    if (tot0) flying0 = false;
+                    if (tot1) flying1 = false;
                     if (by0) { org0 = 8 * slot0_s + min(rel0 - 8 * at0, 127u); lane_start(L0, org0); }
                     if (by1) { org1 = 8 * slot1_s + min(rel1 - 8 * at1, 127u); lane_start(L1, org1); }
                     tot0 = tot1 = 0;
                 }
                 if (kHuff && r == 0) {
-                    if (H0 && staged0 && !sliced0) {
-                        if (mbar_wait(&bar[0], parity0, P.spin_limit)) parity0 ^= 1; else err = ZC_E_DEVICE_TIMEOUT;
-                    }
-                    if (H1 && staged1 && !sliced1) {
-                        if (mbar_wait(&bar[1], parity1, P.spin_limit)) parity1 ^= 1; else err = ZC_E_DEVICE_TIMEOUT;
-                    }
-                    if (__any_sync(0xFFFFFFFFu, err == ZC_E_DEVICE_TIMEOUT)) { err = ZC_E_DEVICE_TIMEOUT; return; }
+                    if (!pieces_here(H0 && staged0 && !sliced0, H1 && staged1 && !sliced1, bar, parity0, parity1, P.spin_limit)) { err = ZC_E_DEVICE_TIMEOUT; return; }
                     if (!sliced0) flying0 = false;
                     if (!sliced1) flying1 = false;
                     // staged: positions count from shared address 0; from global memory: from the piece, and the last
@@ -787,9 +812,8 @@ __device__ __forceinline__ uint32_t run_chunks(const DecParams& P, const DecShar
         };
         if (c < n_full) body(BoolTag<true>{}); else body(BoolTag<false>{});
     }
-    // a copy that was started and not waited for (the loop ended early) must land before the block may leave
-    if (flying0 && !P.skip_copy) mbar_wait(&bar[0], parity0, P.spin_limit);
-    if (flying1 && !P.skip_copy) mbar_wait(&bar[1], parity1, P.spin_limit);
+    if (!P.skip_copy && !settle(flying0, &bar[0], parity0, P.spin_limit)) err = ZC_E_DEVICE_TIMEOUT;
+    if (!P.skip_copy && !settle(flying1, &bar[1], parity1, P.spin_limit)) err = ZC_E_DEVICE_TIMEOUT;
     return err;
 }
 
@@ -961,7 +985,7 @@ __device__ __forceinline__ uint32_t run_small(const DecParams& P, const volatile
     if (c < c_end) {
         if (H1) load_tables(1, c, nx_end1, nx_off1);
         prepare(c);
-        if (kCopyRaw) copy_raw(raw_s, c);
+        if (kCopyRaw && !err) copy_raw(raw_s, c);
     }
 
     for (; c < c_end && !err; c += step) {
@@ -977,9 +1001,7 @@ __device__ __forceinline__ uint32_t run_small(const DecParams& P, const volatile
             LaneBits L0{}, L1{};                                 // (.pos also where the piece is read from global memory)
             for (uint32_t r = 0; r <= last_r; ++r) {
                 if (kHuff && r == 0) {
-                    if (H0 && staged0) { if (mbar_wait(&bar[0], parity0, P.spin_limit)) parity0 ^= 1; else err = ZC_E_DEVICE_TIMEOUT; }
-                    if (H1 && staged1) { if (mbar_wait(&bar[1], parity1, P.spin_limit)) parity1 ^= 1; else err = ZC_E_DEVICE_TIMEOUT; }
-                    if (__any_sync(0xFFFFFFFFu, err == ZC_E_DEVICE_TIMEOUT)) { err = ZC_E_DEVICE_TIMEOUT; return; }
+                    if (!pieces_here(H0 && staged0, H1 && staged1, bar, parity0, parity1, P.spin_limit)) { err = ZC_E_DEVICE_TIMEOUT; return; }
                     if (H0) flying0 = false;
                     if (H1) flying1 = false;
                     if (H0) { if (staged0) lane_start(L0, 8 * (kAhead ? at_s : slot0_s) + start0); else L0.pos = start0; }
@@ -1035,7 +1057,7 @@ __device__ __forceinline__ uint32_t run_small(const DecParams& P, const volatile
                         // the slots are free: the next chunk's pieces travel while this round is merged and written
                         if (!err && c + step < c_end) {
                             if (kAhead) ask_late(); else prepare(c + step);
-                            if (kCopyRaw && kRawBufs == 2) copy_raw(other_raw(), c + step);
+                            if (kCopyRaw && kRawBufs == 2 && !err) copy_raw(other_raw(), c + step);
                         }
                     }
                 }
@@ -1088,9 +1110,8 @@ __device__ __forceinline__ uint32_t run_small(const DecParams& P, const volatile
         };
         if (c < V.n_full) body(BoolTag<true>{}); else body(BoolTag<false>{});
     }
-    // a copy that was started and not waited for (the loop ended early) must land before the block may leave
-    if (flying0 && !P.skip_copy) mbar_wait(&bar[0], parity0, P.spin_limit);
-    if (flying1 && !P.skip_copy) mbar_wait(&bar[1], parity1, P.spin_limit);
+    if (!P.skip_copy && !settle(flying0, &bar[0], parity0, P.spin_limit)) err = ZC_E_DEVICE_TIMEOUT;
+    if (!P.skip_copy && !settle(flying1, &bar[1], parity1, P.spin_limit)) err = ZC_E_DEVICE_TIMEOUT;
     return err;
 }
 
@@ -1575,6 +1596,7 @@ decode_batch_kernel(const __grid_constant__ DecBatchParams B)
     __shared__ uint32_t s_empty, s_piece, s_g, s_g_hi, s_g_t;    // tensor to look at for an empty one; pieces taken of my slice; the rest of a piece
     if (threadIdx.x == 0) {
         s_opened = kNone;
+        block_lost() = 0;
         // Block 0 first walks over the tensors, if there are any without chunks: their headers are still checked.  (The walk takes
         // 0.1 us a tensor, which the block is late for its slice: 64 BF16 pages of 129 chunks 37 us, without it 31 us.)
         s_empty = blockIdx.x == 0 && B.n_empty ? 0u : B.n_tensors;
@@ -1638,10 +1660,11 @@ decode_batch_kernel(const __grid_constant__ DecBatchParams B)
     auto next_part = [&]() {
         uint32_t t = kNone, lo = 0, hi = 0, e = s_empty;
         while (e < B.n_tensors && B.item[e].n_chunks != 0) ++e;
-        if (e < B.n_tensors) {
+        const bool lost = block_lost() != 0;
+        if (e < B.n_tensors && !lost) {
             t = e++;
         } else {
-            bool more = true;
+            bool more = !lost;
             while (s_g >= s_g_hi && more) more = next_piece();
             if (more) {
                 const uint32_t g = s_g;

@@ -187,3 +187,50 @@ def test_output_aligned_to_16_bytes_only(batched):
     back = buf.cpu().numpy()
     assert np.array_equal(back[16: 16 + p.input_bytes], data[: p.input_bytes])
     assert (back[:16] == 0xEE).all() and (back[16 + p.input_bytes:] == 0xEE).all()
+
+
+@pytest.mark.parametrize("damage", ["payload", "first_table_entries", "later_table_entries"])
+@pytest.mark.parametrize("policy", [zc.POLICY_AUTO, zc.POLICY_HUFF_ALL])
+@pytest.mark.parametrize("chunk_bytes", [1024, 3072, 4096, 16384])
+def test_tensors_behind_a_damaged_one_are_decoded(chunk_bytes, policy, damage):
+    """A warp leaves a damaged tensor with a copy still on its way (the next chunk's piece or raw bytes); the copy's phase has to
+    count, or every later wait of the warp is one copy behind.  447 tensors of four to five chunks per warp come to about three
+    tensors per block, of five different contents and every fourth of them damaged: the others must come out whole."""
+    n = 120 * chunk_bytes // 2
+    contents = [torch.from_numpy(_bf16_weights(n, 40 + k, 0.02 * 4.0 ** k)).to(DEV) for k in range(5)]
+    p = zc.plan(zc.FMT_BF16, n, chunk_bytes)
+    ws = torch.zeros(zc.CompressBatch([p] * 5, contents, contents).workspace_bytes, dtype=torch.uint8, device=DEV)
+    hists = zc.histogram_batch(zc.HistogramBatch([p] * 5, contents), torch.zeros((5, 2, 256), dtype=torch.int64, device=DEV))
+    conts = [torch.empty(p.max_compressed_bytes, dtype=torch.uint8, device=DEV) for _ in range(5)]
+    enc = zc.CompressBatch([p] * 5, contents, conts)
+    enc.set_codebooks(zc.build_codebooks([p] * 5, hists.cpu().numpy(), policy))
+    sizes = zc.compress_batch(enc, ws)
+
+    bads = []
+    for cont, size in zip(conts, sizes):
+        bad = cont[:size].cpu().numpy().copy()
+        hd = zo.parse_header(bad)
+        assert hd["streams"][0]["mode"] == zo.HUFF
+        tables = 128 + 256 + 480                                     # header, code lengths, 120 chunk offsets
+        if damage == "payload":
+            bad[hd["total_bytes"] - 16 - hd["payload_bytes"]: hd["total_bytes"] - 16] = 0
+        else:
+            width = 2 if chunk_bytes <= 8192 else 4
+            for c in range(28) if damage == "first_table_entries" else range(30, 120, 9):
+                at = tables + (32 * c + 31) * width                  # the chunk's last subchunk ends before it starts
+                bad[at: at + width] = 0
+        bads.append(torch.from_numpy(bad).to(DEV))
+
+    which = [(t % 5, t % 4 == 1) for t in range(447)]
+    stride = p.input_bytes + 64
+    arena = torch.full((447 * stride,), 0xEE, dtype=torch.uint8, device=DEV)
+    outs = [arena[t * stride: (t + 1) * stride] for t in range(447)]
+    batch = zc.DecompressBatch([p] * 447, [(bads if bad else conts)[k] for k, bad in which], [sizes[k] for k, _ in which], outs)
+    for _ in range(2):
+        arena.fill_(0xEE)
+        zc.decompress_batch(batch, ws)
+        status, tensor = zc.batch_status(ws)
+        assert status == zc.E_CORRUPT and which[tensor][1]
+        for (k, bad), out in zip(which, outs):
+            assert bad or torch.equal(out[: p.input_bytes], contents[k])
+            assert bool((out[p.input_bytes:] == 0xEE).all())
