@@ -1210,7 +1210,7 @@ __device__ __forceinline__ uint32_t open_container(const DecParams& P, const Dec
             for (int s = 0; s < 2; ++s) if (mode[s] == ZC_MODE_RAW) { sec[s] = off; off += (P.n_syms + 15) & ~15ull; }
             const bool any_huff = mode[0] == ZC_MODE_HUFF || mode[1] == ZC_MODE_HUFF;
             const uint64_t total = h64[kHdrTotal / 8], poff = h64[kHdrPayloadOff / 8], pbytes = h64[kHdrPayloadBytes / 8];
-            ok = poff == off && (pbytes & 15) == 0 && total == poff + pbytes + (any_huff ? 16 : 0) && total <= P.comp_bytes;
+            ok = poff == off && (pbytes & 15) == 0 && payload_fits(P.comp_bytes, off, any_huff ? 16 : 0, pbytes, total);
             for (int s = 0; s < 2 && ok; ++s)
                 ok = reinterpret_cast<const unsigned long long*>(h + kHdrStream0 + kHdrStreamStride * s)[3] == sec[s];
             T.mode[0] = mode[0]; T.mode[1] = mode[1];

@@ -550,7 +550,7 @@ zc_status zc_validate_container(const zc_plan_t* p, const void* h_container, siz
     const Layout L = make_layout(*p, mode);
     const bool any_huff = mode[0] == ZC_MODE_HUFF || mode[1] == ZC_MODE_HUFF;
     const uint64_t total = rd(c + kHdrTotal, 8), poff = rd(c + kHdrPayloadOff, 8), pbytes = rd(c + kHdrPayloadBytes, 8);
-    if (poff != L.payload_off || pbytes % 16 || total != poff + pbytes + (any_huff ? 16 : 0) || total > bytes)
+    if (poff != L.payload_off || pbytes % 16 || !payload_fits(bytes, L.payload_off, any_huff ? 16 : 0, pbytes, total))
         return ZC_E_CORRUPT;
     for (int s = 0; s < 2; ++s)
         if (rd(c + kHdrStream0 + kHdrStreamStride * s + kSdSection, 8) != L.section_off[s]) return ZC_E_CORRUPT;

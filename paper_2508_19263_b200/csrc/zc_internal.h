@@ -89,6 +89,18 @@ inline Layout make_layout(const zc_plan_s& p, const uint32_t mode[2])
     return L;
 }
 
+// Whether the sizes that a header states fit each other and the `room` bytes there are: payload_off (worked out from the plan and the
+// streams' modes), the payload area, `guard` bytes.  A damaged header may state any 64-bit values, so none of them is added to before it
+// is known to be small.
+#if defined(__CUDACC__)
+__host__ __device__
+#endif
+inline bool payload_fits(uint64_t room, uint64_t payload_off, uint64_t guard, uint64_t payload_bytes, uint64_t total)
+{
+    return payload_off <= room && guard <= room - payload_off && payload_bytes <= room - payload_off - guard &&
+           total == payload_off + payload_bytes + guard;
+}
+
 // What the encoder accumulates per tensor on the device.
 struct TensorCounters {
     unsigned long long payload_bits[2];

@@ -234,3 +234,27 @@ def test_tensors_behind_a_damaged_one_are_decoded(chunk_bytes, policy, damage):
         for (k, bad), out in zip(which, outs):
             assert bad or torch.equal(out[: p.input_bytes], contents[k])
             assert bool((out[p.input_bytes:] == 0xEE).all())
+
+
+@pytest.mark.parametrize("form", ["payload_of_minus_16", "total_of_a_header"])
+@pytest.mark.parametrize("chunk_bytes", [4096, 16384])
+def test_header_sizes_that_wrap_are_refused(chunk_bytes, form):
+    """total_bytes is payload_off + payload_bytes + guard modulo 2^64 only: refused with nothing written, alone and in a batch."""
+    fmt, n = zc.FMT_BF16, 9 * chunk_bytes // 2
+    data = _bf16_weights(n, 6)
+    cont = _oracle_container(fmt, data, n, chunk_bytes)
+    hd = zo.parse_header(cont)
+    off = hd["total_bytes"] - 16 - hd["payload_bytes"]
+    total, payload = (off, 2 ** 64 - 16) if form == "payload_of_minus_16" else (128, 2 ** 64 + 128 - off - 16)
+    bad = cont.copy()
+    bad[32:40] = np.frombuffer(total.to_bytes(8, "little"), np.uint8)
+    bad[48:56] = np.frombuffer(payload.to_bytes(8, "little"), np.uint8)
+    p = zc.plan(fmt, n, chunk_bytes)
+    d_bad, d_cont = torch.from_numpy(bad).to(DEV), torch.from_numpy(cont).to(DEV)
+    ws = torch.zeros(256, dtype=torch.uint8, device=DEV)
+    outs = [torch.full((p.input_bytes,), 0xEE, dtype=torch.uint8, device=DEV) for _ in range(2)]
+    zc.decompress(p, d_bad, bad.size, outs[0], ws)
+    assert zc.device_status(p, ws) == zc.E_CORRUPT and bool((outs[0] == 0xEE).all())
+    zc.decompress_batch(zc.DecompressBatch([p, p], [d_bad, d_cont], [bad.size, cont.size], outs), ws)
+    assert zc.batch_status(ws) == (zc.E_CORRUPT, 0)
+    assert bool((outs[0] == 0xEE).all()) and np.array_equal(outs[1].cpu().numpy(), data)

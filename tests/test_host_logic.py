@@ -2,6 +2,8 @@
 import ctypes
 import os
 import re
+import subprocess
+import sys
 
 import numpy as np
 import pytest
@@ -318,6 +320,44 @@ def test_validate_accepts_oracle_containers_and_rejects_damage(fmt, policy, cbyt
         assert zc.validate_container(p, bad) == zc.E_CORRUPT
         bad = cont.copy(); bad[-3] = 1                                # guard not zero
         assert zc.validate_container(p, bad) == zc.E_CORRUPT
+
+
+WRAPPED_SIZES = {
+    # total_bytes and payload_bytes whose sum with payload_off and the guard comes out right modulo 2^64
+    "payload_of_minus_16": lambda off: (off, 2 ** 64 - 16),
+    "total_of_a_header": lambda off: (128, 2 ** 64 + 128 - off - 16),
+}
+
+
+@pytest.mark.parametrize("form", sorted(WRAPPED_SIZES))
+def test_header_sizes_that_wrap_are_refused_before_the_tables_are_read(form, tmp_path):
+    """The container is cut off in its tables, at the end of a mapped page with an unreadable one behind it; a process of its own,
+    because a checker that believes the header's sizes reads on."""
+    _, _, _, cont = _container(zo.BF16, 200 * 2048, 4096, zo.POLICY_AUTO)
+    hd = zo.parse_header(cont)
+    off = hd["total_bytes"] - 16 - hd["payload_bytes"]
+    bad = cont.copy()
+    bad[32:40] = np.frombuffer(WRAPPED_SIZES[form](off)[0].to_bytes(8, "little"), np.uint8)
+    bad[48:56] = np.frombuffer(WRAPPED_SIZES[form](off)[1].to_bytes(8, "little"), np.uint8)
+    np.save(tmp_path / "bad.npy", bad[:4096])
+    child = f"""
+import ctypes, mmap, sys
+import numpy as np
+sys.path.insert(0, {ROOT!r})
+from paper_2508_19263_b200 import binding as zc
+bad = np.load({str(tmp_path / "bad.npy")!r})
+page = mmap.PAGESIZE
+area = mmap.mmap(-1, 2 * page)
+at = ctypes.addressof(ctypes.c_char.from_buffer(area))
+assert ctypes.CDLL(None).mprotect(ctypes.c_void_p(at + page), page, 0) == 0
+ctypes.memmove(at + page - bad.size, bad.ctypes.data, bad.size)
+p = zc.plan(zc.FMT_BF16, {200 * 2048}, 4096)
+print("status", zc._lib.zc_validate_container(p._h, ctypes.c_void_p(at + page - bad.size), bad.size), flush=True)
+import os
+os._exit(0)
+"""
+    r = subprocess.run([sys.executable, "-c", child], capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0 and f"status {zc.E_CORRUPT}" in r.stdout, (r.returncode, r.stdout, r.stderr)
 
 
 def test_stats_match_oracle():
