@@ -146,6 +146,8 @@ def _load():
     L.zc_test_encoder_workers.argtypes = [vp, C.c_uint32, C.c_uint32, C.c_uint64]
     L.zc_test_decoder_warps.restype = C.c_uint32
     L.zc_test_decoder_warps.argtypes = [vp, C.c_uint32]
+    L.zc_test_decoder_pieces.restype = C.c_uint32
+    L.zc_test_decoder_pieces.argtypes = [vp, C.c_uint32, C.c_uint64, C.POINTER(C.c_uint32)]
     L.zc_test_debug_counts.restype = C.c_int
     L.zc_test_debug_counts.argtypes = [C.POINTER(C.c_uint32)]
     for name in ("zc_test_set_wait_limit", "zc_test_stall_encoder", "zc_test_stall_decoder"):
@@ -553,3 +555,9 @@ def test_encoder_workers(p: Plan, n_coded: int, any_base: bool, total_chunks: in
 
 def test_decoder_warps(p: Plan, both_coded: bool) -> int:
     return int(_lib.zc_test_decoder_warps(p._h, 1 if both_coded else 0))
+
+
+def test_decoder_pieces(p: Plan, any_base: bool, total_chunks: int):
+    """zc_test_decoder_pieces: where the pieces of a slice end, in 65536ths of it."""
+    end = (C.c_uint32 * 7)()
+    return [int(end[i]) for i in range(_lib.zc_test_decoder_pieces(p._h, int(any_base), total_chunks, end))]

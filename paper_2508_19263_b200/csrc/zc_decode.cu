@@ -48,7 +48,7 @@ struct DecItem {
 // the block's last warp, header, tables, first pieces).  (Dealt out in rounds over the whole index space by a ticket counter, every
 // piece of a block was of another tensor: 1.74 GB of BF16 weights 621 us, now 612; their delta of 872 MB 550 and 524; 18 tensors of
 // 66 MB in all 58 and 53.  In one piece each, the delta takes 659 us.)
-constexpr uint32_t kDecMaxPieces = 5, kDecOneRound = 64;
+constexpr uint32_t kDecMaxPieces = 7, kDecOneRound = 64;
 constexpr uint32_t kDecMaxBlocks = 160, kDecClaimWords = kDecMaxBlocks / 32;
 constexpr size_t kDecClaims = 128;           // where the bits are in the control block: [piece - 1][kDecClaimWords]
 static_assert(sizeof(Control) <= kDecClaims && kDecClaims + 4 * (kDecMaxPieces - 1) * kDecClaimWords <= kControlBytes, "control block");
@@ -1901,6 +1901,28 @@ DecShape split_shape(const zc_plan_t* p, uint32_t n_chunks, uint32_t* groups)
     return s;
 }
 
+// Pieces of a slice of a batched launch (see kDecMaxPieces), as where they end in 65536ths of it; turn = one chunk for every warp.
+// Seven eighths of what is left, until one is down to two chunks per warp; the last one is the rest.  Deltas: half of the slice, then
+// an eighth of it or half of what is left, whichever is less, since slices differ in speed (unchanged stretches take half of the
+// time and less) and the piece that is taken last from a slow one is what the launch ends with.  (15 GB of deltas, most layers
+// unchanged: 6.77 ms; 7.59 ms with a half, a quarter and so on in five pieces, which left a quarter of a slow slice to the block that
+// came first.  872 MB with a quarter, half, three quarters unchanged 608, 514, 439 us against 606, 517, 485; all changed 665 against
+// 655: about 5 us for every piece more.)  With fewer than kDecOneRound chunks per warp in all, another piece costs more than it evens out
+// (FP8 at 16 KiB chunks, 9 chunks per warp: 219 us in one round, 270 us in three; BF16 at 1 KiB chunks, 44 per warp: 119 us in one
+// round, 140 in four).
+uint32_t dec_pieces(uint64_t total, uint64_t turn, bool any_base, uint32_t* piece_end)
+{
+    uint32_t n = 0;
+    for (uint64_t done = 0; done < 65536;) {
+        const uint64_t left = 65536 - done;
+        const uint64_t part = !any_base ? left - left / 8 : done ? std::min<uint64_t>(left / 2, 65536 / 8) : left / 2;
+        const bool last = n + 1 == kDecMaxPieces || total < kDecOneRound * turn || (left - part) * total < 2 * turn * 65536;
+        done = last ? 65536 : done + part;
+        piece_end[n++] = (uint32_t)done;
+    }
+    return n;
+}
+
 // Blocks of a batched launch: one per SM, or fewer.  The chunk index space is cut into equal slices, and a slice that reaches
 // over a tensor's end costs its block a second header, table and walk over a subchunk, one after the other.  A multiple of
 // the number of tensors has no such ranges when the tensors are of one size.  Taken is what is shorter for the block with the
@@ -1961,6 +1983,13 @@ uint32_t zc_test_decoder_warps(const zc_plan_t* p, uint32_t both_coded)
     DecShape sh;
     if (!p || dec_shape(p, both_coded != 0, &sh) != ZC_OK) return 0;
     return sh.warps;
+}
+
+uint32_t zc_test_decoder_pieces(const zc_plan_t* p, uint32_t any_base, uint64_t total_chunks, uint32_t* h_piece_end)
+{
+    DecShape sh;
+    if (!p || !h_piece_end || !total_chunks || dec_shape(p, any_base != 0, &sh) != ZC_OK) return 0;
+    return dec_pieces(total_chunks, std::min<uint64_t>({total_chunks, (uint64_t)sm_count(), kDecMaxBlocks}) * sh.warps, any_base != 0, h_piece_end);
 }
 
 zc_status zc_decompress(const zc_plan_t* p, const void* d_comp, size_t comp_bytes, void* d_out, void* d_workspace,
@@ -2096,19 +2125,8 @@ zc_status zc_decompress_batch_xor(uint32_t n_tensors, const zc_plan_t* const* pl
             B.n_empty += B.item[i].n_chunks == 0;
         }
         const uint32_t grid = batch_grid(B.item, n, n - B.n_empty, total, shape.warps, B.sub);
-        // Pieces of a slice: seven eighths (deltas: half, since unchanged stretches take a fraction of the time) of what is left, until
-        // one is down to two chunks per warp; the last one is the rest.  With fewer than kDecOneRound chunks per warp in all, another
-        // piece costs more than it evens out (FP8 at 16 KiB chunks, 9 chunks per warp: 219 us in one round, 270 us in three; BF16 at
-        // 1 KiB chunks, 44 per warp: 119 us in one round, 140 in four).
-        const uint64_t turn = (uint64_t)grid * shape.warps;      // one chunk per warp
         B.total = (uint32_t)total;
-        B.n_pieces = 0;
-        for (uint64_t done = 0; done < 65536;) {
-            const uint64_t left = 65536 - done, part = any_base ? left / 2 : left - left / 8;
-            const bool last = B.n_pieces + 1 == kDecMaxPieces || total < kDecOneRound * turn || (left - part) * total < 2 * turn * 65536;
-            done = last ? 65536 : done + part;
-            B.piece_end[B.n_pieces++] = (uint32_t)done;
-        }
+        B.n_pieces = dec_pieces(total, (uint64_t)grid * shape.warps, any_base, B.piece_end);
         if (B.n_pieces > 1 && cudaMemsetAsync((uint8_t*)d_workspace + kDecClaims, 0, 4 * (kDecMaxPieces - 1) * kDecClaimWords, st) != cudaSuccess) return ZC_E_CUDA;
         DecRanges R{nullptr, 0, nullptr, 0, d_workspace, sizeof(Control)};
 #if ZC_DEBUG_CHECKS

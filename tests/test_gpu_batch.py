@@ -608,6 +608,35 @@ def test_batched_decoder_deals_chunks_out_in_several_rounds(kind, chunks):
         assert torch.equal(b[:n], x[:n])
 
 
+@pytest.mark.parametrize("unchanged", ["first_half", "every_other", "last_quarter"])
+def test_batched_decoder_with_slices_of_unlike_speed(unchanged):
+    """Deltas whose unchanged stretches are as long as many blocks' slices: blocks that are through take the other slices' pieces,
+    of which there are seven."""
+    chunks, cs = 400_000, 512
+    assert len(zc.test_decoder_pieces(zc.plan(zc.FMT_BF16, cs, 1024), True, chunks)) == 7
+    parts = {"first_half": [(300_000, True), (100_000 - 3, False)], "every_other": [(50_000, k % 2 == 0) for k in range(8)],
+             "last_quarter": [(299_999, False), (100_001, True)]}[unchanged]
+    sizes = [n * cs - 7 * k for k, (n, _) in enumerate(parts)]
+    tile = torch.from_numpy(_weights(zc.FMT_BF16, 8 << 20, 5)).to(DEV)
+    d_ins = [tile.repeat(-(-2 * n // tile.numel()))[: 2 * n].clone() for n in sizes]
+    g = torch.Generator(device=DEV); g.manual_seed(2)
+    d_bases = []
+    for k, (x, (_, same)) in enumerate(zip(d_ins, parts)):
+        step = (torch.rand(x.numel(), generator=g, device=DEV) < 0.3).to(torch.uint8) * 3
+        if same:
+            step[: x.numel() * 2 // 3 if unchanged == "first_half" else x.numel()] = 0
+        d_bases.append(x ^ step)
+    plans, d_outs, got = _encoded_batch(zc.FMT_BF16, 1024, d_ins, sizes, d_bases)
+    ws = torch.zeros(256, dtype=torch.uint8, device=DEV)
+    backs = [torch.zeros_like(x) for x in d_ins]
+    for _ in range(3):
+        zc.decompress_batch(zc.DecompressBatch(plans, d_outs, got, backs, d_bases), ws)
+        assert zc.batch_status(ws) == (zc.OK, None)
+        for b, x in zip(backs, d_ins):
+            assert torch.equal(b, x)
+            b.zero_()
+
+
 @pytest.mark.parametrize("chunk_bytes", [4096, 32768])
 @pytest.mark.parametrize("count", [2, 20, 64, 147, 149])
 def test_batched_decoder_with_tensors_of_one_size_and_of_several(count, chunk_bytes):

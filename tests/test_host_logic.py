@@ -322,6 +322,28 @@ def test_validate_accepts_oracle_containers_and_rejects_damage(fmt, policy, cbyt
         assert zc.validate_container(p, bad) == zc.E_CORRUPT
 
 
+@pytest.mark.parametrize("any_base", [False, True])
+def test_pieces_of_a_slice(any_base):
+    """The pieces add up to the slice and shrink; one below 64 chunks per warp.  With a base, where slices differ in speed, nothing
+    larger than an eighth of a slice is left for others."""
+    p = zc.plan(zc.FMT_BF16, 1 << 20, 4096)
+    turn = 148 * zc.test_decoder_warps(p, any_base)
+    assert zc.test_decoder_pieces(p, any_base, 0) == []
+    seen = set()
+    for turns in [0.001, 1, 63.9, 64, 65, 100, 127, 128, 200, 500, 1024, 5000, 9000, 60000]:
+        end = zc.test_decoder_pieces(p, any_base, max(1, int(turns * turn + 0.5)))
+        seen.add(len(end))
+        length = [b - a for a, b in zip([0] + end, end)]
+        assert 1 <= len(end) <= 7 and end[-1] == 65536 and all(n > 0 for n in length)
+        assert (len(end) == 1) == (turns < 64)
+        assert length == sorted(length, reverse=True)
+        if len(end) > 1:
+            assert length[0] == (32768 if any_base else 57344)
+            assert max(length[1:]) <= 8192
+            assert min(length) * turns >= 2 * 65536 * 0.99       # two chunks per warp and more
+    assert seen == ({1, 7} if any_base else {1, 2, 3, 4, 5})      # plain: one more for every factor of 8; 60000 < 2 * 8 ** 5
+
+
 WRAPPED_SIZES = {
     # total_bytes and payload_bytes whose sum with payload_off and the guard comes out right modulo 2^64
     "payload_of_minus_16": lambda off: (off, 2 ** 64 - 16),
