@@ -35,7 +35,7 @@ zc_status zc_test_merge16(zc_format fmt, const uint8_t* h_e8, const uint8_t* h_s
 uint32_t zc_test_encoder_workers(const zc_plan_t* plan, uint32_t n_coded, uint32_t any_base, uint64_t total_chunks);
 uint32_t zc_test_decoder_warps(const zc_plan_t* plan, uint32_t both_coded);
 /* Number of pieces into which the batched decoder cuts a block's slice of a launch of total_chunks chunks with one block per SM
- * (host arithmetic only; 148 SMs without a GPU); h_piece_end (7 entries) receives where they end, in 65536ths of the slice.  0 =
+ * (host arithmetic only; 148 SMs without a GPU); h_piece_end (5 entries) receives where they end, in 65536ths of the slice.  0 =
  * no plan, no chunks or a plan that the kernels cannot take. */
 uint32_t zc_test_decoder_pieces(const zc_plan_t* plan, uint32_t any_base, uint64_t total_chunks, uint32_t* h_piece_end);
 void zc_test_set_wait_limit(uint32_t polls);

@@ -559,5 +559,5 @@ def test_decoder_warps(p: Plan, both_coded: bool) -> int:
 
 def test_decoder_pieces(p: Plan, any_base: bool, total_chunks: int):
     """zc_test_decoder_pieces: where the pieces of a slice end, in 65536ths of it."""
-    end = (C.c_uint32 * 7)()
+    end = (C.c_uint32 * 5)()
     return [int(end[i]) for i in range(_lib.zc_test_decoder_pieces(p._h, int(any_base), total_chunks, end))]

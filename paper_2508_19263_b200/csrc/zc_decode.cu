@@ -48,7 +48,7 @@ struct DecItem {
 // the block's last warp, header, tables, first pieces).  (Dealt out in rounds over the whole index space by a ticket counter, every
 // piece of a block was of another tensor: 1.74 GB of BF16 weights 621 us, now 612; their delta of 872 MB 550 and 524; 18 tensors of
 // 66 MB in all 58 and 53.  In one piece each, the delta takes 659 us.)
-constexpr uint32_t kDecMaxPieces = 7, kDecOneRound = 64;
+constexpr uint32_t kDecMaxPieces = 5, kDecOneRound = 64;
 constexpr uint32_t kDecMaxBlocks = 160, kDecClaimWords = kDecMaxBlocks / 32;
 constexpr size_t kDecClaims = 128;           // where the bits are in the control block: [piece - 1][kDecClaimWords]
 static_assert(sizeof(Control) <= kDecClaims && kDecClaims + 4 * (kDecMaxPieces - 1) * kDecClaimWords <= kControlBytes, "control block");
@@ -1902,20 +1902,20 @@ DecShape split_shape(const zc_plan_t* p, uint32_t n_chunks, uint32_t* groups)
 }
 
 // Pieces of a slice of a batched launch (see kDecMaxPieces), as where they end in 65536ths of it; turn = one chunk for every warp.
-// Seven eighths of what is left, until one is down to two chunks per warp; the last one is the rest.  Deltas: half of the slice, then
-// an eighth of it or half of what is left, whichever is less, since slices differ in speed (unchanged stretches take half of the
-// time and less) and the piece that is taken last from a slow one is what the launch ends with.  (15 GB of deltas, most layers
-// unchanged: 6.77 ms; 7.59 ms with a half, a quarter and so on in five pieces, which left a quarter of a slow slice to the block that
-// came first.  872 MB with a quarter, half, three quarters unchanged 608, 514, 439 us against 606, 517, 485; all changed 665 against
-// 655: about 5 us for every piece more.)  With fewer than kDecOneRound chunks per warp in all, another piece costs more than it evens out
-// (FP8 at 16 KiB chunks, 9 chunks per warp: 219 us in one round, 270 us in three; BF16 at 1 KiB chunks, 44 per warp: 119 us in one
-// round, 140 in four).
+// Seven eighths of what is left, until one is down to two chunks per warp; the last one is the rest.  Deltas: five eighths of the slice,
+// then an eighth of it or half of what is left, whichever is less, since slices differ in speed (unchanged stretches take half of
+// the time and less) and the piece that is taken last from a slow one is what the launch ends with.  (15 GB of deltas, most layers
+// unchanged: 6.89 ms; 7.59 ms with a half, a quarter and so on, which left a quarter of a slow slice to the block that came first.  872
+// MB with none, a quarter, half, three quarters unchanged: 657, 609, 523, 457 us against 658, 623, 520, 485.  Two more pieces: 6.75 ms,
+// but 668, 611, 532, 457 us: another piece costs about 5 us.)  With fewer than kDecOneRound chunks per warp in all, another piece costs
+// more than it evens out (FP8 at 16 KiB chunks, 9 chunks per warp: 219 us in one round, 270 us in three; BF16 at 1 KiB chunks, 44
+// per warp: 119 us in one round, 140 in four).
 uint32_t dec_pieces(uint64_t total, uint64_t turn, bool any_base, uint32_t* piece_end)
 {
     uint32_t n = 0;
     for (uint64_t done = 0; done < 65536;) {
         const uint64_t left = 65536 - done;
-        const uint64_t part = !any_base ? left - left / 8 : done ? std::min<uint64_t>(left / 2, 65536 / 8) : left / 2;
+        const uint64_t part = !any_base ? left - left / 8 : done ? std::min<uint64_t>(left / 2, 65536 / 8) : left / 8 * 5;
         const bool last = n + 1 == kDecMaxPieces || total < kDecOneRound * turn || (left - part) * total < 2 * turn * 65536;
         done = last ? 65536 : done + part;
         piece_end[n++] = (uint32_t)done;

@@ -334,14 +334,14 @@ def test_pieces_of_a_slice(any_base):
         end = zc.test_decoder_pieces(p, any_base, max(1, int(turns * turn + 0.5)))
         seen.add(len(end))
         length = [b - a for a, b in zip([0] + end, end)]
-        assert 1 <= len(end) <= 7 and end[-1] == 65536 and all(n > 0 for n in length)
+        assert 1 <= len(end) <= 5 and end[-1] == 65536 and all(n > 0 for n in length)
         assert (len(end) == 1) == (turns < 64)
         assert length == sorted(length, reverse=True)
         if len(end) > 1:
-            assert length[0] == (32768 if any_base else 57344)
+            assert length[0] == (40960 if any_base else 57344)
             assert max(length[1:]) <= 8192
             assert min(length) * turns >= 2 * 65536 * 0.99       # two chunks per warp and more
-    assert seen == ({1, 7} if any_base else {1, 2, 3, 4, 5})      # plain: one more for every factor of 8; 60000 < 2 * 8 ** 5
+    assert seen == ({1, 5} if any_base else {1, 2, 3, 4, 5})      # plain: one more for every factor of 8; 60000 < 2 * 8 ** 5
 
 
 WRAPPED_SIZES = {
