@@ -843,6 +843,93 @@ struct DecView {
     uint32_t n_full;                 // complete chunks (every lane has a whole subchunk)
 };
 
+// Merges 16 symbols of either stream (off: where their 32 element bytes are in the tensor, room: those the chunk has from there on).
+template <int FMT, bool XOR, bool FULL>
+__device__ __forceinline__ void merge_part(const volatile DecView& V, uint8_t* const dst, const uint4 ev, const uint4 mv, const uint64_t off,
+                                           const uint32_t room, const bool out32)
+{
+    uint32_t e[4], m[4], o[8];
+    e[0] = ev.x; e[1] = ev.y; e[2] = ev.z; e[3] = ev.w;
+    m[0] = mv.x; m[1] = mv.y; m[2] = mv.z; m[3] = mv.w;
+    merge16<FMT>(e, m, o);
+    merge16<FMT>(e + 2, m + 2, o + 4);
+    if (XOR && V.base) {                                         // delta form: XOR the base tensor back in
+        const uint8_t* const base = V.base;
+        const uint4 b0 = FULL ? ld_nc_v4(base + off) : load16_guarded(base, off, V.input_bytes);
+        const uint4 b1 = FULL ? ld_nc_v4(base + off + 16) : load16_guarded(base, off + 16, V.input_bytes);
+        o[0] ^= b0.x; o[1] ^= b0.y; o[2] ^= b0.z; o[3] ^= b0.w;
+        o[4] ^= b1.x; o[5] ^= b1.y; o[6] ^= b1.z; o[7] ^= b1.w;
+    }
+    if (FULL || room >= 32) {
+        if (out32) {
+            st_cs_v8(dst, o);
+        } else {                                                 // an output that is aligned to 16 bytes only
+            st_cs_v4(dst, make_uint4(o[0], o[1], o[2], o[3]));
+            st_cs_v4(dst + 16, make_uint4(o[4], o[5], o[6], o[7]));
+        }
+    } else {
+#pragma unroll
+        for (int t = 0; t < 32; ++t)
+            if ((uint32_t)t < room) dst[t] = (uint8_t)(o[t >> 2] >> (8 * (t & 3)));
+    }
+}
+
+// The bytes of chunk cc of the base tensor travel to the L2.  One lane calls it.
+__device__ __forceinline__ void prefetch_base_chunk(const volatile DecView& V, const uint32_t cc, const uint32_t chunk_bytes)
+{
+    const uint8_t* const base = V.base;
+    const uint32_t n = cc < V.n_full ? chunk_bytes : (uint32_t)min((unsigned long long)chunk_bytes, V.input_bytes - (uint64_t)cc * chunk_bytes) & ~15u;
+    if (base && n) asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" :: "l"(base + (uint64_t)cc * chunk_bytes), "r"(n) : "memory");
+}
+
+// Neither stream coded (chunks of up to 4 KiB): nothing is decoded, the symbols are merged in address order (a complete chunk
+// is a multiple of the warp's 512 symbols) and the next chunk's bytes travel to the L2 a chunk ahead.  Bound by memory.  (Dealt to the
+// lanes by subchunks and without the prefetch, these containers lived on the L1, of which the pools of this kernel leave 28 KB:
+// at 1, 2, 3, 4 KiB 872 MB of BF16 took 330, 294, 417, 320 us, now 303, 290, 299, 318; as a delta 453, 411, 676, 559 us, now 417, 407,
+// 418, 451; 3.75 GB of FP4 elements 1.53 ms, now 1.44.  By bulk copies into the pools BF16 takes 305 us at 4 KiB, but FP4 4 % more
+// at 2 and 4 KiB.)
+template <int FMT, bool XOR>
+__device__ __forceinline__ uint32_t run_plain(const DecParams& P, const volatile DecView& V, uint32_t c, const uint32_t c_end, const uint32_t step)
+{
+    const uint32_t lane = threadIdx.x & 31, cs = P.cs, chunk_bytes = P.chunk_bytes;
+    const uint8_t* const sec0 = V.sec[0];
+    const uint8_t* const sec1 = V.sec[1];
+    uint8_t* const out = V.out;
+    const uint64_t n_syms = V.n_syms, input_bytes = V.input_bytes;
+    const uint32_t n_full = V.n_full;
+    const bool out32 = ((uintptr_t)out & 16) == 0;
+    for (; c < c_end; c += step) {
+        const uint32_t next = c + step;
+        if (next < c_end) {
+            const uint64_t lo = (uint64_t)next * cs;             // (a raw section is padded to 16 bytes)
+            const uint32_t n = next < n_full ? cs : ((uint32_t)min((uint64_t)cs, n_syms - lo) + 15u) & ~15u;
+            if (lane < 2) asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" :: "l"((lane ? sec1 : sec0) + lo), "r"(n) : "memory");
+            if (XOR && lane == 2) prefetch_base_chunk(V, next, chunk_bytes);
+        }
+        auto body = [&](auto full_tag) {
+            constexpr bool FULL = decltype(full_tag)::value;
+            const uint64_t lo = (uint64_t)c * cs + 16 * lane;    // my first part's symbols
+            const uint32_t syms = FULL ? cs : (uint32_t)min((uint64_t)cs, n_syms - (uint64_t)c * cs);
+            const uint32_t bytes = FULL ? chunk_bytes : (uint32_t)min((uint64_t)chunk_bytes, input_bytes - (uint64_t)c * chunk_bytes);
+            const uint8_t* const e_at = sec0 + lo;
+            const uint8_t* const m_at = sec1 + lo;
+            uint8_t* const dst = out + 2 * lo;                 // two element bytes per symbol in every format
+#pragma unroll 1
+            for (uint32_t at = FULL ? 0u : 16 * lane; at < syms; at += 1024) {   // two parts at a time, 512 symbols apart
+                const bool two = at + 512 < syms;
+                const uint32_t k = at - (FULL ? 0u : 16 * lane);
+                uint4 e1{}, m1{};
+                const uint4 e0 = ld_nc_v4(e_at + k), m0 = ld_nc_v4(m_at + k);
+                if (two) { e1 = ld_nc_v4(e_at + k + 512); m1 = ld_nc_v4(m_at + k + 512); }
+                merge_part<FMT, XOR, FULL>(V, dst + 2 * k, e0, m0, 2 * (lo + k), bytes - (32 * lane + 2 * k), out32);
+                if (two) merge_part<FMT, XOR, FULL>(V, dst + 2 * k + 1024, e1, m1, 2 * (lo + k) + 1024, bytes - (32 * lane + 2 * k + 1024), out32);
+            }
+        };
+        if (c < n_full) body(BoolTag<true>{}); else body(BoolTag<false>{});
+    }
+    return ZC_OK;
+}
+
 // Chunks of up to 4 KiB are decoded as run_chunks does it, but everything a chunk needs comes by bulk copies: its pieces,
 // staged whole, and the bytes of a raw stream, so that the merge reads both streams from shared memory.  Both are requested as
 // soon as the chunk before has been decoded; the raw bytes of 4 KiB chunks, for which the block's memory has one buffer per
@@ -860,6 +947,7 @@ __device__ __forceinline__ uint32_t run_small(const DecParams& P, const volatile
     constexpr uint32_t kLog = PPL == 4 ? 2 : PPL == 2 ? 1 : 0;
     constexpr uint32_t kRowsBytes = 512 * PPL;
     constexpr uint32_t kHuff = (H0 ? 1u : 0u) + (H1 ? 1u : 0u);
+    static_assert(kHuff != 0, "containers without a coded stream: run_plain");
     constexpr bool kCopyRaw = kHuff == 1;                        // one coded stream, one raw
     constexpr int kRaw = H0 ? 1 : 0;                             // the raw one, and its mbarrier
     constexpr uint32_t kRawBufs = small_raw_buffers(PPL);
@@ -875,7 +963,7 @@ __device__ __forceinline__ uint32_t run_small(const DecParams& P, const volatile
     // pool: symbols of stream 0 (if coded), of stream 1 (if coded), raw bytes of a chunk, one staging slot per coded stream
     constexpr uint32_t rows1_off = H0 ? kRowsBytes : 0, raw_off = kHuff * kRowsBytes;
     const uint32_t slots_off = raw_off + (kCopyRaw ? kRawBufs * cs : 0u);
-    const uint32_t slot_bytes = kHuff ? ((pool_bytes - slots_off) / (kHuff ? kHuff : 1)) & ~15u : 0u;
+    const uint32_t slot_bytes = ((pool_bytes - slots_off) / kHuff) & ~15u;
     const uint32_t rows0_s = smem_u32(pool), rows1_s = rows0_s + rows1_off;
     uint32_t raw_s = rows0_s + raw_off;                          // of the chunk that is merged next
     const uint32_t slot0_s = rows0_s + slots_off, slot1_s = slot0_s + (H0 ? slot_bytes : 0u);
@@ -916,6 +1004,8 @@ __device__ __forceinline__ uint32_t run_small(const DecParams& P, const volatile
     };
     // Takes the table entries in nx_* (of chunk cc), checks them, starts the copies, and requests the entries of the chunk
     // after it.  A copy takes 16 bytes more than the piece (the next piece or the guard), for the windows' look-ahead.
+    // (As prefetch_base_chunk has it; but with a call of that the compiler spills in the loop of two coded streams: 15 GB of deltas 10.1 ->
+    // 10.7 ms.)
     auto prefetch_base = [&](const uint32_t cc) {                // the base tensor's bytes travel to the L2
         const uint8_t* const base = V.base;
         const uint32_t n = cc < V.n_full ? chunk_bytes : (uint32_t)min((unsigned long long)chunk_bytes, V.input_bytes - (uint64_t)cc * chunk_bytes) & ~15u;
@@ -927,7 +1017,7 @@ __device__ __forceinline__ uint32_t run_small(const DecParams& P, const volatile
         if (H0) { end0 = nx_end0; off0 = nx_off0; ok = check(end0, off0, start0, piece0); }
         if (H1) { end1 = nx_end1; off1 = nx_off1; ok = check(end1, off1, start1, piece1) && ok; }
         staged0 = staged1 = false;
-        if (kHuff && !__all_sync(0xFFFFFFFFu, ok)) { err = ZC_E_CORRUPT; return; }
+        if (!__all_sync(0xFFFFFFFFu, ok)) { err = ZC_E_CORRUPT; return; }
         if (H0 && piece0 + 16 <= slot_bytes) {
             staged0 = flying0 = true;
             if (lane == 0 && !P.skip_copy) copy(slot0_s, V.payload + 16ull * off0, piece0 + 16, &bar[0]);
@@ -1008,7 +1098,7 @@ __device__ __forceinline__ uint32_t run_small(const DecParams& P, const volatile
             const uint32_t last_r = FULL ? n_rounds - 1 : (min(c_syms, sub) - 1) / R;         // lane 0 has the most symbols
             LaneBits L0{}, L1{};                                 // (.pos also where the piece is read from global memory)
             for (uint32_t r = 0; r <= last_r; ++r) {
-                if (kHuff && r == 0) {
+                if (r == 0) {
                     if (!pieces_here(H0 && staged0, H1 && staged1, bar, parity0, parity1, P.spin_limit)) { err = ZC_E_DEVICE_TIMEOUT; return; }
                     if (H0) flying0 = false;
                     if (H1) flying1 = false;
@@ -1078,11 +1168,11 @@ __device__ __forceinline__ uint32_t run_small(const DecParams& P, const volatile
                     if ((!FULL && k >= c_syms)) continue;
                     uint32_t e[4], m[4];
                     {
-                        const uint4 v = H0 ? lds128(rows0_s + rd_off + 512 * i) : kCopyRaw ? lds128(raw_s + k) : ld_nc_v4(V.sec[0] + c_lo + k);
+                        const uint4 v = H0 ? lds128(rows0_s + rd_off + 512 * i) : lds128(raw_s + k);
                         e[0] = v.x; e[1] = v.y; e[2] = v.z; e[3] = v.w;
                     }
                     {
-                        const uint4 v = H1 ? lds128(rows1_s + rd_off + 512 * i) : kCopyRaw ? lds128(raw_s + k) : ld_nc_v4(V.sec[1] + c_lo + k);
+                        const uint4 v = H1 ? lds128(rows1_s + rd_off + 512 * i) : lds128(raw_s + k);
                         m[0] = v.x; m[1] = v.y; m[2] = v.z; m[3] = v.w;
                     }
                     uint32_t o[8];
@@ -1110,7 +1200,7 @@ __device__ __forceinline__ uint32_t run_small(const DecParams& P, const volatile
                             if (2 * k + t < out_bytes) dst[t] = (uint8_t)(o[t >> 2] >> (8 * (t & 3)));
                     }
                 }
-                if (kHuff) __syncwarp();
+                __syncwarp();
             }
             if (kCopyRaw && kRawBufs == 1 && !err && c + step < c_end) copy_raw(raw_s, c + step);   // everybody has read this chunk's
             if (kCopyRaw && kRawBufs == 2) raw_s = other_raw();
@@ -1322,7 +1412,7 @@ __device__ __forceinline__ uint32_t decode_one(const DecParams& P, const DecSmem
         __syncthreads();
         const volatile DecView& V = s_view;
         if (huff0 && !huff1) return run_small<FMT, PPL, true, false, XOR, SIDE>(P, V, S.pairs0, 0, pool, pool_bytes, M.bar, first_end0, first_off0, c0, c_end, step, parity0, parity1);
-        if (!huff0 && !huff1) return run_small<FMT, PPL, false, false, XOR, SIDE>(P, V, 0, 0, pool, pool_bytes, M.bar, 0, 0, c0, c_end, step, parity0, parity1);
+        if (!huff0 && !huff1) return run_plain<FMT, XOR>(P, V, c0, c_end, step);
         if (huff0) return run_small<FMT, PPL, true, true, XOR, SIDE>(P, V, S.pairs0, S.pairs1, pool, pool_bytes, M.bar, first_end0, first_off0, c0, c_end, step, parity0, parity1);
         return run_small<FMT, PPL, false, true, XOR, SIDE>(P, V, 0, S.pairs1, pool, pool_bytes, M.bar, 0, 0, c0, c_end, step, parity0, parity1);
     } else {

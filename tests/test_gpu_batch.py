@@ -573,14 +573,14 @@ def test_batches_from_one_chunk_to_several_rounds(fmt, chunk_bytes, chunks):
         assert np.array_equal(back[: p.input_bytes], data[: p.input_bytes]) and (back[p.input_bytes:] == 0xEE).all()
 
 
-def _encoded_batch(fmt, chunk_bytes, d_ins, sizes, d_bases=None):
+def _encoded_batch(fmt, chunk_bytes, d_ins, sizes, d_bases=None, policy=None):
     """Containers of tensors on the device, by the library's own encoder (compared with the oracle's elsewhere)."""
     plans = [zc.plan(fmt, n, chunk_bytes) for n in sizes]
     d_hists = torch.zeros((len(plans), 2, 256), dtype=torch.int64, device=DEV)
     zc.histogram_batch(zc.HistogramBatch(plans, d_ins, d_bases), d_hists)
     d_outs = [torch.empty(p.max_compressed_bytes, dtype=torch.uint8, device=DEV) for p in plans]
     enc = zc.CompressBatch(plans, d_ins, d_outs, d_bases)
-    enc.set_codebooks(zc.build_codebooks(plans, d_hists.cpu().numpy(), zc.POLICY_HUFF_ALL if d_bases else zc.POLICY_AUTO))
+    enc.set_codebooks(zc.build_codebooks(plans, d_hists.cpu().numpy(), policy or (zc.POLICY_HUFF_ALL if d_bases else zc.POLICY_AUTO)))
     return plans, d_outs, zc.compress_batch(enc, torch.empty(enc.workspace_bytes, dtype=torch.uint8, device=DEV))
 
 
@@ -685,3 +685,38 @@ def test_decoder_of_small_chunks_with_one_and_two_coded_streams(fmt, chunk_bytes
         zc.decompress(p, out, nbytes, back, ws)
         assert zc.device_status(p, ws) == zc.OK
     check()
+
+
+@pytest.mark.parametrize("fmt", FORMATS)
+@pytest.mark.parametrize("chunk_bytes", [1024, 2048, 3072, 4096, 5120])
+def test_decoder_of_small_chunks_without_coded_streams(fmt, chunk_bytes):
+    """Containers with both streams raw have a loop of their own up to 4 KiB: several chunks per warp, the last one ragged at every kind of
+    place, outputs aligned to 32 and to 16 bytes, batched and alone, plain and (BF16) as a delta."""
+    G = zo.group(fmt)
+    cs = chunk_bytes // 2 * G
+    sizes = [13000 * cs, 9000 * cs - 2, 5000 * cs + 16 * G, 300 * cs + cs // 2 + 8 * G, cs - 2, 2 * cs + 2, 2, 0]
+    nbytes = [zo.input_bytes(fmt, n) for n in sizes]
+    g = torch.Generator(device=DEV); g.manual_seed(chunk_bytes + fmt)
+    d_ins = [torch.randint(0, 256, (max(b, 16),), dtype=torch.uint8, device=DEV, generator=g) for b in nbytes]
+    for delta in (False, True)[: 2 if fmt == zc.FMT_BF16 else 1]:
+        d_bases = [torch.randint(0, 256, (x.numel(),), dtype=torch.uint8, device=DEV, generator=g) for x in d_ins] if delta else None
+        plans, d_outs, got = _encoded_batch(fmt, chunk_bytes, d_ins, sizes, d_bases, zc.POLICY_RAW_ALL)
+        for shift in (0, 16):
+            bufs = [torch.full((b + 64,), 0xEE, dtype=torch.uint8, device=DEV) for b in nbytes]
+            assert all(b.data_ptr() % 32 == 0 for b in bufs)
+            backs = [b[shift:] for b in bufs]
+            ws = torch.zeros(256, dtype=torch.uint8, device=DEV)
+
+            def check():
+                for n, x, b in zip(nbytes, d_ins, bufs):
+                    assert torch.equal(b[shift: shift + n], x[:n]) and bool((b[:shift] == 0xEE).all()) and bool((b[shift + n:] == 0xEE).all())
+                    b.fill_(0xEE)
+
+            zc.decompress_batch(zc.DecompressBatch(plans, d_outs, got, backs, d_bases), ws)
+            assert zc.batch_status(ws) == (zc.OK, None)
+            check()
+            if not delta:
+                for p, out, n, back in zip(plans, d_outs, got, backs):
+                    zc.decompress(p, out, n, back, ws)
+                    assert zc.device_status(p, ws) == zc.OK
+                check()
