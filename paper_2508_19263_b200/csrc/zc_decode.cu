@@ -4,8 +4,9 @@
 // with a bulk asynchronous copy (TMA, non-multicast) completing on an mbarrier.  Work proceeds in
 // rounds: every lane decodes R symbols of its own subchunk into a padded row of shared memory, then the
 // whole warp merges 32 x R symbols with the other stream and writes 16-byte vectors, fully coalesced.
-// Raw sign+mantissa bytes of a round (and, for deltas, the base tensor's bytes) are prefetched into the L2 before the
-// round's decoding, so the DRAM latency hides behind the table lookups.
+// The bytes of a raw stream come by bulk copies too in chunks of up to 4 KiB (run_small); in larger ones those of a round are
+// prefetched into the L2 before it is decoded, as a delta's base tensor is, so that the DRAM latency hides behind the table lookups.
+// Small chunks without a coded stream are only merged (run_plain).
 #include "zc_device.cuh"
 
 #include <atomic>
@@ -32,7 +33,7 @@ struct DecParams {
 };
 
 // One tensor of a batch, and the parameters of a batched launch.  The tensors share format and chunk size;
-// the chunks of all of them form one index space that is cut into contiguous ranges (see kDecMaxPieces).
+// the chunks of all of them form one index space that is cut into contiguous slices (see kDecMaxPieces).
 struct DecItem {
     const uint8_t* comp;
     const uint8_t* base;
@@ -46,8 +47,8 @@ struct DecItem {
 // get through a piece.  Who takes a piece sets its bit in the control block (nobody else takes a slice's first piece).  The next
 // piece of one's own slice is nearly always of the same tensor, whose tables are kept; another one costs about 12 us (waiting for
 // the block's last warp, header, tables, first pieces).  (Dealt out in rounds over the whole index space by a ticket counter, every
-// piece of a block was of another tensor: 1.74 GB of BF16 weights 621 us, now 612; their delta of 872 MB 550 and 524; 18 tensors of
-// 66 MB in all 58 and 53.  In one piece each, the delta takes 659 us.)
+// piece of a block was of another tensor; the step from that to slices, with the chunk loops as they were then: 1.74 GB of BF16 weights
+// 621 -> 612 us, their delta of 872 MB 550 -> 524, 18 tensors of 66 MB in all 58 -> 53.  In one piece each, the delta took 659 us.)
 constexpr uint32_t kDecMaxPieces = 5, kDecOneRound = 64;
 constexpr uint32_t kDecMaxBlocks = 160, kDecClaimWords = kDecMaxBlocks / 32;
 constexpr size_t kDecClaims = 128;           // where the bits are in the control block: [piece - 1][kDecClaimWords]
@@ -88,15 +89,6 @@ __device__ __forceinline__ uint32_t* block_luts()
 constexpr uint32_t kSliceSyms = 128;               // symbols a lane decodes from one slice of its subchunk
 constexpr uint32_t kSliceBytes = 256;              // copied per slice: 15 bytes of alignment + 128 * 12 bits + the window's look-ahead fit
 constexpr uint32_t kSliceSlot = 272;               // a lane's slot
-
-__device__ __forceinline__ uint32_t lds32_if(bool p, uint32_t addr)
-{
-    if (p) ZC_DBG_SHARED(addr, 4, return 0);
-    uint32_t v;
-    asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %2, 0;\n\tmov.u32 %0, 0;\n\t@q ld.shared.u32 %0, [%1];\n\t}"
-                 : "=r"(v) : "r"(addr), "r"((uint32_t)p));
-    return v;
-}
 
 __device__ __forceinline__ void sts128(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d)
 {
@@ -273,11 +265,10 @@ __device__ __forceinline__ uint32_t load_sub_end(const uint8_t* tab, uint32_t wi
     return reinterpret_cast<const uint32_t*>(tab + 128ull * chunk)[lane];
 }
 
-// A lane's place in its chunk's piece is one number, the bit position `pos`.  Piece staged in shared memory: pos
-// counts from shared address 0 (8 * byte address of the slot + bit in the piece), so a window costs a shift, a mask,
-// two loads and a funnel shift, and nothing else has to be kept between lookups (no pointer, no count of valid
-// bits, no second buffer word).  Piece read from global memory: pos counts from the start of the piece and the
-// word index is clamped to `lim`, the last place from which two words can be read.
+// A lane's place in its chunk's piece is the bit position `pos`.  Piece staged in shared memory: pos counts from shared
+// address 0 (8 * byte address of the slot + bit in the piece), and the words around it are kept in registers (LaneBits), so a
+// window is one funnel shift.  Piece read from global memory: pos counts from the start of the piece, a window loads its two
+// words, and the word index is clamped to `lim`, the last place from which two words can be read.
 // Bounds of the staged form: a lane starts inside its piece (checked against the tables before the chunk is
 // decoded) and consumes at most 12 bits per symbol, so it reads less than 1.5 * sub + 16 bytes past the piece
 // whatever the payload bits are; the block's shared memory ends with that much slack behind the last warp's

@@ -633,8 +633,8 @@ encode_kernel(const __grid_constant__ EncParams P)
     } else {
         // =========================== a worker warp ===========================
         // Bounded wait of the whole warp for a phase of an mbarrier; false on the failure flag or when the wait gives up.
-        // (A try_wait sleeps in hardware until the phase completes or a time limit is reached.  With a hint of 2 us for that limit
-        // the compiler makes a loop of short sleeps of it: 872 MB of BF16 weights at 16 KiB 425 -> 419 us without.)
+        // (A try_wait sleeps in hardware until the phase completes or a time limit is reached.  With a hint of 2 us for that limit 872
+        // MB of BF16 weights at 16 KiB take 425 us, without 419.)
         auto wait_phase = [&](uint64_t* bar, const uint32_t parity) -> bool {
             bool ok = mbar_try_wait(bar, parity);
             for (uint32_t k = 0; !ok && k < P.spin_limit; ++k) {

@@ -584,11 +584,14 @@ def _encoded_batch(fmt, chunk_bytes, d_ins, sizes, d_bases=None, policy=None):
     return plans, d_outs, zc.compress_batch(enc, torch.empty(enc.workspace_bytes, dtype=torch.uint8, device=DEV))
 
 
-@pytest.mark.parametrize("kind,chunks", [("plain", 300_000), ("plain", 750_000), ("scale", 200_000), ("delta", 200_000)])
-def test_batched_decoder_deals_chunks_out_in_several_rounds(kind, chunks):
-    """64 chunks per warp and more are dealt out in shrinking rounds, up to five (with 148 SMs: plain 4 and 5, scale 4, delta
-    5): a large tensor, an empty one, a ragged one, one without a base."""
+@pytest.mark.parametrize("kind,chunks,pieces", [("plain", 300_000, 2), ("plain", 750_000, 3), ("plain", 4_400_000, 4), ("scale", 200_000, 2),
+                                                ("delta", 200_000, 5)])
+def test_batched_decoder_deals_chunks_out_in_several_rounds(kind, chunks, pieces):
+    """A block's slice of 64 chunks per warp and more is cut into two to five pieces (numbers for 148 SMs; plain launches have a fifth
+    from 34 million chunks on): a large tensor, an empty one, a ragged one, one without a base."""
     fmt = zc.FMT_SCALE_U8 if kind == "scale" else zc.FMT_BF16
+    if torch.cuda.get_device_properties(0).multi_processor_count == 148:
+        assert len(zc.test_decoder_pieces(zc.plan(fmt, 1 << 20, 1024), kind == "delta", chunks)) == pieces
     cs = 512 * zo.group(fmt)
     sizes = [(chunks * 5 // 8) * cs, 0, (chunks // 4) * cs - 77, (chunks // 8) * cs + 1]
     tile = torch.from_numpy(_weights(fmt, 8 << 20, chunks)).to(DEV)
