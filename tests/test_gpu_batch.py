@@ -584,14 +584,11 @@ def _encoded_batch(fmt, chunk_bytes, d_ins, sizes, d_bases=None, policy=None):
     return plans, d_outs, zc.compress_batch(enc, torch.empty(enc.workspace_bytes, dtype=torch.uint8, device=DEV))
 
 
-@pytest.mark.parametrize("kind,chunks,pieces", [("plain", 300_000, 2), ("plain", 750_000, 3), ("plain", 4_400_000, 4), ("scale", 200_000, 2),
-                                                ("delta", 200_000, 5)])
-def test_batched_decoder_deals_chunks_out_in_several_rounds(kind, chunks, pieces):
-    """A block's slice of 64 chunks per warp and more is cut into two to five pieces (numbers for 148 SMs; plain launches have a fifth
-    from 34 million chunks on): a large tensor, an empty one, a ragged one, one without a base."""
+@pytest.mark.parametrize("kind,chunks", [("plain", 300_000), ("plain", 750_000), ("scale", 200_000), ("delta", 200_000)])
+def test_batched_decoder_deals_chunks_out_in_several_rounds(kind, chunks):
+    """Launches of 64 chunks per warp and more, a block's slice in two to five pieces: a large tensor, an empty one, a ragged one, one
+    without a base."""
     fmt = zc.FMT_SCALE_U8 if kind == "scale" else zc.FMT_BF16
-    if torch.cuda.get_device_properties(0).multi_processor_count == 148:
-        assert len(zc.test_decoder_pieces(zc.plan(fmt, 1 << 20, 1024), kind == "delta", chunks)) == pieces
     cs = 512 * zo.group(fmt)
     sizes = [(chunks * 5 // 8) * cs, 0, (chunks // 4) * cs - 77, (chunks // 8) * cs + 1]
     tile = torch.from_numpy(_weights(fmt, 8 << 20, chunks)).to(DEV)
@@ -609,6 +606,18 @@ def test_batched_decoder_deals_chunks_out_in_several_rounds(kind, chunks, pieces
     assert zc.batch_status(ws) == (zc.OK, None)
     for b, x, n in zip(backs, d_ins, nbytes):
         assert torch.equal(b[:n], x[:n])
+
+
+@pytest.mark.parametrize("kind,chunks,pieces", [("plain", 300_000, 2), ("plain", 750_000, 3), ("plain", 4_400_000, 4), ("scale", 200_000, 2),
+                                                ("delta", 200_000, 5)])
+def test_launches_in_several_rounds_have_two_to_five_pieces(kind, chunks, pieces):
+    """The launches of the test above, and one of four pieces (plain launches have a fifth from 34 million chunks on)."""
+    p = zc.plan(zc.FMT_SCALE_U8 if kind == "scale" else zc.FMT_BF16, 1 << 20, 1024)
+    if torch.cuda.get_device_properties(0).multi_processor_count != 148:
+        pytest.skip("the numbers are those of 148 SMs")
+    assert len(zc.test_decoder_pieces(p, kind == "delta", chunks)) == pieces
+    if pieces == 4:
+        test_batched_decoder_deals_chunks_out_in_several_rounds(kind, chunks)
 
 
 @pytest.mark.parametrize("unchanged", ["first_half", "every_other", "last_quarter"])
