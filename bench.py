@@ -41,7 +41,7 @@ ORACLE_SAMPLE_BYTES = int(os.environ.get("ZC_ORACLE_SAMPLE_BYTES", 768 << 20))  
 # stack of 872.4 MB, 4 KiB chunks, batched kernels); traffic grows in proportion to the input, so the figure for a
 # launch over the whole stack is this ratio times its input bytes.  The write part is undercounted in a capture
 # because some of the output is still in L2 when the kernel ends.
-NCU_DRAM_BYTES_PER_INPUT_BYTE = {"decode_kernel": (603383040.0 + 825236480.0) / 872415232.0,
+NCU_DRAM_BYTES_PER_INPUT_BYTE = {"decode_kernel": (594575360.0 + 824700672.0) / 872415232.0,
                                  "encode_kernel": (872557824.0 + 553053952.0) / 872415232.0}
 
 
